@@ -18,31 +18,18 @@
 
 struct orbg_code {
     int n, k, r, w32;
-    bool has_stride = false;     /* its tables hold strided pair runs (m-segment orders) */
     uint32_t max_cap;
     int device;
     std::vector<uint8_t> H;      /* r x n as used */
-    uint32_t *d_hcol = nullptr;
-    OrbgRun *d_runs = nullptr;
-    uint32_t *d_floor = nullptr;
-    OrbgRun *d_runs_cta = nullptr;
-    uint32_t *d_floor_cta = nullptr;
-    uint32_t *d_trip = nullptr;
-    uint32_t *d_reach = nullptr;
-    uint32_t *d_reach_cta = nullptr;
-    uint8_t *d_flat = nullptr;
-    uint8_t *d_s3 = nullptr;
-    uint32_t *d_x3off = nullptr;
+    unsigned char *d_mem = nullptr; /* every device array of the code */
     OrbgDeviceCode dev;
 };
 
 struct orbg_codeset {
     int ncodes, n_max, w32_max;
     OrbgVariants var;            /* decoder variants and the codes' sort buckets */
-    int has_stride = 0;          /* a code's tables hold strided pair runs */
     int32_t *d_bucket = nullptr; /* [ncodes] sort bucket of each code (var.d_bucket) */
-    uint32_t ntrip_max;
-    uint32_t x3w_max;
+    uint32_t npairs_max;
     orbg_tuning tuning;
     std::vector<int> n_of;       /* n of each code, host copy */
     OrbgDeviceCode code0;        /* host copy of code 0's descriptor */
@@ -230,28 +217,9 @@ struct Stager {
 
 void free_code_device(orbg_code *c)
 {
-    if (c->d_hcol) cudaFree(c->d_hcol);
-    if (c->d_runs) cudaFree(c->d_runs);
-    if (c->d_floor) cudaFree(c->d_floor);
-    if (c->d_runs_cta) cudaFree(c->d_runs_cta);
-    if (c->d_floor_cta) cudaFree(c->d_floor_cta);
-    if (c->d_trip) cudaFree(c->d_trip);
-    if (c->d_reach) cudaFree(c->d_reach);
-    if (c->d_reach_cta) cudaFree(c->d_reach_cta);
-    if (c->d_flat) cudaFree(c->d_flat);
-    if (c->d_s3) cudaFree(c->d_s3);
-    if (c->d_x3off) cudaFree(c->d_x3off);
-    c->d_s3 = nullptr;
-    c->d_x3off = nullptr;
-    c->d_runs_cta = nullptr;
-    c->d_floor_cta = nullptr;
-    c->d_trip = nullptr;
-    c->d_reach = nullptr;
-    c->d_reach_cta = nullptr;
-    c->d_flat = nullptr;
-    c->d_hcol = nullptr;
-    c->d_runs = nullptr;
-    c->d_floor = nullptr;
+    if (c->d_mem)
+        cudaFree(c->d_mem);
+    c->d_mem = nullptr;
 }
 
 }  // namespace
@@ -266,9 +234,7 @@ int orbg_codeset_view(const orbg_codeset *set, OrbgSetView *out)
     out->n_max = set->n_max;
     out->w32_max = set->w32_max;
     out->var = set->var;
-    out->has_stride = set->has_stride;
-    out->ntrip_max = set->ntrip_max;
-    out->x3w_max = set->x3w_max;
+    out->npairs_max = set->npairs_max;
     out->cap_min = set->cap_min;
     out->tuning = set->tuning;
     return 0;
@@ -327,7 +293,6 @@ namespace {
 /* The first `count` patterns of table `table` of tb (orbg_query_order). */
 int64_t expand_tables(const OrbgTables &tb, int n, uint32_t count, int table, int32_t *out)
 {
-    const std::vector<OrbgRun> &runs = table == 0 ? tb.runs : tb.runs_cta;
     const size_t stride = (size_t)n + 1;
     uint64_t total = std::min<uint64_t>(tb.patterns, count);
     if (table == 2) {
@@ -347,19 +312,12 @@ int64_t expand_tables(const OrbgTables &tb, int n, uint32_t count, int table, in
         return (int64_t)total;
     }
     std::memset(out, 0, sizeof(int32_t) * stride * (size_t)total);
-    std::vector<int> v(64);
-    for (const OrbgRun &r : runs) {
-        for (int j = 0; j < r.count; j++) {
-            uint64_t t = (uint64_t)r.tstart + (uint64_t)j;
-            if (t > total)
-                break;
-            int32_t *row = out + (t - 1) * stride;
-            const int w = orbg_run_pattern(r, j, tb.trip.data(), v.data());
-            row[0] = w;
-            for (int i = 0; i < w; i++)
-                row[1 + i] = v[i];
-        }
-    }
+    orbg_expand_tables(tb, n, total, [&](uint32_t t, const int *v, int w) {
+        int32_t *row = out + (size_t)(t - 1) * stride;
+        row[0] = w;
+        for (int i = 0; i < w; i++)
+            row[1 + i] = v[i];
+    });
     return (int64_t)total;
 }
 
@@ -534,67 +492,61 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
         delete c;
         return ORBG_ELIMIT;
     }
-    for (const OrbgRun &run : tb.runs)
-        c->has_stride |= run.kind == ORBG_RUN_STRIDE;
-    for (const OrbgRun &run : tb.runs_cta)
-        c->has_stride |= run.kind == ORBG_RUN_STRIDE;
     cudaError_t e;
     if ((e = cudaGetDevice(&c->device)) != cudaSuccess) {
         delete c;
         return cuda_fail(e);
     }
-    /* device copies: hcol, both run tables with their floors, the triples */
+    /* the device arrays, one after another in one allocation and one copy */
     struct Up {
-        void **dst;
+        const void **dst;
         const void *src;
         size_t bytes;
     };
-    Up ups[] = {
-        {(void **)&c->d_hcol, hcol.data(), hcol.size() * sizeof(uint32_t)},
-        {(void **)&c->d_runs, tb.runs.data(), tb.runs.size() * sizeof(OrbgRun)},
-        {(void **)&c->d_floor, tb.group_floor.data(), tb.group_floor.size() * sizeof(uint32_t)},
-        {(void **)&c->d_runs_cta, tb.runs_cta.data(), tb.runs_cta.size() * sizeof(OrbgRun)},
-        {(void **)&c->d_floor_cta, tb.group_floor_cta.data(),
-         tb.group_floor_cta.size() * sizeof(uint32_t)},
-        {(void **)&c->d_trip, tb.trip.data(), tb.trip.size() * 4},
-        {(void **)&c->d_reach, tb.reach.data(), tb.reach.size() * 4},
-        {(void **)&c->d_reach_cta, tb.reach_cta.data(), tb.reach_cta.size() * 4},
-        {(void **)&c->d_flat, tb.flat.data(), tb.flat.size()},
-        {(void **)&c->d_s3, tb.s3_cta.data(), tb.s3_cta.size()},
-        {(void **)&c->d_x3off, tb.x3off.data(), tb.x3off.size() * 4},
+    OrbgDeviceCode &d = c->dev;
+    const Up ups[] = {
+        {(const void **)&d.hcol, hcol.data(), hcol.size() * sizeof(uint32_t)},
+        {(const void **)&d.pairs, tb.pairs.data(), tb.pairs.size() * 2},
+        {(const void **)&d.pinfo, tb.pinfo.data(), tb.pinfo.size() * 4},
+        {(const void **)&d.pre, tb.pre.data(), tb.pre.size() * 8},
+        {(const void **)&d.pext, tb.pext.data(), tb.pext.size() * 8},
+        {(const void **)&d.pre1, tb.pre1.data(), tb.pre1.size() * 8},
+        {(const void **)&d.gmeta, tb.gmeta.data(), tb.gmeta.size() * 4},
+        {(const void **)&d.pmeta, tb.pmeta.data(), tb.pmeta.size() * 4},
+        {(const void **)&d.start, tb.start.data(), tb.start.size() * 4},
+        {(const void **)&d.single, tb.single.data(), tb.single.size() * 4},
+        {(const void **)&d.light, tb.light, sizeof(tb.light)},
+        {(const void **)&d.flat, tb.flat.data(), tb.flat.size()},
     };
-    for (const Up &u : ups) {
-        const size_t bytes = std::max<size_t>(u.bytes, 4);
-        if ((e = cudaMalloc(u.dst, bytes)) != cudaSuccess ||
-            (u.bytes && (e = cudaMemcpy(*u.dst, u.src, u.bytes, cudaMemcpyHostToDevice)) !=
-                            cudaSuccess)) {
-            free_code_device(c);
-            delete c;
-            return cuda_fail(e);
-        }
+    size_t total = 0;
+    for (const Up &u : ups)
+        total += (u.bytes + 255) & ~(size_t)255;
+    std::vector<unsigned char> image(total);
+    if ((e = cudaMalloc((void **)&c->d_mem, total)) != cudaSuccess) {
+        delete c;
+        return cuda_fail(e);
     }
-    c->dev.hcol = c->d_hcol;
-    c->dev.warp.runs = c->d_runs;
-    c->dev.warp.group_floor = c->d_floor;
-    c->dev.warp.nruns = (uint32_t)tb.runs.size();
-    c->dev.warp.ngroups = (uint32_t)tb.group_floor.size();
-    c->dev.warp.group_reach = c->d_reach;
-    c->dev.warp.flat_group = tb.flat_group;
-    c->dev.cta.runs = c->d_runs_cta;
-    c->dev.cta.group_floor = c->d_floor_cta;
-    c->dev.cta.nruns = (uint32_t)tb.runs_cta.size();
-    c->dev.cta.ngroups = (uint32_t)tb.group_floor_cta.size();
-    c->dev.cta.group_reach = c->d_reach_cta;
-    c->dev.cta.group_s3 = c->d_s3;
-    c->dev.x3off = c->d_x3off;
-    c->dev.s3max = tb.s3max;
-    c->dev.exact16 = r <= 16 ? 1 : 0;
-    c->dev.x3w = tb.x3off[std::min(ORBG_X3_WARP_S3, tb.s3max) + 1];
-    c->dev.cta.flat_group = tb.flat_group_cta;
-    c->dev.flat = reinterpret_cast<const uint32_t *>(c->d_flat);
-    c->dev.nflat = tb.nflat;
-    c->dev.trip = c->d_trip;
-    c->dev.ntrip = (uint32_t)tb.trip.size();
+    size_t at = 0;
+    for (const Up &u : ups) {
+        *u.dst = u.bytes ? c->d_mem + at : nullptr;
+        if (u.bytes)
+            std::memcpy(image.data() + at, u.src, u.bytes);
+        at += (u.bytes + 255) & ~(size_t)255;
+    }
+    if ((e = cudaMemcpy(c->d_mem, image.data(), total, cudaMemcpyHostToDevice)) != cudaSuccess) {
+        free_code_device(c);
+        delete c;
+        return cuda_fail(e);
+    }
+    d.npairs = (uint32_t)tb.pairs.size();
+    d.npre = tb.npre;
+    d.ngroups = (uint32_t)(tb.gmeta.size() / 2);
+    d.npre1 = tb.npre1;
+    for (int i = 0; i < ORBG_BANDS; i++) {
+        d.band_pairs[i] = tb.band_pairs[i];
+        d.band_end[i] = tb.band_end[i];
+    }
+    d.nflat = tb.nflat;
     c->dev.max_cap = cap;
     c->dev.n = n;
     c->dev.r = r;
@@ -708,8 +660,7 @@ int orbg_codeset_create(const orbg_code *const *codes, int ncodes, orbg_codeset 
     s->n_max = 0;
     s->w32_max = 1;
     s->cap_min = 0xFFFFFFFFu;
-    s->ntrip_max = 0;
-    s->x3w_max = 0;
+    s->npairs_max = 0;
     s->tuning = kDefaultTuning;
     for (int i = 0; i < ncodes; i++) {
         if (!codes[i]) {
@@ -723,9 +674,7 @@ int orbg_codeset_create(const orbg_code *const *codes, int ncodes, orbg_codeset 
         s->n_max = std::max(s->n_max, codes[i]->n);
         s->w32_max = std::max(s->w32_max, codes[i]->w32);
         s->cap_min = std::min(s->cap_min, codes[i]->max_cap);
-        s->ntrip_max = std::max(s->ntrip_max, codes[i]->dev.ntrip);
-        s->x3w_max = std::max(s->x3w_max, codes[i]->dev.x3w);
-        s->has_stride |= codes[i]->has_stride ? 1 : 0;
+        s->npairs_max = std::max(s->npairs_max, codes[i]->dev.npairs);
     }
     /* the decoder variants the kernels specialise on: keys per lane from n
      * (n <= 32, 64, 128, 256: 1, 2, 4, 8) and the syndrome words (1, 2, or
@@ -955,7 +904,6 @@ int decode_batched_pipelined(const orbg_codeset *set, const int32_t *code_id,
     a.n_max = set->n_max;
     a.w32_max = set->w32_max;
     a.var = set->var;
-    a.has_stride = set->has_stride;
     a.cap = query_cap;
     a.budget = t.warp_budget < query_cap ? t.warp_budget : query_cap;
     a.scratch = scratch;
@@ -963,8 +911,7 @@ int decode_batched_pipelined(const orbg_codeset *set, const int32_t *code_id,
     a.ctas_per_sm = t.ctas_per_sm;
     a.grab = t.blocks_per_grab;
     a.heavy_warps = t.heavy_warps;
-    a.ntrip_max = set->ntrip_max;
-    a.x3w_max = set->x3w_max;
+    a.npairs_max = set->npairs_max;
     a.scratch_B = B;
     bool declined = false;
     std::vector<cudaEvent_t> chunk_done;
@@ -1210,7 +1157,6 @@ int orbg_decode_batched(const orbg_codeset *set, const int32_t *code_id,
     a.n_max = set->n_max;
     a.w32_max = set->w32_max;
     a.var = set->var;
-    a.has_stride = set->has_stride;
     a.code_id = d_cid;
     a.llr_off = d_lo;
     a.llr = d_llr;
@@ -1226,8 +1172,7 @@ int orbg_decode_batched(const orbg_codeset *set, const int32_t *code_id,
     a.ctas_per_sm = t.ctas_per_sm;
     a.grab = t.blocks_per_grab;
     a.heavy_warps = t.heavy_warps;
-    a.ntrip_max = set->ntrip_max;
-    a.x3w_max = set->x3w_max;
+    a.npairs_max = set->npairs_max;
     a.stream = st;
     int le = orbg_launch_batched(a);
     cudaFreeAsync(scratch, st);
@@ -1516,7 +1461,6 @@ int orbg_fitted_decode(orbg_fitted *f, const float *llr, int64_t B, uint32_t que
         a.n_max = set->n_max;
         a.w32_max = set->w32_max;
         a.var = set->var;
-        a.has_stride = set->has_stride;
         a.code_id = d_cid;
         a.llr_off = nullptr;
         a.llr = llr;
@@ -1532,8 +1476,7 @@ int orbg_fitted_decode(orbg_fitted *f, const float *llr, int64_t B, uint32_t que
         a.ctas_per_sm = t.ctas_per_sm;
         a.grab = t.blocks_per_grab;
         a.heavy_warps = t.heavy_warps;
-        a.ntrip_max = set->ntrip_max;
-        a.x3w_max = set->x3w_max;
+        a.npairs_max = set->npairs_max;
         a.stream = st;
         const int le = orbg_launch_batched(a);
         if (le != 0)

@@ -192,12 +192,12 @@ int orbg_launch_code_sort(const int32_t *code_id, const int32_t *bucket, int64_t
 }
 
 int orbg_launch_exact(int K, int W, const OrbgBatchedArgs &a, const OrbgScratch &s,
-                      unsigned long long *queue, int blo, int bhi, int pdl, int stride)
+                      unsigned long long *queue, int blo, int bhi, int pdl)
 {
 #define ORBG_EX(KK)                                                                         \
-    return W <= 1   ? orbg_launch_exact_k##KK##w1(a, s, queue, blo, bhi, pdl, stride)       \
-           : W == 2 ? orbg_launch_exact_k##KK##w2(a, s, queue, blo, bhi, pdl, stride)       \
-                    : orbg_launch_exact_k##KK##w4(a, s, queue, blo, bhi, pdl, stride);
+    return W <= 1   ? orbg_launch_exact_k##KK##w1(a, s, queue, blo, bhi, pdl)       \
+           : W == 2 ? orbg_launch_exact_k##KK##w2(a, s, queue, blo, bhi, pdl)       \
+                    : orbg_launch_exact_k##KK##w4(a, s, queue, blo, bhi, pdl);
     if (K <= 1)
         ORBG_EX(1)
     if (K == 2)
@@ -217,8 +217,7 @@ int orbg_launch_batched(const OrbgBatchedArgs &args)
         /* every block is code 0: size everything for it alone */
         a.n_max = a.code0->n;
         a.w32_max = a.code0->w32;
-        a.ntrip_max = a.code0->ntrip;
-        a.x3w_max = a.code0->x3w;
+        a.npairs_max = a.code0->npairs;
     }
 #define ORBG_BW(K)                                           \
     return a.w32_max <= 1   ? orbg_launch_batched_k##K##w1(a) \

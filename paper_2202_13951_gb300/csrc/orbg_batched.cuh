@@ -35,28 +35,17 @@ using namespace orbg_dev;
 
 constexpr int kCounters = ORBG_BATCHED_COUNTERS;
 
-/* resident phase-1 CTAs per SM the register allocation is sized for: three
- * for one code or one decoder variant (80 registers, no spills), two for
- * the kernel that dispatches per block (holding every variant it spilled at
- * 80; at two it holds them in registers) */
+/* resident phase-1 CTAs per SM the register allocation is sized for */
 #ifndef ORBG_PHASE1_MIN_CTAS
 #define ORBG_PHASE1_MIN_CTAS 3
 #endif
-#ifndef ORBG_PHASE1_MIN_CTAS_MIXED
-#define ORBG_PHASE1_MIN_CTAS_MIXED 2
-#endif
 
-/* How a phase-1 kernel finds each block's decoder: P1_ONE every block is
- * the code in the kernel's parameters; P1_GENERIC each block's code from the
- * device array, dispatched to K <= KMAX, W <= WMAX; P1_EXACT each block's
- * code from the device array, all of keys per lane KMAX and width WMAX (one
- * decoder variant per launch, the blocks taken from their sort buckets). */
-enum { P1_ONE = 0, P1_GENERIC = 1, P1_EXACT = 2 };
-
-template <int KMAX, int WMAX, int MODE, bool STRIDE = true>
-__global__ void __launch_bounds__(256, MODE == P1_GENERIC ? ORBG_PHASE1_MIN_CTAS_MIXED
-                                                          : ORBG_PHASE1_MIN_CTAS)
-    orbg_batched_kernel(
+/* ONE: every block is the code in the kernel's parameters; otherwise each
+ * block's code comes from the device array, all of keys per lane K and width
+ * W (one decoder variant per launch, the blocks taken from their sort
+ * buckets). */
+template <int K, int W, bool ONE>
+__global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel(
     const OrbgDeviceCode *__restrict__ codes, int ncodes, const int32_t *__restrict__ code_id,
     const int64_t *__restrict__ llr_off, const float *__restrict__ llr, int64_t B, uint32_t cap,
     uint32_t budget, uint8_t *__restrict__ cw, const int64_t *__restrict__ cw_off,
@@ -64,10 +53,9 @@ __global__ void __launch_bounds__(256, MODE == P1_GENERIC ? ORBG_PHASE1_MIN_CTAS
     unsigned long long *__restrict__ queue, unsigned long long *__restrict__ heavy,
     const uint32_t *__restrict__ perm,
     unsigned char *__restrict__ hand, uint32_t hand_cap, unsigned long long b_base,
-    uint32_t bstride, uint32_t x3w_bytes, int grab, const uint32_t *__restrict__ range_count,
+    uint32_t bstride, int grab, const uint32_t *__restrict__ range_count,
     int blo, int bhi, const __grid_constant__ OrbgDeviceCode code0)
 {
-    constexpr bool ONE = MODE == P1_ONE;
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -75,11 +63,11 @@ __global__ void __launch_bounds__(256, MODE == P1_GENERIC ? ORBG_PHASE1_MIN_CTAS
     unsigned char *bsm = smem + warp * bstride;
     /* two LLR slots per warp: the block being decoded and the next one,
      * copied in asynchronously while the current one is decoded */
-    constexpr int kSlot = 32 * KMAX;
+    constexpr int kSlot = 32 * K;
     float *ring = reinterpret_cast<float *>(smem + nwarps * bstride) + warp * 2 * kSlot;
-    /* the warp's own triple table (sums <= ORBG_X3_WARP_S3), filled lazily */
-    uint16_t *X3w = reinterpret_cast<uint16_t *>(smem + nwarps * (bstride + 2 * kSlot * 4) +
-                                                 warp * x3w_bytes);
+    /* the warp's own hash set (search_band) */
+    uint32_t *set = reinterpret_cast<uint32_t *>(smem + nwarps * (bstride + 2 * kSlot * 4) +
+                                                  warp * kWarpSetBytes);
     const int64_t n0 = ONE ? code0.n : codes[0].n;
 
     /* the queue's slots: all B, or (range_count: the per-bucket counts of
@@ -131,7 +119,7 @@ __global__ void __launch_bounds__(256, MODE == P1_GENERIC ? ORBG_PHASE1_MIN_CTAS
                 const int n = ONE ? code0.n : codes[cid].n;
                 const int64_t lo = llr_off ? llr_off[b] : b * n0;
 #pragma unroll
-                for (int k = 0; k < KMAX; k++) {
+                for (int k = 0; k < K; k++) {
                     const int i = k * 32 + lane;
                     if (i < n)
                         __pipeline_memcpy_async(ring + slot * kSlot + i, llr + lo + i, 4);
@@ -152,36 +140,24 @@ __global__ void __launch_bounds__(256, MODE == P1_GENERIC ? ORBG_PHASE1_MIN_CTAS
         const int cid = ONE ? 0 : code_id ? code_id[b] : 0;
         const int64_t co = cw_off ? cw_off[b] : b * n0;
         const float *l = ring + slot * kSlot;
+        /* the 256-key sort stays rolled; the others are unrolled */
         if (ONE) {
-            /* one code, read from the kernel's parameters: K and W are exact;
-             * its sort is unrolled unless it is the 256-key one (for mixed
-             * codes, where several decoder variants share the instruction
-             * cache, the sort's stage loops stay rolled) */
-            decode_block_warp<KMAX, WMAX, true, true, (KMAX <= 4), (KMAX >= 8)>(code0, l, cw + co, q + b, ab + b,
-                                                            cap, budget, bsm, lane, heavy,
-                                                            &counters[1],
-                                                            b_base + (unsigned long long)b, X3w,
-                                                            hand, hand_cap);
+            decode_block_warp<K, W, true, (K >= 8)>(code0, l, cw + co, q + b, ab + b, cap, budget,
+                                                    bsm, lane, set, heavy, &counters[1],
+                                                    b_base + (unsigned long long)b, hand,
+                                                    hand_cap);
         } else if (cid < 0 || cid >= ncodes) {
             if (lane == 0) {
                 q[b] = 0u;
                 ab[b] = 2;
             }
-        } else if (MODE == P1_EXACT) {
-            /* one decoder variant: K and W exact; the block's descriptor is
-             * read where it is used (a register copy of it spilled) */
-            decode_block_warp<KMAX, WMAX, true, true, (KMAX <= 4), (KMAX >= 8), STRIDE>(
-                codes[cid], l, cw + co, q + b, ab + b, cap, budget, bsm, lane, heavy, &counters[1],
-                b_base + (unsigned long long)b, X3w, hand, hand_cap);
         } else {
-            const OrbgDeviceCode code = codes[cid];
-#define ORBG_CALL_WARP(KK, WW)                                                                 \
-    decode_block_warp<KK, WW, true, true, false, true>(code, l, cw + co, q + b, ab + b, cap, \
-                                                 budget, bsm, lane, heavy, &counters[1],    \
-                                                 b_base + (unsigned long long)b, X3w, hand,  \
-                                                 hand_cap)
-            ORBG_DISPATCH(KMAX, WMAX, ORBG_CALL_WARP);
-#undef ORBG_CALL_WARP
+            /* the block's descriptor is read where it is used (a register
+             * copy of it spilled) */
+            decode_block_warp<K, W, true, (K >= 8)>(codes[cid], l, cw + co, q + b, ab + b, cap,
+                                                    budget, bsm, lane, set, heavy, &counters[1],
+                                                    b_base + (unsigned long long)b, hand,
+                                                    hand_cap);
         }
         __syncwarp(); /* slot is free before it is refilled */
         b = bn;
@@ -196,12 +172,18 @@ __global__ void __launch_bounds__(256, MODE == P1_GENERIC ? ORBG_PHASE1_MIN_CTAS
 }
 
 
+/* Shared memory of a phase-1 warp: one block's working set, two LLR slots
+ * and its own hash set. */
+template <int K> constexpr uint32_t warp_smem_bytes(uint32_t bstride)
+{
+    return bstride + 2u * 32u * K * (uint32_t)sizeof(float) + kWarpSetBytes;
+}
+
 /* Phase 1 of one decoder variant (K, W): the blocks of sort buckets
  * [blo, bhi) of ss.perm (blo < 0: every block, in order), on its own queue.
  * pdl: the launch may begin while the previous launch in the stream (the
- * previous variant's) finishes its last blocks.  STRIDE: the set holds
- * codes with strided pair runs. */
-template <int K, int W, bool STRIDE>
+ * previous variant's) finishes its last blocks. */
+template <int K, int W>
 int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned long long *queue,
                    int blo, int bhi, int pdl)
 {
@@ -209,9 +191,8 @@ int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned lon
     const int g = a.grab < 1 ? 1 : a.grab;
     const int nk = a.n_max < 32 * K ? a.n_max : 32 * K;
     const uint32_t bstride = block_smem_bytes(nk, W);
-    auto k1 = orbg_batched_kernel<K, W, P1_EXACT, STRIDE>;
-    const uint32_t x3w_bytes = triple_table_bytes(a.x3w_max);
-    const size_t smem1 = ((size_t)bstride + 2u * 32u * K * sizeof(float) + x3w_bytes) * wpc;
+    auto k1 = orbg_batched_kernel<K, W, false>;
+    const size_t smem1 = (size_t)warp_smem_bytes<K>(bstride) * wpc;
     int grid = 0;
     int rc = orbg_grid_for((const void *)k1, wpc * 32, smem1, a.ctas_per_sm, &grid);
     if (rc != 0)
@@ -237,7 +218,7 @@ int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned lon
         &cfg, k1, a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, a.budget, a.cw,
         a.cw_off, a.q, a.ab, ss.counters, queue, ss.heavy,
         sorted ? (const uint32_t *)ss.perm : (const uint32_t *)nullptr, ss.hand, ss.hand_cap,
-        (unsigned long long)a.scratch_base, bstride, x3w_bytes, g,
+        (unsigned long long)a.scratch_base, bstride, g,
         sorted ? (const uint32_t *)ss.count : (const uint32_t *)nullptr, blo, bhi, c0);
 }
 
@@ -280,8 +261,7 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
             (e = cudaMemsetAsync(ss.count, 0, 2 * nc * sizeof(uint32_t), st)) != cudaSuccess)
             return e;
     }
-    if (!ONE && a.code_id != nullptr && a.var.n >= 1 && a.var.n <= ORBG_MAX_VARIANTS &&
-        a.var.d_bucket != nullptr) {
+    if constexpr (!ONE) {
         /* per-block codes: one launch per decoder variant, each a kernel of
          * that variant alone; with several variants the blocks are first
          * grouped by variant (a counting sort by bucket), and each launch
@@ -292,44 +272,36 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
             return (cudaError_t)rc;
         for (int v = 0; v < a.var.n; v++) {
             rc = orbg_launch_exact(a.var.k[v], a.var.w[v], a, ss, vqueue + v,
-                                   sorted ? a.var.blo[v] : -1, a.var.bhi[v], v > 0,
-                                   a.has_stride);
+                                   sorted ? a.var.blo[v] : -1, a.var.bhi[v], v > 0);
             if (rc != 0)
                 return (cudaError_t)rc;
         }
     } else {
-        /* phase 1: per warp, one block's working set, two LLR slots and its
-         * own triple table */
-        auto k1 = orbg_batched_kernel<KMAX, WMAX, ONE ? P1_ONE : P1_GENERIC>;
-        const uint32_t x3w_bytes = triple_table_bytes(a.x3w_max);
-        size_t smem1 = ((size_t)bstride + 2u * 32u * KMAX * sizeof(float) + x3w_bytes) * wpc;
+        auto k1 = orbg_batched_kernel<KMAX, WMAX, true>;
+        const size_t smem1 = (size_t)warp_smem_bytes<KMAX>(bstride) * wpc;
         if ((rc = orbg_grid_for((const void *)k1, wpc * 32, smem1, a.ctas_per_sm, &grid)) != 0)
             return (cudaError_t)rc;
         int64_t units = (a.B + g - 1) / g;
         int64_t need = (units + wpc - 1) / wpc;
         if (grid > need) grid = (int)(need > 0 ? need : 1);
-        OrbgDeviceCode c0{};
-        if (ONE)
-            c0 = *a.code0;
         k1<<<grid, wpc * 32, smem1, st>>>(a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B,
                                           a.cap, a.budget, a.cw, a.cw_off, a.q, a.ab, counters,
                                           queue, heavy, nullptr, sc.hand, sc.hand_cap,
-                                          (unsigned long long)a.scratch_base, bstride, x3w_bytes,
-                                          g, nullptr, 0, 0, c0);
+                                          (unsigned long long)a.scratch_base, bstride, g, nullptr,
+                                          0, 0, *a.code0);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }
-    /* phase 2 runs whatever the budget: a phase-1 walk on the CTA table also
-     * stops, open, where it needs triple sums past the warp's own table
-     * (decode_block_warp), so the list can hold blocks with a budget at or
-     * above the cap too (with an empty list the launch only reads its
+    /* phase 2 runs whatever the budget: phase 1 also leaves a block open
+     * after its last band (with an empty list the launch only reads its
      * length) */
     if (a.stage == 1)
         return cudaSuccess; /* phase 2 comes later, over every chunk's list */
     return launch_heavy_t<KMAX, WMAX, ONE>(a, counters, heavy, sc.hand);
 }
 
-/* Phases 1 and 2 for keys-per-lane bound KMAX and syndrome width WMAX. */
+/* Phases 1 and 2 for keys-per-lane bound KMAX and syndrome width WMAX: one
+ * code (a.code0), or per-block codes. */
 template <int KMAX, int WMAX>
 int launch_kw(const OrbgBatchedArgs &a)
 {

@@ -14,19 +14,18 @@
  *      sorting networks as one option, Sec. IV-B);
  *   3. permuted columns hperm[p] = H[:, pi_p] into shared memory, after a
  *      zero column read by unused prefix slots;
- *   4. the query order as runs (orbg_internal.h): lane l of a warp step
- *      takes run l of a group of 32, XORs its prefix columns into s0 and
- *      walks the run, testing s0 (+) prefix (+) hperm[a] (+) hperm[b] == 0;
- *      the smallest hit index is kept and the search stops once no later
- *      group can hold a smaller one, or the cap is passed;
+ *   4. past the flat table, every pattern of weight >= 2 is a prefix and a
+ *      pair of its last two positions: the block's pairs go into a hash set
+ *      of their syndromes, and each prefix is one look-up of s0 (+) prefix
+ *      (orbg_internal.h says why the first pair of a syndrome is enough, how
+ *      a hit's query index is formed and when no later prefix can beat it);
  *   5. codeword y (+) z* (or y if abandoned), query count, abandon flag.
  *
- * Two ways to run step 4: one warp walks all groups of its block
- * (decode_block_warp), or all warps of a CTA share one block and take its
- * groups in turn, with the best index in shared memory (decode_block_cta).
- * The second keeps a block that needs 1e6 queries from running on a single
- * warp.  Every loop is bounded by the table size or the run length; no
- * thread waits on another's progress beyond __syncthreads.
+ * Two ways to run step 4: one warp takes its block through the first bands
+ * of the order (decode_block_warp), with a small table of its own; all warps
+ * of a CTA share one block and its whole set of pairs (decode_block_cta).
+ * Every loop is bounded by the tables' sizes or the hash sets'; no thread
+ * waits on another's progress beyond __syncthreads.
  */
 #pragma once
 #include <cuda_runtime.h>
@@ -97,25 +96,6 @@ __host__ __device__ __forceinline__ uint32_t block_smem_bytes(int n, int w32)
     return h + h0 + 256u + 256u;
 }
 
-/* Triple table: X3[i] = low 16 bits of h0[c0] ^ h0[a0] ^ h0[b0] for triple
- * i of the code's triple list (a match is verified on the whole syndrome
- * unless n - k <= 16, where 16 bits are the whole syndrome). */
-__host__ __device__ __forceinline__ uint32_t triple_table_bytes(uint32_t ntrip)
-{
-    return (ntrip * 2u + 15u) & ~15u;
-}
-
-/* Fills X3[lo, hi) from the triple list; `stride` threads starting at `t`. */
-__device__ __forceinline__ void build_x3(const OrbgDeviceCode &code, const uint32_t *h0,
-                                         uint16_t *X3, uint32_t lo, uint32_t hi, uint32_t t,
-                                         uint32_t stride)
-{
-    for (uint32_t i = lo + t; i < hi; i += stride) {
-        const uint32_t c = __ldg(code.trip + i);
-        X3[i] = (uint16_t)(h0[c & 0xFFu] ^ h0[(c >> 8) & 0xFFu] ^ h0[(c >> 16) & 0xFFu]);
-    }
-}
-
 /* h[r] (and h0[r]) is the column of sorted position r, 0 <= r < n; the
  * entry before it, h[-1], is the zero column, so a 1-based position p (0 =
  * none) reads h[p - 1] with no test. */
@@ -143,6 +123,24 @@ template <int W> struct BlockSmem {
 __device__ __forceinline__ uint32_t first_word(uint32_t v) { return v; }
 __device__ __forceinline__ uint32_t first_word(uint2 v) { return v.x; }
 __device__ __forceinline__ uint32_t first_word(uint4 v) { return v.x; }
+
+/* A 32-bit key of a syndrome, linear over GF(2) so that the key of a sum is
+ * the XOR of the keys; the syndrome itself up to 32 bits.  Longer ones add
+ * the further words through an invertible linear mix (xorshift steps, after
+ * Marsaglia): with the first word alone, the unit columns of a systematic H
+ * beyond row 32 would all have key 0 and share their sums' keys. */
+__device__ __forceinline__ uint32_t key_mix(uint32_t v)
+{
+    v ^= v << 13;
+    v ^= v >> 17;
+    return v ^ (v << 5);
+}
+__device__ __forceinline__ uint32_t syn_key(uint32_t v) { return v; }
+__device__ __forceinline__ uint32_t syn_key(uint2 v) { return v.x ^ key_mix(v.y); }
+__device__ __forceinline__ uint32_t syn_key(uint4 v)
+{
+    return v.x ^ key_mix(v.y ^ key_mix(v.z ^ key_mix(v.w)));
+}
 
 /* LLR reads: from shared memory (LS, staged ahead by the batched kernel)
  * or from global memory through the read-only path. */
@@ -428,7 +426,7 @@ __device__ __forceinline__ void build_perm(const OrbgDeviceCode &code, const uin
             const typename Syn<W>::T col = load_col<W>(code.hcol, idx);
             sm.h[e] = col;
             if (W > 1)
-                sm.h0[e] = first_word(col);
+                sm.h0[e] = syn_key(col);
         }
     }
     if (lane == 0) {
@@ -502,7 +500,7 @@ __device__ __forceinline__ void perm_ranks(const OrbgDeviceCode &code, uint32_t 
         const typename Syn<W>::T col = load_col<W>(code.hcol, idx);
         sm.h[lane] = col;
         if (W > 1)
-            sm.h0[lane] = first_word(col);
+            sm.h0[lane] = syn_key(col);
     }
 }
 
@@ -521,305 +519,285 @@ __device__ __forceinline__ void make_keys(const float *__restrict__ llr, int n, 
     }
 }
 
-/* -------------------------------------------------- step 4: one run */
+/* ------------------------------------------- step 4: pair look-ups */
 
-/* A run record (orbg_internal.h) as two 16-byte loads:
- * v0.x tstart, v0.y count | npre << 16 | kind << 24, v0.z aux,
- * v0.w prefix positions 0..3, v1 prefix positions 4..19. */
-__device__ __forceinline__ int run_count(const uint4 &v0) { return (int)(v0.y & 0xFFFFu); }
-__device__ __forceinline__ int run_npre(const uint4 &v0) { return (int)((v0.y >> 16) & 0xFFu); }
-__device__ __forceinline__ int run_kind(const uint4 &v0) { return (int)(v0.y >> 24); }
-
-/* Syndrome of a run's prefix: s0 (+) the prefix columns, over the W-word
- * syndromes h or over their first words h0.  Prefix positions are stored
- * 1-based with 0 in the unused slots, which read the zero column h[-1]:
- * the first eight loads need no test of npre. */
-template <typename T>
-__device__ __forceinline__ T prefix_syndrome(const uint4 &v0, const uint4 &v1,
-                                             const T *__restrict__ h, const T s0, int npre)
+/*
+ * A hash set of pairs: 2^bits 32-bit slots, linear probing.  An entry is the
+ * pair's index in the chunk of pairs the set holds (low 12 bits) under a tag,
+ * the hash bits below the slot's: with the slot they are the key itself up to
+ * two bits, and resolve_pair checks the whole syndrome.  Of pairs of equal
+ * syndrome the first stays.  The hash is multiplicative (the high bits of
+ * the key times an odd constant near 2^32 / golden ratio).
+ */
+constexpr uint32_t kIdMask = 0xFFFu;
+constexpr uint32_t kPairChunk = 4095; /* pairs of one set; entry kEmpty is never a pair's */
+constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t slot_hash(uint32_t v) { return v * 0x9E3779B1u; }
+__device__ __forceinline__ uint32_t slot_tag(uint32_t hash, uint32_t bits)
 {
-    T p[8];
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-        const uint32_t wd = i < 4 ? v0.w : v1.x;
-        p[i] = h[(int)((wd >> (8 * (i & 3))) & 0xFFu) - 1];
-    }
-    T P = sx(sx(sx(s0, p[0]), sx(p[1], p[2])), sx(sx(p[3], p[4]), sx(p[5], sx(p[6], p[7]))));
-    if (npre > 8) {
-#pragma unroll
-        for (int i = 8; i < ORBG_RUN_MAX_PRE; i++) {
-            if (i >= npre)
-                break;
-            const uint32_t wd = (i < 12) ? v1.y : (i < 16) ? v1.z : v1.w;
-            P = sx(P, h[(int)((wd >> (8 * (i & 3))) & 0xFFu) - 1]);
-        }
-    }
-    return P;
+    return (hash << bits) & ~kIdMask;
 }
 
-/* Positions (0-based) a query flips besides the prefix: kind 1 hit value
- * is a (1-based), the pair (a, S - a); kind 2 hit value is the pattern's
- * offset j in the run, the pair (a_0 + j da, b_0 - j db); kind 3 hit value
- * is the triple index.  Writes up to three positions, returns how many. */
-template <bool STRIDE = true>
-__device__ __forceinline__ int query_tail(const uint4 &v0, uint32_t hit, const uint32_t *trip,
-                                          int *pos)
+/* A warp's own set: 1,024 slots hold the 225 pairs of the first band at a
+ * load of 0.22 and the 484 of the second at 0.47. */
+constexpr uint32_t kWarpSetBits = 10;
+constexpr uint32_t kWarpSetBytes = 4u << kWarpSetBits;
+static_assert(ORBG_BAND2_PAIRS * 2 <= (1 << kWarpSetBits), "set too small for the last band");
+
+/* A CTA's set for a code of `npairs` pairs, taken in chunks of at most
+ * kPairChunk: at least four slots a pair up to 2,048 pairs (cap 1e6 has
+ * 1,640), two beyond. */
+__host__ __device__ __forceinline__ uint32_t pair_slot_bits(uint32_t npairs)
 {
-    const int kind = run_kind(v0);
-    if (kind == ORBG_RUN_PAIRS) {
-        const int S = (int)(v0.z & 0xFFu), a = (int)hit;
-        pos[0] = a - 1;
-        pos[1] = S - a - 1;
-        return 2;
-    }
-    if (STRIDE && kind == ORBG_RUN_STRIDE) {
-        const int j = (int)hit;
-        pos[0] = (int)(v0.z & 0xFFu) + j * (int)((v0.z >> 16) & 0xFFu) - 1;
-        pos[1] = (int)((v0.z >> 8) & 0xFFu) - j * (int)(v0.z >> 24) - 1;
-        return 2;
-    }
-    if (kind == ORBG_RUN_TRIPLES) {
-        const uint32_t t = __ldg(trip + hit);
-        pos[0] = (int)(t & 0xFFu);
-        pos[1] = (int)((t >> 8) & 0xFFu);
-        pos[2] = (int)((t >> 16) & 0xFFu);
-        return 3;
-    }
-    return 0;
+    const uint32_t np = npairs < kPairChunk ? npairs : kPairChunk;
+    uint32_t b = 8;
+    while (b < 13 && (1u << b) < 4u * np)
+        b++;
+    return b;
+}
+/* Keys of the subsets of the eight lightest positions, then of the next
+ * eight: a prefix record names its light positions by two bytes. */
+constexpr uint32_t kMaskBytes = 512 * 4;
+__host__ __device__ __forceinline__ uint32_t pair_smem_bytes(uint32_t npairs)
+{
+    return kMaskBytes + (4u << pair_slot_bits(npairs));
 }
 
-/* Full-width check of a query whose first word matched (rare: kept out of
- * line so it costs the scan loops no registers). */
+/* Pair id (of the chunk from lo) into the set.  Returns true if its key is
+ * zero but its syndrome is not (such a pair is looked up by resolve_pair; a
+ * pair of syndrome zero is part of no first hit). */
 template <int W>
-__device__ __noinline__ bool verify_query(const uint4 &v0, const uint4 &v1,
-                                          const typename Syn<W>::T *__restrict__ h,
-                                          const typename Syn<W>::T s0, int n, uint32_t hit,
-                                          const uint32_t *trip)
+__device__ __forceinline__ bool insert_pair(const OrbgDeviceCode &code, const BlockSmem<W> &sm,
+                                            uint32_t *set, uint32_t bits, uint32_t lo,
+                                            uint32_t id)
 {
-    typedef typename Syn<W>::T T;
-    T P = prefix_syndrome<T>(v0, v1, h, s0, run_npre(v0));
-    int pos[3];
-    const int k = query_tail(v0, hit, trip, pos);
-    for (int i = 0; i < k; i++)
-        P = sx(P, h[pos[i]]);
-    return sz(P);
-}
-
-/* Pair run: queries (a, b) = (a_0 + j da, b_0 - j db), j = 0, 1, ... (kind
- * 1: a_0 = a_lo, b_0 = S - a_lo, da = db = 1; kind 2, only where STRIDE: as
- * stored); two queries per step, first words from h0; a first-word match is
- * checked on all W words outside the scan loop (a false match, probability
- * 2^-32 per query, resumes it).  Returns the offset of the first hit or -1,
- * and the hit value for query_tail in *hit (kind 1: a; kind 2: the offset).
- * STRIDE = false (kernels of code sets without strided runs) compiles the
- * kind-1 walk alone: the extra registers cost the mixed-code kernels. */
-template <int W, bool STRIDE>
-__device__ __forceinline__ int walk_pairs(const uint4 &v0, const uint4 &v1,
-                                          const typename Syn<W>::T *__restrict__ h,
-                                          const uint32_t *__restrict__ h0,
-                                          const typename Syn<W>::T s0, uint32_t P0, int n,
-                                          uint32_t *hit)
-{
-    const int len = run_count(v0);
-    if constexpr (!STRIDE) {
-        const int S = (int)(v0.z & 0xFFu);
-        const int a_first = (int)((v0.z >> 8) & 0xFFu);
-        int j = 0;
-        for (;;) {
-            int cand = -1;
-            for (; j < len; j += 2) {
-                const int a = a_first + j;
-                const int b = S - a;
-                /* the second slot is clamped into the table and masked past the run */
-                const int a1 = min(a + 1, n), b1 = max(b - 1, 1);
-                const bool m0 = (h0[a - 1] ^ h0[b - 1]) == P0;
-                const bool m1 = ((h0[a1 - 1] ^ h0[b1 - 1]) == P0) && (j + 1 < len);
-                if (m0 || m1) {
-                    cand = j + (m0 ? 0 : 1);
-                    break;
-                }
-            }
-            if (cand < 0)
-                return -1;
-            if (W == 1 ||
-                verify_query<W>(v0, v1, h, s0, n, (uint32_t)(a_first + cand), nullptr)) {
-                *hit = (uint32_t)(a_first + cand);
-                return cand;
-            }
-            j = cand + 1;
-        }
-    }
-    const bool stride = run_kind(v0) == ORBG_RUN_STRIDE;
-    const int a_first = stride ? (int)(v0.z & 0xFFu) : (int)((v0.z >> 8) & 0xFFu);
-    const int b_first =
-        stride ? (int)((v0.z >> 8) & 0xFFu) : (int)(v0.z & 0xFFu) - a_first;
-    const int da = stride ? (int)((v0.z >> 16) & 0xFFu) : 1;
-    const int db = stride ? (int)(v0.z >> 24) : 1;
-    int j = 0;
+    const uint32_t p = __ldg(code.pairs + id);
+    const uint32_t v = sm.h0[p & 0xFFu] ^ sm.h0[p >> 8];
+    if (v == 0u)
+        return W > 1 && !sz(sx(sm.h[p & 0xFFu], sm.h[p >> 8]));
+    const uint32_t x = slot_hash(v), e = slot_tag(x, bits) | (id - lo);
+    uint32_t slot = x >> (32u - bits);
     for (;;) {
-        int cand = -1;
-        int a = a_first + j * da, b = b_first - j * db;
-        for (; j < len; j += 2, a += 2 * da, b -= 2 * db) {
-            /* the second slot is clamped into the table and masked past the run */
-            const int a1 = min(a + da, n), b1 = max(b - db, 1);
-            const bool m0 = (h0[a - 1] ^ h0[b - 1]) == P0;
-            const bool m1 = ((h0[a1 - 1] ^ h0[b1 - 1]) == P0) && (j + 1 < len);
-            if (m0 || m1) {
-                cand = j + (m0 ? 0 : 1);
-                break;
+        const uint32_t old = atomicCAS(set + slot, kEmpty, e);
+        if (old == kEmpty)
+            return false;
+        if ((old ^ e) <= kIdMask) {
+            /* the same tag: the same syndrome? */
+            const uint32_t o = __ldg(code.pairs + lo + (old & kIdMask));
+            if (sz(sx(sx(sm.h[p & 0xFFu], sm.h[p >> 8]), sx(sm.h[o & 0xFFu], sm.h[o >> 8])))) {
+                atomicMin(set + slot, e);
+                return false;
             }
         }
-        if (cand < 0)
-            return -1;
-        const uint32_t hv = stride ? (uint32_t)cand : (uint32_t)(a_first + cand);
-        if (W == 1 || verify_query<W>(v0, v1, h, s0, n, hv, nullptr)) {
-            *hit = hv;
-            return cand;
-        }
-        j = cand + 1;
+        slot = (slot + 1u) & ((1u << bits) - 1u);
     }
 }
 
-/* Walk one run of the warp table unless it cannot beat `best`.  Returns the
- * run's first hit index (or ORBG_NONE) and the hit value for the flips. */
-template <int W, bool STRIDE = true>
-__device__ __forceinline__ uint32_t search_run_warp(const uint4 &v0, const uint4 &v1,
-                                                    const typename Syn<W>::T *__restrict__ h,
-                                                    const uint32_t *__restrict__ h0,
-                                                    const typename Syn<W>::T s0, uint32_t best,
-                                                    uint32_t cap, int n, uint32_t *hit)
+/* The entry whose tag is that of key v, or kEmpty. */
+__device__ __forceinline__ uint32_t find_pair(const uint32_t *set, uint32_t bits, uint32_t v)
 {
-    const uint32_t tstart = v0.x;
-    if (!(tstart < best && tstart <= cap))
-        return ORBG_NONE;
-    const uint32_t P0 = prefix_syndrome<uint32_t>(v0, v1, h0, first_word(s0), run_npre(v0));
-    if (run_kind(v0) == ORBG_RUN_SINGLE) {
-        if (P0 == 0u && (W == 1 || verify_query<W>(v0, v1, h, s0, n, 0u, nullptr))) {
-            *hit = 0u;
-            return tstart;
-        }
-        return ORBG_NONE;
+    const uint32_t x = slot_hash(v), tag = slot_tag(x, bits);
+    uint32_t slot = x >> (32u - bits);
+    uint32_t e = set[slot];
+    while (e != kEmpty && (e ^ tag) > kIdMask) {
+        slot = (slot + 1u) & ((1u << bits) - 1u);
+        e = set[slot];
     }
-    const int j = walk_pairs<W, STRIDE>(v0, v1, h, h0, s0, P0, n, hit);
-    return j < 0 ? ORBG_NONE : tstart + (uint32_t)j;
+    return e;
 }
 
-/* Nonzero iff one of the two 16-bit halves of t is zero (the lowest zero
- * half always sets its flag; a borrow can only add flags above it). */
-__device__ __forceinline__ uint32_t zero16(uint32_t t)
+/* A hit: its query index, its prefix (or kSingle) and its pair (or the
+ * 0-based position). */
+constexpr uint32_t kSingle = 0xFFFFFFFEu;
+struct PairHit {
+    uint32_t t, pre, pair;
+};
+
+/* s0 (+) the columns of prefix i, whole width. */
+template <int W>
+__device__ __forceinline__ typename Syn<W>::T prefix_target(const OrbgDeviceCode &code,
+                                                            const typename Syn<W>::T *h,
+                                                            typename Syn<W>::T s0, uint32_t i)
 {
-    return (t - 0x00010001u) & ~t & 0x80008000u;
+    typename Syn<W>::T v = s0;
+    const uint2 r = __ldg(reinterpret_cast<const uint2 *>(code.pre) + i);
+    for (uint32_t m = r.x & 0xFFFFu; m; m &= m - 1u)
+        v = sx(v, h[(int)__ldg(code.light + (__ffs(m) - 1)) - 1]);
+    v = sx(v, sx(h[(int)((r.x >> 16) & 0xFFu) - 1], h[(int)(r.x >> 24) - 1]));
+    for (uint32_t y = r.y; y; y >>= 8)
+        v = sx(v, h[(int)(y & 0xFFu) - 1]);
+    if (code.pext) {
+        const uint2 e = __ldg(reinterpret_cast<const uint2 *>(code.pext) + i);
+        for (uint32_t y = e.x; y; y >>= 8)
+            v = sx(v, h[(int)(y & 0xFFu) - 1]);
+        for (uint32_t y = e.y; y; y >>= 8)
+            v = sx(v, h[(int)(y & 0xFFu) - 1]);
+    }
+    return v;
 }
 
-/* Walk one run of the CTA table: kind 3 tests the X3 range [aux, aux +
- * count) against the low 16 bits of the prefix syndrome, four queries per
- * step.  Entries at or past x3lim are not built: those queries are formed
- * from the triple list instead (slower, used only near the end of a warp's
- * own table). */
-template <int W, bool STRIDE = true>
-__device__ __forceinline__ uint32_t search_run_cta(const uint4 &v0, const uint4 &v1,
-                                                   const typename Syn<W>::T *__restrict__ h,
-                                                   const uint32_t *__restrict__ h0,
-                                                   const uint16_t *__restrict__ X3,
-                                                   uint32_t x3lim,
-                                                   const uint32_t *__restrict__ trip,
-                                                   const typename Syn<W>::T s0, uint32_t best,
-                                                   uint32_t cap, int n, bool exact16,
-                                                   uint32_t *hit)
+/* Query index of prefix i with the first of the pairs [lo, hi) that makes
+ * it a hit, and that pair in *pair; ORBG_NONE if there is none, it does not
+ * lie after the prefix, or the table ends before it.  id: the pair the set
+ * named (checked here), or ORBG_NONE.  Each lane for itself (rare: kept out
+ * of line). */
+template <int W>
+__device__ __noinline__ uint32_t resolve_pair(const OrbgDeviceCode &code,
+                                              const typename Syn<W>::T *h,
+                                              typename Syn<W>::T s0, uint32_t i, uint32_t id,
+                                              uint32_t lo, uint32_t hi, uint32_t *pair)
 {
-    const uint32_t tstart = v0.x;
-    if (!(tstart < best && tstart <= cap))
+    const uint2 *pm = reinterpret_cast<const uint2 *>(code.pmeta);
+    const uint2 m = __ldg(pm + i);
+    const uint32_t end = __ldg(pm + i + 1).x;
+    const typename Syn<W>::T v = prefix_target<W>(code, h, s0, i);
+    uint32_t p = id != ORBG_NONE ? __ldg(code.pairs + id) : 0u;
+    if (id == ORBG_NONE || !sz(sx(sx(h[p & 0xFFu], h[p >> 8]), v))) {
+        /* an equal tag of another syndrome: look through all pairs */
+        for (id = lo; id < hi; id++) {
+            p = __ldg(code.pairs + id);
+            if (sz(sx(sx(h[p & 0xFFu], h[p >> 8]), v)))
+                break;
+        }
+        if (id >= hi)
+            return ORBG_NONE;
+    }
+    const uint32_t q = m.y & 0xFFFFu, info = __ldg(code.pinfo + id);
+    if ((p & 0xFFu) + 1u <= q)
         return ORBG_NONE;
-    const uint32_t P0 = prefix_syndrome<uint32_t>(v0, v1, h0, first_word(s0), run_npre(v0));
-    const int kind = run_kind(v0);
-    if (kind == ORBG_RUN_TRIPLES) {
-        const int len = run_count(v0);
-        const uint32_t x0 = v0.z;
-        const uint16_t p16 = (uint16_t)P0;
-        const bool exact = W == 1 && exact16;
-        int j = 0;
-        if (x0 + (uint32_t)len <= x3lim) {
-            /* aligned 16-byte chunks of eight entries (the table starts on
-             * a 16-byte boundary and its allocation is a whole number of
-             * chunks), tested at once for an entry equal to p16; a step
-             * with one is re-read entry by entry, skipping the entries
-             * outside the run */
-            const uint32_t end = x0 + (uint32_t)len;
-            const uint32_t pp = (uint32_t)p16 * 0x00010001u;
-            const uint4 *X4 = reinterpret_cast<const uint4 *>(X3);
-            /* two chunks per step; the second is read only inside the run
-             * (past its end the table may end) */
-            for (uint32_t c = x0 & ~7u; c < end; c += 16u) {
-                const uint4 va = X4[c >> 3];
-                const bool two = c + 8u < end;
-                const uint4 vb = two ? X4[(c >> 3) + 1u] : va;
-                if (zero16(va.x ^ pp) | zero16(va.y ^ pp) | zero16(va.z ^ pp) |
-                    zero16(va.w ^ pp) | zero16(vb.x ^ pp) | zero16(vb.y ^ pp) |
-                    zero16(vb.z ^ pp) | zero16(vb.w ^ pp)) {
-                    for (uint32_t e = max(c, x0); e < min(c + 16u, end); e++) {
-                        if (X3[e] == p16 &&
-                            (exact || verify_query<W>(v0, v1, h, s0, n, e, trip))) {
-                            *hit = e;
-                            return tstart + (e - x0);
-                        }
-                    }
+    const uint32_t at = m.x + ((info & 0xFFFFu) - (m.y >> 16));
+    if (at >= end)
+        return ORBG_NONE;
+    /* the first pair of its group after the prefix */
+    uint32_t a = info >> 16, b = id;
+    while (a < b) {
+        const uint32_t mid = (a + b) >> 1;
+        if ((uint32_t)(__ldg(code.pairs + mid) & 0xFFu) + 1u > q)
+            b = mid;
+        else
+            a = mid + 1u;
+    }
+    *pair = id;
+    return __ldg(code.start + at) + (id - a);
+}
+
+/* Single positions: the first whose column is s0.  `step` threads, thread t
+ * takes positions t, t + step, ...; returns the thread's first hit. */
+template <int W>
+__device__ __forceinline__ PairHit single_hits(const OrbgDeviceCode &code,
+                                               const typename Syn<W>::T *h,
+                                               typename Syn<W>::T s0, uint32_t t, uint32_t step)
+{
+    PairHit best{ORBG_NONE, kSingle, 0u};
+    for (uint32_t j = t; j < (uint32_t)code.n; j += step)
+        if (sz(sx(h[j], s0))) {
+            const uint32_t x = __ldg(code.single + j);
+            if (x != 0u && x < best.t) {
+                best.t = x;
+                best.pair = j;
+            }
+        }
+    return best;
+}
+
+/* The warp's best of its lanes' hits, in every lane. */
+__device__ __forceinline__ PairHit warp_best(const PairHit &mine)
+{
+    PairHit h;
+    h.t = __reduce_min_sync(FULL_MASK, mine.t);
+    const int src = __ffs(__ballot_sync(FULL_MASK, mine.t == h.t)) - 1;
+    h.pre = __shfl_sync(FULL_MASK, mine.pre, src);
+    h.pair = __shfl_sync(FULL_MASK, mine.pair, src);
+    return h;
+}
+
+/*
+ * One warp searches band k of its block: the band's pairs from np on go into
+ * its set, then every prefix before the band's end is looked up, unless
+ * `best` or the cap ends the search first.  Returns the best hit, `best` or
+ * one found here.  Every pattern before the band's end is covered, so a hit
+ * below it is final.
+ */
+template <int W>
+__device__ __forceinline__ PairHit search_band(const OrbgDeviceCode &code,
+                                               const BlockSmem<W> &sm,
+                                               const typename Syn<W>::T s0, uint32_t cap, int k,
+                                               uint32_t np, uint32_t *set, int lane, PairHit best,
+                                               bool *zero)
+{
+    const uint32_t end = code.band_end[k], hi = code.band_pairs[k];
+#pragma unroll 1
+    for (uint32_t id = np + (uint32_t)lane; id < hi; id += 32u)
+        *zero |= insert_pair<W>(code, sm, set, kWarpSetBits, 0u, id);
+    __syncwarp();
+    if (W > 1)
+        *zero = __any_sync(FULL_MASK, *zero);
+    const uint32_t s0w = syn_key(s0);
+    const uint2 *gm = reinterpret_cast<const uint2 *>(code.gmeta);
+    const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre1);
+    PairHit mine = best;
+#pragma unroll 1
+    for (uint32_t g = 0; g < code.ngroups; g++) {
+        const uint2 m = __ldg(gm + g);
+        if (m.x >= end || m.x >= best.t || m.x > cap)
+            break;
+        const uint32_t i = g * ORBG_GROUP + (uint32_t)lane;
+        const uint2 r = __ldg(pre + i);
+        uint32_t v = s0w;
+        const int kmax = (int)(m.y >> 8);
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            if (j >= kmax)
+                break;
+            v ^= sm.h0[(int)(((j < 4 ? r.x : r.y) >> (8 * (j & 3))) & 0xFFu) - 1];
+        }
+        const uint32_t e = find_pair(set, kWarpSetBits, v);
+        const bool found = (e != kEmpty || (W > 1 && v == 0u && *zero)) && i < code.npre1;
+        if (__any_sync(FULL_MASK, found)) {
+            if (found) {
+                uint32_t pair = 0;
+                const uint32_t t = resolve_pair<W>(code, sm.h, s0, i,
+                                                   e != kEmpty ? e & kIdMask : ORBG_NONE, 0u, hi,
+                                                   &pair);
+                if (t < mine.t) {
+                    mine.t = t;
+                    mine.pre = i;
+                    mine.pair = pair;
                 }
             }
-            return ORBG_NONE;
+            best = warp_best(mine);
         }
-        for (; j < len; j++) { /* entries not built: form each triple */
-            const uint32_t t = x0 + (uint32_t)j;
-            const uint32_t c = __ldg(trip + t);
-            const uint32_t v = h0[c & 0xFFu] ^ h0[(c >> 8) & 0xFFu] ^ h0[(c >> 16) & 0xFFu];
-            if (v == P0 && (W == 1 || verify_query<W>(v0, v1, h, s0, n, t, trip))) {
-                *hit = t;
-                return tstart + (uint32_t)j;
-            }
-        }
-        return ORBG_NONE;
     }
-    if (kind == ORBG_RUN_SINGLE) {
-        if (P0 == 0u && (W == 1 || verify_query<W>(v0, v1, h, s0, n, 0u, nullptr))) {
-            *hit = 0u;
-            return tstart;
-        }
-        return ORBG_NONE;
-    }
-    const int j = walk_pairs<W, STRIDE>(v0, v1, h, h0, s0, P0, n, hit);
-    return j < 0 ? ORBG_NONE : tstart + (uint32_t)j;
-}
-
-__device__ __forceinline__ void load_run(const OrbgTable &tb, uint32_t e, uint4 *v0, uint4 *v1)
-{
-    if (e < tb.nruns) {
-        const uint4 *runs4 = reinterpret_cast<const uint4 *>(tb.runs);
-        *v0 = __ldg(runs4 + 2 * e);
-        *v1 = __ldg(runs4 + 2 * e + 1);
-    } else {
-        *v0 = make_uint4(ORBG_NONE, 0u, 0u, 0u); /* tstart = NONE: never searched */
-        *v1 = make_uint4(0u, 0u, 0u, 0u);
-    }
+    return best;
 }
 
 /* ----------------------------------------------------- step 5: output */
 
-/* The owner of the winning run applies its flips to the staged codeword. */
-template <bool STRIDE = true>
-__device__ __forceinline__ void apply_flips(const OrbgTable &tb, uint32_t run, uint32_t hit,
-                                            const uint32_t *trip, const uint8_t *pi,
-                                            uint8_t *cw)
+/* Flips of a hit into the staged codeword (one thread). */
+static __device__ __noinline__ void apply_pair_flips(const OrbgDeviceCode &code, const PairHit &hit,
+                                              const uint8_t *pi, uint8_t *cw)
 {
-    const uint4 *runs4 = reinterpret_cast<const uint4 *>(tb.runs);
-    const uint4 v0 = __ldg(runs4 + 2 * run), v1 = __ldg(runs4 + 2 * run + 1);
-    const int npre = run_npre(v0);
-    for (int i = 0; i < npre; i++) {
-        const uint32_t wd = i < 4 ? v0.w : i < 8 ? v1.x : i < 12 ? v1.y : i < 16 ? v1.z : v1.w;
-        cw[pi[(int)((wd >> (8 * (i & 3))) & 0xFFu) - 1]] ^= 1;
+    if (hit.pre == kSingle) {
+        cw[pi[hit.pair]] ^= 1;
+        return;
     }
-    int pos[3];
-    const int k = query_tail<STRIDE>(v0, hit, trip, pos);
-    for (int i = 0; i < k; i++)
-        cw[pi[pos[i]]] ^= 1;
+    const uint32_t p = __ldg(code.pairs + hit.pair);
+    cw[pi[p & 0xFFu]] ^= 1;
+    cw[pi[p >> 8]] ^= 1;
+    const uint2 r = __ldg(reinterpret_cast<const uint2 *>(code.pre) + hit.pre);
+    for (uint32_t m = r.x & 0xFFFFu; m; m &= m - 1u)
+        cw[pi[__ldg(code.light + (__ffs(m) - 1)) - 1]] ^= 1;
+    for (uint32_t y = r.x >> 16; y; y >>= 8)
+        cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+    for (uint32_t y = r.y; y; y >>= 8)
+        cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+    if (code.pext) {
+        const uint2 e = __ldg(reinterpret_cast<const uint2 *>(code.pext) + hit.pre);
+        for (uint32_t y = e.x; y; y >>= 8)
+            cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+        for (uint32_t y = e.y; y; y >>= 8)
+            cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+    }
 }
 
 /* ---------------------------------------------------- the flat table */
@@ -853,7 +831,7 @@ __device__ __forceinline__ bool flat_test(const typename Syn<W>::T *__restrict__
                                           int wmax = ORBG_FLAT_POS)
 {
     typedef typename Syn<W>::T T;
-    uint32_t P0 = first_word(s0);
+    uint32_t P0 = syn_key(s0);
 #pragma unroll
     for (int i = 0; i < ORBG_FLAT_POS; i++) {
         if (i >= wmax)
@@ -876,22 +854,6 @@ __device__ __forceinline__ bool flat_test(const typename Syn<W>::T *__restrict__
     return true;
 }
 
-/* Lane's query of flat step `base` (queries base+1 .. base+32): returns its
- * index if it is a hit, else ORBG_NONE. */
-template <int W>
-__device__ __forceinline__ uint32_t flat_query(const OrbgDeviceCode &code,
-                                               const typename Syn<W>::T *__restrict__ h,
-                                               const uint32_t *__restrict__ h0,
-                                               const typename Syn<W>::T s0, uint32_t base,
-                                               uint32_t cap, int lane)
-{
-    const uint32_t t = base + (uint32_t)lane + 1u;
-    if (t > code.nflat || t > cap)
-        return ORBG_NONE;
-    const uint2 e = flat_entry(code, t, cap);
-    return flat_test<W>(h, h0, s0, e, code.n) ? t : ORBG_NONE;
-}
-
 /* Flips of flat pattern t into the staged codeword. */
 __device__ __forceinline__ void apply_flat_flips(const OrbgDeviceCode &code, uint32_t t,
                                                  const uint8_t *pi, uint8_t *cw)
@@ -904,62 +866,39 @@ __device__ __forceinline__ void apply_flat_flips(const OrbgDeviceCode &code, uin
     }
 }
 
-/* First group of `tb` holding a query >= q (reach is non-decreasing). */
-__device__ __forceinline__ uint32_t group_reaching(const OrbgTable &tb, uint32_t q)
-{
-    uint32_t lo = 0, hi = tb.ngroups;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (__ldg(tb.group_reach + mid) >= q)
-            hi = mid;
-        else
-            lo = mid + 1;
-    }
-    return lo;
-}
-
 /* ------------------------------------------------ one warp, one block */
 
 /*
- * Decode one block with one warp over the warp table.  Groups are walked
- * from 0 while their floor (the smallest first index of any later run) is
- * below the best hit, at most `cap`, and at most `budget`.  If the walk
- * stops on the budget with the result still open, the block is not
- * written: its index is appended to heavy[] (when heavy != NULL) for
- * decode_block_cta, with its reliability order and starting syndrome in
- * the handover record of the same slot when one is free (hand_cap; bit 63
- * of the heavy[] entry says so).  On the CTA table (TRIP) a walk that
- * reaches groups needing triple sums past the warp's own table
- * (ORBG_X3_WARP_S3) with no hit stops there and is listed the same way,
- * whatever the budget; on the warp table, with budget >= cap every block
- * finishes here.  LS: llr points into shared memory (the batched kernel
- * stages it there).
+ * Decode one block with one warp: the flat table, then the bands
+ * (search_bands) while no hit is known and the next one starts within
+ * `budget`.  A block still open after them is not written: its index is
+ * appended to heavy[] for decode_block_cta, with its reliability order and
+ * starting syndrome in the handover record of the same slot when one is free
+ * (hand_cap; bit 63 of the heavy[] entry says so); with heavy NULL the
+ * caller takes it up.  Returns whether the block was written.  LS: llr
+ * points into shared memory (the batched kernel stages it there).
  */
-template <int K, int W, bool LS = false, bool TRIP = false, bool PF = true, bool ROLL = true,
-          bool STRIDE = true>
-__device__ void decode_block_warp(const OrbgDeviceCode &code, const float *__restrict__ llr,
+template <int K, int W, bool LS = false, bool ROLL = true>
+__device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__restrict__ llr,
                                   uint8_t *__restrict__ cw_out, uint32_t *__restrict__ q_out,
                                   uint8_t *__restrict__ ab_out, uint32_t cap, uint32_t budget,
-                                  unsigned char *__restrict__ bsm, int lane,
+                                  unsigned char *__restrict__ bsm, int lane, uint32_t *set,
                                   unsigned long long *heavy, unsigned long long *heavy_count,
-                                  unsigned long long block_index, uint16_t *X3w = nullptr,
+                                  unsigned long long block_index,
                                   unsigned char *hand = nullptr, uint32_t hand_cap = 0)
 {
     typedef typename Syn<W>::T T;
     const int n = code.n;
-    const OrbgTable &tb = TRIP ? code.cta : code.warp;
     BlockSmem<W> sm(bsm, n);
     uint32_t key[K];
     bool nan;
     const T s0 = load_block<K, W, LS>(code, llr, key, sm.cw, lane, &nan);
-    uint32_t best = ORBG_NONE, my_t = ORBG_NONE, my_run = 0, my_hit = 0;
-    uint32_t handover = 0;
+    PairHit hit{ORBG_NONE, ORBG_NONE, 0u}; /* prefix NONE: a flat-table hit */
+    bool flat_mine = false;
     bool done = true;
-    if (nan) {
-        best = ORBG_NONE - 1; /* marker: NaN block */
-    } else if (sz(s0)) {
-        best = 1u;            /* query 1, the zero pattern, is a codeword */
-    } else {
+    if (!nan && sz(s0)) {
+        hit.t = 1u; /* query 1, the zero pattern, is a codeword */
+    } else if (!nan) {
         /* the flat table: 32 consecutive queries per step, in query order,
          * so the first step with a hit holds the answer.  Ranks are
          * extracted as the steps need them (one more than needed, so that a
@@ -1000,106 +939,41 @@ __device__ void decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     : ORBG_NONE;
             const uint32_t gbest = __reduce_min_sync(FULL_MASK, mine);
             if (gbest != ORBG_NONE) {
-                best = gbest;
-                if (mine == gbest) {
-                    my_t = mine;
-                    my_run = ORBG_NONE; /* a flat-table hit */
-                }
+                hit.t = gbest;
+                flat_mine = mine == gbest;
                 break;
             }
         }
-        if (best == ORBG_NONE && !sorted && cap > code.nflat) {
-            /* leaving the flat table: every rank is needed (unless the
-             * cap ended the search inside it: the walk below then stops at
-             * its first floor, past the cap) */
-            make_keys<K, LS>(llr, n, lane, key);
-            sort_block<K, LS, ROLL>(key, llr, n, lane);
-            build_perm<K, W>(code, key, sm, lane);
+        if (hit.t == ORBG_NONE && cap > code.nflat) {
+            /* leaving the flat table: every rank is needed */
+            if (!sorted) {
+                make_keys<K, LS>(llr, n, lane, key);
+                sort_block<K, LS, ROLL>(key, llr, n, lane);
+                build_perm<K, W>(code, key, sm, lane);
+                __syncwarp();
+            }
+            hit = warp_best(single_hits<W>(code, sm.h, s0, (uint32_t)lane, 32u));
+            uint4 *clear = reinterpret_cast<uint4 *>(set);
+            for (uint32_t i = (uint32_t)lane; i < kWarpSetBytes / 16u; i += 32u)
+                clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
             __syncwarp();
-        }
-        uint32_t stop = ORBG_NONE;
-        if (best == ORBG_NONE) {
-            /* then the runs, from the first group past the flat table; the
-             * budget (and, on the CTA table, the warp's own triple table)
-             * only ends the walk while no hit is known */
-            const uint32_t g0 = tb.flat_group;
-            int built = 5;         /* triple sums whose X3 entries exist */
-            uint32_t x3lim = 0;    /* X3 entries built */
-            /* PF: group g + 1's runs, floor and triple need are loaded while
-             * g is searched (costs registers: off where they are short) */
-            uint4 n0, n1;
-            uint32_t nfloor = 0;
-            int nneed = 0;
-            if (PF) {
-                load_run(tb, g0 * ORBG_GROUP + (uint32_t)lane, &n0, &n1);
-                nfloor = g0 < tb.ngroups ? __ldg(tb.group_floor + g0) : ORBG_NONE;
-                nneed = TRIP && g0 < tb.ngroups ? (int)__ldg(tb.group_s3 + g0) : 0;
-            }
-            for (uint32_t g = g0; g < tb.ngroups; g++) {
-                uint4 v0, v1;
-                uint32_t floor;
-                int need_g = 0;
-                if (PF) {
-                    floor = nfloor;
-                    need_g = nneed;
-                    v0 = n0;
-                    v1 = n1;
-                } else {
-                    floor = __ldg(tb.group_floor + g);
-                }
-                if (floor >= best || floor > cap || (best == ORBG_NONE && floor > budget)) {
-                    stop = floor;
+            uint32_t tested = code.nflat + 1u, np = 0;
+            bool zero = false;
+#pragma unroll 1
+            for (int k = 0; k < ORBG_BANDS; k++) {
+                if (hit.t < tested || tested > cap || tested > budget)
                     break;
-                }
-                if (PF && g + 1u < tb.ngroups) {
-                    load_run(tb, (g + 1u) * ORBG_GROUP + (uint32_t)lane, &n0, &n1);
-                    nfloor = __ldg(tb.group_floor + g + 1u);
-                    if (TRIP)
-                        nneed = (int)__ldg(tb.group_s3 + g + 1u);
-                }
-                if (TRIP) {
-                    const int need = PF ? need_g : (int)__ldg(tb.group_s3 + g);
-                    if (need > built) {
-                        if (best == ORBG_NONE && need > ORBG_X3_WARP_S3) {
-                            stop = floor;
-                            break;
-                        }
-                        const int upto = min(need, ORBG_X3_WARP_S3);
-                        if (upto > built) {
-                            const uint32_t lo = __ldg(code.x3off + built + 1);
-                            x3lim = __ldg(code.x3off + upto + 1);
-                            build_x3(code, sm.h0, X3w, lo, x3lim, (uint32_t)lane, 32u);
-                            __syncwarp();
-                            built = upto;
-                        }
-                    }
-                }
-                if (!PF)
-                    load_run(tb, g * ORBG_GROUP + (uint32_t)lane, &v0, &v1);
-                uint32_t hv = 0;
-                uint32_t mine;
-                if (TRIP)
-                    mine = search_run_cta<W, STRIDE>(v0, v1, sm.h, sm.h0, X3w, x3lim, code.trip, s0,
-                                             best, cap, n, code.exact16 != 0, &hv);
-                else
-                    mine = search_run_warp<W, STRIDE>(v0, v1, sm.h, sm.h0, s0, best, cap, n, &hv);
-                const uint32_t gbest = __reduce_min_sync(FULL_MASK, mine);
-                if (gbest < best) {
-                    best = gbest;
-                    if (mine == gbest) {
-                        my_t = mine;
-                        my_run = g * ORBG_GROUP + (uint32_t)lane;
-                        my_hit = hv;
-                    }
-                }
+                if (code.band_end[k] <= tested)
+                    continue;
+                hit = search_band<W>(code, sm, s0, cap, k, np, set, lane, hit, &zero);
+                np = code.band_pairs[k];
+                tested = code.band_end[k];
             }
+            done = hit.t < tested || tested > cap;
         }
-        done = stop >= best || stop > cap; /* exhausted tables give stop = NONE */
-        handover = stop;
     }
     if (!done) {
-        /* every query below `handover` was tested without a hit; the block
-         * is fully sorted here (the walk past the flat table sorts it) */
+        /* the block is fully sorted here */
         if (heavy != nullptr) {
             unsigned long long slot = 0;
             if (lane == 0)
@@ -1118,19 +992,17 @@ __device__ void decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     *reinterpret_cast<T *>(rec + 256) = s0;
             }
             if (lane == 0)
-                heavy[slot] = block_index | ((unsigned long long)handover << 32) |
-                              (keep ? 1ull << 63 : 0ull);
+                heavy[slot] = block_index | (keep ? 1ull << 63 : 0ull);
         }
         __syncwarp();
-        return;
+        return false;
     }
-    const bool is_nan = best == ORBG_NONE - 1;
-    const bool hit = !is_nan && best <= cap;
-    if (hit && my_t == best) {
-        if (my_run == ORBG_NONE)
-            apply_flat_flips(code, my_t, sm.pi, sm.cw);
-        else
-            apply_flips<STRIDE>(tb, my_run, my_hit, code.trip, sm.pi, sm.cw);
+    const bool found = !nan && hit.t <= cap;
+    if (found) {
+        if (flat_mine)
+            apply_flat_flips(code, hit.t, sm.pi, sm.cw);
+        else if (hit.pre != ORBG_NONE && lane == 0)
+            apply_pair_flips(code, hit, sm.pi, sm.cw);
     }
     __syncwarp();
 #pragma unroll
@@ -1140,36 +1012,41 @@ __device__ void decode_block_warp(const OrbgDeviceCode &code, const float *__res
             cw_out[i] = sm.cw[i];
     }
     if (lane == 0) {
-        *q_out = is_nan ? 0u : hit ? best : cap;
-        *ab_out = is_nan ? 2 : hit ? 0 : 1;
+        *q_out = nan ? 0u : found ? hit.t : cap;
+        *ab_out = nan ? 2 : found ? 0 : 1;
     }
     __syncwarp();
+    return true;
 }
 
 /* ------------------------------------------------ one CTA, one block */
 
 /*
- * All warps of the CTA decode one block over the CTA table.  Warp 0 loads
- * and sorts; all threads then fill the triple table X3 from the permuted
- * first-word columns; then warp w walks groups w, w + nw, w + 2 nw, ...
- * Each warp stops at its first group whose floor is at least the shared
- * best (or above the cap): floors never decrease with the group index and
- * the best never increases, so no group that could hold the final best is
- * skipped.
+ * All warps of the CTA decode one block.  Its order comes from phase 1's
+ * handover record, or warp 0 loads and sorts; all threads then build the
+ * subset tables of the light positions and the hash set of the block's pairs
+ * (several sets in turn for an order of more than kPairChunk pairs); then
+ * warp w looks up the prefixes of groups w, w + nw, w + 2 nw, ...  Each warp
+ * stops at its first group whose floor is at least the shared best (or above
+ * the cap): floors never decrease with the group index and the best never
+ * increases, so no group that could hold the final best is skipped.
+ * pair_sm: pair_smem_bytes(code.npairs) bytes.
  */
-template <int K, int W, bool STRIDE = true>
+template <int K, int W>
 __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__restrict__ llr,
                                  uint8_t *__restrict__ cw_out, uint32_t *__restrict__ q_out,
                                  uint8_t *__restrict__ ab_out, uint32_t cap,
-                                 unsigned char *__restrict__ bsm, uint16_t *__restrict__ X3,
-                                 uint32_t *s_best, typename Syn<W>::T *s_s0, uint32_t from,
+                                 unsigned char *__restrict__ bsm, unsigned char *pair_sm,
+                                 uint32_t *s_best, uint32_t *s_zero, typename Syn<W>::T *s_s0,
                                  int warp, int lane, int nwarps,
                                  const unsigned char *__restrict__ rec = nullptr)
 {
     typedef typename Syn<W>::T T;
     const int n = code.n;
-    const OrbgTable &tb = code.cta;
     BlockSmem<W> sm(bsm, n);
+    uint32_t *mask = reinterpret_cast<uint32_t *>(pair_sm);
+    uint32_t *set = reinterpret_cast<uint32_t *>(pair_sm + kMaskBytes);
+    const uint32_t bits = pair_slot_bits(code.npairs);
     if (rec != nullptr) {
         /* phase 1's handover record: the block's order and starting
          * syndrome; every thread takes a share of the positions */
@@ -1180,7 +1057,7 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
             const T col = load_col<W>(code.hcol, idx);
             sm.h[i] = col;
             if (W > 1)
-                sm.h0[i] = first_word(col);
+                sm.h0[i] = syn_key(col);
         }
         if (threadIdx.x == 0) {
             sm.h[-1] = szero<T>();
@@ -1206,83 +1083,99 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
             }
         }
     }
+    if (threadIdx.x == 0)
+        *s_zero = 0u;
     __syncthreads();
     const uint32_t start = *s_best;
-    if (start == ORBG_NONE)
-        build_x3(code, sm.h0, X3, 0u, code.ntrip, threadIdx.x, blockDim.x);
     __syncthreads();
-    uint32_t my_t = ORBG_NONE, my_run = 0, my_hit = 0;
+    PairHit mine{ORBG_NONE, ORBG_NONE, 0u};
     if (start == ORBG_NONE) {
         const T s0 = *s_s0;
-        bool stopped = false;
-        uint32_t g = (uint32_t)warp;
-        if (from <= code.nflat) {
-            /* flat table, steps interleaved over the warps: a warp that sees
-             * a hit, or a step at or past the best, has nothing left to do
-             * below the best (every query <= nflat is some warp's step) */
-            for (uint32_t base = 32u * (uint32_t)warp; base < code.nflat && base < cap;
-                 base += 32u * (uint32_t)nwarps) {
-                if (base + 1u >= *((volatile uint32_t *)s_best)) {
-                    stopped = true;
-                    break;
-                }
-                const uint32_t mine = flat_query<W>(code, sm.h, sm.h0, s0, base, cap, lane);
-                const uint32_t gbest = __reduce_min_sync(FULL_MASK, mine);
-                if (gbest != ORBG_NONE) {
-                    if (mine == gbest) {
-                        my_t = mine;
-                        my_run = ORBG_NONE;
-                        atomicMin(s_best, mine);
-                    }
-                    stopped = true;
-                    break;
-                }
+        const uint32_t s0w = syn_key(s0);
+        mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x);
+        if (mine.t != ORBG_NONE)
+            atomicMin(s_best, mine.t);
+        for (uint32_t e = threadIdx.x; e < 512u; e += blockDim.x) {
+            uint32_t v = 0;
+#pragma unroll
+            for (int b = 0; b < 8; b++) {
+                const int p = (int)__ldg(code.light + (e >> 8) * 8u + (uint32_t)b);
+                if (e >> b & 1u)
+                    v ^= sm.h0[p - 1];
             }
-            g += tb.flat_group;
-        } else {
-            /* every query below `from` was tested by the warp pass */
-            g += group_reaching(tb, from);
+            mask[e] = v;
         }
-        if (!stopped) {
-            uint4 n0, n1;
-            load_run(tb, g * ORBG_GROUP + (uint32_t)lane, &n0, &n1);
-            uint32_t nfloor = g < tb.ngroups ? __ldg(tb.group_floor + g) : ORBG_NONE;
-            for (; g < tb.ngroups; g += (uint32_t)nwarps) {
-                const uint32_t floor = nfloor;
+        const uint2 *gm = reinterpret_cast<const uint2 *>(code.gmeta);
+        const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre);
+#pragma unroll 1
+        for (uint32_t lo = 0; lo < code.npairs; lo += kPairChunk) {
+            const uint32_t hi = min(code.npairs, lo + kPairChunk);
+            uint4 *clear = reinterpret_cast<uint4 *>(set);
+            for (uint32_t i = threadIdx.x; i < (1u << bits) / 4u; i += blockDim.x)
+                clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+            __syncthreads();
+            for (uint32_t id = lo + threadIdx.x; id < hi; id += blockDim.x)
+                if (insert_pair<W>(code, sm, set, bits, lo, id))
+                    *s_zero = 1u;
+            __syncthreads();
+            const bool zero = W > 1 && *s_zero != 0u;
+            uint32_t g = (uint32_t)warp;
+            uint2 nm = make_uint2(ORBG_NONE, 0u), nr = make_uint2(0u, 0u);
+            if (g < code.ngroups) {
+                nm = __ldg(gm + g);
+                nr = __ldg(pre + g * ORBG_GROUP + (uint32_t)lane);
+            }
+#pragma unroll 1
+            for (; g < code.ngroups; g += (uint32_t)nwarps) {
+                const uint2 m = nm, r = nr;
                 const uint32_t best = *((volatile uint32_t *)s_best);
-                if (floor >= best || floor > cap)
+                if (m.x >= best || m.x > cap)
                     break;
-                const uint4 v0 = n0, v1 = n1;
                 /* the warp's next group, loaded while this one is searched */
                 const uint32_t gn = g + (uint32_t)nwarps;
-                load_run(tb, gn * ORBG_GROUP + (uint32_t)lane, &n0, &n1);
-                nfloor = gn < tb.ngroups ? __ldg(tb.group_floor + gn) : ORBG_NONE;
-                uint32_t hv = 0;
-                const uint32_t mine =
-                    search_run_cta<W, STRIDE>(v0, v1, sm.h, sm.h0, X3, code.ntrip, code.trip, s0, best,
-                                      cap, n, code.exact16 != 0, &hv);
-                const uint32_t gbest = __reduce_min_sync(FULL_MASK, mine);
-                if (gbest != ORBG_NONE) {
-                    if (mine == gbest) {
-                        my_t = mine;
-                        my_run = g * ORBG_GROUP + (uint32_t)lane;
-                        my_hit = hv;
-                        atomicMin(s_best, mine);
+                if (gn < code.ngroups) {
+                    nm = __ldg(gm + gn);
+                    nr = __ldg(pre + gn * ORBG_GROUP + (uint32_t)lane);
+                }
+                const uint32_t i = g * ORBG_GROUP + (uint32_t)lane;
+                uint32_t v = s0w ^ mask[r.x & 0xFFu] ^ mask[256u + ((r.x >> 8) & 0xFFu)];
+                const int kmax = (int)(m.y & 0xFFu);
+#pragma unroll
+                for (int j = 0; j < ORBG_PRE_POS; j++) {
+                    if (j >= kmax)
+                        break;
+                    const uint32_t p = j < 2 ? r.x >> (16 + 8 * j) : r.y >> (8 * (j - 2));
+                    v ^= sm.h0[(int)(p & 0xFFu) - 1];
+                }
+                if (kmax > ORBG_PRE_POS) {
+                    const uint2 x = __ldg(reinterpret_cast<const uint2 *>(code.pext) + i);
+                    for (int j = 0; j < 8; j++)
+                        v ^= sm.h0[(int)(((j < 4 ? x.x : x.y) >> (8 * (j & 3))) & 0xFFu) - 1];
+                }
+                const uint32_t e = find_pair(set, bits, v);
+                if ((e != kEmpty || (W > 1 && v == 0u && zero)) && i < code.npre) {
+                    uint32_t pair = 0;
+                    const uint32_t t = resolve_pair<W>(
+                        code, sm.h, s0, i, e != kEmpty ? lo + (e & kIdMask) : ORBG_NONE, lo, hi,
+                        &pair);
+                    if (t < mine.t) {
+                        mine.t = t;
+                        mine.pre = i;
+                        mine.pair = pair;
+                        atomicMin(s_best, t);
                     }
                 }
+                __syncwarp();
             }
+            __syncthreads(); /* the set is free before the next chunk's pairs */
         }
     }
     __syncthreads();
     const uint32_t best = *s_best;
     const bool is_nan = best == ORBG_NONE - 1;
     const bool hit = !is_nan && best <= cap;
-    if (start == ORBG_NONE && hit && my_t == best) {
-        if (my_run == ORBG_NONE)
-            apply_flat_flips(code, my_t, sm.pi, sm.cw);
-        else
-            apply_flips<STRIDE>(tb, my_run, my_hit, code.trip, sm.pi, sm.cw);
-    }
+    if (start == ORBG_NONE && hit && mine.t == best)
+        apply_pair_flips(code, mine, sm.pi, sm.cw);
     __syncthreads();
     for (int i = warp * 32 + lane; i < n; i += nwarps * 32)
         cw_out[i] = sm.cw[i];

@@ -19,7 +19,7 @@ using namespace orbg_dev;
 #define ORBG_PHASE2_MIN_CTAS 2
 #endif
 
-template <int KMAX, int WMAX, bool ONE, bool STRIDE>
+template <int KMAX, int WMAX, bool ONE>
 __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
     const OrbgDeviceCode *__restrict__ codes, int ncodes, const int32_t *__restrict__ code_id,
     const int64_t *__restrict__ llr_off, const float *__restrict__ llr, uint32_t cap,
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_block, s_slot;
-    __shared__ uint32_t s_best;
+    __shared__ uint32_t s_best, s_zero;
     __shared__ uint4 s_s0;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
         if (threadIdx.x == 0) {
             const unsigned long long nheavy = *((volatile unsigned long long *)&counters[1]);
             const unsigned long long slot = atomicAdd(&counters[2], 1ull);
-            /* block | tested-below << 32 | handover record << 63 */
+            /* block | handover record << 63 */
             /* code sets take the list from its end: its phase-1 launches run
              * by decoder variant, shortest codes first, so the longest codes'
              * blocks, which search longest, list last and start first here */
@@ -53,23 +53,22 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
         if (bb == ~0ull)
             break; /* uniform: every thread read the same s_block */
         const int64_t b = (int64_t)(bb & 0xFFFFFFFFull);
-        const uint32_t from = (uint32_t)((bb >> 32) & 0x7FFFFFFFull);
         const unsigned char *rec = (bb >> 63) ? hand + s_slot * ORBG_HANDOVER_BYTES : nullptr;
         const int64_t lo = llr_off ? llr_off[b] : b * n0;
         const int64_t co = cw_off ? cw_off[b] : b * n0;
         if (ONE) {
-            decode_block_cta<KMAX, WMAX, STRIDE>(code0, llr + lo, cw + co, q + b, ab + b, cap, smem,
-                                         reinterpret_cast<uint16_t *>(smem + bstride), &s_best,
-                                         reinterpret_cast<typename Syn<WMAX>::T *>(&s_s0), from,
-                                         warp, lane, nwarps, rec);
+            decode_block_cta<KMAX, WMAX>(code0, llr + lo, cw + co, q + b, ab + b, cap, smem,
+                                         smem + bstride, &s_best, &s_zero,
+                                         reinterpret_cast<typename Syn<WMAX>::T *>(&s_s0), warp,
+                                         lane, nwarps, rec);
             continue;
         }
         const int cid = code_id ? code_id[b] : 0; /* checked in phase 1 */
-        const OrbgDeviceCode code = codes[cid];
-#define ORBG_CALL_CTA(KK, WW)                                                               \
-    decode_block_cta<KK, WW, STRIDE>(code, llr + lo, cw + co, q + b, ab + b, cap, smem,              \
-                             reinterpret_cast<uint16_t *>(smem + bstride), &s_best,          \
-                             reinterpret_cast<typename Syn<WW>::T *>(&s_s0), from, warp, lane,  \
+        const OrbgDeviceCode &code = codes[cid];
+#define ORBG_CALL_CTA(KK, WW)                                                             \
+    decode_block_cta<KK, WW>(code, llr + lo, cw + co, q + b, ab + b, cap, smem,           \
+                             smem + bstride, &s_best, &s_zero,                            \
+                             reinterpret_cast<typename Syn<WW>::T *>(&s_s0), warp, lane,  \
                              nwarps, rec)
         ORBG_DISPATCH(KMAX, WMAX, ORBG_CALL_CTA);
 #undef ORBG_CALL_CTA
@@ -77,14 +76,15 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
     (void)ncodes;
 }
 
-template <int KMAX, int WMAX, bool ONE, bool STRIDE>
-cudaError_t launch_heavy_k(const OrbgBatchedArgs &a, unsigned long long *counters,
+template <int KMAX, int WMAX, bool ONE>
+cudaError_t launch_heavy_t(const OrbgBatchedArgs &a, unsigned long long *counters,
                            const unsigned long long *heavy, const unsigned char *hand)
 {
-    auto k2 = orbg_heavy_kernel<KMAX, WMAX, ONE, STRIDE>;
-    const int hw = a.heavy_warps > 0 ? a.heavy_warps : 16;
+    auto k2 = orbg_heavy_kernel<KMAX, WMAX, ONE>;
+    const int hw = a.heavy_warps > 0 ? a.heavy_warps : 8;
+    /* 16-byte aligned: block_smem_bytes is a multiple of 16 */
     const uint32_t bstride = block_smem_bytes(a.n_max, a.w32_max);
-    const size_t smem = (size_t)bstride + triple_table_bytes(a.ntrip_max);
+    const size_t smem = (size_t)bstride + pair_smem_bytes(a.npairs_max);
     int grid = 0;
     int rc = orbg_grid_for((const void *)k2, hw * 32, smem, 0, &grid);
     if (rc != 0)
@@ -97,19 +97,6 @@ cudaError_t launch_heavy_k(const OrbgBatchedArgs &a, unsigned long long *counter
                                                         a.q, a.ab, counters, heavy, hand, bstride,
                                                         c0);
     return cudaGetLastError();
-}
-
-/* One code: strided runs always handled (no cost measured there); code
- * sets: the kernel with them only where a code has them. */
-template <int KMAX, int WMAX, bool ONE>
-cudaError_t launch_heavy_t(const OrbgBatchedArgs &a, unsigned long long *counters,
-                           const unsigned long long *heavy, const unsigned char *hand)
-{
-    if constexpr (ONE)
-        return launch_heavy_k<KMAX, WMAX, true, true>(a, counters, heavy, hand);
-    else
-        return a.has_stride ? launch_heavy_k<KMAX, WMAX, false, true>(a, counters, heavy, hand)
-                            : launch_heavy_k<KMAX, WMAX, false, false>(a, counters, heavy, hand);
 }
 
 }  // namespace orbg_batched_impl

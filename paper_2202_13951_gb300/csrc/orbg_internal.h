@@ -2,69 +2,49 @@
  * orbg_internal.h -- data shared between the host side of the library and
  * its CUDA kernels.
  *
- * The query order (Sec. III-B: increasing logistic weight W; this library's
- * tie reading: Hamming weight w ascending, then positions lexicographic) is
- * held as tables of "runs" of consecutive query indices.  Two tables per
- * code, each covering the whole order:
+ * The query order (position weights rho_j of the sorted positions; patterns
+ * by increasing weight, then Hamming weight w, then positions) is held per
+ * code as prefixes and pairs.  A pattern of weight w >= 2 is its prefix P,
+ * the first w - 2 positions, and the pair a < b of the last two.  With h_j
+ * the parity-check column of sorted position j, it is a hit iff h_a ^ h_b =
+ * s0 ^ sum over P of h: the pairs of a block go into a hash set of their
+ * syndromes, and one look-up per prefix then tests every pattern the prefix
+ * starts, of whatever weight.  A search up to 1,004,225 queries (cap 1e6, n
+ * >= 82) makes 15,552 look-ups over 1,640 pairs.
  *
- * Warp table (one warp decodes a block):
- *   kind 0  one pattern of weight 0 or 1 (the prefix is the pattern);
- *   kind 1  a prefix v_1 < ... < v_{w-2} and every pair a < b <= n after it
- *           with a + b = S, a ascending from a_lo;
- *   kind 2  (m-segment orders) a prefix and the pairs (a_0 + j da, b_0 - j db),
- *           j = 0, 1, ...: a pair whose positions lie in two segments of
- *           slopes beta, beta' with beta da = beta' db keeps its weight.
- * CTA table (a CTA decodes a block and first builds the block's triple
- * table X3: the first syndrome word of every triple c < a < b <= n with
- * c + a + b <= S3max, ordered by that sum, then c, then a):
- *   kind 0  as above;
- *   kind 1  as above, used for w = 2 and for triples beyond S3max;
- *   kind 3  a prefix v_1 < ... < v_{w-3} and every triple after it with
- *           c + a + b = S3: a contiguous range of X3, tested against one
- *           prefix syndrome.  Cut into chunks of at most 8..255 queries
- *           (longer deeper in the order).
- * Runs are stored class by class ((W, w) ascending); inside a class they are
- * sorted by length so that the 32 lanes of a warp, which take 32
- * consecutive runs, loop for about the same number of queries.  Every run
- * keeps its own first query index, so the decoder still reports the first
- * hit of the paper's order; a group floor (the smallest first index over
- * runs of groups >= g) tells a warp when no later group can hold an earlier
- * hit.
+ * Only one pair per syndrome matters, the first in the order (weight, a, b):
+ * if the first hit of the order is P + {a, b} and a pair {c, d} before {a, b}
+ * has the same syndrome, then exchanging {a, b} for {c, d} (both flipped
+ * twice cancel) gives a hit that is lighter, or as heavy with fewer
+ * positions, or as heavy and as many and lexicographically smaller.  For the
+ * same reason a look-up that finds a pair not wholly after its prefix can
+ * be passed over.
+ *
+ * The prefixes are listed by the least weight m(P) of a pattern they start;
+ * the floor of a group of 32, the first query index of that weight, bounds
+ * from below every hit of it and later groups, which ends a search.  The
+ * index of P + {a, b}: start[] holds, per prefix and group of equally heavy
+ * pairs, the index of the first one after P, and the pairs of a group
+ * follow in the order of a.
  */
 #ifndef ORBG_INTERNAL_H
 #define ORBG_INTERNAL_H
 
 #include <stdint.h>
 
-#define ORBG_GROUP 32          /* runs per warp step: one per lane */
-#define ORBG_RUN_MAX_PRE 20    /* prefix positions stored per run */
-#define ORBG_MAX_LOGISTIC 255  /* deepest logistic weight a table may reach */
-#define ORBG_X3_MAX 16384      /* triple-table entries (32 KiB of shared memory, 16 bits each) */
-#define ORBG_X3_WARP_S3 44     /* triple sums a phase-1 warp keeps in its own table */
+#define ORBG_GROUP 32          /* prefixes per warp step: one per lane */
+#define ORBG_MAX_FLIPS 22      /* largest Hamming weight of an order's patterns */
+#define ORBG_MAX_LOGISTIC 255  /* deepest logistic weight of a line's order */
+#define ORBG_PRE_POS 6         /* positions of a prefix record besides the sixteen lightest */
 
-enum { ORBG_RUN_SINGLE = 0, ORBG_RUN_PAIRS = 1, ORBG_RUN_STRIDE = 2, ORBG_RUN_TRIPLES = 3 };
-
-/* One run: 32 bytes, read by a lane as two 16-byte loads. */
-struct OrbgRun {
-    uint32_t tstart;    /* 1-based query index of the run's first pattern */
-    uint16_t count;     /* patterns in the run, >= 1 */
-    uint8_t npre;       /* prefix positions used */
-    uint8_t kind;       /* ORBG_RUN_* */
-    uint32_t aux;       /* kind 1: S | a_lo << 8 (1-based); kind 2: a_0 | b_0 << 8 | da << 16 |
-                         * db << 24 (pattern j's pair is a_0 + j da, b_0 - j db); kind 3:
-                         * first X3 index */
-    uint8_t pre[ORBG_RUN_MAX_PRE]; /* 1-based prefix positions, ascending; 0 = unused */
-};
-
-struct OrbgTable {
-    const OrbgRun *runs;         /* [nruns] */
-    const uint32_t *group_floor; /* [ngroups] */
-    const uint32_t *group_reach; /* [ngroups]: largest query index in groups <= g */
-    const uint8_t *group_s3;     /* [ngroups]: largest triple sum any run in groups <= g reads */
-    uint32_t nruns;
-    uint32_t ngroups;
-    uint32_t flat_group;         /* first group holding a query beyond the flat table */
-};
+/* Phase 1 (one warp a block) searches in bands: the pairs of the leading
+ * pair groups, and the prefixes that lie before the first group left out.
+ * For basic ORBGRAND the bands end after logistic weights 31 and 45 (queries
+ * 2,375 and 16,857), with 225 and 484 pairs, 84 and 438 prefixes. */
+#define ORBG_BANDS 2
+#define ORBG_BAND1_PAIRS 225
+#define ORBG_BAND2_PAIRS 500
+#define ORBG_PRE1_MAX 1024
 
 /* The flat table: the first `nflat` patterns of the order, 8 bytes each:
  * up to 7 positions, 1-based (0 = unused), then a byte describing the
@@ -79,14 +59,25 @@ struct OrbgTable {
 /* What a kernel needs of one code (passed by value or from a device array). */
 struct OrbgDeviceCode {
     const uint32_t *hcol;        /* [n][w32]: column j of H, row i at bit i%32 of word i/32 */
-    OrbgTable warp;              /* runs of kinds 0, 1 */
-    OrbgTable cta;               /* runs of kinds 0, 1, 3 */
-    const uint32_t *trip;        /* [ntrip]: c0 | a0 << 8 | b0 << 16 (0-based), X3 order */
-    const uint32_t *x3off;       /* [s3max + 2]: first X3 index of each triple sum */
-    uint32_t ntrip;
-    int32_t s3max;               /* largest triple sum in X3 */
-    uint32_t x3w;                /* X3 entries of sums <= ORBG_X3_WARP_S3 (a warp's own table) */
-    int32_t exact16;             /* n - k <= 16: 16-bit X3 entries are whole syndromes */
+    const uint16_t *pairs;       /* [npairs] a0 | b0 << 8, 0-based, by (weight, a, b) */
+    const uint32_t *pinfo;       /* [npairs] its group of equally heavy pairs | first pair of the
+                                  * group << 16 */
+    const uint32_t *pre;         /* [2 * npre, padded to groups] prefix records, 8 bytes: bit i
+                                  * position light[i], then ORBG_PRE_POS further positions,
+                                  * 1-based, 0 = none */
+    const uint32_t *pext;        /* NULL, or as pre: eight positions past those */
+    const uint32_t *pre1;        /* as pre: all positions of a prefix of up to eight */
+    const uint32_t *gmeta;       /* [2 * ngroups] floor of the group; the most positions of its
+                                  * pre (low byte) and pre1 records (next byte) */
+    const uint32_t *pmeta;       /* [2 * (npre + 1)] first entry of the prefix in start[]; its
+                                  * last position | the first pair group after it << 16 */
+    const uint32_t *start;       /* query index of the first pair of a (prefix, group) */
+    const uint32_t *single;      /* [n] query index of each single position, 0 = past the table */
+    const uint8_t *light;        /* [16] the lightest positions, 1-based, 0 = none */
+    uint32_t npairs, npre, ngroups;
+    uint32_t npre1;              /* leading prefixes phase 1 may walk */
+    uint32_t band_pairs[ORBG_BANDS]; /* pairs of each band */
+    uint32_t band_end[ORBG_BANDS];   /* first query index past the band */
     const uint32_t *flat;        /* [2 * nflat] flat-table patterns, 8 bytes each */
     uint32_t nflat;
     uint32_t max_cap;
@@ -95,27 +86,21 @@ struct OrbgDeviceCode {
     int32_t w32;                 /* syndrome words: 1, 2 or 4 */
 };
 
-#ifdef __cplusplus
-static_assert(sizeof(OrbgRun) == 32, "run record must be 32 bytes");
-#endif
-
 /* Host-side table builder (orbg_tables.cpp). */
 #ifdef __cplusplus
+#include <functional>
 #include <vector>
+/* The arrays of OrbgDeviceCode, see there. */
 struct OrbgTables {
-    std::vector<OrbgRun> runs;           /* warp table */
-    std::vector<uint32_t> group_floor;
-    std::vector<OrbgRun> runs_cta;       /* CTA table */
-    std::vector<uint32_t> group_floor_cta;
-    std::vector<uint32_t> trip;          /* X3 order */
+    std::vector<uint16_t> pairs, pgroup; /* pgroup: a pair's group */
+    std::vector<uint32_t> pinfo;
+    std::vector<uint64_t> pre, pre1, pext;
+    std::vector<uint32_t> gmeta, pmeta, start, single;
+    uint8_t light[16] = {};
     std::vector<uint8_t> flat;           /* 8 bytes per pattern */
-    std::vector<uint32_t> reach, reach_cta;
-    std::vector<uint8_t> s3_cta;         /* group_s3 of the CTA table */
-    std::vector<uint32_t> x3off;
-    int s3max = 0;
-    uint32_t nflat = 0, flat_group = 0, flat_group_cta = 0;
+    uint32_t npre = 0, npre1 = 0, nflat = 0;
+    uint32_t band_pairs[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
     uint64_t patterns = 0;  /* query indices covered (last index) */
-    int wmax_logistic = 0;  /* deepest logistic weight in the table */
 };
 /* The tables for the order of increasing reliability weight J0 w + beta W
  * (one-line full ORBGRAND; J0 = 0, beta = 1 is basic ORBGRAND). */
@@ -133,10 +118,12 @@ struct OrbgModel {
     long beta[ORBG_MAX_SEG];
 };
 /* The tables for the m-segment order (reliability weight, then Hamming
- * weight, then positions lexicographically): single, pair and strided pair
- * runs. */
+ * weight, then positions lexicographically). */
 int orbg_build_tables_model(int n, uint64_t cap, const OrbgModel &md, OrbgTables *out);
-int orbg_run_pattern(const OrbgRun &r, int j, const uint32_t *trip, int *v);
+/* Calls f(t, positions, w) for every pattern of query index t <= count, in
+ * no particular order: positions 1-based, ascending. */
+void orbg_expand_tables(const OrbgTables &tb, int n, uint64_t count,
+                        const std::function<void(uint32_t, const int *, int)> &f);
 
 /* GF(2) helpers on dense 0/1 byte matrices (row-major). */
 int orbg_gf2_rank(const uint8_t *M, int rows, int cols);
@@ -168,7 +155,6 @@ struct OrbgBatchedArgs {
     const OrbgDeviceCode *code0;
     int ncodes, n_max, w32_max;
     OrbgVariants var;            /* the set's decoder variants (mixed-code calls) */
-    int has_stride;              /* a code of the set has strided pair runs (kind 2) */
     const int32_t *code_id;
     const int64_t *llr_off;
     const float *llr;
@@ -180,7 +166,7 @@ struct OrbgBatchedArgs {
     uint8_t *ab;
     unsigned long long *scratch;
     int warps_per_cta, ctas_per_sm, grab, heavy_warps;
-    uint32_t ntrip_max, x3w_max;
+    uint32_t npairs_max;         /* most pairs of a code of the set */
     void *stream;
     /* Staged calls (the host-buffer pipeline: phase 1 chunk by chunk as the
      * LLRs arrive, then one phase 2 over every chunk's open blocks).
@@ -206,8 +192,7 @@ struct OrbgScratch;
 #define ORBG_DECLARE_BATCHED(K, W)                                                   \
     int orbg_launch_batched_k##K##w##W(const OrbgBatchedArgs &a);                    \
     int orbg_launch_exact_k##K##w##W(const OrbgBatchedArgs &a, const OrbgScratch &s, \
-                                     unsigned long long *queue, int blo, int bhi, int pdl, \
-                                     int stride);
+                                     unsigned long long *queue, int blo, int bhi, int pdl);
 ORBG_DECLARE_BATCHED(1, 1) ORBG_DECLARE_BATCHED(1, 2) ORBG_DECLARE_BATCHED(1, 4)
 ORBG_DECLARE_BATCHED(2, 1) ORBG_DECLARE_BATCHED(2, 2) ORBG_DECLARE_BATCHED(2, 4)
 ORBG_DECLARE_BATCHED(4, 1) ORBG_DECLARE_BATCHED(4, 2) ORBG_DECLARE_BATCHED(4, 4)
@@ -267,7 +252,7 @@ int orbg_launch_code_sort(const int32_t *code_id, const int32_t *bucket, int64_t
                           const OrbgScratch &s, void *stream);
 /* orbg_launch_exact_k*w* for keys per lane K and syndrome words W. */
 int orbg_launch_exact(int K, int W, const OrbgBatchedArgs &a, const OrbgScratch &s,
-                      unsigned long long *queue, int blo, int bhi, int pdl, int stride);
+                      unsigned long long *queue, int blo, int bhi, int pdl);
 /* Outputs of the blocks phase 2 decoded, gathered after the last launch of a
  * batch whose other results already went to the host.  At `out` (memory the
  * device writes, here host-mapped) the heavy list's length (uint64).  With
@@ -310,9 +295,7 @@ struct OrbgSetView {
     OrbgDeviceCode code0;        /* host copy of code 0's descriptor */
     int ncodes, n_max, w32_max;
     OrbgVariants var;
-    int has_stride;
-    uint32_t ntrip_max;
-    uint32_t x3w_max;
+    uint32_t npairs_max;
     uint32_t cap_min;
     orbg_tuning tuning;
 };

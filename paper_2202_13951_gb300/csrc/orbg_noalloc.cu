@@ -117,7 +117,6 @@ extern "C" int orbg_decode_batched_noalloc(const orbg_codeset *set, const int32_
     a.ncodes = v.ncodes;
     a.n_max = v.n_max;
     a.var = v.var;
-    a.has_stride = v.has_stride;
     a.w32_max = v.w32_max;
     a.code_id = code_id;
     a.llr_off = llr_offset;
@@ -134,8 +133,7 @@ extern "C" int orbg_decode_batched_noalloc(const orbg_codeset *set, const int32_
     a.ctas_per_sm = v.tuning.ctas_per_sm;
     a.grab = v.tuning.blocks_per_grab;
     a.heavy_warps = v.tuning.heavy_warps;
-    a.ntrip_max = v.ntrip_max;
-    a.x3w_max = v.x3w_max;
+    a.npairs_max = v.npairs_max;
     a.stream = cuda_stream;
     e = orbg_launch_batched(a);
     return e != 0 ? orbg_note_cuda_error(e) : ORBG_OK;

@@ -1,6 +1,9 @@
 /*
  * orbg_plain.cu -- the plain form: one launch, one warp per block in a static
- * grid (Algorithm 1 per block; see orbg_decode_block.cuh).
+ * grid (Algorithm 1 per block; see orbg_decode_block.cuh).  A block that its
+ * warp's bands leave open is searched by the whole CTA once all its warps
+ * are through (the CTA's pair set then takes over their shared memory): one
+ * warp alone would hold the launch for a search of a million queries.
  */
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -11,39 +14,65 @@ using namespace orbg_dev;
 
 namespace {
 
+constexpr int kPlainWarps = 8;
+
 template <int K, int W>
-__global__ void __launch_bounds__(256) orbg_plain_kernel(OrbgDeviceCode code,
-                                                         const float *__restrict__ llr,
-                                                         int64_t B, uint32_t cap,
-                                                         uint8_t *__restrict__ cw,
-                                                         uint32_t *__restrict__ q,
-                                                         uint8_t *__restrict__ ab,
-                                                         uint32_t wstride)
+__global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
+    const __grid_constant__ OrbgDeviceCode code, const float *__restrict__ llr, int64_t B,
+    uint32_t cap, uint8_t *__restrict__ cw, uint32_t *__restrict__ q, uint8_t *__restrict__ ab,
+    uint32_t bstride)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_best, s_zero;
+    __shared__ uint4 s_s0;
+    __shared__ uint32_t s_open;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (b >= B)
-        return; /* whole warp */
-    const int64_t off = b * (int64_t)code.n;
-    decode_block_warp<K, W, false, false, true, (K >= 8)>(code, llr + off, cw + off, q + b,
-                                                          ab + b, cap, cap, smem + warp * wstride,
-                                                          lane, nullptr, nullptr, 0ull);
+    const int64_t b0 = (int64_t)blockIdx.x * kPlainWarps;
+    if (threadIdx.x == 0)
+        s_open = 0u;
+    __syncthreads();
+    const int64_t b = b0 + warp;
+    if (b < B) {
+        const int64_t off = b * (int64_t)code.n;
+        unsigned char *own = smem + warp * (bstride + kWarpSetBytes);
+        const bool done = decode_block_warp<K, W, false, (K >= 8)>(
+            code, llr + off, cw + off, q + b, ab + b, cap, cap, own, lane,
+            reinterpret_cast<uint32_t *>(own + bstride), nullptr, nullptr, 0ull);
+        if (!done && lane == 0)
+            atomicOr(&s_open, 1u << warp);
+    }
+    __syncthreads();
+    for (uint32_t open = s_open; open; open &= open - 1u) {
+        const int64_t bo = b0 + __ffs(open) - 1;
+        const int64_t off = bo * (int64_t)code.n;
+        decode_block_cta<K, W>(code, llr + off, cw + off, q + bo, ab + bo, cap, smem,
+                               smem + bstride, &s_best, &s_zero,
+                               reinterpret_cast<typename Syn<W>::T *>(&s_s0), warp, lane,
+                               kPlainWarps);
+    }
 }
 
 template <int K, int W>
 cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t B, uint32_t cap,
                            uint8_t *cw, uint32_t *q, uint8_t *ab, cudaStream_t st)
 {
-    const int wpc = 8;
-    uint32_t wstride = block_smem_bytes(code.n, W);
-    size_t smem = (size_t)wstride * wpc;
-    int64_t grid = (B + wpc - 1) / wpc;
+    const uint32_t bstride = block_smem_bytes(code.n, W);
+    size_t smem = (size_t)(bstride + kWarpSetBytes) * kPlainWarps;
+    const size_t cta = (size_t)bstride + pair_smem_bytes(code.npairs);
+    if (smem < cta)
+        smem = cta;
+    int64_t grid = (B + kPlainWarps - 1) / kPlainWarps;
     if (grid > 0x7FFFFFFF)
         return cudaErrorInvalidValue;
-    orbg_plain_kernel<K, W><<<(unsigned)grid, wpc * 32, smem, st>>>(code, llr, B, cap, cw, q, ab,
-                                                                      wstride);
+    auto k = orbg_plain_kernel<K, W>;
+    if (smem > 47 * 1024) { /* static + dynamic past 48 KB: opt in */
+        const cudaError_t e = cudaFuncSetAttribute(
+            k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess)
+            return e;
+    }
+    k<<<(unsigned)grid, kPlainWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, bstride);
     return cudaGetLastError();
 }
 

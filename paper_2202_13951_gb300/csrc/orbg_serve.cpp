@@ -277,7 +277,6 @@ bool dispatch_one(orbg_server *s)
         a.ncodes = s->view.ncodes;
         a.n_max = s->view.n_max;
         a.var = s->view.var;
-        a.has_stride = s->view.has_stride;
         a.w32_max = s->view.w32_max;
         a.code_id = reinterpret_cast<const int32_t *>(d + bt.L.code_id);
         a.llr_off = reinterpret_cast<const int64_t *>(d + bt.L.llr_off);
@@ -294,8 +293,7 @@ bool dispatch_one(orbg_server *s)
         a.ctas_per_sm = s->view.tuning.ctas_per_sm;
         a.grab = s->view.tuning.blocks_per_grab;
         a.heavy_warps = s->view.tuning.heavy_warps;
-        a.ntrip_max = s->view.ntrip_max;
-        a.x3w_max = s->view.x3w_max;
+        a.npairs_max = s->view.npairs_max;
         a.stream = st;
         le = orbg_launch_batched(a);
     }

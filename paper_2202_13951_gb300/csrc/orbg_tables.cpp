@@ -1,289 +1,436 @@
 /*
  * orbg_tables.cpp -- host-side tables of the query order, and GF(2) helpers.
  *
- * The order is basic ORBGRAND's (Sec. III-B): logistic weight
- * W = sum_i v_i over the flipped sorted positions v (Eq. lw) ascending,
- * split by Hamming weight w (Eq. fractionation) ascending, and inside one
- * (W, w) the distinct-part partitions v_1 < ... < v_w <= n of W (Eq.
- * intpart) in lexicographic order, the order Algorithm 2 (Landslide)
- * generates.  This file enumerates that order directly, as lexicographic
- * prefixes followed by a run of pairs or of triples (see orbg_internal.h),
- * not with Landslide.  The one-line order of full ORBGRAND (Sec. III-D)
- * reorders the same (W, w) classes; the m-segment order (Eq. relest_seg)
- * is built pattern by pattern (orbg_build_tables_model).
+ * Every order this library decodes in is one of position weights: sorted
+ * position j weighs rho_j >= 0 (basic ORBGRAND, Sec. III-B: rho_j = j; one
+ * line, Sec. III-D: J_0 + beta j; m segments, Eq. relest_seg), and noise
+ * patterns come in increasing weight R = sum of rho over the flipped
+ * positions, then Hamming weight w, then positions lexicographically.  The
+ * tables (orbg_internal.h) name every pattern of weight w >= 2 as a prefix,
+ * its first w - 2 positions, and the pair of its last two, and give each
+ * one's index in that order.
  */
 #include <algorithm>
+#include <cstdint>
 #include <cstring>
-#include <queue>
 #include <vector>
 
 #include "orbg_internal.h"
 
 namespace {
 
-/* Pairs a < b <= n (1-based) with a + b = S and a >= lo: a in
- * [max(lo, S - n), (S - 1) / 2]. */
-inline int pair_lo(int S, int lo, int n) { return std::max(lo, S - n); }
-inline int pair_hi(int S) { return (S - 1) / 2; }
+/* Patterns counted up to this many are counted exactly. */
+constexpr uint64_t kCountMax = 1ull << 40;
+/* Weights up to here are counted by one array over the weights. */
+constexpr long kDenseMax = 4096;
 
-/* Triples c < a < b <= n with c + a + b = S3 and c >= lo: the c that admit a
- * pair form [max(lo, S3 - (2n - 1)), (S3 - 3) / 3]. */
-inline int trip_c_lo(int S3, int lo, int n) { return std::max(lo, S3 - (2 * n - 1)); }
-inline int trip_c_hi(int S3) { return (S3 - 3) / 3; }
+/* One prefix during the build. */
+struct Prefix {
+    long R;        /* its weight */
+    long m;        /* least weight of a pattern it starts */
+    int32_t up;    /* the prefix without its last position, -1 for the empty one */
+    int16_t q;     /* its last position, 0 for the empty one */
+    uint8_t len;
+    uint8_t extra; /* positions outside the sixteen lightest */
+};
 
-/* Longest chunk a triple run starting at query t is cut into: short early
- * in the order (a warp step over 32 chunks should not overshoot a hit by
- * much) and long deep in it (the per-chunk setup is amortised). */
-int chunk_len(uint64_t t)
-{
-    const uint64_t c = t / 512;
-    return (int)(c < 8 ? 8 : c > 255 ? 255 : c);
-}
-
-struct Builder {
+/* The patterns of an order given by position weights. */
+struct Order {
     int n;
-    bool cta;                      /* build the CTA table (triple runs) */
-    int s3max = 0;                 /* triple sums covered by X3 */
-    const std::vector<uint32_t> *x3off = nullptr; /* first X3 index of each sum */
-    uint64_t t = 1;                /* next query index */
-    std::vector<OrbgRun> cls;      /* runs of the current (W, w) class */
-    int pre[64];
-    bool overflow = false;
-    long J0 = 0, beta = 1;         /* the line: reliability J0 + beta j */
-
-    OrbgRun blank(int kind, int npre) {
-        OrbgRun r;
-        std::memset(&r, 0, sizeof(r));
-        r.tstart = (uint32_t)t;
-        r.kind = (uint8_t)kind;
-        r.npre = (uint8_t)npre;
-        for (int i = 0; i < npre; i++) {
-            overflow |= pre[i] > 255; /* a byte holds positions 1..255 */
-            r.pre[i] = (uint8_t)pre[i]; /* 1-based; 0 marks an unused slot */
+    const std::vector<long> &rho;   /* [n + 1], rho[j] of position j = 1..n */
+    std::vector<long> x;            /* the weights ascending */
+    explicit Order(int n_, const std::vector<long> &rho_) : n(n_), rho(rho_), x(rho_.begin() + 1,
+                                                                               rho_.end())
+    {
+        std::sort(x.begin(), x.end());
+    }
+    /* patterns of weight <= R with least rank >= k (the empty one left out),
+     * at least `most` if there are that many */
+    uint64_t count_from(size_t k, long R, uint64_t most) const
+    {
+        const size_t end = (size_t)(std::upper_bound(x.begin() + (long)k, x.end(), R) - x.begin());
+        uint64_t c = end - k;
+        for (size_t i = k; i + 1 < end && c < most; i++) {
+            if (x[i] + x[i + 1] > R)
+                break;
+            c += count_from(i + 1, R - x[i], most - c);
         }
-        return r;
+        return c;
     }
-
-    void emit(OrbgRun r, uint64_t count) {
-        if (count > 0xFFFF || count == 0) {
-            overflow |= count > 0xFFFF;
-            return;
+    /* The least weight up to which there are at least `cap` patterns (the
+     * heaviest pattern's if there are fewer in all), and the number of
+     * patterns up to it. */
+    long depth(uint64_t cap, uint64_t *patterns) const
+    {
+        long all = 0;
+        for (long w : x)
+            all += w;
+        const long top = std::min(all, kDenseMax);
+        std::vector<uint64_t> c((size_t)top + 1, 0);
+        c[0] = 1;
+        long reach = 0;
+        for (long w : x) {
+            reach = std::min(top, reach + w);
+            for (long R = reach; R >= w; R--)
+                c[(size_t)R] = std::min(kCountMax, c[(size_t)R] + c[(size_t)(R - w)]);
         }
-        r.count = (uint16_t)count;
-        cls.push_back(r);
-        t += count;
-    }
-
-    void single(int np) { emit(blank(ORBG_RUN_SINGLE, np), 1); }
-
-    /* pairs of sum S after a prefix of `depth` positions ending at q */
-    void pairs(int depth, int q, int S) {
-        const int lo = pair_lo(S, q + 1, n), hi = pair_hi(S);
-        if (lo > hi)
-            return;
-        OrbgRun r = blank(ORBG_RUN_PAIRS, depth);
-        r.aux = (uint32_t)S | ((uint32_t)lo << 8);
-        emit(r, (uint64_t)(hi - lo + 1));
-    }
-
-    /* triples of sum S3 after a prefix ending at q: one X3 range, chunked */
-    void triples(int depth, int q, int S3) {
-        const int c_lo = trip_c_lo(S3, q + 1, n), c_hi = trip_c_hi(S3);
-        if (c_lo > c_hi)
-            return;
-        /* X3 index of the first triple with c >= c_lo, and the range length */
-        uint32_t x = (*x3off)[S3];
-        for (int c = trip_c_lo(S3, 1, n); c < c_lo; c++)
-            x += (uint32_t)(pair_hi(S3 - c) - pair_lo(S3 - c, c + 1, n) + 1);
-        uint64_t total = 0;
-        for (int c = c_lo; c <= c_hi; c++)
-            total += (uint64_t)(pair_hi(S3 - c) - pair_lo(S3 - c, c + 1, n) + 1);
-        while (total > 0) {
-            const uint64_t len = std::min<uint64_t>(total, (uint64_t)chunk_len(t));
-            OrbgRun r = blank(ORBG_RUN_TRIPLES, depth);
-            r.aux = x;
-            emit(r, len);
-            x += (uint32_t)len;
-            total -= len;
+        uint64_t sum = 0;
+        long last = 0;
+        for (long R = 0; R <= top; R++) {
+            if (!c[(size_t)R])
+                continue;
+            sum = std::min(kCountMax, sum + c[(size_t)R]);
+            last = R;
+            if (sum >= cap || (top == all && R == all)) {
+                *patterns = sum;
+                return last;
+            }
         }
-    }
-
-    /* Prefixes of `need` more positions, each >= lo, with `rem` left for
-     * them and the final `tail` (2 = pair, 3 = triple) positions. */
-    void prefixes(int depth, int need, int lo, int rem, int tail) {
-        if (need == 0) {
-            if (tail == 2)
-                pairs(depth, lo - 1, rem);
+        long lo = top + 1, hi = all; /* the depth is in [lo, hi] */
+        while (lo < hi) {
+            const long mid = lo + (hi - lo) / 2;
+            if (1 + count_from(0, mid, cap) >= cap)
+                hi = mid;
             else
-                triples(depth, lo - 1, rem);
-            return;
+                lo = mid + 1;
         }
-        const int m = need - 1 + tail; /* positions after v, all above it */
-        for (int v = lo; v <= n; v++) {
-            long min_rest = (long)m * v + (long)m * (m + 1) / 2;
-            long max_rest = (long)m * n - (long)m * (m - 1) / 2;
-            if (v + min_rest > rem)
-                break;
-            if (v + max_rest < rem)
-                continue;
-            pre[depth] = v;
-            prefixes(depth + 1, need - 1, v + 1, rem - v, tail);
-        }
-    }
-
-    void flush(std::vector<OrbgRun> *out) {
-        /* longest runs first; equal lengths keep the query order */
-        std::stable_sort(cls.begin(), cls.end(),
-                         [](const OrbgRun &a, const OrbgRun &b) {
-                             return a.count > b.count;
-                         });
-        out->insert(out->end(), cls.begin(), cls.end());
-        cls.clear();
-    }
-
-    /* The whole order up to the class holding query `cap`: classes (W, w)
-     * of logistic weight W and Hamming weight w in increasing reliability
-     * weight R = J0 w + beta W (one-line full ORBGRAND, Sec. III-D; basic
-     * ORBGRAND is J0 = 0, beta = 1, R = W), w ascending within R. */
-    int build(uint64_t cap, std::vector<OrbgRun> *out, uint64_t *patterns, int *wdeep) {
-        t = 1;
-        single(0); /* R = 0: the zero pattern */
-        flush(out);
-        *wdeep = 0;
-        const long Rlast = J0 * n + beta * ((long)n * (n + 1) / 2);
-        for (long R = 1; R <= Rlast && t <= cap; R++) {
-            for (int w = 1; w <= n; w++) {
-                if (R - J0 * w < 0)
-                    break;                 /* larger w only weigh more */
-                if ((R - J0 * w) % beta)
-                    continue;              /* no integer logistic weight */
-                const long W = (R - J0 * w) / beta;
-                if (W < (long)w * (w + 1) / 2)
-                    break;                 /* below the lightest w-subset */
-                if (W > (long)w * (w + 1) / 2 + (long)w * (n - w))
-                    continue;              /* above the heaviest w-subset */
-                if (W > ORBG_MAX_LOGISTIC)
-                    return -2;
-                if (w == 1) {
-                    if (W <= n) {
-                        pre[0] = (int)W;
-                        single(1);
-                    }
-                } else if (cta && w >= 3) {
-                    /* triple runs where the prefix leaves a sum inside X3,
-                     * pair runs (prefix extended by c) where it does not */
-                    if (w - 2 > ORBG_RUN_MAX_PRE)
-                        return -2;
-                    prefixes_split(0, w - 3, 1, (int)W);
-                } else {
-                    if (w - 2 > ORBG_RUN_MAX_PRE)
-                        return -2;
-                    prefixes(0, w - 2, 1, (int)W, 2);
-                }
-                flush(out);
-                *wdeep = std::max(*wdeep, (int)W);
-            }
-        }
-        *patterns = t - 1;
-        return overflow ? -2 : 0;
-    }
-
-    /* CTA table, w >= 3: (w-3)-prefixes in lexicographic order; each one's
-     * triples become an X3 range if their sum fits X3, else the prefix is
-     * extended by every valid c (in order) and the pairs after it form
-     * pair runs -- the same patterns in the same order. */
-    void prefixes_split(int depth, int need, int lo, int rem) {
-        if (need == 0) {
-            if (rem <= s3max) {
-                triples(depth, lo - 1, rem);
-            } else {
-                const int c_lo = trip_c_lo(rem, lo, n), c_hi = trip_c_hi(rem);
-                for (int c = c_lo; c <= c_hi; c++) {
-                    pre[depth] = c;
-                    pairs(depth + 1, c, rem - c);
-                }
-            }
-            return;
-        }
-        const int m = need - 1 + 3;
-        for (int v = lo; v <= n; v++) {
-            long min_rest = (long)m * v + (long)m * (m + 1) / 2;
-            long max_rest = (long)m * n - (long)m * (m - 1) / 2;
-            if (v + min_rest > rem)
-                break;
-            if (v + max_rest < rem)
-                continue;
-            pre[depth] = v;
-            prefixes_split(depth + 1, need - 1, v + 1, rem - v);
-        }
+        *patterns = 1 + count_from(0, lo, kCountMax);
+        return lo;
     }
 };
 
-/* reach[g]: the largest query index in groups 0..g; and the first group
- * holding a query beyond `nflat` */
-void reaches(const std::vector<OrbgRun> &runs, uint32_t nflat, std::vector<uint32_t> *out,
-             uint32_t *flat_group)
-{
-    const size_t nr = runs.size();
-    const size_t ng = (nr + ORBG_GROUP - 1) / ORBG_GROUP;
-    out->assign(ng, 0u);
-    uint32_t reach = 0;
-    *flat_group = (uint32_t)ng;
-    for (size_t g = 0; g < ng; g++) {
-        bool beyond = false;
-        for (size_t i = g * ORBG_GROUP; i < std::min(nr, (g + 1) * ORBG_GROUP); i++) {
-            const uint32_t last = runs[i].tstart + runs[i].count - 1u;
-            reach = std::max(reach, last);
-            beyond |= last > nflat;
+struct TableBuilder {
+    int n;
+    std::vector<long> rho;          /* [n + 2] */
+    long Rmax = 0;
+    OrbgTables *out;
+    std::vector<long> sufpair;      /* least pair weight over q < a < b */
+    std::vector<long> gsum;         /* weight of each pair group */
+    std::vector<uint8_t> is_light;  /* [n + 1] one of the sixteen lightest */
+    std::vector<Prefix> pre;        /* in lexicographic (depth-first) order */
+    bool monotone = true;
+
+    void make_pairs()
+    {
+        std::vector<std::pair<long, uint32_t>> v;
+        for (int a = 1; a < n; a++)
+            for (int b = a + 1; b <= n; b++)
+                if (rho[(size_t)a] + rho[(size_t)b] <= Rmax)
+                    v.push_back({rho[(size_t)a] + rho[(size_t)b],
+                                 (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1)});
+        std::sort(v.begin(), v.end());
+        for (const auto &e : v) {
+            if (gsum.empty() || gsum.back() != e.first)
+                gsum.push_back(e.first);
+            out->pairs.push_back((uint16_t)((e.second >> 8) | (e.second & 0xFFu) << 8));
+            out->pgroup.push_back((uint16_t)(gsum.size() - 1));
+            const size_t k = out->pgroup.size() - 1;
+            const uint32_t first = k && out->pgroup[k] == out->pgroup[k - 1]
+                                       ? out->pinfo[k - 1] >> 16
+                                       : (uint32_t)k;
+            out->pinfo.push_back((uint32_t)out->pgroup[k] | first << 16);
         }
-        (*out)[g] = reach;
-        if (beyond && *flat_group == ng)
-            *flat_group = (uint32_t)g;
-    }
-}
-
-void floors(const std::vector<OrbgRun> &runs, std::vector<uint32_t> *out)
-{
-    const size_t nr = runs.size();
-    const size_t ng = (nr + ORBG_GROUP - 1) / ORBG_GROUP;
-    out->assign(ng, 0xFFFFFFFFu);
-    uint32_t floor = 0xFFFFFFFFu;
-    for (size_t g = ng; g-- > 0;) {
-        for (size_t i = g * ORBG_GROUP; i < std::min(nr, (g + 1) * ORBG_GROUP); i++)
-            floor = std::min(floor, runs[i].tstart);
-        (*out)[g] = floor;
-    }
-}
-
-/* Group floors and reaches, the flat table and the CTA table's triple
- * needs, from the two run tables (and X3) of `out`. */
-void finish_tables(OrbgTables *out)
-{
-    const uint64_t patterns = out->patterns;
-    const int s3max = out->s3max;
-    floors(out->runs, &out->group_floor);
-    floors(out->runs_cta, &out->group_floor_cta);
-    /* flat table: the leading patterns of weight <= ORBG_FLAT_POS, at most
-     * ORBG_FLAT_MAX of them, in query order */
-    std::vector<std::vector<int>> first((size_t)std::min<uint64_t>(patterns, ORBG_FLAT_MAX));
-    std::vector<int> v(64);
-    for (const OrbgRun &r : out->runs)
-        for (int j = 0; j < r.count; j++) {
-            const uint64_t t = (uint64_t)r.tstart + (uint64_t)j;
-            if (t <= first.size()) {
-                const int w = orbg_run_pattern(r, j, out->trip.data(), v.data());
-                first[t - 1].assign(v.begin(), v.begin() + w);
+        sufpair.assign((size_t)n + 2, INT64_MAX / 4);
+        long least = INT64_MAX / 4; /* lightest single position after a */
+        for (int a = n - 1; a >= 0; a--) {
+            /* pairs with least position a + 1 */
+            if (a + 2 <= n) {
+                least = std::min(least, rho[(size_t)a + 2]);
+                sufpair[(size_t)a] = std::min(sufpair[(size_t)a + 1], rho[(size_t)a + 1] + least);
             }
         }
-    uint32_t nflat = 0;
-    while (nflat < first.size() && first[nflat].size() <= ORBG_FLAT_POS)
-        nflat++;
-    /* per step of 32 patterns: the ranks it needs in sorted order (its
-     * largest position, non-decreasing over the steps; the table ends before
-     * the first step needing more than ORBG_FLAT_RANKS) and its largest
-     * Hamming weight */
-    std::vector<uint8_t> need;
+    }
+
+    /* every prefix that starts a pattern of weight <= Rmax */
+    void make_prefixes()
     {
+        struct Step {
+            int id, v;
+        };
+        std::vector<Step> st;
+        if (n < 2 || sufpair[0] > Rmax)
+            return;
+        pre.push_back(Prefix{0, sufpair[0], -1, 0, 0, 0});
+        st.push_back(Step{0, 1});
+        while (!st.empty()) {
+            const int id = st.back().id, v = st.back().v;
+            const long R = pre[(size_t)id].R;
+            if (v + 2 > n || R + sufpair[(size_t)v] > Rmax ||
+                (monotone && R + rho[(size_t)v] + sufpair[(size_t)v] > Rmax)) {
+                st.pop_back(); /* no later position leads to a pattern either */
+                continue;
+            }
+            st.back().v++;
+            const long m = R + rho[(size_t)v] + sufpair[(size_t)v];
+            if (m > Rmax)
+                continue;
+            Prefix p{R + rho[(size_t)v], m, id, (int16_t)v, (uint8_t)(pre[(size_t)id].len + 1),
+                     (uint8_t)(pre[(size_t)id].extra + (is_light[(size_t)v] ? 0 : 1))};
+            pre.push_back(p);
+            st.push_back(Step{(int)pre.size() - 1, v + 1});
+        }
+    }
+
+    /* A model's order is limited to patterns of 20 positions, and of 22 where
+     * the last two can be written as a + j da, b - j db of one run of
+     * patterns with bytes for a and b.  Is any pattern outside that? */
+    bool past_model_limit() const
+    {
+        for (const Prefix &p : pre) {
+            if (p.len < ORBG_MAX_FLIPS - 3)
+                continue;
+            for (size_t k = 0; k < out->pairs.size();) {
+                size_t e = k;
+                std::vector<std::pair<int, int>> run;
+                for (; e < out->pairs.size() && out->pgroup[e] == out->pgroup[k]; e++) {
+                    const int a = (out->pairs[e] & 0xFF) + 1, b = (out->pairs[e] >> 8) + 1;
+                    if (a > p.q)
+                        run.push_back({a, b});
+                }
+                if (p.R + gsum[out->pgroup[k]] > Rmax)
+                    break;
+                for (size_t s = 0; s < run.size();) {
+                    int da = 1, db = 1;
+                    if (s + 1 < run.size()) {
+                        da = run[s + 1].first - run[s].first;
+                        db = run[s].second - run[s + 1].second;
+                    }
+                    if (da < 1 || db < 1)
+                        da = db = 1;
+                    size_t f = s + 1;
+                    while (f < run.size() &&
+                           run[f].first == run[s].first + da * (int)(f - s) &&
+                           run[f].second == run[s].second - db * (int)(f - s))
+                        f++;
+                    const bool pairs = da == 1 && db == 1 &&
+                                       run[s].first + run[s].second <= 255;
+                    if (!pairs && (f - s < 2 || run[s].second > 255))
+                        return true;
+                    s = f;
+                }
+                k = e;
+            }
+        }
+        return false;
+    }
+
+    /* positions of prefix id, ascending */
+    int positions(int id, int *v) const
+    {
+        const int w = pre[(size_t)id].len;
+        for (int i = w - 1; i >= 0; i--) {
+            v[i] = pre[(size_t)id].q;
+            id = pre[(size_t)id].up;
+        }
+        return w;
+    }
+
+    /* first query index of the patterns of weight R and more */
+    std::vector<std::pair<long, uint32_t>> first_of; /* (weight, first index), ascending */
+    uint32_t first_at(long R) const
+    {
+        const auto it = std::lower_bound(first_of.begin(), first_of.end(),
+                                         std::make_pair(R, (uint32_t)0));
+        return it == first_of.end() ? (uint32_t)out->patterns + 1u : it->second;
+    }
+
+    int build(bool model)
+    {
+        const int light_n = std::min(n, 16);
+        std::vector<std::pair<long, int>> by;
+        for (int j = 1; j <= n; j++) {
+            by.push_back({rho[(size_t)j], j});
+            monotone &= j == 1 || rho[(size_t)j] >= rho[(size_t)j - 1];
+        }
+        std::sort(by.begin(), by.end());
+        is_light.assign((size_t)n + 1, 0);
+        std::vector<int> bit((size_t)n + 1, 0);
+        std::memset(out->light, 0, sizeof(out->light));
+        for (int i = 0; i < light_n; i++) {
+            const int j = by[(size_t)i].second;
+            out->light[i] = (uint8_t)j; /* at most position 256 of n = 256, cut below */
+            is_light[(size_t)j] = 1;
+            bit[(size_t)j] = i;
+            if (j > 255)
+                is_light[(size_t)j] = 0, out->light[i] = 0; /* no prefix holds position 256 */
+        }
+        make_pairs();
+        make_prefixes();
+        if (model && past_model_limit())
+            return -2;
+        const uint32_t npre = (uint32_t)pre.size();
+        /* the prefixes by the least weight they start; equal ones by the
+         * loads they cost */
+        std::vector<uint32_t> ord(npre);
+        for (uint32_t i = 0; i < npre; i++)
+            ord[i] = i;
+        std::stable_sort(ord.begin(), ord.end(), [&](uint32_t a, uint32_t b) {
+            return pre[a].m != pre[b].m ? pre[a].m < pre[b].m : pre[a].extra < pre[b].extra;
+        });
+        /* per last position q: the first group with a pair after q, and how
+         * many pairs after q each group from there on holds */
+        const uint32_t ngrp = (uint32_t)gsum.size();
+        std::vector<std::vector<uint16_t>> after((size_t)n + 1);
+        std::vector<uint32_t> g0((size_t)n + 1, 0);
+        std::vector<uint32_t> place(npre); /* of lexicographic prefix i in the final order */
+        out->pmeta.resize(2 * ((size_t)npre + 1));
+        uint64_t rows = 0;
+        for (uint32_t i = 0; i < npre; i++) {
+            const Prefix &p = pre[ord[i]];
+            place[ord[i]] = i;
+            const size_t q = (size_t)p.q;
+            if (after[q].empty()) {
+                std::vector<uint16_t> c(ngrp, 0);
+                for (size_t k = 0; k < out->pairs.size(); k++)
+                    c[out->pgroup[k]] += (size_t)(out->pairs[k] & 0xFFu) + 1 > q;
+                uint32_t g = 0;
+                while (c[g] == 0)
+                    g++;
+                g0[q] = g;
+                after[q].assign(c.begin() + g, c.end());
+            }
+            out->pmeta[2 * i] = (uint32_t)rows;
+            out->pmeta[2 * i + 1] = (uint32_t)p.q | g0[q] << 16;
+            const uint32_t g1 = (uint32_t)(std::upper_bound(gsum.begin(), gsum.end(), Rmax - p.R) -
+                                           gsum.begin());
+            rows += g1 - g0[q];
+        }
+        out->pmeta[2 * (size_t)npre] = (uint32_t)rows;
+        out->pmeta[2 * (size_t)npre + 1] = 0;
+        out->start.assign((size_t)rows, 0u);
+        out->single.assign((size_t)n, 0u);
+        /* the runs (prefix, group) and the single positions, ordered by
+         * (weight, w); generated in lexicographic order, which a stable sort
+         * keeps inside one (weight, w) */
+        struct Run {
+            uint32_t at;    /* entry of start[], or of single[] */
+            uint16_t count; /* patterns; 0 marks a single position */
+        };
+        std::vector<Run> runs;
+        std::vector<uint64_t> key;
+        for (int j = 1; j <= n; j++)
+            if (rho[(size_t)j] <= Rmax) {
+                runs.push_back(Run{(uint32_t)j - 1u, 0});
+                key.push_back((uint64_t)rho[(size_t)j] << 5 | 1u);
+            }
+        for (uint32_t l = 0; l < npre; l++) {
+            const uint32_t i = place[l];
+            const uint32_t lo = out->pmeta[2 * i], hi = out->pmeta[2 * i + 2];
+            const size_t q = (size_t)pre[l].q;
+            for (uint32_t k = lo; k < hi; k++) {
+                const uint16_t c = after[q][k - lo];
+                if (!c)
+                    continue;
+                runs.push_back(Run{k, c});
+                key.push_back((uint64_t)(pre[l].R + gsum[g0[q] + (k - lo)]) << 5 |
+                              (uint64_t)(pre[l].len + 2));
+            }
+        }
+        std::vector<uint32_t> ro(runs.size());
+        if (Rmax <= kDenseMax) {
+            std::vector<uint32_t> c((size_t)(Rmax + 1) * 32 + 1, 0);
+            for (uint64_t k : key)
+                c[(size_t)k + 1]++;
+            for (size_t k = 1; k < c.size(); k++)
+                c[k] += c[k - 1];
+            for (size_t r = 0; r < runs.size(); r++)
+                ro[c[(size_t)key[r]]++] = (uint32_t)r;
+        } else {
+            for (size_t r = 0; r < runs.size(); r++)
+                ro[r] = (uint32_t)r;
+            std::stable_sort(ro.begin(), ro.end(),
+                             [&](uint32_t a, uint32_t b) { return key[a] < key[b]; });
+        }
+        uint32_t t = 2; /* the zero pattern is query 1 */
+        first_of.push_back({0, 1u});
+        for (uint32_t r : ro) {
+            const long R = (long)(key[r] >> 5);
+            if (R != first_of.back().first)
+                first_of.push_back({R, t});
+            if (runs[r].count) {
+                out->start[runs[r].at] = t;
+                t += runs[r].count;
+            } else {
+                out->single[runs[r].at] = t++;
+            }
+        }
+        /* the records the kernels read, 32 prefixes to a group */
+        const uint32_t ng = (npre + ORBG_GROUP - 1) / ORBG_GROUP;
+        out->npre = npre;
+        out->pre.assign((size_t)ng * ORBG_GROUP, 0);
+        out->pre1.assign((size_t)ng * ORBG_GROUP, 0);
+        out->gmeta.assign(2 * (size_t)ng, 0);
+        uint32_t npre1 = npre; /* leading prefixes a phase-1 warp walks */
+        int v[64];
+        for (uint32_t i = 0; i < npre; i++) {
+            const Prefix &p = pre[ord[i]];
+            positions((int)ord[i], v);
+            uint64_t rec = 0, rec1 = 0, ext = 0;
+            int x = 0;
+            for (int k = 0; k < p.len; k++) {
+                if (is_light[(size_t)v[k]]) {
+                    rec |= 1ull << bit[(size_t)v[k]];
+                } else {
+                    if (x < ORBG_PRE_POS)
+                        rec |= (uint64_t)v[k] << (16 + 8 * x);
+                    else
+                        ext |= (uint64_t)v[k] << (8 * (x - ORBG_PRE_POS));
+                    x++;
+                }
+                if (k < 8)
+                    rec1 |= (uint64_t)v[k] << (8 * k);
+            }
+            if (p.len > 8 && npre1 == npre)
+                npre1 = i;
+            out->pre[i] = rec;
+            out->pre1[i] = rec1;
+            if (x > ORBG_PRE_POS) {
+                out->pext.resize((size_t)ng * ORBG_GROUP, 0);
+                out->pext[i] = ext;
+            }
+            uint32_t &gm = out->gmeta[2 * (size_t)(i / ORBG_GROUP) + 1];
+            gm = std::max(gm & 0xFFu, (uint32_t)x) |
+                 std::max(gm >> 8, (uint32_t)std::min<int>(p.len, 8)) << 8;
+            if (i % ORBG_GROUP == 0)
+                out->gmeta[2 * (size_t)(i / ORBG_GROUP)] = first_at(p.m);
+        }
+        npre1 = std::min<uint32_t>(npre1, ORBG_PRE1_MAX);
+        out->npre1 = npre1;
+        /* phase 1's bands: the pairs of the leading groups, and the first
+         * query index not covered by them and the leading prefixes */
+        const uint32_t aim[ORBG_BANDS] = {ORBG_BAND1_PAIRS, ORBG_BAND2_PAIRS};
+        const uint32_t none = (uint32_t)out->patterns + 1u;
+        const uint32_t lim1 = npre1 < npre ? first_at(pre[ord[npre1]].m) : none;
+        for (int k = 0; k < ORBG_BANDS; k++) {
+            uint32_t np = std::min<uint32_t>(aim[k], (uint32_t)out->pairs.size());
+            while (np > 0 && np < out->pairs.size() && out->pgroup[np] == out->pgroup[np - 1])
+                np--;
+            out->band_pairs[k] = np;
+            const uint32_t end =
+                np < out->pairs.size() ? first_at(gsum[out->pgroup[np]]) : none;
+            out->band_end[k] = std::min(end, lim1);
+        }
+        make_flat();
+        return 0;
+    }
+
+    /* Flat table: the leading patterns of weight <= ORBG_FLAT_POS, at most
+     * ORBG_FLAT_MAX of them, in query order. */
+    void make_flat()
+    {
+        const uint32_t most = (uint32_t)std::min<uint64_t>(out->patterns, ORBG_FLAT_MAX);
+        std::vector<std::vector<int>> first((size_t)most);
+        orbg_expand_tables(*out, n, most, [&](uint32_t t, const int *v, int w) {
+            first[t - 1].assign(v, v + w);
+        });
+        uint32_t nflat = 0;
+        while (nflat < first.size() && first[nflat].size() <= ORBG_FLAT_POS)
+            nflat++;
+        /* per step of 32 patterns: the ranks it needs in sorted order (its
+         * largest position, non-decreasing over the steps; the table ends
+         * before the first step needing more than ORBG_FLAT_RANKS) and its
+         * largest Hamming weight */
+        std::vector<uint8_t> need;
         int mx = 0;
         uint32_t keep = 0;
         for (uint32_t base = 0; base < nflat; base += 32) {
@@ -300,38 +447,40 @@ void finish_tables(OrbgTables *out)
             keep = end;
         }
         nflat = keep;
-    }
-    out->nflat = nflat;
-    out->flat.assign((size_t)std::max<uint32_t>(nflat, 1) * 8, 0);
-    for (uint32_t t = 0; t < nflat; t++) {
-        uint8_t *e = &out->flat[(size_t)t * 8];
-        for (size_t i = 0; i < first[t].size(); i++)
-            e[i] = (uint8_t)first[t][i];
-        e[7] = need[t / 32];
-    }
-    reaches(out->runs, nflat, &out->reach, &out->flat_group);
-    reaches(out->runs_cta, nflat, &out->reach_cta, &out->flat_group_cta);
-    /* largest triple sum read by the runs of groups <= g: an X3 index falls
-     * in the sum whose range holds it */
-    {
-        const size_t nr = out->runs_cta.size();
-        const size_t ng = (nr + ORBG_GROUP - 1) / ORBG_GROUP;
-        out->s3_cta.assign(ng, 0);
-        int s3 = 0;
-        for (size_t g = 0; g < ng; g++) {
-            for (size_t i = g * ORBG_GROUP; i < std::min(nr, (g + 1) * ORBG_GROUP); i++) {
-                const OrbgRun &r = out->runs_cta[i];
-                if (r.kind != ORBG_RUN_TRIPLES)
-                    continue;
-                const uint32_t last = r.aux + r.count - 1u;
-                int S = 6;
-                while (S < s3max && out->x3off[S + 1] <= last)
-                    S++;
-                s3 = std::max(s3, S);
-            }
-            out->s3_cta[g] = (uint8_t)s3;
+        out->nflat = nflat;
+        out->flat.assign((size_t)std::max<uint32_t>(nflat, 1) * 8, 0);
+        for (uint32_t t = 0; t < nflat; t++) {
+            uint8_t *e = &out->flat[(size_t)t * 8];
+            for (size_t i = 0; i < first[t].size(); i++)
+                e[i] = (uint8_t)first[t][i];
+            e[7] = need[t / 32];
         }
     }
+};
+
+/* Some pattern of weight <= Rmax flips more than ORBG_MAX_FLIPS positions. */
+bool too_heavy(const Order &o, long Rmax)
+{
+    long s = 0;
+    for (int i = 0; i < o.n && i <= ORBG_MAX_FLIPS; i++)
+        s += o.x[(size_t)i];
+    return o.n > ORBG_MAX_FLIPS && s <= Rmax;
+}
+
+int build_order(int n, const std::vector<long> &rho, uint64_t patterns, long Rmax, bool model,
+                OrbgTables *out)
+{
+    if (patterns >= 0xFFFFFFFFull)
+        return -3;
+    *out = OrbgTables();
+    out->patterns = patterns;
+    TableBuilder b;
+    b.n = n;
+    b.rho = rho;
+    b.rho.push_back(0);
+    b.Rmax = Rmax;
+    b.out = out;
+    return b.build(model);
 }
 
 }  // namespace
@@ -341,226 +490,22 @@ int orbg_build_tables(int n, uint64_t cap, OrbgTables *out, long J0, long beta)
     if (n < 1 || n > 256 || cap < 1 || J0 < 0 || beta < 1 || J0 > ORBG_MAX_LINE ||
         beta > ORBG_MAX_LINE)
         return -1;
-    /* warp table */
-    Builder bw;
-    bw.n = n;
-    bw.cta = false;
-    bw.J0 = J0;
-    bw.beta = beta;
-    out->runs.clear();
+    std::vector<long> rho((size_t)n + 1, 0);
+    for (int j = 1; j <= n; j++)
+        rho[(size_t)j] = J0 + beta * j;
+    const Order o(n, rho);
     uint64_t patterns = 0;
-    int wdeep = 0;
-    int rc = bw.build(cap, &out->runs, &patterns, &wdeep);
-    if (rc)
-        return rc;
-    out->patterns = patterns;
-    out->wmax_logistic = wdeep;
-    if (patterns >= 0xFFFFFFFFull)
-        return -3;
-    /* X3: every triple c < a < b <= n by sum (<= the table's depth, within
-     * ORBG_X3_MAX entries), then c, then a */
-    std::vector<uint32_t> x3off(ORBG_MAX_LOGISTIC + 2, 0);
-    out->trip.clear();
-    int s3max = 0;
-    for (int S3 = 6; S3 <= wdeep; S3++) {
-        size_t cnt = 0;
-        for (int c = trip_c_lo(S3, 1, n); c <= trip_c_hi(S3); c++)
-            cnt += (size_t)(pair_hi(S3 - c) - pair_lo(S3 - c, c + 1, n) + 1);
-        if (out->trip.size() + cnt > ORBG_X3_MAX)
-            break;
-        x3off[S3] = (uint32_t)out->trip.size();
-        for (int c = trip_c_lo(S3, 1, n); c <= trip_c_hi(S3); c++)
-            for (int a = pair_lo(S3 - c, c + 1, n); a <= pair_hi(S3 - c); a++)
-                out->trip.push_back((uint32_t)(c - 1) | ((uint32_t)(a - 1) << 8) |
-                                    ((uint32_t)(S3 - c - a - 1) << 16));
-        s3max = S3;
+    const long Rmax = o.depth(cap, &patterns);
+    if (too_heavy(o, Rmax))
+        return -2;
+    /* lines stop at logistic weight ORBG_MAX_LOGISTIC */
+    for (long w = 1; w <= n; w++) {
+        const long W = std::max<long>(ORBG_MAX_LOGISTIC + 1, w * (w + 1) / 2);
+        if (W <= w * (w + 1) / 2 + w * (n - w) && J0 * w + beta * W <= Rmax)
+            return -2;
     }
-    out->s3max = s3max;
-    out->x3off.assign(x3off.begin(), x3off.begin() + (s3max + 2));
-    out->x3off[s3max + 1] = (uint32_t)out->trip.size();
-    /* CTA table */
-    Builder bc;
-    bc.n = n;
-    bc.cta = true;
-    bc.J0 = J0;
-    bc.beta = beta;
-    bc.s3max = s3max;
-    bc.x3off = &x3off;
-    out->runs_cta.clear();
-    uint64_t patterns_c = 0;
-    int wdeep_c = 0;
-    rc = bc.build(cap, &out->runs_cta, &patterns_c, &wdeep_c);
-    if (rc)
-        return rc;
-    if (patterns_c != patterns)
-        return -5;
-    finish_tables(out);
-    return 0;
+    return build_order(n, rho, patterns, Rmax, false, out);
 }
-
-namespace {
-
-/*
- * m-segment full ORBGRAND (Sec. III-D, Eq. relest_seg): position j of
- * segment i, I_{i-1} < j <= I_i, weighs rho_j = J_{i-1} + beta_i (j -
- * I_{i-1}) >= 0, and patterns come in increasing reliability weight (the
- * sum of rho over the flipped positions), then Hamming weight, then
- * positions lexicographically.
- *
- * Patterns of increasing weight come from a best-first walk over subsets
- * of the positions ranked by weight, x_0 <= x_1 <= ...: a subset whose
- * highest rank is k leads to the subset with rank k + 1 added and to the
- * one with rank k replaced by k + 1.  Every non-empty subset is reached
- * exactly once, from {0}, and never weighs less than the subset it comes
- * from, so a min-heap pops weights in order.  All subsets of one weight R
- * are collected, ordered by (w, positions) and cut into runs: consecutive
- * patterns (p, a, b), (p, a + 1, b - 1), ... with one prefix p become one
- * pair run, and consecutive (p, a, b), (p, a + da, b - db), ... (a pair
- * across two segments whose slopes balance, beta da = beta' db) one strided
- * pair run; the rest are single runs.
- */
-struct ModelBuilder {
-    Builder b;                           /* run records and class flush */
-    std::vector<long> x;                 /* weights by rank, lightest first */
-    std::vector<int> pos;                /* 1-based position of each rank */
-    struct Node {
-        int parent;                      /* the subset without `rank`, -1 = empty */
-        int rank;
-    };
-    std::vector<Node> nodes;
-
-    /* one weight's patterns, back to back: pattern q is pos_all[start[q] ..
-     * start[q] + len[q]) ascending */
-    std::vector<int> pos_all;
-    std::vector<uint32_t> start;
-    std::vector<uint16_t> len;
-    std::vector<uint32_t> order;  /* pattern indices in (w, positions) order */
-
-    int build(uint64_t cap, std::vector<OrbgRun> *out, uint64_t *patterns) {
-        const int n = b.n;
-        typedef std::pair<long, int> Item;   /* (weight, node) */
-        std::priority_queue<Item, std::vector<Item>, std::greater<Item>> heap;
-        nodes.clear();
-        nodes.push_back(Node{-1, 0});
-        heap.push(Item(x[0], 0));
-        b.t = 1;
-        long R = 0;
-        bool first = true;
-        while (b.t <= cap && (first || !heap.empty())) {
-            pos_all.clear();
-            start.clear();
-            len.clear();
-            if (first) {                 /* the empty pattern, weight 0 */
-                start.push_back(0);
-                len.push_back(0);
-            } else {
-                R = heap.top().first;
-            }
-            first = false;
-            while (!heap.empty() && heap.top().first == R) {
-                const int id = heap.top().second;
-                heap.pop();
-                const int k = nodes[id].rank;
-                if (k + 1 < n) {
-                    const int par = nodes[id].parent;
-                    nodes.push_back(Node{id, k + 1});
-                    heap.push(Item(R + x[k + 1], (int)nodes.size() - 1));
-                    nodes.push_back(Node{par, k + 1});
-                    heap.push(Item(R - x[k] + x[k + 1], (int)nodes.size() - 1));
-                }
-                const size_t s0 = pos_all.size();
-                for (int q = id; q >= 0; q = nodes[q].parent)
-                    pos_all.push_back(pos[nodes[q].rank]);
-                std::sort(pos_all.begin() + (long)s0, pos_all.end());
-                start.push_back((uint32_t)s0);
-                len.push_back((uint16_t)(pos_all.size() - s0));
-            }
-            if (nodes.size() > (size_t)1 << 30 || pos_all.size() > 0xFFFFFFFFull)
-                return -2;
-            order.resize(start.size());
-            for (size_t q = 0; q < order.size(); q++)
-                order[q] = (uint32_t)q;
-            std::sort(order.begin(), order.end(), [this](uint32_t p, uint32_t q) {
-                if (len[p] != len[q])
-                    return len[p] < len[q];
-                const int *a = pos_all.data() + start[p], *c = pos_all.data() + start[q];
-                return std::lexicographical_compare(a, a + len[p], c, c + len[q]);
-            });
-            if (emit_bucket(out))
-                return -2;
-        }
-        *patterns = b.t - 1;
-        return b.overflow ? -2 : 0;
-    }
-
-    const int *pat(size_t i) const { return pos_all.data() + start[order[i]]; }
-    int wof(size_t i) const { return len[order[i]]; }
-
-    /* Runs of one weight's patterns, class by class (one class per w). */
-    int emit_bucket(std::vector<OrbgRun> *out) {
-        const size_t np = order.size();
-        size_t i = 0;
-        while (i < np) {
-            const int w = wof(i);
-            size_t end = i;
-            while (end < np && wof(end) == w)
-                end++;
-            if (w - 2 > ORBG_RUN_MAX_PRE)
-                return -2;
-            for (size_t s = i; s < end;) {
-                const int *v = pat(s);
-                size_t e = s + 1;
-                if (w >= 2) {
-                    const int a = v[w - 2], bb = v[w - 1];
-                    /* the step from this pattern to the next, if it keeps the prefix */
-                    int da = 1, db = 1;
-                    if (e < end && std::equal(v, v + w - 2, pat(e))) {
-                        da = pat(e)[w - 2] - a;
-                        db = bb - pat(e)[w - 1];
-                    }
-                    if (da < 1 || db < 1 || da > 255 || db > 255)
-                        da = db = 1;
-                    while (e < end && std::equal(v, v + w - 2, pat(e)) &&
-                           pat(e)[w - 2] == a + da * (int)(e - s) &&
-                           pat(e)[w - 1] == bb - db * (int)(e - s))
-                        e++;
-                    if (da == 1 && db == 1 && a + bb <= 255) {
-                        for (int q = 0; q < w - 2; q++)
-                            b.pre[q] = v[q];
-                        OrbgRun r = b.blank(ORBG_RUN_PAIRS, w - 2);
-                        r.aux = (uint32_t)(a + bb) | ((uint32_t)a << 8);
-                        b.emit(r, (uint64_t)(e - s));
-                        s = e;
-                        continue;
-                    }
-                    if (e - s >= 2 && bb <= 255) {
-                        for (int q = 0; q < w - 2; q++)
-                            b.pre[q] = v[q];
-                        OrbgRun r = b.blank(ORBG_RUN_STRIDE, w - 2);
-                        r.aux = (uint32_t)a | ((uint32_t)bb << 8) | ((uint32_t)da << 16) |
-                                ((uint32_t)db << 24);
-                        b.emit(r, (uint64_t)(e - s));
-                        s = e;
-                        continue;
-                    }
-                }
-                if (w > ORBG_RUN_MAX_PRE)
-                    return -2;
-                for (size_t q = s; q < e; q++) {
-                    for (int z = 0; z < w; z++)
-                        b.pre[z] = pat(q)[z];
-                    b.single(w);
-                }
-                s = e;
-            }
-            b.flush(out);
-            i = end;
-        }
-        return 0;
-    }
-};
-
-}  // namespace
 
 int orbg_build_tables_model(int n, uint64_t cap, const OrbgModel &md, OrbgTables *out)
 {
@@ -571,57 +516,72 @@ int orbg_build_tables_model(int n, uint64_t cap, const OrbgModel &md, OrbgTables
         if (md.I[i + 1] <= md.I[i] || md.beta[i] < 1 || md.beta[i] > ORBG_MAX_MODEL ||
             md.J[i] < -md.beta[i] || md.J[i] > ORBG_MAX_MODEL)
             return -1;
-    ModelBuilder mb;
-    mb.b.n = n;
-    mb.b.cta = false;
-    std::vector<std::pair<long, int>> w;
+    std::vector<long> rho((size_t)n + 1, 0);
     for (int i = 0; i < md.m; i++)
         for (int j = md.I[i] + 1; j <= md.I[i + 1]; j++)
-            w.push_back(std::make_pair(md.J[i] + md.beta[i] * (long)(j - md.I[i]), j));
-    std::sort(w.begin(), w.end());
-    for (const auto &e : w) {
-        mb.x.push_back(e.first);
-        mb.pos.push_back(e.second);
-    }
-    out->runs.clear();
+            rho[(size_t)j] = md.J[i] + md.beta[i] * (long)(j - md.I[i]);
+    const Order o(n, rho);
     uint64_t patterns = 0;
-    const int rc = mb.build(cap, &out->runs, &patterns);
-    if (rc)
-        return rc;
-    if (patterns >= 0xFFFFFFFFull)
-        return -3;
-    out->patterns = patterns;
-    out->wmax_logistic = 0;
-    /* no triple runs: the CTA table is the warp table, X3 is empty */
-    out->runs_cta = out->runs;
-    out->trip.clear();
-    out->s3max = 0;
-    out->x3off.assign(2, 0u);
-    finish_tables(out);
-    return 0;
+    const long Rmax = o.depth(cap, &patterns);
+    /* position 256 does not fit a byte of a model's order */
+    if (too_heavy(o, Rmax) || (n == 256 && rho[256] <= Rmax))
+        return -2;
+    return build_order(n, rho, patterns, Rmax, true, out);
 }
 
-/* Expands run r's j-th pattern into v (1-based sorted positions, ascending);
- * returns its Hamming weight.  trip is the table's X3 triple list. */
-int orbg_run_pattern(const OrbgRun &r, int j, const uint32_t *trip, int *v)
+/* Calls f(t, positions, w) for every pattern of index t <= count: positions
+ * 1-based, ascending.  Expanded from the tables the kernels read. */
+void orbg_expand_tables(const OrbgTables &tb, int n, uint64_t count,
+                        const std::function<void(uint32_t, const int *, int)> &f)
 {
-    int w = 0;
-    for (int i = 0; i < r.npre; i++)
-        v[w++] = r.pre[i];
-    if (r.kind == ORBG_RUN_PAIRS) {
-        const int S = (int)(r.aux & 0xFFu), a = (int)(r.aux >> 8) + j;
-        v[w++] = a;
-        v[w++] = S - a;
-    } else if (r.kind == ORBG_RUN_STRIDE) {
-        v[w++] = (int)(r.aux & 0xFFu) + j * (int)((r.aux >> 16) & 0xFFu);
-        v[w++] = (int)((r.aux >> 8) & 0xFFu) - j * (int)(r.aux >> 24);
-    } else if (r.kind == ORBG_RUN_TRIPLES) {
-        const uint32_t t = trip[r.aux + (uint32_t)j];
-        v[w++] = (int)(t & 0xFFu) + 1;
-        v[w++] = (int)((t >> 8) & 0xFFu) + 1;
-        v[w++] = (int)((t >> 16) & 0xFFu) + 1;
+    int v[64];
+    if (count >= 1)
+        f(1u, v, 0);
+    for (int j = 1; j <= n; j++)
+        if (tb.single[(size_t)j - 1] && tb.single[(size_t)j - 1] <= count) {
+            v[0] = j;
+            f(tb.single[(size_t)j - 1], v, 1);
+        }
+    /* first pair of each group */
+    std::vector<uint32_t> gfirst;
+    for (size_t k = 0; k < tb.pairs.size(); k++)
+        if (k == 0 || tb.pgroup[k] != tb.pgroup[k - 1])
+            gfirst.push_back((uint32_t)k);
+    gfirst.push_back((uint32_t)tb.pairs.size());
+    for (uint32_t i = 0; i < tb.npre; i++) {
+        if (tb.gmeta[2 * (size_t)(i / ORBG_GROUP)] > count)
+            break;
+        int w = 0;
+        const uint64_t rec = tb.pre[i], ext = i < tb.pext.size() ? tb.pext[i] : 0;
+        for (int b = 0; b < 16; b++)
+            if (rec >> b & 1)
+                v[w++] = tb.light[b];
+        for (int k = 0; k < ORBG_PRE_POS; k++)
+            if (rec >> (16 + 8 * k) & 0xFF)
+                v[w++] = (int)(rec >> (16 + 8 * k) & 0xFF);
+        for (int k = 0; k < 8; k++)
+            if (ext >> (8 * k) & 0xFF)
+                v[w++] = (int)(ext >> (8 * k) & 0xFF);
+        std::sort(v, v + w);
+        const int q = (int)(tb.pmeta[2 * (size_t)i + 1] & 0xFFFFu);
+        const uint32_t g0 = tb.pmeta[2 * (size_t)i + 1] >> 16;
+        for (uint32_t k = tb.pmeta[2 * (size_t)i]; k < tb.pmeta[2 * (size_t)i + 2]; k++) {
+            const uint32_t g = g0 + (k - tb.pmeta[2 * (size_t)i]);
+            uint32_t t = tb.start[k];
+            if (t == 0)
+                continue;
+            for (uint32_t e = gfirst[g]; e < gfirst[g + 1]; e++) {
+                if ((tb.pairs[e] & 0xFF) + 1 <= q)
+                    continue;
+                if (t <= count) {
+                    v[w] = (tb.pairs[e] & 0xFF) + 1;
+                    v[w + 1] = (tb.pairs[e] >> 8) + 1;
+                    f(t, v, w + 2);
+                }
+                t++;
+            }
+        }
     }
-    return w;
 }
 
 /* ------------------------------------------------------------- GF(2) -- */
