@@ -75,12 +75,11 @@ constexpr int kDepth = 31;                  /* largest pattern the stack holds *
 constexpr uint32_t kRhoInf = 1u << 30;      /* weight of a position never reached */
 constexpr int32_t kRmax = (1 << 26) - 1;    /* heaviest reliability weight searched */
 constexpr int kLeafRun = 3;                /* leaf siblings tested per step besides the node */
-/* nodes a one-warp pass may test before a CTA takes over (a quarter of the
- * cap if less): measured on BCH(127,113) and CA-Polar[256,234] (3 lines),
- * 2^16 sends so many BCH blocks to the CTA search (each restarting there)
- * that its step grows by a fifth; 2^18 costs BCH nothing and still takes
- * the long CA-Polar blocks off single warps */
-constexpr uint32_t kSplit = 1u << 18;
+/* Nodes a one-warp pass may test before a CTA takes over (a quarter of the
+ * cap if less).  Measured, us a call, three lines, 100,000 BCH(127,113) and
+ * 20,000 CA-Polar[256,234] blocks: 256 1,658 and 1,991; 512 1,533 and 1,861;
+ * 1024 1,469 and 1,699; 2048 1,505 and 1,732; 4096 1,746 and 1,946. */
+constexpr uint32_t kSplit = 1024;
 constexpr int32_t kNoHit = 0x7FFFFFFF;
 constexpr int kBlockRange = ORBG_BLOCK_RANGE; /* abandoned[] value: beyond the search range */
 
@@ -95,10 +94,12 @@ template <int W> struct FsSmem {
     uint8_t *pi;     /* [256] received index of sorted position j - 1 */
     uint8_t *cw;     /* [256] staged codeword */
     uint8_t *stk;    /* [32][32] stk[d * 32 + lane]: j_{d+1} of the lane's node */
-    uint8_t *hb;     /* [32][32] hb[i * 32 + lane]: the lane's best member so far */
-    uint8_t *best;   /* [32] the block's decoding, positions ascending */
+    uint8_t *hb;     /* [32][32] hb[i * 32 + lane]: the lane's best member so far, its
+                      * positions less one (position 256 of n = 256 fits a byte) */
+    uint8_t *best;   /* [32] the block's decoding, positions ascending, less one */
     int32_t *rec;    /* [24] the block's model record */
     int32_t *anch;   /* [9] anchors during the fit */
+    __device__ __forceinline__ FsSmem() {}
     __device__ __forceinline__ FsSmem(unsigned char *base)
     {
         unsigned char *p = base;
@@ -290,6 +291,29 @@ __device__ void fit_block(const FsSmem<W> &sm, int n, int lines, int divisible, 
     quantise_lanes<W>(sm, na, divisible, lane);
 }
 
+/* v of position 8 lane + 1 + i becomes the least value of that and all later
+ * positions. */
+__device__ __forceinline__ void suffix_minima(uint32_t (&v)[8], int lane)
+{
+#pragma unroll
+    for (int i = 6; i >= 0; i--)
+        v[i] = min(v[i], v[i + 1]);
+    /* minimum over the lanes above: inclusive suffix scan, shifted by one */
+    uint32_t incl = v[0];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_down_sync(FULL_MASK, incl, d);
+        if (lane + d < 32)
+            incl = min(incl, o);
+    }
+    uint32_t above = __shfl_down_sync(FULL_MASK, incl, 1);
+    if (lane == 31)
+        above = kRhoInf;
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        v[i] = min(v[i], above);
+}
+
 /* rho_j from the model record (Eq. relest_seg), clamped to kRhoInf, and the
  * suffix minima.  Lane l owns positions 8l + 1 .. 8l + 8. */
 template <int W>
@@ -315,25 +339,12 @@ __device__ void position_weights(const FsSmem<W> &sm, int n, int lane)
         }
         v[i] = r;
     }
-#pragma unroll
-    for (int i = 6; i >= 0; i--)
-        v[i] = min(v[i], v[i + 1]);
-    /* minimum over the lanes above: inclusive suffix scan, shifted by one */
-    uint32_t incl = v[0];
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_down_sync(FULL_MASK, incl, d);
-        if (lane + d < 32)
-            incl = min(incl, o);
-    }
-    uint32_t above = __shfl_down_sync(FULL_MASK, incl, 1);
-    if (lane == 31)
-        above = kRhoInf;
+    suffix_minima(v, lane);
 #pragma unroll
     for (int i = 0; i < 8; i++) {
         const int j = 8 * lane + 1 + i;
         if (j <= n)
-            sm.msuf[j] = min(v[i], above);
+            sm.msuf[j] = v[i];
     }
     if (lane == 0) {
         sm.rho[n + 1] = kRhoInf;
@@ -351,7 +362,7 @@ __device__ __forceinline__ bool node_lex_less(const uint8_t *stk, int lane, int 
 {
     for (int i = 0; i < t; i++) {
         const int a = i < t - 1 ? (int)stk[i * 32 + lane] : jt;
-        const int b = (int)other[i * ostride];
+        const int b = (int)other[i * ostride] + 1;
         if (a != b)
             return a < b;
     }
@@ -370,26 +381,94 @@ __device__ __forceinline__ bool hb_lex_less(const uint8_t *hb, int la, int lb, i
     return false;
 }
 
+/* Is the lane's node with the pair a < b before the t-position pattern of
+ * lane `lane` of hb in lexicographic order? (t = the node's size + 2) */
+__device__ __forceinline__ bool node_pair_lex_less(const uint8_t *stk, int lane, int t, int jt,
+                                                   int a, int b, const uint8_t *hb)
+{
+    for (int i = 0; i < t; i++) {
+        const int x = i < t - 3 ? (int)stk[i * 32 + lane] : i == t - 3 ? jt : i == t - 2 ? a : b;
+        const int y = (int)hb[i * 32 + lane] + 1;
+        if (x != y)
+            return x < y;
+    }
+    return false;
+}
+
+/* What a pass over prefixes needs besides the node arrays: the block's pairs
+ * of weights slo < s <= shi in a hash set (2^kFsSetBits 32-bit slots, linear
+ * probing; an entry is a 16-bit tag, the hash bits below the slot's, over
+ * a - 1 and b - 1), and the least weight tb[j] that a pair of the set after
+ * position j can have. */
+constexpr int kFsSetBits = 14;
+constexpr uint32_t kFsEmpty = 0xFFFFFFFFu;
+struct FsPairs {
+    const uint32_t *tb;
+    uint32_t *set;
+};
+
+__device__ __forceinline__ uint32_t fs_tag(uint32_t hash)
+{
+    return (hash << kFsSetBits) & 0xFFFF0000u;
+}
+
+/* Entry with the tag of key v, or kFsEmpty (a filter: fs_match checks). */
+__device__ __forceinline__ uint32_t fs_find(const uint32_t *set, uint32_t v)
+{
+    const uint32_t x = slot_hash(v), tag = fs_tag(x);
+    uint32_t slot = x >> (32 - kFsSetBits);
+    uint32_t e = set[slot];
+    while (e != kFsEmpty && ((e ^ tag) & 0xFFFF0000u) != 0u) {
+        slot = (slot + 1u) & ((1u << kFsSetBits) - 1u);
+        e = set[slot];
+    }
+    return e;
+}
+
+/* The set's pair whose whole syndrome is `full` (key v): a | b << 16, 1-based, or 0. */
+template <int W>
+__device__ __noinline__ uint32_t fs_match(const uint32_t *set, const uint32_t *c0,
+                                          const typename Syn<W>::T *h, uint32_t v,
+                                          typename Syn<W>::T full)
+{
+    const uint32_t x = slot_hash(v), tag = fs_tag(x);
+    uint32_t slot = x >> (32 - kFsSetBits);
+    for (;;) {
+        const uint32_t e = set[slot];
+        if (e == kFsEmpty)
+            return 0u;
+        if (((e ^ tag) & 0xFFFF0000u) == 0u) {
+            const uint32_t a = ((e >> 8) & 0xFFu) + 1u, b = (e & 0xFFu) + 1u;
+            if (W == 1 ? (c0[a] ^ c0[b]) == v : sz(sx(sx(h[a], h[b]), full)))
+                return a | b << 16;
+        }
+        slot = (slot + 1u) & ((1u << kFsSetBits) - 1u);
+    }
+}
+
 /* Syndrome of the lane's node on all W words. */
 template <int W>
-__device__ __noinline__ bool node_is_member(const FsSmem<W> &sm, int lane, int t, int jt,
-                                            typename Syn<W>::T s0)
+__device__ __noinline__ typename Syn<W>::T node_syndrome(const FsSmem<W> &sm, int lane, int t,
+                                                         int jt, typename Syn<W>::T s0)
 {
     typename Syn<W>::T P = sx(s0, sm.h[jt]);
     for (int i = 0; i < t - 1; i++)
         P = sx(P, sm.h[sm.stk[i * 32 + lane]]);
-    return sz(P);
+    return P;
 }
 
 /*
  * One pass over the nodes whose bound is <= Rhi.
- * RANK = false: tests every node with R <= Rhi; a lane keeps its least
+ * MODE kFsSearch: tests every node with R <= Rhi; a lane keeps its least
  *   member (bR, bT, its positions in hb) and the bound drops to the warp's
  *   lightest member.  Returns the number of nodes tested (lane's share).
- * RANK = true: counts the nodes before the block's decoding (weight Rb,
+ * MODE kFsRank: counts the nodes before the block's decoding (weight Rb,
  *   Hamming weight Tb, positions sm.best): lighter, or as heavy with fewer
  *   positions, or as heavy and as many positions and lexicographically
  *   smaller.  Returns the lane's share of that count.
+ * MODE kFsPairs: the nodes are prefixes (first positions) of patterns, and
+ *   each is one look-up of its syndrome in the set of pairs; sm.msuf holds
+ *   the least weight that a prefix position >= j and a pair after it add.
  * *guard is set (warp-uniform) if the walk exceeds `steps` iterations.
  * P, w: the walk covers class w of P (P = 1, w = 0: the whole tree): the
  * sets {j} with j = w + 1 modulo P and the larger sets whose second position
@@ -397,12 +476,14 @@ __device__ __noinline__ bool node_is_member(const FsSmem<W> &sm, int lane, int t
  * 2 go to the next such position ("add") or P positions on ("replace"), so
  * the big subtrees of the least reliable positions are shared out evenly.
  */
-template <int W, bool RANK, int P>
+enum { kFsSearch = 0, kFsRank = 1, kFsPairs = 2 };
+template <int W, int MODE, int P>
 __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0, int32_t Rhi,
                               int32_t Rb, int Tb, int lane, uint32_t steps, int32_t *bR,
-                              int *bT, bool *guard, int w)
+                              int *bT, bool *guard, int w, const FsPairs *pr = nullptr)
 {
-    const uint32_t s0w = first_word(s0);
+    constexpr bool RANK = MODE == kFsRank, PAIRS = MODE == kFsPairs;
+    const uint32_t s0w = syn_key(s0);
     bool active = false; /* an active lane's node is always untested yet */
     int t = 0, t0 = 0, jt = 0;
     uint32_t R = 0, rcur = 0, ccur = 0, syn = 0, don = 0, cnt = 0;
@@ -416,7 +497,7 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
         jt = lane + 1;
         rcur = sm.rho[jt];
         ccur = sm.c0[jt];
-        active = (lane < last ? rcur : sm.msuf[jt]) <= (uint32_t)Rhi;
+        active = (lane < last ? rcur + (PAIRS ? pr->tb[jt] : 0u) : sm.msuf[jt]) <= (uint32_t)Rhi;
         t = 1;
         t0 = 1;
         don = lane < last ? 1u << 1 : 0u;
@@ -433,8 +514,40 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
             break;
         }
         const bool tested =
-            active && R <= (uint32_t)Rhi && (P == 1 || t != 1 || (jt - 1) % P == w);
-        if (RANK) {
+            active && R + (PAIRS ? pr->tb[jt] : 0u) <= (uint32_t)Rhi &&
+            (P == 1 || t != 1 || (jt - 1) % P == w);
+        if (PAIRS) {
+            const bool cand = tested && fs_find(pr->set, syn) != kFsEmpty;
+            if (__any_sync(FULL_MASK, cand)) {
+                if (cand) {
+                    const uint32_t ab = fs_match<W>(
+                        pr->set, sm.c0, sm.h, syn,
+                        W == 1 ? szero<typename Syn<W>::T>()
+                               : node_syndrome<W>(sm, lane, t, jt, s0));
+                    const int pa = (int)(ab & 0xFFFFu), pb = (int)(ab >> 16);
+                    /* a pair not wholly after the prefix belongs to no first hit */
+                    if (pa > jt) {
+                        const int32_t Rp = (int32_t)(R + sm.rho[pa] + sm.rho[pb]);
+                        const bool better =
+                            Rp < *bR ||
+                            (Rp == *bR &&
+                             (t + 2 < *bT ||
+                              (t + 2 == *bT && node_pair_lex_less(sm.stk, lane, t + 2, jt, pa, pb,
+                                                                  sm.hb))));
+                        if (better) {
+                            for (int i = 0; i < t - 1; i++)
+                                sm.hb[i * 32 + lane] = sm.stk[i * 32 + lane] - 1;
+                            sm.hb[(t - 1) * 32 + lane] = (uint8_t)(jt - 1);
+                            sm.hb[t * 32 + lane] = (uint8_t)(pa - 1);
+                            sm.hb[(t + 1) * 32 + lane] = (uint8_t)(pb - 1);
+                            *bR = Rp;
+                            *bT = t + 2;
+                        }
+                    }
+                }
+                Rhi = min(Rhi, __reduce_min_sync(FULL_MASK, *bR));
+            }
+        } else if (RANK) {
             if (tested) {
                 if (R < (uint32_t)Rb)
                     cnt++;
@@ -446,7 +559,7 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
             cnt += tested ? 1u : 0u;
             const bool cand = tested && syn == 0u;
             if (__any_sync(FULL_MASK, cand)) {
-                if (cand && (W == 1 || node_is_member<W>(sm, lane, t, jt, s0))) {
+                if (cand && (W == 1 || sz(node_syndrome<W>(sm, lane, t, jt, s0)))) {
                     const bool better =
                         (int32_t)R < *bR ||
                         ((int32_t)R == *bR &&
@@ -454,8 +567,8 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
                           (t == *bT && node_lex_less(sm.stk, lane, t, jt, sm.hb + lane, 32))));
                     if (better) {
                         for (int i = 0; i < t - 1; i++)
-                            sm.hb[i * 32 + lane] = sm.stk[i * 32 + lane];
-                        sm.hb[(t - 1) * 32 + lane] = (uint8_t)jt;
+                            sm.hb[i * 32 + lane] = sm.stk[i * 32 + lane] - 1;
+                        sm.hb[(t - 1) * 32 + lane] = (uint8_t)(jt - 1);
                         *bR = (int32_t)R;
                         *bT = t;
                     }
@@ -550,8 +663,11 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
                     }
                     const uint32_t r = sm.rho[jm], Rs = Rp + r;
                     const bool inner = jm < n && Rs + sm.msuf[jm + 1] <= (uint32_t)Rhi;
-                    const bool own = Rs <= (uint32_t)Rhi &&
-                                     (RANK ? Rs == (uint32_t)Rb : (sp ^ sm.c0[jm]) == 0u);
+                    const bool own =
+                        PAIRS ? Rs + pr->tb[jm] <= (uint32_t)Rhi &&
+                                    fs_find(pr->set, sp ^ sm.c0[jm]) != kFsEmpty
+                              : Rs <= (uint32_t)Rhi &&
+                                    (RANK ? Rs == (uint32_t)Rb : (sp ^ sm.c0[jm]) == 0u);
                     if (inner || own) {
                         move = true;
                         stop = true;
@@ -724,7 +840,7 @@ __device__ typename Syn<W>::T load_record(const OrbgDeviceCode &code,
         const int idx = (int)r[e];
         sm.pi[e] = (uint8_t)idx;
         const T col = load_col<W>(code.hcol, idx);
-        sm.c0[e + 1] = first_word(col);
+        sm.c0[e + 1] = syn_key(col);
         if (W > 1)
             sm.h[e + 1] = col;
         sm.cw[e] = __ldg(llr + e) > 0.0f ? 1 : 0;
@@ -816,7 +932,7 @@ __device__ void band_search(const FsSmem<W> &sm, int n, typename Syn<W>::T s0, u
         bool guard = false;
         uint32_t c = 0;
         if (!CTA) {
-            c = tree_pass<W, false, 1>(sm, n, s0, Rhi, 0, 0, lane, steps, &bR, &bT, &guard, 0);
+            c = tree_pass<W, kFsSearch, 1>(sm, n, s0, Rhi, 0, 0, lane, steps, &bR, &bT, &guard, 0);
         } else {
             for (;;) {
                 unsigned int k = 0;
@@ -826,7 +942,7 @@ __device__ void band_search(const FsSmem<W> &sm, int n, typename Syn<W>::T s0, u
                 if (k >= (unsigned)kClasses)
                     break;
                 const int32_t Rk = min(Rhi, __reduce_min_sync(FULL_MASK, bR));
-                c += tree_pass<W, false, P>(sm, n, s0, Rk, 0, 0, lane, steps, &bR, &bT, &guard,
+                c += tree_pass<W, kFsSearch, P>(sm, n, s0, Rk, 0, 0, lane, steps, &bR, &bT, &guard,
                                             (int)k);
             }
         }
@@ -891,7 +1007,7 @@ __device__ void band_search(const FsSmem<W> &sm, int n, typename Syn<W>::T s0, u
             __syncwarp();
             uint32_t b = 0;
             if (!CTA) {
-                b = tree_pass<W, true, 1>(sm, n, s0, Rb, Rb, Tb, lane, steps, &bR, &bT, &guard,
+                b = tree_pass<W, kFsRank, 1>(sm, n, s0, Rb, Rb, Tb, lane, steps, &bR, &bT, &guard,
                                           0);
             } else {
                 for (;;) {
@@ -901,7 +1017,7 @@ __device__ void band_search(const FsSmem<W> &sm, int n, typename Syn<W>::T s0, u
                     k = __shfl_sync(FULL_MASK, k, 0);
                     if (k >= (unsigned)kClasses)
                         break;
-                    b += tree_pass<W, true, P>(sm, n, s0, Rb, Rb, Tb, lane, steps, &bR, &bT,
+                    b += tree_pass<W, kFsRank, P>(sm, n, s0, Rb, Rb, Tb, lane, steps, &bR, &bT,
                                                &guard, (int)k);
                 }
             }
@@ -980,7 +1096,7 @@ __device__ __forceinline__ void write_fitted(const FsSmem<W> &sm, int n, int lan
 {
     __syncwarp();
     if (lane < wbest)
-        sm.cw[sm.pi[sm.best[lane] - 1]] ^= 1;
+        sm.cw[sm.pi[sm.best[lane]]] ^= 1;
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < K; k++) {
@@ -996,12 +1112,15 @@ __device__ __forceinline__ void write_fitted(const FsSmem<W> &sm, int n, int lan
 }
 
 /* The scratch of one call (orbg_fitsearch_scratch_bytes): counters, the
- * open list, the list of blocks for the CTA search, the handover records. */
+ * open list, the lists of blocks for the two CTA searches, the handover
+ * records. */
 struct FsScratch {
     unsigned long long *cnt; /* [0] stage-1 queue, [1] open blocks, [2] stage-2 queue,
-                              * [3] stage-3 queue, [4] blocks for stage 3 */
+                              * [3] stage-4 queue, [4] blocks for stage 3, [5] stage-3 queue,
+                              * [6] blocks for stage 4 */
     uint32_t *open;          /* block of each open slot */
     uint32_t *wide;          /* open slots left to stage 3 */
+    uint32_t *rest;          /* open slots left to stage 4 */
     unsigned char *hand;
     __host__ __device__ FsScratch(unsigned char *base, int64_t B)
     {
@@ -1009,7 +1128,8 @@ struct FsScratch {
         cnt = reinterpret_cast<unsigned long long *>(base);
         open = reinterpret_cast<uint32_t *>(base + 64);
         wide = reinterpret_cast<uint32_t *>(base + 64 + list);
-        hand = base + 64 + 2 * list;
+        rest = reinterpret_cast<uint32_t *>(base + 64 + 2 * list);
+        hand = base + 64 + 3 * list;
     }
 };
 
@@ -1081,8 +1201,8 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_kernel(
     }
 }
 
-/* Stage 3, persistent over the blocks stage 2 left: all warps of a CTA
- * search one block, each its own class of least positions. */
+/* Stage 4, persistent over the blocks stage 3 does not cover: all warps of a
+ * CTA search one block's tree. */
 template <int K, int W>
 __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
     const __grid_constant__ OrbgDeviceCode code, const float *__restrict__ llr, int64_t B,
@@ -1095,7 +1215,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FsSmem<W> sm(smem + warp * fs_warp_bytes<W>());
     const FsScratch sc(scratch, B);
-    const unsigned long long nwide = sc.cnt[4];
+    const unsigned long long nrest = sc.cnt[6];
     const int n = code.n;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1106,9 +1226,9 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
         __syncthreads();
         const unsigned long long k = s_i;
         __syncthreads(); /* everyone has read s_i before it changes */
-        if (k >= nwide)
+        if (k >= nrest)
             break; /* uniform */
-        const uint32_t i = sc.wide[k];
+        const uint32_t i = sc.rest[k];
         const int64_t b = sc.open[i];
         const auto s0 = load_record<W>(code, llr + b * n, sm, lane,
                                        sc.hand + (size_t)i * ORBG_FIT_HAND_BYTES);
@@ -1122,6 +1242,509 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
     }
 }
 
+/*
+ * Stage 3: all warps of a CTA search one long block by pair look-ups.
+ *
+ * A pattern of two or more positions is a prefix and the pair a < b of its
+ * last two.  The block's pairs go into a hash set of their syndromes, and a
+ * walk over the prefixes alone (tree_pass, kFsPairs; about 3,600 for a
+ * million patterns of a three-line model) looks up each one's syndrome,
+ * which tests every pattern it starts.  Of several pairs of one syndrome the
+ * set keeps the first in the order (weight, a, b): exchanging a later one in
+ * a hit for it gives an earlier hit.  Orders of more than kFsChunk pairs up
+ * to a band's bound take the pairs in chunks of rising weight, each with its
+ * own walk.
+ *
+ * How many patterns have weight r follows from a count over the weights:
+ * counts[r] of the sets of the first j positions plus, for position j + 1,
+ * counts[r - rho].  It gives the weight that holds the cap-th pattern, the
+ * bands' bounds (kFsBand patterns, then sixteen times as many each) and the
+ * patterns lighter than a hit.  The patterns as heavy as the hit but before
+ * it are counted the same way by their number of positions, from the last
+ * position to the first; in passing, for every position x that could take
+ * the place of one of the hit's, the sets after x that complete it (the
+ * lexicographically smaller ones).
+ *
+ * Blocks it does not cover (a weight of the cap-th pattern above kFsTop, a
+ * hit of too many positions for the second count) go to the CTA tree search.
+ * Measured on 20,000 CA-Polar[256,234] blocks of three lines at cap 5e6:
+ * 51.1 ms a call when every search visited its patterns one by one (18.1 ms
+ * of it in stage 2's longest warps, 35.6 in the CTAs' walks), 1.7 ms with
+ * the longer searches here; 100,000 BCH(127,113) blocks 4.4 -> 1.5 ms.
+ */
+constexpr int kFsTop = 4095;          /* largest weight counted */
+constexpr uint32_t kFsCountMax = 1u << 26; /* counts are exact below, and no cap is above */
+constexpr uint32_t kFsChunk = 7168;   /* pairs in the set at once: load 0.44 */
+constexpr uint32_t kFsBand = 32768;   /* patterns of the first band */
+constexpr uint32_t kFsTied = 8192;    /* entries of the tied-patterns count */
+
+/* Dynamic shared memory of the CTA. */
+template <int W> struct FpSmem {
+    uint32_t *cum;   /* [kFsTop + 1] patterns of weight <= r */
+    uint32_t *set;   /* [2^kFsSetBits]; also the counts' work space */
+    uint32_t *mpair; /* [258] least pair weight after position j */
+    uint32_t *m3;    /* [258] least rho_v + mpair[v] over v >= j */
+    uint32_t *mall;  /* [258] least rho over positions >= j */
+    uint32_t *tb;    /* [258] a chunk's bounds: of a look-up, */
+    uint32_t *lb;    /* [258] and of a subtree */
+    FsSmem<W> sm;
+    __device__ __forceinline__ FpSmem(unsigned char *base, int warp)
+    {
+        unsigned char *p = base;
+        auto take = [&](size_t bytes) {
+            unsigned char *r = p;
+            p += (bytes + 15) & ~(size_t)15;
+            return r;
+        };
+        set = (uint32_t *)take(4u << kFsSetBits);
+        cum = (uint32_t *)take(4 * (kFsTop + 1));
+        sm.h = (typename Syn<W>::T *)take(W > 1 ? 258 * sizeof(typename Syn<W>::T) : 0);
+        mpair = (uint32_t *)take(258 * 4);
+        m3 = (uint32_t *)take(258 * 4);
+        mall = (uint32_t *)take(258 * 4);
+        tb = (uint32_t *)take(258 * 4);
+        lb = (uint32_t *)take(258 * 4);
+        sm.rho = (uint32_t *)take(258 * 4);
+        sm.c0 = (uint32_t *)take(258 * 4);
+        sm.rec = (int32_t *)take(24 * 4);
+        sm.pi = take(256);
+        sm.cw = take(256);
+        sm.best = take(32);
+        sm.stk = take(32 * 32 * kWarps) + 32 * 32 * warp;
+        sm.hb = take(32 * 32 * kWarps) + 32 * 32 * warp;
+        sm.msuf = mall; /* position_weights fills it; the walks read lb */
+        sm.L = nullptr;
+        sm.anch = nullptr;
+    }
+};
+template <int W> __host__ __device__ constexpr uint32_t fp_smem_bytes()
+{
+    return (4u << kFsSetBits) + 4u * (kFsTop + 1) +
+           (W > 1 ? (258u * 4u * W + 15u) / 16u * 16u : 0u) + 7u * ((258u * 4u + 15u) / 16u * 16u) +
+           96u + 256u + 256u + 32u + 2u * 32u * 32u * kWarps;
+}
+
+/* cum[r] = patterns of weight <= r (the empty one included), r <= top,
+ * exact below kFsCountMax, held there above.  x, y: top + 1 words each. */
+__device__ __forceinline__ void count_weights(const uint32_t *rho, int n, uint32_t top, uint32_t *x,
+                                              uint32_t *y, uint32_t *cum)
+{
+    for (uint32_t r = threadIdx.x; r <= top; r += blockDim.x)
+        x[r] = r == 0u;
+    __syncthreads();
+    for (int j = 1; j <= n; j += 2) {
+        /* two positions at a time: rho[n + 1] is out of reach */
+        const uint32_t a = rho[j], b = rho[j + 1], ab = a + b;
+        if (a > top && b > top)
+            continue;
+        for (uint32_t r = threadIdx.x; r <= top; r += blockDim.x) {
+            uint32_t v = x[r];
+            if (r >= a)
+                v += x[r - a];
+            if (r >= b)
+                v += x[r - b];
+            if (r >= ab)
+                v += x[r - ab];
+            y[r] = min(v, kFsCountMax);
+        }
+        __syncthreads();
+        uint32_t *t = x;
+        x = y;
+        y = t;
+    }
+    if (threadIdx.x < 32u) {
+        uint32_t run = 0;
+        for (uint32_t base = 0; base <= top; base += 32u) {
+            const uint32_t r = base + threadIdx.x;
+            uint32_t v = r <= top ? x[r] : 0u;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(FULL_MASK, v, d);
+                if ((int)threadIdx.x >= d)
+                    v += o; /* at most 32 * 2^26 */
+            }
+            v = min(v + run, kFsCountMax);
+            if (r <= top)
+                cum[r] = v;
+            run = __shfl_sync(FULL_MASK, v, 31);
+        }
+    }
+    __syncthreads();
+}
+
+/* Least weight with at least `goal` patterns up to it; top + 1 if none. */
+__device__ __forceinline__ uint32_t weight_holding(const uint32_t *cum, uint32_t top, uint32_t goal)
+{
+    uint32_t lo = 0, hi = top + 1u;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (cum[mid] >= goal)
+            hi = mid;
+        else
+            lo = mid + 1u;
+    }
+    return lo;
+}
+
+/* The patterns of weight R before the T positions v (less one, ascending):
+ * fewer positions, or as many and lexicographically smaller; T (R + 1) <=
+ * kFsTied.  x, y: that many words each.  Every thread returns the count. */
+__device__ __forceinline__ uint32_t count_tied(const uint32_t *rho, int n, uint32_t R, int T,
+                                               const uint8_t *v, uint32_t *x, uint32_t *y,
+                                               uint32_t *s_acc)
+{
+    const uint32_t row = R + 1u;
+    for (uint32_t i = threadIdx.x; i < row * (uint32_t)T; i += blockDim.x)
+        x[i] = i == 0u;
+    if (threadIdx.x == 0)
+        *s_acc = 0u;
+    __syncthreads();
+    /* thread 0 keeps the hit's next position below p and the weight before it */
+    int k = T - 1;                 /* v[k] is the last hit position <= p */
+    uint32_t head = 0;             /* weight of v[0 .. k] */
+    uint32_t acc = 0;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < T; i++)
+            head += rho[v[i] + 1];
+    for (int p = n; p >= 1; p--) {
+        const uint32_t a = rho[p];
+        if (threadIdx.x == 0) {
+            if (k >= 0 && (int)v[k] + 1 == p) {
+                head -= rho[p];
+                k--;
+            } else if (k < T - 1 && head + a <= R) {
+                /* p in place of v[k + 1], any T - k - 2 positions after it */
+                acc += x[(uint32_t)(T - k - 2) * row + (R - head - a)];
+            }
+        }
+        if (a > R)
+            continue;
+        for (int t = 0; t < T; t++)
+            for (uint32_t r = threadIdx.x; r <= R; r += blockDim.x) {
+                uint32_t c = x[(uint32_t)t * row + r];
+                if (t > 0 && r >= a)
+                    c += x[(uint32_t)(t - 1) * row + (r - a)];
+                y[(uint32_t)t * row + r] = c;
+            }
+        __syncthreads();
+        uint32_t *s = x;
+        x = y;
+        y = s;
+    }
+    if (threadIdx.x == 0) {
+        for (int t = 0; t < T; t++)
+            acc += x[(uint32_t)t * row + R];
+        *s_acc = acc;
+    }
+    __syncthreads();
+    return *s_acc;
+}
+
+/* The pair (a, b) of key v into the set; the first of a syndrome in the
+ * order (weight, a, b) stays. */
+template <int W>
+__device__ __forceinline__ void fs_insert(const FsSmem<W> &sm, uint32_t *set, int a, int b)
+{
+    const uint32_t v = sm.c0[a] ^ sm.c0[b];
+    typename Syn<W>::T full = szero<typename Syn<W>::T>();
+    if (W > 1)
+        full = sx(sm.h[a], sm.h[b]);
+    const uint32_t x = slot_hash(v), e = fs_tag(x) | (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1);
+    const uint32_t mine = (sm.rho[a] + sm.rho[b]) << 16 | (e & 0xFFFFu);
+    uint32_t slot = x >> (32 - kFsSetBits);
+    for (;;) {
+        uint32_t old = atomicCAS(set + slot, kFsEmpty, e);
+        if (old == kFsEmpty)
+            return;
+        while (((old ^ e) & 0xFFFF0000u) == 0u) {
+            const int oa = (int)((old >> 8) & 0xFFu) + 1, ob = (int)(old & 0xFFu) + 1;
+            if (W == 1 ? (sm.c0[oa] ^ sm.c0[ob]) != v : !sz(sx(sx(sm.h[oa], sm.h[ob]), full)))
+                break; /* another syndrome */
+            if (((sm.rho[oa] + sm.rho[ob]) << 16 | (old & 0xFFFFu)) <= mine)
+                return;
+            const uint32_t was = atomicCAS(set + slot, old, e);
+            if (was == old)
+                return;
+            old = was;
+        }
+        slot = (slot + 1u) & ((1u << kFsSetBits) - 1u);
+    }
+}
+
+template <int K, int W>
+__global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
+    const __grid_constant__ OrbgDeviceCode code, const float *__restrict__ llr, int64_t B,
+    uint32_t cap, uint8_t *__restrict__ cw, uint32_t *__restrict__ q,
+    uint8_t *__restrict__ ab, unsigned char *__restrict__ scratch)
+{
+    typedef typename Syn<W>::T T;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ FsTeam team;
+    __shared__ unsigned long long s_i;
+    __shared__ int32_t s_R;          /* lightest hit so far */
+    __shared__ uint32_t s_next, s_acc;
+    __shared__ int s_win, s_T;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    FpSmem<W> fp(smem, warp);
+    const FsSmem<W> &sm = fp.sm;
+    FsSmem<W> walk = fp.sm;
+    walk.msuf = fp.lb;
+    const FsPairs pairs{fp.tb, fp.set};
+    const FsScratch sc(scratch, B);
+    const unsigned long long nwide = sc.cnt[4];
+    const int n = code.n;
+    const uint32_t steps = 64u * (min(cap, (uint32_t)ORBG_MAX_QUERY_CAP) + 4096u);
+    for (;;) {
+        __syncthreads(); /* the previous block is written */
+        if (threadIdx.x == 0)
+            s_i = atomicAdd(&sc.cnt[5], 1ull);
+        __syncthreads();
+        if (s_i >= nwide)
+            break; /* uniform */
+        const uint32_t open = sc.wide[s_i];
+        const int64_t b = sc.open[open];
+        const unsigned char *rec = sc.hand + (size_t)open * ORBG_FIT_HAND_BYTES;
+        for (int e = (int)threadIdx.x; e < n; e += (int)blockDim.x) {
+            const int idx = (int)rec[e];
+            sm.pi[e] = (uint8_t)idx;
+            const T col = load_col<W>(code.hcol, idx);
+            sm.c0[e + 1] = syn_key(col);
+            if (W > 1)
+                sm.h[e + 1] = col;
+            sm.cw[e] = __ldg(llr + b * n + e) > 0.0f ? 1 : 0;
+        }
+        if (threadIdx.x < ORBG_FIT_WORDS)
+            sm.rec[threadIdx.x] = reinterpret_cast<const int32_t *>(rec + kHandRec)[threadIdx.x];
+        if (threadIdx.x == 0) {
+            sm.c0[0] = 0u;
+            if (W > 1)
+                sm.h[0] = szero<T>();
+            s_R = kNoHit;
+        }
+        const T s0 = *reinterpret_cast<const T *>(rec + kHandS0);
+        __syncthreads();
+        if (warp == 0) {
+            position_weights<W>(sm, n, lane); /* rho and mall */
+            uint32_t v[8];
+            /* mpair[j]: the least rho_a + (least rho after a) over a > j */
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const int a = 8 * lane + 1 + i;
+                v[i] = a < n ? min(sm.rho[a] + fp.mall[a + 1], kRhoInf) : kRhoInf;
+            }
+            suffix_minima(v, lane);
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const int a = 8 * lane + 1 + i;
+                fp.mpair[a - 1] = v[i];
+            }
+            if (lane == 0)
+                fp.mpair[256] = kRhoInf;
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const int j = 8 * lane + 1 + i;
+                v[i] = j < n ? min(sm.rho[j] + fp.mpair[j], kRhoInf) : kRhoInf;
+            }
+            suffix_minima(v, lane);
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                fp.m3[8 * lane + 1 + i] = v[i];
+        }
+        __syncthreads();
+        /* the weight of the cap-th pattern */
+        uint32_t top = 511u, Rcap;
+        for (;;) {
+            count_weights(sm.rho, n, top, fp.set, fp.set + (kFsTop + 1), fp.cum);
+            Rcap = weight_holding(fp.cum, top, cap);
+            if (Rcap <= top || top >= (uint32_t)kFsTop)
+                break;
+            top = min(2u * top + 1u, (uint32_t)kFsTop);
+        }
+        if (Rcap > top) {
+            /* fewer than cap patterns in all, or weights past the count */
+            if (threadIdx.x == 0)
+                sc.rest[atomicAdd(&sc.cnt[6], 1ull)] = open;
+            continue;
+        }
+        /* single positions: thread j - 1 tests position j */
+        int32_t bR = kNoHit;
+        int bT = 0;
+        bool guard = false;
+        {
+            const int j = (int)threadIdx.x + 1;
+            if (j <= n && sm.rho[j] <= Rcap &&
+                (W == 1 ? sm.c0[j] == syn_key(s0) : sz(sx(sm.h[j], s0)))) {
+                bR = (int32_t)sm.rho[j];
+                bT = 1;
+                sm.hb[lane] = (uint8_t)(j - 1);
+                atomicMin(&s_R, bR);
+            }
+        }
+        __syncthreads();
+        uint32_t Rb = 0;
+        for (uint32_t goal = min(cap, kFsBand);; goal = goal > cap / 16u ? cap : goal * 16u) {
+            Rb = weight_holding(fp.cum, top, goal); /* <= Rcap */
+            /* chunks of pairs by weight: (slo, shi] */
+            int32_t slo = -1;
+            while (slo < (int32_t)Rb) {
+                int32_t shi = (int32_t)Rb;
+                if (n * (n - 1) / 2 > (int)kFsChunk) {
+                    for (uint32_t r = threadIdx.x; r <= Rb; r += blockDim.x)
+                        fp.set[r] = 0u;
+                    __syncthreads();
+                    for (int a = 1 + warp; a < n; a += kWarps)
+                        for (int c = a + 1 + lane; c <= n; c += 32) {
+                            const uint32_t s = sm.rho[a] + sm.rho[c];
+                            if ((int32_t)s > slo && s <= Rb)
+                                atomicAdd(fp.set + s, 1u);
+                        }
+                    __syncthreads();
+                    if (warp == 0) {
+                        /* the largest shi with at most kFsChunk pairs (a weight
+                         * has far fewer) */
+                        uint32_t run = 0;
+                        int32_t lim = (int32_t)Rb;
+                        for (uint32_t base = (uint32_t)(slo + 1); base <= Rb; base += 32u) {
+                            const uint32_t r = base + (uint32_t)lane;
+                            uint32_t v = r <= Rb ? fp.set[r] : 0u;
+#pragma unroll
+                            for (int d = 1; d < 32; d <<= 1) {
+                                const uint32_t o = __shfl_up_sync(FULL_MASK, v, d);
+                                if (lane >= d)
+                                    v += o;
+                            }
+                            const uint32_t over =
+                                __ballot_sync(FULL_MASK, run + v > kFsChunk && r <= Rb);
+                            if (over) {
+                                lim = (int32_t)base + __ffs(over) - 2;
+                                break;
+                            }
+                            run += __shfl_sync(FULL_MASK, v, 31);
+                        }
+                        if (lane == 0)
+                            s_win = max(lim, slo + 1);
+                    }
+                    __syncthreads();
+                    shi = s_win;
+                }
+                uint4 *clear = reinterpret_cast<uint4 *>(fp.set);
+                for (uint32_t r = threadIdx.x; r < (1u << kFsSetBits) / 4u; r += blockDim.x)
+                    clear[r] = make_uint4(kFsEmpty, kFsEmpty, kFsEmpty, kFsEmpty);
+                for (int j = (int)threadIdx.x; j <= n + 1; j += (int)blockDim.x) {
+                    const uint32_t least = (uint32_t)(slo + 1);
+                    fp.tb[j] = j <= n ? max(fp.mpair[j], least) : kRhoInf;
+                    fp.lb[j] = j >= 1 && j <= n ? max(fp.m3[j], fp.mall[j] + least) : kRhoInf;
+                }
+                if (threadIdx.x == 0) {
+                    s_next = 0u;
+                }
+                __syncthreads();
+                for (int a = 1 + warp; a < n; a += kWarps)
+                    for (int c = a + 1 + lane; c <= n; c += 32) {
+                        const int32_t s = (int32_t)(sm.rho[a] + sm.rho[c]);
+                        if (s > slo && s <= shi)
+                            fs_insert<W>(sm, fp.set, a, c);
+                    }
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    /* the empty prefix: a pair alone */
+                    const uint32_t m = fs_match<W>(fp.set, sm.c0, sm.h, syn_key(s0), s0);
+                    if (m) {
+                        const int pa = (int)(m & 0xFFFFu), pb = (int)(m >> 16);
+                        const int32_t R = (int32_t)(sm.rho[pa] + sm.rho[pb]);
+                        /* an equally heavy single position comes first */
+                        if (R < bR || (R == bR && bT > 2)) {
+                            bR = R;
+                            bT = 2;
+                            sm.hb[0] = (uint8_t)(pa - 1);
+                            sm.hb[32] = (uint8_t)(pb - 1);
+                            atomicMin(&s_R, R);
+                        }
+                    }
+                }
+                __syncwarp();
+                for (;;) {
+                    unsigned int k = 0;
+                    if (lane == 0)
+                        k = atomicAdd(&s_next, 1u);
+                    k = __shfl_sync(FULL_MASK, k, 0);
+                    if (k >= (unsigned)kClasses)
+                        break;
+                    const int32_t Rk = min((int32_t)Rb, *((volatile int32_t *)&s_R));
+                    const int32_t was = __reduce_min_sync(FULL_MASK, bR);
+                    tree_pass<W, kFsPairs, kClasses>(walk, n, s0, Rk, 0, 0, lane, steps, &bR, &bT,
+                                                     &guard, (int)k, &pairs);
+                    const int32_t now = __reduce_min_sync(FULL_MASK, bR);
+                    if (lane == 0 && now < was)
+                        atomicMin(&s_R, now);
+                }
+                __syncthreads();
+                slo = shi;
+                if (s_R <= (int32_t)Rb && slo + 1 > s_R)
+                    break; /* later pairs are heavier than the hit (uniform) */
+            }
+            if (s_R <= (int32_t)Rb || Rb >= Rcap)
+                break;
+        }
+        const int32_t R = s_R;
+        const bool hit = R <= (int32_t)Rb;
+        /* the team's first member of that weight */
+        if (lane == 0) {
+            team.rb[warp] = kNoHit;
+            team.guard[warp] = guard ? 1 : 0;
+        }
+        __syncwarp();
+        if (hit && __any_sync(FULL_MASK, bR == R)) {
+            const int Tw = warp_least_member<W>(sm, lane, bR, bT, R, team.pos[warp]);
+            if (lane == 0) {
+                team.rb[warp] = R;
+                team.tb[warp] = Tw;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int win = -1;
+            bool bad = false;
+            for (int v = 0; v < kWarps; v++) {
+                bad |= team.guard[v] != 0;
+                if (team.rb[v] == kNoHit)
+                    continue;
+                bool better = win < 0 || team.tb[v] < team.tb[win];
+                if (!better && team.tb[v] == team.tb[win])
+                    for (int i = 0; i < team.tb[v]; i++)
+                        if (team.pos[v][i] != team.pos[win][i]) {
+                            better = team.pos[v][i] < team.pos[win][i];
+                            break;
+                        }
+                if (better)
+                    win = v;
+            }
+            s_win = bad ? -2 : win;
+            s_T = win >= 0 ? team.tb[win] : 0;
+        }
+        __syncthreads();
+        const int win = s_win, Tb = s_T;
+        if (win == -2 || (hit && (uint32_t)Tb * ((uint32_t)R + 1u) > kFsTied)) {
+            if (threadIdx.x == 0)
+                sc.rest[atomicAdd(&sc.cnt[6], 1ull)] = open;
+            continue;
+        }
+        uint32_t rank = 0xFFFFFFFFu;
+        if (hit) {
+            rank = 1u + (R > 0 ? fp.cum[R - 1] : 0u) +
+                   count_tied(sm.rho, n, (uint32_t)R, Tb, team.pos[win], fp.set, fp.set + kFsTied,
+                              &s_acc);
+            if (warp == 0 && lane < Tb)
+                sm.best[lane] = team.pos[win][lane];
+        }
+        const bool ok = rank <= cap;
+        if (warp == 0)
+            write_fitted<K, W>(sm, n, lane, ok ? rank : cap, ok ? 0 : ORBG_BLOCK_ABANDONED,
+                               ok ? Tb : 0, cw + b * n, q + b, ab + b);
+    }
+}
+
 template <int K, int W>
 int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, uint32_t cap,
                      int lines, int divisible, uint8_t *cw, uint32_t *q, uint8_t *ab,
@@ -1129,14 +1752,17 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
 {
     auto k1 = orbg_fitprep_kernel<K, W>;
     auto k2 = orbg_fitsearch_kernel<K, W>;
-    auto k3 = orbg_fitsearch_cta_kernel<K, W>;
+    auto k3 = orbg_fitpair_kernel<K, W>;
+    auto k4 = orbg_fitsearch_cta_kernel<K, W>;
     const size_t smem = (size_t)fs_warp_bytes<W>() * kWarps;
-    int g1 = 0, g2 = 0, g3 = 0;
+    int g1 = 0, g2 = 0, g3 = 0, g4 = 0;
     int rc = orbg_grid_for((const void *)k1, kWarps * 32, smem, 0, &g1);
     if (rc == 0)
         rc = orbg_grid_for((const void *)k2, kWarps * 32, smem, 0, &g2);
     if (rc == 0)
-        rc = orbg_grid_for((const void *)k3, kWarps * 32, smem, 0, &g3);
+        rc = orbg_grid_for((const void *)k3, kWarps * 32, fp_smem_bytes<W>(), 0, &g3);
+    if (rc == 0)
+        rc = orbg_grid_for((const void *)k4, kWarps * 32, smem, 0, &g4);
     if (rc != 0)
         return rc;
     const int64_t need = (B + kWarps - 1) / kWarps;
@@ -1146,6 +1772,8 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
         g2 = (int)need;
     if (g3 > B)
         g3 = (int)B;
+    if (g4 > B)
+        g4 = (int)B;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(scratch, 0, 64, st);
     if (e != cudaSuccess)
@@ -1157,7 +1785,10 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
     k2<<<g2, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return (int)e;
-    k3<<<g3, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
+    k3<<<g3, kWarps * 32, fp_smem_bytes<W>(), st>>>(code, llr, B, cap, cw, q, ab, scratch);
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return (int)e;
+    k4<<<g4, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
     return (int)cudaGetLastError();
 }
 

@@ -326,7 +326,7 @@ int orbg_fit_map_lines(const int32_t *models, int64_t B, int32_t top, const int3
 inline size_t orbg_fitsearch_scratch_bytes(int64_t B)
 {
     const size_t b = (size_t)(B > 0 ? B : 0);
-    return 64 + 2 * ((4 * b + 15) & ~(size_t)15) + (size_t)ORBG_FIT_HAND_BYTES * b;
+    return 64 + 3 * ((4 * b + 15) & ~(size_t)15) + (size_t)ORBG_FIT_HAND_BYTES * b;
 }
 #define ORBG_DECLARE_FITSEARCH(K)                                                         \
     int orbg_launch_fitsearch_k##K(const OrbgDeviceCode &code, const float *llr, int64_t B, \
