@@ -541,11 +541,14 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
     d.npairs = (uint32_t)tb.pairs.size();
     d.npre = tb.npre;
     d.ngroups = (uint32_t)(tb.gmeta.size() / 2);
-    d.npre1 = tb.npre1;
     for (int i = 0; i < ORBG_BANDS; i++) {
         d.band_pairs[i] = tb.band_pairs[i];
+        d.band_pre[i] = tb.band_pre[i];
+        d.band_ranks[i] = tb.band_ranks[i];
         d.band_end[i] = tb.band_end[i];
     }
+    d.lead_pairs = tb.lead_pairs;
+    d.lead_end = tb.lead_end;
     d.nflat = tb.nflat;
     c->dev.max_cap = cap;
     c->dev.n = n;

@@ -65,9 +65,9 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
      * copied in asynchronously while the current one is decoded */
     constexpr int kSlot = 32 * K;
     float *ring = reinterpret_cast<float *>(smem + nwarps * bstride) + warp * 2 * kSlot;
-    /* the warp's own hash set (search_band) */
-    uint32_t *set = reinterpret_cast<uint32_t *>(smem + nwarps * (bstride + 2 * kSlot * 4) +
-                                                  warp * kWarpSetBytes);
+    /* the warp's own pairs (search_band) */
+    uint32_t *filter = reinterpret_cast<uint32_t *>(smem + nwarps * (bstride + 2 * kSlot * 4) +
+                                                  warp * kWarpPairBytes);
     const int64_t n0 = ONE ? code0.n : codes[0].n;
 
     /* the queue's slots: all B, or (range_count: the per-bucket counts of
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
         /* the 256-key sort stays rolled; the others are unrolled */
         if (ONE) {
             decode_block_warp<K, W, true, (K >= 8)>(code0, l, cw + co, q + b, ab + b, cap, budget,
-                                                    bsm, lane, set, heavy, &counters[1],
+                                                    bsm, lane, filter, heavy, &counters[1],
                                                     b_base + (unsigned long long)b, hand,
                                                     hand_cap);
         } else if (cid < 0 || cid >= ncodes) {
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
             /* the block's descriptor is read where it is used (a register
              * copy of it spilled) */
             decode_block_warp<K, W, true, (K >= 8)>(codes[cid], l, cw + co, q + b, ab + b, cap,
-                                                    budget, bsm, lane, set, heavy, &counters[1],
+                                                    budget, bsm, lane, filter, heavy, &counters[1],
                                                     b_base + (unsigned long long)b, hand,
                                                     hand_cap);
         }
@@ -173,10 +173,10 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
 
 
 /* Shared memory of a phase-1 warp: one block's working set, two LLR slots
- * and its own hash set. */
+ * and its own pairs. */
 template <int K> constexpr uint32_t warp_smem_bytes(uint32_t bstride)
 {
-    return bstride + 2u * 32u * K * (uint32_t)sizeof(float) + kWarpSetBytes;
+    return bstride + 2u * 32u * K * (uint32_t)sizeof(float) + kWarpPairBytes;
 }
 
 /* Phase 1 of one decoder variant (K, W): the blocks of sort buckets
@@ -237,7 +237,7 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
     int grid = 0, rc;
     if (a.stage == 2) {
         /* phase 2 over the open blocks every chunk's phase 1 listed */
-        return launch_heavy_t<KMAX, WMAX, ONE>(a, counters, heavy, sc.hand);
+        return launch_heavy_t<WMAX, ONE>(a, counters, heavy, sc.hand);
     }
     /* this launch's slot: its queue heads, bucket counts and cursors, and
      * its blocks' part of the order array */
@@ -297,7 +297,7 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
      * length) */
     if (a.stage == 1)
         return cudaSuccess; /* phase 2 comes later, over every chunk's list */
-    return launch_heavy_t<KMAX, WMAX, ONE>(a, counters, heavy, sc.hand);
+    return launch_heavy_t<WMAX, ONE>(a, counters, heavy, sc.hand);
 }
 
 /* Phases 1 and 2 for keys-per-lane bound KMAX and syndrome width WMAX: one

@@ -459,48 +459,55 @@ __device__ __forceinline__ void sort_lane(uint32_t (&key)[K])
         }
 }
 
-/* Extracts ranks have .. upto-1 (upto <= 32): lane r keeps rank r's key in
- * *mine.  Returns true if two consecutive ranks (this call's or the last
- * earlier one, in *prev) have equal truncated reliabilities: then the
- * truncated order may differ from the exact one and the caller sorts
- * exactly instead. */
+/* Extracts ranks have .. upto-1 (upto <= 64): lane r keeps rank r's key in
+ * mine[0], rank r + 32's in mine[1].  Returns true if two consecutive ranks
+ * (this call's or the last earlier one, in *prev) have equal truncated
+ * reliabilities: then the truncated order may differ from the exact one and
+ * the caller sorts exactly instead. */
 template <int K>
 __device__ __forceinline__ bool extract_ranks(uint32_t (&key)[K], int have, int upto,
-                                              uint32_t *prev, uint32_t *mine, int lane)
+                                              uint32_t *prev, uint32_t (&mine)[2], int lane)
 {
     typedef KeyBits<K> KB;
     bool tie = false;
-    uint32_t pv = *prev, mn = *mine;
-    for (int r = have; r < upto; r++) {
-        const uint32_t g = __reduce_min_sync(FULL_MASK, key[0]);
-        tie |= (g >> KB::IB) == (pv >> KB::IB);
-        if (key[0] == g) {
+    uint32_t pv = *prev;
 #pragma unroll
-            for (int k = 0; k + 1 < K; k++)
-                key[k] = key[k + 1];
-            key[K - 1] = 0xFFFFFFFFu;
+    for (int half = 0; half < 2; half++) {
+        const int end = min(upto, 32 * half + 32);
+        for (int r = max(have, 32 * half); r < end; r++) {
+            const uint32_t g = __reduce_min_sync(FULL_MASK, key[0]);
+            tie |= (g >> KB::IB) == (pv >> KB::IB);
+            if (key[0] == g) {
+#pragma unroll
+                for (int k = 0; k + 1 < K; k++)
+                    key[k] = key[k + 1];
+                key[K - 1] = 0xFFFFFFFFu;
+            }
+            if (lane == r - 32 * half)
+                mine[half] = g;
+            pv = g;
         }
-        if (lane == r)
-            mn = g;
-        pv = g;
     }
     *prev = pv;
-    *mine = mn;
     return tie;
 }
 
 /* Permuted columns of ranks lo .. hi-1 from the lanes holding them. */
 template <int K, int W>
-__device__ __forceinline__ void perm_ranks(const OrbgDeviceCode &code, uint32_t mine, int lo,
-                                           int hi, const BlockSmem<W> &sm, int lane)
+__device__ __forceinline__ void perm_ranks(const OrbgDeviceCode &code, const uint32_t (&mine)[2],
+                                           int lo, int hi, const BlockSmem<W> &sm, int lane)
 {
-    if (lane >= lo && lane < hi) {
-        const int idx = (int)(mine & KeyBits<K>::IMASK);
-        sm.pi[lane] = (uint8_t)idx;
-        const typename Syn<W>::T col = load_col<W>(code.hcol, idx);
-        sm.h[lane] = col;
-        if (W > 1)
-            sm.h0[lane] = syn_key(col);
+#pragma unroll
+    for (int half = 0; half < 2; half++) {
+        const int r = lane + 32 * half;
+        if (r >= lo && r < hi) {
+            const int idx = (int)(mine[half] & KeyBits<K>::IMASK);
+            sm.pi[r] = (uint8_t)idx;
+            const typename Syn<W>::T col = load_col<W>(code.hcol, idx);
+            sm.h[r] = col;
+            if (W > 1)
+                sm.h0[r] = syn_key(col);
+        }
     }
 }
 
@@ -522,88 +529,93 @@ __device__ __forceinline__ void make_keys(const float *__restrict__ llr, int n, 
 /* ------------------------------------------- step 4: pair look-ups */
 
 /*
- * A hash set of pairs: 2^bits 32-bit slots, linear probing.  An entry is the
- * pair's index in the chunk of pairs the set holds (low 12 bits) under a tag,
- * the hash bits below the slot's: with the slot they are the key itself up to
- * two bits, and resolve_pair checks the whole syndrome.  Of pairs of equal
- * syndrome the first stays.  The hash is multiplicative (the high bits of
- * the key times an odd constant near 2^32 / golden ratio).
+ * The pairs of a block are looked up through a filter: 2^bits bits, of which
+ * each pair sets two.  A look-up reads two words and needs no loop: with a
+ * hash set alone a warp step waited for its longest probe sequence (80 warp
+ * instructions a step of 32 look-ups, 45 with the filter).  Both hashes are
+ * multiplicative (the high bits of the key times an odd constant, the first
+ * near 2^32 / golden ratio): the low bits of one product would repeat where
+ * the code's columns differ in few rows.
  */
-constexpr uint32_t kIdMask = 0xFFFu;
-constexpr uint32_t kPairChunk = 4095; /* pairs of one set; entry kEmpty is never a pair's */
-constexpr uint32_t kEmpty = 0xFFFFFFFFu;
-__device__ __forceinline__ uint32_t slot_hash(uint32_t v) { return v * 0x9E3779B1u; }
-__device__ __forceinline__ uint32_t slot_tag(uint32_t hash, uint32_t bits)
+__device__ __forceinline__ uint32_t pair_hash(uint32_t v) { return v * 0x9E3779B1u; }
+__device__ __forceinline__ void filter_add(uint32_t *filter, uint32_t bits, uint32_t v)
 {
-    return (hash << bits) & ~kIdMask;
+    const uint32_t i = pair_hash(v) >> (32u - bits), j = (v * 0x85EBCA6Bu) >> (32u - bits);
+    atomicOr(filter + (i >> 5), 1u << (i & 31u));
+    atomicOr(filter + (j >> 5), 1u << (j & 31u));
+}
+/* May the filter hold a pair of key v? */
+__device__ __forceinline__ bool filter_has(const uint32_t *filter, uint32_t bits, uint32_t v)
+{
+    const uint32_t i = pair_hash(v) >> (32u - bits), j = (v * 0x85EBCA6Bu) >> (32u - bits);
+    return ((filter[i >> 5] >> (i & 31u)) & (filter[j >> 5] >> (j & 31u)) & 1u) != 0u;
 }
 
-/* A warp's own set: 1,024 slots hold the 225 pairs of the first band at a
- * load of 0.22 and the 484 of the second at 0.47. */
-constexpr uint32_t kWarpSetBits = 10;
-constexpr uint32_t kWarpSetBytes = 4u << kWarpSetBits;
-static_assert(ORBG_BAND2_PAIRS * 2 <= (1 << kWarpSetBits), "set too small for the last band");
+/* A warp's own: 2^14 bits for the 484 pairs of the second band, so that 0.3 %
+ * of look-ups pass by chance, and the pairs' keys in order, which the warp
+ * looks through for a key that passed. */
+constexpr uint32_t kWarpFilterBits = 14;
+constexpr uint32_t kWarpFilterBytes = (1u << kWarpFilterBits) / 8u;
+constexpr uint32_t kWarpPairBytes = kWarpFilterBytes + ((ORBG_BAND2_PAIRS * 4u + 15u) & ~15u);
 
-/* A CTA's set for a code of `npairs` pairs, taken in chunks of at most
- * kPairChunk: at least four slots a pair up to 2,048 pairs (cap 1e6 has
- * 1,640), two beyond. */
-__host__ __device__ __forceinline__ uint32_t pair_slot_bits(uint32_t npairs)
+/* A CTA's for a code of `npairs` pairs, taken in chunks of at most
+ * kPairChunk: at least 64 bits a pair (2^17 for the 1,640 of cap 1e6), and a
+ * hash set behind it of at least two slots a pair, linear probing, in which
+ * every lane finds its own pair (codes of few parity bits hit often).  An
+ * entry is the pair's index in the chunk (low 12 bits) under the hash bits
+ * below the slot's; of pairs of equal syndrome the first stays. */
+constexpr uint32_t kIdMask = 0xFFFu;
+constexpr uint32_t kPairChunk = ORBG_PAIR_CHUNK; /* 4095: entry kEmpty is never a pair's */
+constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+__host__ __device__ __forceinline__ uint32_t pair_filter_bits(uint32_t npairs)
 {
     const uint32_t np = npairs < kPairChunk ? npairs : kPairChunk;
-    uint32_t b = 8;
-    while (b < 13 && (1u << b) < 4u * np)
+    uint32_t b = 12;
+    while (b < 18 && (1u << b) < 64u * np)
         b++;
     return b;
+}
+__host__ __device__ __forceinline__ uint32_t pair_slot_bits(uint32_t npairs)
+{
+    return pair_filter_bits(npairs) - 5u;
 }
 /* Keys of the subsets of the eight lightest positions, then of the next
  * eight: a prefix record names its light positions by two bytes. */
 constexpr uint32_t kMaskBytes = 512 * 4;
 __host__ __device__ __forceinline__ uint32_t pair_smem_bytes(uint32_t npairs)
 {
-    return kMaskBytes + (4u << pair_slot_bits(npairs));
+    return kMaskBytes + (1u << pair_filter_bits(npairs)) / 8u + (4u << pair_slot_bits(npairs));
+}
+__device__ __forceinline__ uint32_t slot_tag(uint32_t hash, uint32_t bits)
+{
+    return (hash << bits) & ~kIdMask;
 }
 
-/* Pair id (of the chunk from lo) into the set.  Returns true if its key is
- * zero but its syndrome is not (such a pair is looked up by resolve_pair; a
- * pair of syndrome zero is part of no first hit). */
+/* Pair id (of the chunk from lo) into the CTA's filter and set. */
 template <int W>
-__device__ __forceinline__ bool insert_pair(const OrbgDeviceCode &code, const BlockSmem<W> &sm,
-                                            uint32_t *set, uint32_t bits, uint32_t lo,
-                                            uint32_t id)
+__device__ __forceinline__ void insert_pair(const OrbgDeviceCode &code, const BlockSmem<W> &sm,
+                                            uint32_t *filter, uint32_t fbits, uint32_t *set,
+                                            uint32_t bits, uint32_t lo, uint32_t id)
 {
     const uint32_t p = __ldg(code.pairs + id);
     const uint32_t v = sm.h0[p & 0xFFu] ^ sm.h0[p >> 8];
-    if (v == 0u)
-        return W > 1 && !sz(sx(sm.h[p & 0xFFu], sm.h[p >> 8]));
-    const uint32_t x = slot_hash(v), e = slot_tag(x, bits) | (id - lo);
+    filter_add(filter, fbits, v);
+    const uint32_t x = pair_hash(v), e = slot_tag(x, bits) | (id - lo);
     uint32_t slot = x >> (32u - bits);
     for (;;) {
         const uint32_t old = atomicCAS(set + slot, kEmpty, e);
         if (old == kEmpty)
-            return false;
+            return;
         if ((old ^ e) <= kIdMask) {
             /* the same tag: the same syndrome? */
             const uint32_t o = __ldg(code.pairs + lo + (old & kIdMask));
             if (sz(sx(sx(sm.h[p & 0xFFu], sm.h[p >> 8]), sx(sm.h[o & 0xFFu], sm.h[o >> 8])))) {
                 atomicMin(set + slot, e);
-                return false;
+                return;
             }
         }
         slot = (slot + 1u) & ((1u << bits) - 1u);
     }
-}
-
-/* The entry whose tag is that of key v, or kEmpty. */
-__device__ __forceinline__ uint32_t find_pair(const uint32_t *set, uint32_t bits, uint32_t v)
-{
-    const uint32_t x = slot_hash(v), tag = slot_tag(x, bits);
-    uint32_t slot = x >> (32u - bits);
-    uint32_t e = set[slot];
-    while (e != kEmpty && (e ^ tag) > kIdMask) {
-        slot = (slot + 1u) & ((1u << bits) - 1u);
-        e = set[slot];
-    }
-    return e;
 }
 
 /* A hit: its query index, its prefix (or kSingle) and its pair (or the
@@ -636,35 +648,17 @@ __device__ __forceinline__ typename Syn<W>::T prefix_target(const OrbgDeviceCode
     return v;
 }
 
-/* Query index of prefix i with the first of the pairs [lo, hi) that makes
- * it a hit, and that pair in *pair; ORBG_NONE if there is none, it does not
- * lie after the prefix, or the table ends before it.  id: the pair the set
- * named (checked here), or ORBG_NONE.  Each lane for itself (rare: kept out
- * of line). */
-template <int W>
-__device__ __noinline__ uint32_t resolve_pair(const OrbgDeviceCode &code,
-                                              const typename Syn<W>::T *h,
-                                              typename Syn<W>::T s0, uint32_t i, uint32_t id,
-                                              uint32_t lo, uint32_t hi, uint32_t *pair)
+/* Query index of prefix i with pair id = p; ORBG_NONE if the pair does not
+ * lie after the prefix or the table ends before it. */
+__device__ __forceinline__ uint32_t pattern_index(const OrbgDeviceCode &code, uint32_t i,
+                                                  uint32_t id, uint32_t p)
 {
     const uint2 *pm = reinterpret_cast<const uint2 *>(code.pmeta);
     const uint2 m = __ldg(pm + i);
-    const uint32_t end = __ldg(pm + i + 1).x;
-    const typename Syn<W>::T v = prefix_target<W>(code, h, s0, i);
-    uint32_t p = id != ORBG_NONE ? __ldg(code.pairs + id) : 0u;
-    if (id == ORBG_NONE || !sz(sx(sx(h[p & 0xFFu], h[p >> 8]), v))) {
-        /* an equal tag of another syndrome: look through all pairs */
-        for (id = lo; id < hi; id++) {
-            p = __ldg(code.pairs + id);
-            if (sz(sx(sx(h[p & 0xFFu], h[p >> 8]), v)))
-                break;
-        }
-        if (id >= hi)
-            return ORBG_NONE;
-    }
-    const uint32_t q = m.y & 0xFFFFu, info = __ldg(code.pinfo + id);
+    const uint32_t q = m.y & 0xFFFFu;
     if ((p & 0xFFu) + 1u <= q)
         return ORBG_NONE;
+    const uint32_t end = __ldg(pm + i + 1).x, info = __ldg(code.pinfo + id);
     const uint32_t at = m.x + ((info & 0xFFFFu) - (m.y >> 16));
     if (at >= end)
         return ORBG_NONE;
@@ -677,19 +671,75 @@ __device__ __noinline__ uint32_t resolve_pair(const OrbgDeviceCode &code,
         else
             a = mid + 1u;
     }
-    *pair = id;
     return __ldg(code.start + at) + (id - a);
 }
 
-/* Single positions: the first whose column is s0.  `step` threads, thread t
- * takes positions t, t + step, ...; returns the thread's first hit. */
+/* Query index of prefix i with the first of `np` pairs (their keys in
+ * `keys`) that makes it a hit, and that pair in *pair, or ORBG_NONE; v: the
+ * key to find.  The whole warp together (rare: kept out of line). */
+template <int W>
+__device__ __noinline__ uint32_t resolve_listed(const OrbgDeviceCode &code,
+                                                const typename Syn<W>::T *h,
+                                                typename Syn<W>::T s0, uint32_t i,
+                                                const uint32_t *keys, uint32_t v, uint32_t np,
+                                                int lane, uint32_t *pair)
+{
+    for (uint32_t base = 0; base < np; base += 32u) {
+        const uint32_t k = base + (uint32_t)lane;
+        uint32_t f = __ballot_sync(FULL_MASK, k < np && keys[k] == v);
+        for (; f; f &= f - 1u) {
+            const uint32_t id = base + (uint32_t)__ffs(f) - 1u;
+            const uint32_t p = __ldg(code.pairs + id);
+            if (W == 1 || sz(sx(sx(h[p & 0xFFu], h[p >> 8]), prefix_target<W>(code, h, s0, i)))) {
+                *pair = id;
+                return pattern_index(code, i, id, p);
+            }
+        }
+    }
+    return ORBG_NONE;
+}
+
+/* The same from a CTA's hash set of the pairs from lo, each lane for itself. */
+template <int W>
+__device__ __noinline__ uint32_t resolve_hashed(const OrbgDeviceCode &code,
+                                                const typename Syn<W>::T *h,
+                                                typename Syn<W>::T s0, uint32_t i,
+                                                const uint32_t *set, uint32_t bits, uint32_t v,
+                                                uint32_t lo, uint32_t *pair)
+{
+    const uint32_t x = pair_hash(v), tag = slot_tag(x, bits);
+    uint32_t slot = x >> (32u - bits);
+    typename Syn<W>::T full = s0;
+    bool have = W == 1;
+    for (;; slot = (slot + 1u) & ((1u << bits) - 1u)) {
+        const uint32_t e = set[slot];
+        if (e == kEmpty)
+            return ORBG_NONE;
+        if ((e ^ tag) > kIdMask)
+            continue;
+        const uint32_t id = lo + (e & kIdMask), p = __ldg(code.pairs + id);
+        if (!have) {
+            full = prefix_target<W>(code, h, s0, i);
+            have = true;
+        }
+        if (W == 1 ? (syn_key(h[p & 0xFFu]) ^ syn_key(h[p >> 8])) == v
+                   : sz(sx(sx(h[p & 0xFFu], h[p >> 8]), full))) {
+            *pair = id;
+            return pattern_index(code, i, id, p);
+        }
+    }
+}
+
+/* Single positions before `end`: the first whose column is s0.  Thread t of
+ * `step` takes positions t, t + step, ...; returns the thread's first hit. */
 template <int W>
 __device__ __forceinline__ PairHit single_hits(const OrbgDeviceCode &code,
                                                const typename Syn<W>::T *h,
-                                               typename Syn<W>::T s0, uint32_t t, uint32_t step)
+                                               typename Syn<W>::T s0, uint32_t t, uint32_t step,
+                                               uint32_t end)
 {
     PairHit best{ORBG_NONE, kSingle, 0u};
-    for (uint32_t j = t; j < (uint32_t)code.n; j += step)
+    for (uint32_t j = t; j < end; j += step)
         if (sz(sx(h[j], s0))) {
             const uint32_t x = __ldg(code.single + j);
             if (x != 0u && x < best.t) {
@@ -713,36 +763,47 @@ __device__ __forceinline__ PairHit warp_best(const PairHit &mine)
 
 /*
  * One warp searches band k of its block: the band's pairs from np on go into
- * its set, then every prefix before the band's end is looked up, unless
- * `best` or the cap ends the search first.  Returns the best hit, `best` or
- * one found here.  Every pattern before the band's end is covered, so a hit
- * below it is final.
+ * its filter, then every prefix of the band is looked up, unless `best` or
+ * the cap ends the search first.  Returns the best hit, `best` or one found
+ * here.  Every pattern before the band's end is covered, so a hit below it
+ * is final.  Single positions before the band's are in `best`; only the
+ * band's leading sorted positions need be known.
  */
 template <int W>
 __device__ __forceinline__ PairHit search_band(const OrbgDeviceCode &code,
                                                const BlockSmem<W> &sm,
                                                const typename Syn<W>::T s0, uint32_t cap, int k,
-                                               uint32_t np, uint32_t *set, int lane, PairHit best,
-                                               bool *zero)
+                                               uint32_t np, uint32_t *filter, int lane,
+                                               PairHit best)
 {
-    const uint32_t end = code.band_end[k], hi = code.band_pairs[k];
+    uint32_t *keys = filter + kWarpFilterBytes / 4u;
+    const uint32_t end = code.band_end[k], hi = code.band_pairs[k], npre = code.band_pre[k];
 #pragma unroll 1
-    for (uint32_t id = np + (uint32_t)lane; id < hi; id += 32u)
-        *zero |= insert_pair<W>(code, sm, set, kWarpSetBits, 0u, id);
+    for (uint32_t id = np + (uint32_t)lane; id < hi; id += 32u) {
+        const uint32_t p = __ldg(code.pairs + id);
+        const uint32_t v = sm.h0[p & 0xFFu] ^ sm.h0[p >> 8];
+        keys[id] = v;
+        filter_add(filter, kWarpFilterBits, v);
+    }
     __syncwarp();
-    if (W > 1)
-        *zero = __any_sync(FULL_MASK, *zero);
     const uint32_t s0w = syn_key(s0);
     const uint2 *gm = reinterpret_cast<const uint2 *>(code.gmeta);
     const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre1);
-    PairHit mine = best;
+    if (npre == 0u)
+        return best;
+    const uint32_t ng = (npre + ORBG_GROUP - 1u) / ORBG_GROUP;
+    uint2 nm = __ldg(gm), nr = __ldg(pre + lane);
 #pragma unroll 1
-    for (uint32_t g = 0; g < code.ngroups; g++) {
-        const uint2 m = __ldg(gm + g);
+    for (uint32_t g = 0; g < ng; g++) {
+        const uint2 m = nm, r = nr;
         if (m.x >= end || m.x >= best.t || m.x > cap)
             break;
+        /* the next group, loaded while this one is looked up */
+        if (g + 1u < ng) {
+            nm = __ldg(gm + g + 1u);
+            nr = __ldg(pre + (g + 1u) * ORBG_GROUP + (uint32_t)lane);
+        }
         const uint32_t i = g * ORBG_GROUP + (uint32_t)lane;
-        const uint2 r = __ldg(pre + i);
         uint32_t v = s0w;
         const int kmax = (int)(m.y >> 8);
 #pragma unroll
@@ -751,21 +812,18 @@ __device__ __forceinline__ PairHit search_band(const OrbgDeviceCode &code,
                 break;
             v ^= sm.h0[(int)(((j < 4 ? r.x : r.y) >> (8 * (j & 3))) & 0xFFu) - 1];
         }
-        const uint32_t e = find_pair(set, kWarpSetBits, v);
-        const bool found = (e != kEmpty || (W > 1 && v == 0u && *zero)) && i < code.npre1;
-        if (__any_sync(FULL_MASK, found)) {
-            if (found) {
-                uint32_t pair = 0;
-                const uint32_t t = resolve_pair<W>(code, sm.h, s0, i,
-                                                   e != kEmpty ? e & kIdMask : ORBG_NONE, 0u, hi,
-                                                   &pair);
-                if (t < mine.t) {
-                    mine.t = t;
-                    mine.pre = i;
-                    mine.pair = pair;
-                }
+        uint32_t f = __ballot_sync(FULL_MASK, i < npre && filter_has(filter, kWarpFilterBits, v));
+        for (; f; f &= f - 1u) {
+            const int src = __ffs(f) - 1;
+            uint32_t pair = 0;
+            const uint32_t t =
+                resolve_listed<W>(code, sm.h, s0, g * ORBG_GROUP + (uint32_t)src, keys,
+                                  __shfl_sync(FULL_MASK, v, src), hi, lane, &pair);
+            if (t < best.t) {
+                best.t = t;
+                best.pre = g * ORBG_GROUP + (uint32_t)src;
+                best.pair = pair;
             }
-            best = warp_best(mine);
         }
     }
     return best;
@@ -882,7 +940,7 @@ template <int K, int W, bool LS = false, bool ROLL = true>
 __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__restrict__ llr,
                                   uint8_t *__restrict__ cw_out, uint32_t *__restrict__ q_out,
                                   uint8_t *__restrict__ ab_out, uint32_t cap, uint32_t budget,
-                                  unsigned char *__restrict__ bsm, int lane, uint32_t *set,
+                                  unsigned char *__restrict__ bsm, int lane, uint32_t *filter,
                                   unsigned long long *heavy, unsigned long long *heavy_count,
                                   unsigned long long block_index,
                                   unsigned char *hand = nullptr, uint32_t hand_cap = 0)
@@ -896,6 +954,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
     PairHit hit{ORBG_NONE, ORBG_NONE, 0u}; /* prefix NONE: a flat-table hit */
     bool flat_mine = false;
     bool done = true;
+    int have = 0; /* leading ranks known; n: all, sorted in full */
     if (!nan && sz(s0)) {
         hit.t = 1u; /* query 1, the zero pattern, is a codeword */
     } else if (!nan) {
@@ -909,71 +968,88 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
             if (W > 1)
                 sm.h0[-1] = 0u;
         }
-        bool sorted = false;
-        int have = 0;
-        uint32_t prev = 0xFFFFFFFFu, mine_key = 0xFFFFFFFFu;
-        for (uint32_t base = 0; base < code.nflat && base < cap; base += 32u) {
-            const uint32_t t = base + (uint32_t)lane + 1u;
-            const uint2 e = flat_entry(code, t, cap);
-            /* every entry of a step carries the step byte; entries past the
-             * table are zero */
-            const uint32_t step = __reduce_max_sync(FULL_MASK, flat_step(e));
-            if (!sorted) {
-                const int upto = min((int)(step & 31u) + 1, n);
-                if (upto > have) {
-                    if (extract_ranks<K>(key, have, upto, &prev, &mine_key, lane)) {
-                        make_keys<K, LS>(llr, n, lane, key);
-                        sort_block<K, LS, ROLL>(key, llr, n, lane);
-                        build_perm<K, W>(code, key, sm, lane);
-                        sorted = true;
-                    } else {
-                        perm_ranks<K, W>(code, mine_key, have, upto, sm, lane);
-                        have = upto;
-                    }
+        uint32_t prev = 0xFFFFFFFFu, mine_key[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+        uint32_t base = 0, tested = 1u, np = 0;
+        int k = -1; /* the band; -1: the flat table */
+#pragma unroll 1
+        for (;;) {
+            /* what comes next, and the ranks it needs (one more than needed,
+             * so that a tie across the boundary is seen) */
+            uint2 e = make_uint2(0u, 0u);
+            uint32_t step = 0;
+            int upto;
+            if (k < 0 && base < code.nflat && base < cap) {
+                e = flat_entry(code, base + (uint32_t)lane + 1u, cap);
+                /* every entry of a step carries the step byte; entries past
+                 * the table are zero */
+                step = __reduce_max_sync(FULL_MASK, flat_step(e));
+                upto = (int)(step & 31u) + 1;
+            } else {
+                if (k < 0) {
+                    if (cap <= code.nflat)
+                        break;
+                    tested = code.nflat + 1u;
+                    uint4 *clear = reinterpret_cast<uint4 *>(filter);
+                    for (uint32_t i = (uint32_t)lane; i < kWarpFilterBytes / 16u; i += 32u)
+                        clear[i] = make_uint4(0u, 0u, 0u, 0u);
                     __syncwarp();
                 }
+                for (k++; k < ORBG_BANDS && code.band_end[k] <= tested;)
+                    k++;
+                if (hit.t < tested || tested > cap)
+                    break;
+                if (k < ORBG_BANDS && tested <= budget) {
+                    upto = (int)code.band_ranks[k] + 1;
+                } else {
+                    done = false;
+                    if (heavy == nullptr)
+                        break;
+                    k = ORBG_BANDS;
+                    upto = n; /* the handover record holds them all */
+                }
             }
-            const uint32_t mine =
-                (e.x | e.y << 8) != 0u && flat_test<W>(sm.h, sm.h0, s0, e, n, (int)(step >> 5))
-                    ? t
-                    : ORBG_NONE;
-            const uint32_t gbest = __reduce_min_sync(FULL_MASK, mine);
-            if (gbest != ORBG_NONE) {
-                hit.t = gbest;
-                flat_mine = mine == gbest;
+            upto = min(upto, n);
+            if (upto > have) {
+                /* a tie among the ranks, or more than 64, sorts everything
+                 * exactly */
+                if (upto > 64 || extract_ranks<K>(key, have, upto, &prev, mine_key, lane)) {
+                    make_keys<K, LS>(llr, n, lane, key);
+                    sort_block<K, LS, ROLL>(key, llr, n, lane);
+                    build_perm<K, W>(code, key, sm, lane);
+                    have = n;
+                } else {
+                    perm_ranks<K, W>(code, mine_key, have, upto, sm, lane);
+                    have = upto;
+                }
+                __syncwarp();
+            }
+            if (k < 0) {
+                /* 32 consecutive queries in query order: the first step with
+                 * a hit holds the answer */
+                const uint32_t mine =
+                    (e.x | e.y << 8) != 0u &&
+                            flat_test<W>(sm.h, sm.h0, s0, e, n, (int)(step >> 5))
+                        ? base + (uint32_t)lane + 1u
+                        : ORBG_NONE;
+                const uint32_t gbest = __reduce_min_sync(FULL_MASK, mine);
+                if (gbest != ORBG_NONE) {
+                    hit.t = gbest;
+                    flat_mine = mine == gbest;
+                    break;
+                }
+                base += 32u;
+            } else if (k < ORBG_BANDS) {
+                hit = warp_best(single_hits<W>(code, sm.h, s0, (uint32_t)lane, 32u,
+                                               code.band_ranks[k]));
+                hit = search_band<W>(code, sm, s0, cap, k, np, filter, lane, hit);
+                np = code.band_pairs[k];
+                tested = code.band_end[k];
+            } else {
                 break;
             }
         }
-        if (hit.t == ORBG_NONE && cap > code.nflat) {
-            /* leaving the flat table: every rank is needed */
-            if (!sorted) {
-                make_keys<K, LS>(llr, n, lane, key);
-                sort_block<K, LS, ROLL>(key, llr, n, lane);
-                build_perm<K, W>(code, key, sm, lane);
-                __syncwarp();
-            }
-            hit = warp_best(single_hits<W>(code, sm.h, s0, (uint32_t)lane, 32u));
-            uint4 *clear = reinterpret_cast<uint4 *>(set);
-            for (uint32_t i = (uint32_t)lane; i < kWarpSetBytes / 16u; i += 32u)
-                clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
-            __syncwarp();
-            uint32_t tested = code.nflat + 1u, np = 0;
-            bool zero = false;
-#pragma unroll 1
-            for (int k = 0; k < ORBG_BANDS; k++) {
-                if (hit.t < tested || tested > cap || tested > budget)
-                    break;
-                if (code.band_end[k] <= tested)
-                    continue;
-                hit = search_band<W>(code, sm, s0, cap, k, np, set, lane, hit, &zero);
-                np = code.band_pairs[k];
-                tested = code.band_end[k];
-            }
-            done = hit.t < tested || tested > cap;
-        }
     }
     if (!done) {
-        /* the block is fully sorted here */
         if (heavy != nullptr) {
             unsigned long long slot = 0;
             if (lane == 0)
@@ -982,12 +1058,8 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
             const bool keep = slot < (unsigned long long)hand_cap;
             if (keep) {
                 unsigned char *rec = hand + slot * ORBG_HANDOVER_BYTES;
-#pragma unroll
-                for (int k = 0; k < K; k++) {
-                    const int e = lane * K + k;
-                    if (e < n)
-                        rec[e] = sm.pi[e];
-                }
+                for (int e = lane; e < n; e += 32)
+                    rec[e] = sm.pi[e];
                 if (lane == 0)
                     *reinterpret_cast<T *>(rec + 256) = s0;
             }
@@ -1019,25 +1091,57 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
     return true;
 }
 
+/* The block loaded and sorted by one warp (rare: a block past phase 1's
+ * handover records, and the plain form's open ones): hard decision, order,
+ * permuted columns and *s0.  Returns 0, 1 for a code word, 2 for a NaN
+ * block. */
+template <int K, int W>
+__device__ __noinline__ int load_and_sort_k(const OrbgDeviceCode &code, const float *llr,
+                                            unsigned char *bsm, int lane,
+                                            typename Syn<W>::T *s0)
+{
+    const int n = code.n;
+    const BlockSmem<W> sm(bsm, n);
+    uint32_t key[K];
+    bool nan;
+    *s0 = load_block<K, W>(code, llr, key, sm.cw, lane, &nan);
+    if (nan)
+        return 2;
+    if (sz(*s0))
+        return 1;
+    sort_block<K>(key, llr, n, lane);
+    build_perm<K, W>(code, key, sm, lane);
+    return 0;
+}
+template <int W>
+__device__ __forceinline__ int load_and_sort(const OrbgDeviceCode &code, const float *llr,
+                                             unsigned char *bsm, int lane, typename Syn<W>::T *s0)
+{
+    return code.n <= 32    ? load_and_sort_k<1, W>(code, llr, bsm, lane, s0)
+           : code.n <= 64  ? load_and_sort_k<2, W>(code, llr, bsm, lane, s0)
+           : code.n <= 128 ? load_and_sort_k<4, W>(code, llr, bsm, lane, s0)
+                           : load_and_sort_k<8, W>(code, llr, bsm, lane, s0);
+}
+
 /* ------------------------------------------------ one CTA, one block */
 
 /*
  * All warps of the CTA decode one block.  Its order comes from phase 1's
  * handover record, or warp 0 loads and sorts; all threads then build the
- * subset tables of the light positions and the hash set of the block's pairs
- * (several sets in turn for an order of more than kPairChunk pairs); then
+ * subset tables of the light positions and the filter of the block's pairs
+ * (several in turn for an order of more than kPairChunk pairs); then
  * warp w looks up the prefixes of groups w, w + nw, w + 2 nw, ...  Each warp
  * stops at its first group whose floor is at least the shared best (or above
  * the cap): floors never decrease with the group index and the best never
  * increases, so no group that could hold the final best is skipped.
  * pair_sm: pair_smem_bytes(code.npairs) bytes.
  */
-template <int K, int W>
+template <int W>
 __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__restrict__ llr,
                                  uint8_t *__restrict__ cw_out, uint32_t *__restrict__ q_out,
                                  uint8_t *__restrict__ ab_out, uint32_t cap,
                                  unsigned char *__restrict__ bsm, unsigned char *pair_sm,
-                                 uint32_t *s_best, uint32_t *s_zero, typename Syn<W>::T *s_s0,
+                                 uint32_t *s_best, typename Syn<W>::T *s_s0,
                                  int warp, int lane, int nwarps,
                                  const unsigned char *__restrict__ rec = nullptr)
 {
@@ -1045,8 +1149,9 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
     const int n = code.n;
     BlockSmem<W> sm(bsm, n);
     uint32_t *mask = reinterpret_cast<uint32_t *>(pair_sm);
-    uint32_t *set = reinterpret_cast<uint32_t *>(pair_sm + kMaskBytes);
-    const uint32_t bits = pair_slot_bits(code.npairs);
+    const uint32_t fbits = pair_filter_bits(code.npairs), bits = pair_slot_bits(code.npairs);
+    uint32_t *filter = reinterpret_cast<uint32_t *>(pair_sm + kMaskBytes);
+    uint32_t *set = filter + (1u << fbits) / 32u;
     if (rec != nullptr) {
         /* phase 1's handover record: the block's order and starting
          * syndrome; every thread takes a share of the positions */
@@ -1067,24 +1172,15 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
             *s_s0 = *reinterpret_cast<const T *>(rec + 256);
         }
     } else if (warp == 0) {
-        uint32_t key[K];
-        bool nan;
-        const T s0 = load_block<K, W>(code, llr, key, sm.cw, lane, &nan);
-        if (nan || sz(s0)) {
-            /* not expected here (the warp pass finishes these), but exact */
-            if (lane == 0)
-                *s_best = nan ? ORBG_NONE - 1 : 1u;
-        } else {
-            sort_block<K>(key, llr, n, lane);
-            build_perm<K, W>(code, key, sm, lane);
-            if (lane == 0) {
-                *s_best = ORBG_NONE;
-                *s_s0 = s0;
-            }
+        /* not expected to end here (the warp pass finishes such blocks), but
+         * exact: a NaN block, or a code word */
+        T s0;
+        const int what = load_and_sort<W>(code, llr, bsm, lane, &s0);
+        if (lane == 0) {
+            *s_best = what == 0 ? ORBG_NONE : what == 1 ? 1u : ORBG_NONE - 1u;
+            *s_s0 = s0;
         }
     }
-    if (threadIdx.x == 0)
-        *s_zero = 0u;
     __syncthreads();
     const uint32_t start = *s_best;
     __syncthreads();
@@ -1092,82 +1188,123 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
     if (start == ORBG_NONE) {
         const T s0 = *s_s0;
         const uint32_t s0w = syn_key(s0);
-        mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x);
+        mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x, (uint32_t)n);
         if (mine.t != ORBG_NONE)
             atomicMin(s_best, mine.t);
+        const uint4 light = __ldg(reinterpret_cast<const uint4 *>(code.light));
         for (uint32_t e = threadIdx.x; e < 512u; e += blockDim.x) {
+            const uint32_t w0 = e < 256u ? light.x : light.z, w1 = e < 256u ? light.y : light.w;
             uint32_t v = 0;
 #pragma unroll
             for (int b = 0; b < 8; b++) {
-                const int p = (int)__ldg(code.light + (e >> 8) * 8u + (uint32_t)b);
-                if (e >> b & 1u)
-                    v ^= sm.h0[p - 1];
+                const int p = (int)(((b < 4 ? w0 : w1) >> (8 * (b & 3))) & 0xFFu);
+                const uint32_t c = sm.h0[p - 1];
+                v ^= e >> b & 1u ? c : 0u;
             }
             mask[e] = v;
         }
-        const uint2 *gm = reinterpret_cast<const uint2 *>(code.gmeta);
+        const uint4 *gm = reinterpret_cast<const uint4 *>(code.gmeta);
         const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre);
+        /* first the pairs and prefixes of the order's leading part alone, most
+         * blocks' share; then the rest, chunk by chunk of pairs */
+        uint32_t lo = 0, hi = 0;
+        bool lead = true;
 #pragma unroll 1
-        for (uint32_t lo = 0; lo < code.npairs; lo += kPairChunk) {
-            const uint32_t hi = min(code.npairs, lo + kPairChunk);
-            uint4 *clear = reinterpret_cast<uint4 *>(set);
-            for (uint32_t i = threadIdx.x; i < (1u << bits) / 4u; i += blockDim.x)
-                clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        while (hi < code.npairs || lead) {
+            uint32_t end = ORBG_NONE;
+            if (lead && code.lead_pairs < code.npairs) {
+                hi = code.lead_pairs;
+                end = code.lead_end;
+            } else {
+                /* after the lead, all pairs again: its filter holds them */
+                lo = lead || hi == code.lead_pairs ? 0u : hi;
+                hi = min(code.npairs, lo + kPairChunk);
+            }
+            const bool fresh = lead || lo != 0u;
+            const uint32_t from = fresh ? lo : code.lead_pairs;
+            lead = false;
+            if (fresh) {
+                uint4 *clear = reinterpret_cast<uint4 *>(filter);
+                for (uint32_t i = threadIdx.x; i < (1u << fbits) / 128u; i += blockDim.x)
+                    clear[i] = make_uint4(0u, 0u, 0u, 0u);
+                clear = reinterpret_cast<uint4 *>(set);
+                for (uint32_t i = threadIdx.x; i < (1u << bits) / 4u; i += blockDim.x)
+                    clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+            }
             __syncthreads();
-            for (uint32_t id = lo + threadIdx.x; id < hi; id += blockDim.x)
-                if (insert_pair<W>(code, sm, set, bits, lo, id))
-                    *s_zero = 1u;
+            for (uint32_t id = from + threadIdx.x; id < hi; id += blockDim.x)
+                insert_pair<W>(code, sm, filter, fbits, set, bits, lo, id);
             __syncthreads();
-            const bool zero = W > 1 && *s_zero != 0u;
+            /* two groups a warp step: their loads overlap, and the step's
+             * overhead is shared (60 -> 48 warp instructions a group) */
+            const uint32_t ng2 = (code.ngroups + 1u) / 2u;
             uint32_t g = (uint32_t)warp;
-            uint2 nm = make_uint2(ORBG_NONE, 0u), nr = make_uint2(0u, 0u);
-            if (g < code.ngroups) {
+            uint4 nm = make_uint4(ORBG_NONE, 0u, ORBG_NONE, 0u);
+            uint2 nr0 = make_uint2(0u, 0u), nr1 = nr0;
+            if (g < ng2) {
                 nm = __ldg(gm + g);
-                nr = __ldg(pre + g * ORBG_GROUP + (uint32_t)lane);
+                nr0 = __ldg(pre + g * 64u + (uint32_t)lane);
+                nr1 = __ldg(pre + g * 64u + 32u + (uint32_t)lane);
             }
 #pragma unroll 1
-            for (; g < code.ngroups; g += (uint32_t)nwarps) {
-                const uint2 m = nm, r = nr;
+            for (; g < ng2; g += (uint32_t)nwarps) {
+                const uint4 m = nm;
+                const uint2 r0 = nr0, r1 = nr1;
                 const uint32_t best = *((volatile uint32_t *)s_best);
-                if (m.x >= best || m.x > cap)
+                if (m.x >= min(best, end) || m.x > cap)
                     break;
-                /* the warp's next group, loaded while this one is searched */
+                /* the warp's next groups, loaded while these are searched */
                 const uint32_t gn = g + (uint32_t)nwarps;
-                if (gn < code.ngroups) {
+                if (gn < ng2) {
                     nm = __ldg(gm + gn);
-                    nr = __ldg(pre + gn * ORBG_GROUP + (uint32_t)lane);
+                    nr0 = __ldg(pre + gn * 64u + (uint32_t)lane);
+                    nr1 = __ldg(pre + gn * 64u + 32u + (uint32_t)lane);
                 }
-                const uint32_t i = g * ORBG_GROUP + (uint32_t)lane;
-                uint32_t v = s0w ^ mask[r.x & 0xFFu] ^ mask[256u + ((r.x >> 8) & 0xFFu)];
-                const int kmax = (int)(m.y & 0xFFu);
+                const uint32_t i = g * 64u + (uint32_t)lane;
+                uint32_t v0 = s0w ^ mask[r0.x & 0xFFu] ^ mask[256u + ((r0.x >> 8) & 0xFFu)];
+                uint32_t v1 = s0w ^ mask[r1.x & 0xFFu] ^ mask[256u + ((r1.x >> 8) & 0xFFu)];
+                const int kmax = (int)max(m.y & 0xFFu, m.w & 0xFFu);
 #pragma unroll
                 for (int j = 0; j < ORBG_PRE_POS; j++) {
                     if (j >= kmax)
                         break;
-                    const uint32_t p = j < 2 ? r.x >> (16 + 8 * j) : r.y >> (8 * (j - 2));
-                    v ^= sm.h0[(int)(p & 0xFFu) - 1];
+                    const uint32_t p0 = j < 2 ? r0.x >> (16 + 8 * j) : r0.y >> (8 * (j - 2));
+                    const uint32_t p1 = j < 2 ? r1.x >> (16 + 8 * j) : r1.y >> (8 * (j - 2));
+                    v0 ^= sm.h0[(int)(p0 & 0xFFu) - 1];
+                    v1 ^= sm.h0[(int)(p1 & 0xFFu) - 1];
                 }
                 if (kmax > ORBG_PRE_POS) {
-                    const uint2 x = __ldg(reinterpret_cast<const uint2 *>(code.pext) + i);
-                    for (int j = 0; j < 8; j++)
-                        v ^= sm.h0[(int)(((j < 4 ? x.x : x.y) >> (8 * (j & 3))) & 0xFFu) - 1];
-                }
-                const uint32_t e = find_pair(set, bits, v);
-                if ((e != kEmpty || (W > 1 && v == 0u && zero)) && i < code.npre) {
-                    uint32_t pair = 0;
-                    const uint32_t t = resolve_pair<W>(
-                        code, sm.h, s0, i, e != kEmpty ? lo + (e & kIdMask) : ORBG_NONE, lo, hi,
-                        &pair);
-                    if (t < mine.t) {
-                        mine.t = t;
-                        mine.pre = i;
-                        mine.pair = pair;
-                        atomicMin(s_best, t);
+                    const uint2 *ext = reinterpret_cast<const uint2 *>(code.pext);
+                    const uint2 x0 = __ldg(ext + i), x1 = __ldg(ext + i + 32u);
+                    for (int j = 0; j < 8; j++) {
+                        v0 ^= sm.h0[(int)(((j < 4 ? x0.x : x0.y) >> (8 * (j & 3))) & 0xFFu) - 1];
+                        v1 ^= sm.h0[(int)(((j < 4 ? x1.x : x1.y) >> (8 * (j & 3))) & 0xFFu) - 1];
                     }
                 }
-                __syncwarp();
+                const bool maybe0 = filter_has(filter, fbits, v0);
+                const bool maybe1 = filter_has(filter, fbits, v1);
+                if (__any_sync(FULL_MASK, maybe0 | maybe1)) {
+#pragma unroll 1
+                    for (int w = 0; w < 2; w++) {
+                        const uint32_t iw = i + 32u * (uint32_t)w;
+                        if (!(w ? maybe1 : maybe0) || iw >= code.npre)
+                            continue;
+                        uint32_t pair = 0;
+                        const uint32_t t = resolve_hashed<W>(code, sm.h, s0, iw, set, bits,
+                                                             w ? v1 : v0, lo, &pair);
+                        if (t < mine.t) {
+                            mine.t = t;
+                            mine.pre = iw;
+                            mine.pair = pair;
+                            atomicMin(s_best, t);
+                        }
+                    }
+                    __syncwarp();
+                }
             }
-            __syncthreads(); /* the set is free before the next chunk's pairs */
+            __syncthreads(); /* the filter is free before the next pairs */
+            if (end != ORBG_NONE && (*((volatile uint32_t *)s_best) < end || end > cap))
+                break; /* every pattern before `end` is covered (uniform) */
         }
     }
     __syncthreads();
@@ -1188,34 +1325,19 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
 
 /* ----------------------------------------------------------- dispatch */
 
-/* Runtime dispatch on (n, syndrome width), warp-uniform; only variants up to
- * (KMAX keys per lane, WMAX syndrome words) are instantiated. */
-#define ORBG_DISPATCH(KMAX, WMAX, CALL)                                   \
+/* Runtime dispatch on the syndrome width, uniform over the CTA; only widths
+ * up to WMAX are instantiated. */
+#define ORBG_DISPATCH_W(WMAX, CALL)                                       \
     do {                                                                  \
-        const int n_ = code.n, w_ = code.w32;                             \
-        bool done_ = false;                                               \
-        if constexpr (KMAX >= 8) {                                        \
-            if (!done_ && n_ > 128) { ORBG_DISPATCH_W(8, WMAX, CALL); done_ = true; } \
-        }                                                                 \
-        if constexpr (KMAX >= 4) {                                        \
-            if (!done_ && n_ > 64) { ORBG_DISPATCH_W(4, WMAX, CALL); done_ = true; } \
-        }                                                                 \
-        if constexpr (KMAX >= 2) {                                        \
-            if (!done_ && n_ > 32) { ORBG_DISPATCH_W(2, WMAX, CALL); done_ = true; } \
-        }                                                                 \
-        if (!done_) { ORBG_DISPATCH_W(1, WMAX, CALL); }                  \
-    } while (0)
-
-#define ORBG_DISPATCH_W(KK, WMAX, CALL)                                   \
-    do {                                                                  \
+        const int w_ = code.w32;                                          \
         bool dw_ = false;                                                 \
         if constexpr (WMAX >= 4) {                                        \
-            if (w_ > 2) { CALL(KK, 4); dw_ = true; }                      \
+            if (w_ > 2) { CALL(4); dw_ = true; }                          \
         }                                                                 \
         if constexpr (WMAX >= 2) {                                        \
-            if (!dw_ && w_ == 2) { CALL(KK, 2); dw_ = true; }             \
+            if (!dw_ && w_ == 2) { CALL(2); dw_ = true; }                 \
         }                                                                 \
-        if (!dw_) { CALL(KK, 1); }                                        \
+        if (!dw_) { CALL(1); }                                            \
     } while (0)
 
 }  // namespace orbg_dev

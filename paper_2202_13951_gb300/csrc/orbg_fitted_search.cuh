@@ -407,6 +407,10 @@ struct FsPairs {
     uint32_t *set;
 };
 
+/* multiplicative: the high bits of v times an odd constant near 2^32 /
+ * golden ratio */
+__device__ __forceinline__ uint32_t fs_hash(uint32_t v) { return v * 0x9E3779B1u; }
+
 __device__ __forceinline__ uint32_t fs_tag(uint32_t hash)
 {
     return (hash << kFsSetBits) & 0xFFFF0000u;
@@ -415,7 +419,7 @@ __device__ __forceinline__ uint32_t fs_tag(uint32_t hash)
 /* Entry with the tag of key v, or kFsEmpty (a filter: fs_match checks). */
 __device__ __forceinline__ uint32_t fs_find(const uint32_t *set, uint32_t v)
 {
-    const uint32_t x = slot_hash(v), tag = fs_tag(x);
+    const uint32_t x = fs_hash(v), tag = fs_tag(x);
     uint32_t slot = x >> (32 - kFsSetBits);
     uint32_t e = set[slot];
     while (e != kFsEmpty && ((e ^ tag) & 0xFFFF0000u) != 0u) {
@@ -431,7 +435,7 @@ __device__ __noinline__ uint32_t fs_match(const uint32_t *set, const uint32_t *c
                                           const typename Syn<W>::T *h, uint32_t v,
                                           typename Syn<W>::T full)
 {
-    const uint32_t x = slot_hash(v), tag = fs_tag(x);
+    const uint32_t x = fs_hash(v), tag = fs_tag(x);
     uint32_t slot = x >> (32 - kFsSetBits);
     for (;;) {
         const uint32_t e = set[slot];
@@ -1449,7 +1453,7 @@ __device__ __forceinline__ void fs_insert(const FsSmem<W> &sm, uint32_t *set, in
     typename Syn<W>::T full = szero<typename Syn<W>::T>();
     if (W > 1)
         full = sx(sm.h[a], sm.h[b]);
-    const uint32_t x = slot_hash(v), e = fs_tag(x) | (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1);
+    const uint32_t x = fs_hash(v), e = fs_tag(x) | (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1);
     const uint32_t mine = (sm.rho[a] + sm.rho[b]) << 16 | (e & 0xFFFFu);
     uint32_t slot = x >> (32 - kFsSetBits);
     for (;;) {

@@ -19,7 +19,7 @@ using namespace orbg_dev;
 #define ORBG_PHASE2_MIN_CTAS 2
 #endif
 
-template <int KMAX, int WMAX, bool ONE>
+template <int WMAX, bool ONE>
 __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
     const OrbgDeviceCode *__restrict__ codes, int ncodes, const int32_t *__restrict__ code_id,
     const int64_t *__restrict__ llr_off, const float *__restrict__ llr, uint32_t cap,
@@ -30,8 +30,9 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_block, s_slot;
-    __shared__ uint32_t s_best, s_zero;
+    __shared__ uint32_t s_best;
     __shared__ uint4 s_s0;
+    __shared__ OrbgDeviceCode s_code;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int nwarps = blockDim.x >> 5;
@@ -57,30 +58,35 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
         const int64_t lo = llr_off ? llr_off[b] : b * n0;
         const int64_t co = cw_off ? cw_off[b] : b * n0;
         if (ONE) {
-            decode_block_cta<KMAX, WMAX>(code0, llr + lo, cw + co, q + b, ab + b, cap, smem,
-                                         smem + bstride, &s_best, &s_zero,
-                                         reinterpret_cast<typename Syn<WMAX>::T *>(&s_s0), warp,
-                                         lane, nwarps, rec);
+            decode_block_cta<WMAX>(code0, llr + lo, cw + co, q + b, ab + b, cap, smem,
+                                   smem + bstride, &s_best,
+                                   reinterpret_cast<typename Syn<WMAX>::T *>(&s_s0), warp, lane,
+                                   nwarps, rec);
             continue;
         }
+        /* the block's descriptor, into shared memory */
         const int cid = code_id ? code_id[b] : 0; /* checked in phase 1 */
-        const OrbgDeviceCode &code = codes[cid];
-#define ORBG_CALL_CTA(KK, WW)                                                             \
-    decode_block_cta<KK, WW>(code, llr + lo, cw + co, q + b, ab + b, cap, smem,           \
-                             smem + bstride, &s_best, &s_zero,                            \
-                             reinterpret_cast<typename Syn<WW>::T *>(&s_s0), warp, lane,  \
-                             nwarps, rec)
-        ORBG_DISPATCH(KMAX, WMAX, ORBG_CALL_CTA);
+        constexpr unsigned kWords = sizeof(OrbgDeviceCode) / 4;
+        for (unsigned i = threadIdx.x; i < kWords; i += blockDim.x)
+            reinterpret_cast<uint32_t *>(&s_code)[i] =
+                __ldg(reinterpret_cast<const uint32_t *>(codes + cid) + i);
+        __syncthreads();
+        const OrbgDeviceCode &code = s_code;
+#define ORBG_CALL_CTA(WW)                                                               \
+    decode_block_cta<WW>(code, llr + lo, cw + co, q + b, ab + b, cap, smem,             \
+                         smem + bstride, &s_best,                                       \
+                         reinterpret_cast<typename Syn<WW>::T *>(&s_s0), warp, lane, nwarps, rec)
+        ORBG_DISPATCH_W(WMAX, ORBG_CALL_CTA);
 #undef ORBG_CALL_CTA
     }
     (void)ncodes;
 }
 
-template <int KMAX, int WMAX, bool ONE>
+template <int WMAX, bool ONE>
 cudaError_t launch_heavy_t(const OrbgBatchedArgs &a, unsigned long long *counters,
                            const unsigned long long *heavy, const unsigned char *hand)
 {
-    auto k2 = orbg_heavy_kernel<KMAX, WMAX, ONE>;
+    auto k2 = orbg_heavy_kernel<WMAX, ONE>;
     const int hw = a.heavy_warps > 0 ? a.heavy_warps : 8;
     /* 16-byte aligned: block_smem_bytes is a multiple of 16 */
     const uint32_t bstride = block_smem_bytes(a.n_max, a.w32_max);

@@ -45,6 +45,13 @@
 #define ORBG_BAND1_PAIRS 225
 #define ORBG_BAND2_PAIRS 500
 #define ORBG_PRE1_MAX 1024
+/* Phase 2 (a CTA a block) holds up to ORBG_PAIR_CHUNK pairs at a time.  An
+ * order of more takes its first ORBG_LEAD_PAIRS alone before all of them in
+ * chunks: most blocks end there (three-segment model of BCH(127,113), 6,441
+ * pairs: 216 -> 190 us on 100,000 blocks); with one chunk the repeated
+ * look-ups cost more (CA-Polar(128,94) 1,030 -> 1,110 us). */
+#define ORBG_PAIR_CHUNK 4095
+#define ORBG_LEAD_PAIRS 900
 
 /* The flat table: the first `nflat` patterns of the order, 8 bytes each:
  * up to 7 positions, 1-based (0 = unused), then a byte describing the
@@ -62,7 +69,7 @@ struct OrbgDeviceCode {
     const uint16_t *pairs;       /* [npairs] a0 | b0 << 8, 0-based, by (weight, a, b) */
     const uint32_t *pinfo;       /* [npairs] its group of equally heavy pairs | first pair of the
                                   * group << 16 */
-    const uint32_t *pre;         /* [2 * npre, padded to groups] prefix records, 8 bytes: bit i
+    const uint32_t *pre;         /* [2 * npre, padded to two groups] prefix records, 8 bytes: bit i
                                   * position light[i], then ORBG_PRE_POS further positions,
                                   * 1-based, 0 = none */
     const uint32_t *pext;        /* NULL, or as pre: eight positions past those */
@@ -73,11 +80,14 @@ struct OrbgDeviceCode {
                                   * last position | the first pair group after it << 16 */
     const uint32_t *start;       /* query index of the first pair of a (prefix, group) */
     const uint32_t *single;      /* [n] query index of each single position, 0 = past the table */
-    const uint8_t *light;        /* [16] the lightest positions, 1-based, 0 = none */
+    const uint8_t *light;        /* [16] the lightest positions, 1-based, 0 = none (aligned) */
     uint32_t npairs, npre, ngroups;
-    uint32_t npre1;              /* leading prefixes phase 1 may walk */
-    uint32_t band_pairs[ORBG_BANDS]; /* pairs of each band */
-    uint32_t band_end[ORBG_BANDS];   /* first query index past the band */
+    uint32_t band_pairs[ORBG_BANDS]; /* phase 1: pairs of each band, */
+    uint32_t band_pre[ORBG_BANDS];   /* prefixes, */
+    uint32_t band_ranks[ORBG_BANDS]; /* sorted positions they and the band's patterns take, */
+    uint32_t band_end[ORBG_BANDS];   /* and the first query index past the band */
+    uint32_t lead_pairs;         /* phase 2: pairs of the order's leading part, */
+    uint32_t lead_end;           /* and the first query index past it */
     const uint32_t *flat;        /* [2 * nflat] flat-table patterns, 8 bytes each */
     uint32_t nflat;
     uint32_t max_cap;
@@ -98,8 +108,10 @@ struct OrbgTables {
     std::vector<uint32_t> gmeta, pmeta, start, single;
     uint8_t light[16] = {};
     std::vector<uint8_t> flat;           /* 8 bytes per pattern */
-    uint32_t npre = 0, npre1 = 0, nflat = 0;
-    uint32_t band_pairs[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
+    uint32_t npre = 0, nflat = 0;
+    uint32_t band_pairs[ORBG_BANDS] = {}, band_pre[ORBG_BANDS] = {};
+    uint32_t band_ranks[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
+    uint32_t lead_pairs = 0, lead_end = 0;
     uint64_t patterns = 0;  /* query indices covered (last index) */
 };
 /* The tables for the order of increasing reliability weight J0 w + beta W

@@ -14,7 +14,7 @@ using namespace orbg_dev;
 
 namespace {
 
-constexpr int kPlainWarps = 8;
+constexpr int kPlainWarps = 4;
 
 template <int K, int W>
 __global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
     uint32_t bstride)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint32_t s_best, s_zero;
+    __shared__ uint32_t s_best;
     __shared__ uint4 s_s0;
     __shared__ uint32_t s_open;
     const int warp = threadIdx.x >> 5;
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
     const int64_t b = b0 + warp;
     if (b < B) {
         const int64_t off = b * (int64_t)code.n;
-        unsigned char *own = smem + warp * (bstride + kWarpSetBytes);
+        unsigned char *own = smem + warp * (bstride + kWarpPairBytes);
         const bool done = decode_block_warp<K, W, false, (K >= 8)>(
             code, llr + off, cw + off, q + b, ab + b, cap, cap, own, lane,
             reinterpret_cast<uint32_t *>(own + bstride), nullptr, nullptr, 0ull);
@@ -46,9 +46,8 @@ __global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
     for (uint32_t open = s_open; open; open &= open - 1u) {
         const int64_t bo = b0 + __ffs(open) - 1;
         const int64_t off = bo * (int64_t)code.n;
-        decode_block_cta<K, W>(code, llr + off, cw + off, q + bo, ab + bo, cap, smem,
-                               smem + bstride, &s_best, &s_zero,
-                               reinterpret_cast<typename Syn<W>::T *>(&s_s0), warp, lane,
+        decode_block_cta<W>(code, llr + off, cw + off, q + bo, ab + bo, cap, smem,
+                               smem + bstride, &s_best, reinterpret_cast<typename Syn<W>::T *>(&s_s0), warp, lane,
                                kPlainWarps);
     }
 }
@@ -58,7 +57,7 @@ cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t
                            uint8_t *cw, uint32_t *q, uint8_t *ab, cudaStream_t st)
 {
     const uint32_t bstride = block_smem_bytes(code.n, W);
-    size_t smem = (size_t)(bstride + kWarpSetBytes) * kPlainWarps;
+    size_t smem = (size_t)(bstride + kWarpPairBytes) * kPlainWarps;
     const size_t cta = (size_t)bstride + pair_smem_bytes(code.npairs);
     if (smem < cta)
         smem = cta;

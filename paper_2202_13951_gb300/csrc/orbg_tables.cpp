@@ -355,11 +355,13 @@ struct TableBuilder {
             }
         }
         /* the records the kernels read, 32 prefixes to a group */
-        const uint32_t ng = (npre + ORBG_GROUP - 1) / ORBG_GROUP;
+        /* an even number of groups: a CTA's warps take two at a time */
+        const uint32_t ng = (npre + 2 * ORBG_GROUP - 1) / (2 * ORBG_GROUP) * 2;
         out->npre = npre;
+        for (uint32_t g = 0; g < ng; g++)
+            out->gmeta.push_back(0xFFFFFFFFu), out->gmeta.push_back(0u);
         out->pre.assign((size_t)ng * ORBG_GROUP, 0);
         out->pre1.assign((size_t)ng * ORBG_GROUP, 0);
-        out->gmeta.assign(2 * (size_t)ng, 0);
         uint32_t npre1 = npre; /* leading prefixes a phase-1 warp walks */
         int v[64];
         for (uint32_t i = 0; i < npre; i++) {
@@ -395,21 +397,41 @@ struct TableBuilder {
                 out->gmeta[2 * (size_t)(i / ORBG_GROUP)] = first_at(p.m);
         }
         npre1 = std::min<uint32_t>(npre1, ORBG_PRE1_MAX);
-        out->npre1 = npre1;
-        /* phase 1's bands: the pairs of the leading groups, and the first
-         * query index not covered by them and the leading prefixes */
+        /* phase 1's bands: the pairs of the leading groups; the first weight
+         * not covered by them and the leading prefixes; how many prefixes
+         * and positions the patterns below it take */
         const uint32_t aim[ORBG_BANDS] = {ORBG_BAND1_PAIRS, ORBG_BAND2_PAIRS};
-        const uint32_t none = (uint32_t)out->patterns + 1u;
-        const uint32_t lim1 = npre1 < npre ? first_at(pre[ord[npre1]].m) : none;
+        const long past = Rmax + 1;
+        const long lim1 = npre1 < npre ? pre[ord[npre1]].m : past;
         for (int k = 0; k < ORBG_BANDS; k++) {
             uint32_t np = std::min<uint32_t>(aim[k], (uint32_t)out->pairs.size());
             while (np > 0 && np < out->pairs.size() && out->pgroup[np] == out->pgroup[np - 1])
                 np--;
+            const long end =
+                std::min(lim1, np < out->pairs.size() ? gsum[out->pgroup[np]] : past);
             out->band_pairs[k] = np;
-            const uint32_t end =
-                np < out->pairs.size() ? first_at(gsum[out->pgroup[np]]) : none;
-            out->band_end[k] = std::min(end, lim1);
+            out->band_end[k] = first_at(end);
+            uint32_t c = 0;
+            while (c < npre1 && pre[ord[c]].m < end)
+                c++;
+            out->band_pre[k] = c;
+            uint32_t top = 0;
+            for (int j = 1; j <= n; j++)
+                if (rho[(size_t)j] < end)
+                    top = (uint32_t)j;
+            for (uint32_t i = 0; i < np; i++)
+                top = std::max(top, (uint32_t)(out->pairs[i] >> 8) + 1u);
+            out->band_ranks[k] = top;
         }
+        /* phase 2's leading part, likewise, where one CTA's set does not hold
+         * all pairs */
+        uint32_t np = (uint32_t)out->pairs.size();
+        if (np > ORBG_PAIR_CHUNK)
+            np = ORBG_LEAD_PAIRS;
+        while (np > 0 && np < out->pairs.size() && out->pgroup[np] == out->pgroup[np - 1])
+            np--;
+        out->lead_pairs = np;
+        out->lead_end = first_at(np < out->pairs.size() ? gsum[out->pgroup[np]] : past);
         make_flat();
         return 0;
     }
