@@ -485,6 +485,13 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
         for (int j = 0; j < n; j++)
             if (c->H[(size_t)i * n + j])
                 hcol[(size_t)j * c->w32 + i / 32] |= 1u << (i % 32);
+    /* and rows, for the starting syndrome: see OrbgDeviceCode::hrow */
+    const int kw = n <= 32 ? 1 : n <= 64 ? 2 : n <= 128 ? 4 : 8;
+    std::vector<uint32_t> hrow((size_t)c->w32 * kw * 32, 0);
+    for (int i = 0; i < r; i++)
+        for (int j = 0; j < n; j++)
+            if (c->H[(size_t)i * n + j])
+                hrow[((size_t)(i / 32) * kw + j / 32) * 32 + i % 32] |= 1u << (j % 32);
     OrbgTables tb;
     int trc = md ? orbg_build_tables_model(n, cap, *md, &tb)
                  : orbg_build_tables(n, cap, &tb, J0, beta);
@@ -506,6 +513,7 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
     OrbgDeviceCode &d = c->dev;
     const Up ups[] = {
         {(const void **)&d.hcol, hcol.data(), hcol.size() * sizeof(uint32_t)},
+        {(const void **)&d.hrow, hrow.data(), hrow.size() * sizeof(uint32_t)},
         {(const void **)&d.pairs, tb.pairs.data(), tb.pairs.size() * 2},
         {(const void **)&d.pinfo, tb.pinfo.data(), tb.pinfo.size() * 4},
         {(const void **)&d.pre, tb.pre.data(), tb.pre.size() * 8},

@@ -70,9 +70,9 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
                                                   warp * kWarpPairBytes);
     const int64_t n0 = ONE ? code0.n : codes[0].n;
 
-    /* the queue's slots: all B, or (range_count: the per-bucket counts of
-     * the sort into perm) the slots of buckets [blo, bhi) */
-    int64_t slot_lo = 0, slot_hi = B;
+    /* the queue's slots: all B (< 2^32), or (range_count: the per-bucket
+     * counts of the sort into perm) the slots of buckets [blo, bhi) */
+    uint32_t slot_lo = 0, slot_hi = (uint32_t)B;
     if (range_count) {
         uint32_t before = 0, inside = 0;
         for (int i = lane; i < bhi; i += 32) {
@@ -82,70 +82,85 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
             else
                 inside += c;
         }
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) {
-            before += __shfl_xor_sync(FULL_MASK, before, m);
-            inside += __shfl_xor_sync(FULL_MASK, inside, m);
-        }
-        slot_lo = before;
-        slot_hi = (int64_t)before + inside;
+        slot_lo = __reduce_add_sync(FULL_MASK, before);
+        slot_hi = slot_lo + __reduce_add_sync(FULL_MASK, inside);
     }
     /* the warp's block sequence: `grab` consecutive queue slots per atomic;
      * with perm (mixed codes) slot i holds the block perm[i], so that the
-     * blocks of one decoder variant are decoded together.  A warp that finds
-     * the queue empty lets a programmatically dependent launch (the next
-     * variant's) start on the SMs this one's last blocks leave idle. */
-    int64_t pos = 0, end = 0;
-    auto next_block = [&]() -> int64_t {
-        if (pos >= end) {
-            unsigned long long c = 0;
-            if (lane == 0)
-                c = atomicAdd(queue, (unsigned long long)grab);
-            c = __shfl_sync(FULL_MASK, c, 0);
-            pos = slot_lo + (int64_t)c;
-            end = min(pos + (int64_t)grab, slot_hi);
-            if (pos >= slot_hi) {
-                asm volatile("griddepcontrol.launch_dependents;");
-                return B;
+     * blocks of one decoder variant are decoded together.  The slots' blocks
+     * are read once per grab, a lane a slot, and their layout entries
+     * prefetched (read block by block, each waited for its slot's load).  A
+     * warp that finds the queue empty lets a programmatically dependent
+     * launch (the next variant's) start on the SMs this one's last blocks
+     * leave idle. */
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    uint32_t pos = 0, end = 0;  /* slots of the grab not yet read */
+    int have = 0, next = 0;     /* blocks held in the lanes, and the next one to take */
+    uint32_t held = 0;
+    auto next_block = [&]() -> uint32_t {
+        if (next >= have) {
+            if (pos >= end) {
+                unsigned long long c = 0;
+                if (lane == 0)
+                    c = atomicAdd(queue, (unsigned long long)grab);
+                c = __shfl_sync(FULL_MASK, c, 0);
+                if (c >= (unsigned long long)(slot_hi - slot_lo)) {
+                    asm volatile("griddepcontrol.launch_dependents;");
+                    return kNone;
+                }
+                pos = slot_lo + (uint32_t)c;
+                end = slot_hi - pos > (uint32_t)grab ? pos + (uint32_t)grab : slot_hi;
             }
+            have = (int)min(end - pos, 32u);
+            next = 0;
+            if (lane < have) {
+                held = perm ? __ldg(perm + pos + lane) : pos + (uint32_t)lane;
+                if (!ONE && code_id)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(code_id + held));
+                if (llr_off)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(llr_off + held));
+                if (cw_off)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(cw_off + held));
+            }
+            pos += (uint32_t)have;
         }
-        const int64_t slot = pos++;
-        return perm ? (int64_t)__ldg(perm + slot) : slot;
+        return __shfl_sync(FULL_MASK, held, next++);
     };
-    auto stage = [&](int64_t b, int slot) {
-        if (b < B) {
-            const int cid = ONE ? 0 : code_id ? code_id[b] : 0;
+    /* copies block b's LLRs into the ring's slot; returns its code id */
+    auto stage = [&](uint32_t b, int slot) -> int {
+        int cid = 0;
+        if (b != kNone) {
+            cid = !ONE && code_id ? code_id[b] : 0;
             if (cid >= 0 && cid < ncodes) {
                 const int n = ONE ? code0.n : codes[cid].n;
-                const int64_t lo = llr_off ? llr_off[b] : b * n0;
+                const float *src = llr + (llr_off ? llr_off[b] : (int64_t)b * n0);
 #pragma unroll
                 for (int k = 0; k < K; k++) {
                     const int i = k * 32 + lane;
                     if (i < n)
-                        __pipeline_memcpy_async(ring + slot * kSlot + i, llr + lo + i, 4);
+                        __pipeline_memcpy_async(ring + slot * kSlot + i, src + i, 4);
                 }
             }
         }
         __pipeline_commit();
+        return cid;
     };
 
-    int64_t b = next_block();
+    uint32_t b = next_block();
     int slot = 0;
-    stage(b, slot);
-    int64_t bn = next_block();
-    while (b < B) {
-        stage(bn, slot ^ 1);
+    int cid = stage(b, slot);
+    while (b != kNone) {
+        const uint32_t bn = next_block();
+        const int cidn = stage(bn, slot ^ 1);
         __pipeline_wait_prior(1); /* block b's copies have landed */
         __syncwarp();
-        const int cid = ONE ? 0 : code_id ? code_id[b] : 0;
-        const int64_t co = cw_off ? cw_off[b] : b * n0;
+        uint8_t *out = cw + (cw_off ? cw_off[b] : (int64_t)b * n0);
         const float *l = ring + slot * kSlot;
         /* the 256-key sort stays rolled; the others are unrolled */
         if (ONE) {
-            decode_block_warp<K, W, true, (K >= 8)>(code0, l, cw + co, q + b, ab + b, cap, budget,
-                                                    bsm, lane, filter, heavy, &counters[1],
-                                                    b_base + (unsigned long long)b, hand,
-                                                    hand_cap);
+            decode_block_warp<K, W, true, (K >= 8)>(code0, l, out, q + b, ab + b, cap, budget, bsm,
+                                                    lane, filter, heavy, &counters[1], b_base + b,
+                                                    hand, hand_cap);
         } else if (cid < 0 || cid >= ncodes) {
             if (lane == 0) {
                 q[b] = 0u;
@@ -154,14 +169,13 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
         } else {
             /* the block's descriptor is read where it is used (a register
              * copy of it spilled) */
-            decode_block_warp<K, W, true, (K >= 8)>(codes[cid], l, cw + co, q + b, ab + b, cap,
-                                                    budget, bsm, lane, filter, heavy, &counters[1],
-                                                    b_base + (unsigned long long)b, hand,
-                                                    hand_cap);
+            decode_block_warp<K, W, true, (K >= 8)>(codes[cid], l, out, q + b, ab + b, cap, budget,
+                                                    bsm, lane, filter, heavy, &counters[1],
+                                                    b_base + b, hand, hand_cap);
         }
         __syncwarp(); /* slot is free before it is refilled */
         b = bn;
-        bn = next_block();
+        cid = cidn;
         slot ^= 1;
     }
     __pipeline_wait_prior(0);

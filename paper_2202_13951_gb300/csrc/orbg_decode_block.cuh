@@ -85,15 +85,14 @@ __device__ __forceinline__ uint64_t shfl_xor_u64(uint64_t v, int m)
 }
 
 /* Shared memory of one block in flight: hperm[n+1] full syndromes, then
- * (for W > 1) h0[n+1], the first 32-bit word of each, then pi[256] and the
- * staged codeword cw[256].  Entry 0 of hperm and h0 is a zero column
- * (BlockSmem). */
+ * (for W > 1) h0[n+1], the key of each, then pi[256].  Entry 0 of hperm and
+ * h0 is a zero column (BlockSmem). */
 __host__ __device__ __forceinline__ uint32_t block_smem_bytes(int n, int w32)
 {
     uint32_t h = (uint32_t)(n + 1) * 4u * (uint32_t)w32;
     h = (h + 15u) & ~15u;
     uint32_t h0 = w32 > 1 ? (((uint32_t)(n + 1) * 4u + 15u) & ~15u) : 0u;
-    return h + h0 + 256u + 256u;
+    return h + h0 + 256u;
 }
 
 /* h[r] (and h0[r]) is the column of sorted position r, 0 <= r < n; the
@@ -104,7 +103,6 @@ template <int W> struct BlockSmem {
     T *h;
     uint32_t *h0;
     uint8_t *pi;
-    uint8_t *cw;
     __device__ __forceinline__ BlockSmem(unsigned char *base, int n)
     {
         h = reinterpret_cast<T *>(base) + 1;
@@ -116,7 +114,6 @@ template <int W> struct BlockSmem {
             h0 = reinterpret_cast<uint32_t *>(base) + 1;
         }
         pi = p;
-        cw = pi + 256;
     }
 };
 
@@ -165,38 +162,62 @@ template <int K> struct KeyBits {
 
 /* ------------------------------------------------------- step 1: load */
 
-/* Loads the block, writes y into cw, builds the K 32-bit sort keys per lane
- * and returns s0 (identical in every lane).  *nan is warp-uniform. */
+/* A sort key of received position i from the bits of |L_i|. */
+template <int K> __device__ __forceinline__ uint32_t make_key(uint32_t bits, int i)
+{
+    typedef KeyBits<K> KB;
+    return ((bits >> KB::DROP) << KB::IB) | ((uint32_t)i & KB::IMASK);
+}
+
+/* Loads the block: the hard decision y into cw (if not NULL), the bits of
+ * |L| of the lane's K positions (all ones past n) into bits[], and returns
+ * s0 = H y, identical in every lane.  *nan is warp-uniform.  The warp's
+ * ballots of L > 0 are y; lane i holds row i of H (and rows 32 + i, ... of
+ * longer syndromes), and the parity of its AND with y is bit i of s0: the
+ * row loads do not wait for the LLRs, and nothing is summed over lanes. */
 template <int K, int W, bool LS = false>
 __device__ __forceinline__ typename Syn<W>::T load_block(const OrbgDeviceCode &code,
                                                          const float *__restrict__ llr,
-                                                         uint32_t (&key)[K], uint8_t *cw,
+                                                         uint32_t (&bits)[K], uint8_t *cw,
                                                          int lane, bool *nan_out)
 {
-    typedef typename Syn<W>::T T;
-    typedef KeyBits<K> KB;
     const int n = code.n;
-    T s0 = szero<T>();
+    uint32_t row[W][K], y[K];
+#pragma unroll
+    for (int w = 0; w < W; w++)
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            row[w][k] = __ldg(code.hrow + (w * K + k) * 32 + lane);
     bool nan = false;
 #pragma unroll
     for (int k = 0; k < K; k++) {
-        int i = k * 32 + lane;
-        uint32_t bits = 0xFFFFFFFFu; /* padding sorts last */
-        if (i < n) {
-            float L = llr_at<LS>(llr, i);
-            nan |= (L != L);
-            bits = __float_as_uint(L) & 0x7FFFFFFFu;
-            uint8_t y = L > 0.0f ? 1 : 0;
-            cw[i] = y;
-            if (y)
-                s0 = sx(s0, load_col<W>(code.hcol, i));
-        }
-        key[k] = ((bits >> KB::DROP) << KB::IB) | ((uint32_t)i & KB::IMASK);
+        const int i = k * 32 + lane;
+        const bool in = i < n;
+        const float L = in ? llr_at<LS>(llr, i) : 0.0f;
+        const uint32_t a = __float_as_uint(L) & 0x7FFFFFFFu;
+        nan |= a > 0x7F800000u;
+        y[k] = __ballot_sync(FULL_MASK, L > 0.0f);
+        if (in && cw != nullptr)
+            cw[i] = L > 0.0f ? 1 : 0;
+        bits[k] = in ? a : 0xFFFFFFFFu;
     }
+    uint32_t s[W];
 #pragma unroll
-    for (int m = 16; m >= 1; m >>= 1)
-        s0 = sx(s0, shfl_xor_all(s0, m));
+    for (int w = 0; w < W; w++) {
+        uint32_t acc = 0;
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            acc ^= row[w][k] & y[k];
+        s[w] = __ballot_sync(FULL_MASK, (__popc(acc) & 1) != 0);
+    }
     *nan_out = __any_sync(FULL_MASK, nan);
+    typename Syn<W>::T s0;
+    if constexpr (W == 1)
+        s0 = s[0];
+    else if constexpr (W == 2)
+        s0 = make_uint2(s[0], s[1]);
+    else
+        s0 = make_uint4(s[0], s[1], s[2], s[3]);
     return s0;
 }
 
@@ -511,18 +532,17 @@ __device__ __forceinline__ void perm_ranks(const OrbgDeviceCode &code, const uin
     }
 }
 
-/* The K truncated keys of a lane, in load order (as load_block makes them). */
+/* The K truncated keys of a lane, in load order. */
 template <int K, bool LS>
 __device__ __forceinline__ void make_keys(const float *__restrict__ llr, int n, int lane,
                                           uint32_t (&key)[K])
 {
-    typedef KeyBits<K> KB;
 #pragma unroll
     for (int k = 0; k < K; k++) {
         const int i = k * 32 + lane;
         const uint32_t bits =
             i < n ? (__float_as_uint(llr_at<LS>(llr, i)) & 0x7FFFFFFFu) : 0xFFFFFFFFu;
-        key[k] = ((bits >> KB::DROP) << KB::IB) | ((uint32_t)i & KB::IMASK);
+        key[k] = make_key<K>(bits, i);
     }
 }
 
@@ -831,31 +851,47 @@ __device__ __forceinline__ PairHit search_band(const OrbgDeviceCode &code,
 
 /* ----------------------------------------------------- step 5: output */
 
-/* Flips of a hit into the staged codeword (one thread). */
-static __device__ __noinline__ void apply_pair_flips(const OrbgDeviceCode &code, const PairHit &hit,
-                                              const uint8_t *pi, uint8_t *cw)
+/* Calls flip(received index) for every position of a hit (one thread). */
+template <typename F>
+__device__ __forceinline__ void pair_flips(const OrbgDeviceCode &code, const PairHit &hit,
+                                           const uint8_t *pi, F flip)
 {
     if (hit.pre == kSingle) {
-        cw[pi[hit.pair]] ^= 1;
+        flip(pi[hit.pair]);
         return;
     }
     const uint32_t p = __ldg(code.pairs + hit.pair);
-    cw[pi[p & 0xFFu]] ^= 1;
-    cw[pi[p >> 8]] ^= 1;
+    flip(pi[p & 0xFFu]);
+    flip(pi[p >> 8]);
     const uint2 r = __ldg(reinterpret_cast<const uint2 *>(code.pre) + hit.pre);
     for (uint32_t m = r.x & 0xFFFFu; m; m &= m - 1u)
-        cw[pi[__ldg(code.light + (__ffs(m) - 1)) - 1]] ^= 1;
+        flip(pi[__ldg(code.light + (__ffs(m) - 1)) - 1]);
     for (uint32_t y = r.x >> 16; y; y >>= 8)
-        cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+        flip(pi[(y & 0xFFu) - 1u]);
     for (uint32_t y = r.y; y; y >>= 8)
-        cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+        flip(pi[(y & 0xFFu) - 1u]);
     if (code.pext) {
         const uint2 e = __ldg(reinterpret_cast<const uint2 *>(code.pext) + hit.pre);
         for (uint32_t y = e.x; y; y >>= 8)
-            cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+            flip(pi[(y & 0xFFu) - 1u]);
         for (uint32_t y = e.y; y; y >>= 8)
-            cw[pi[(y & 0xFFu) - 1u]] ^= 1;
+            flip(pi[(y & 0xFFu) - 1u]);
     }
+}
+
+/* A hit's flips on the hard decision of llr, already in cw: from the LLRs
+ * (no read of cw), or, where they are not at hand, on cw itself. */
+static __device__ __noinline__ void write_pair_flips(const OrbgDeviceCode &code,
+                                                     const PairHit &hit, const uint8_t *pi,
+                                                     const float *llr, uint8_t *cw)
+{
+    pair_flips(code, hit, pi, [=](uint32_t i) { cw[i] = llr[i] > 0.0f ? 0 : 1; });
+}
+static __device__ __noinline__ void toggle_pair_flips(const OrbgDeviceCode &code,
+                                                      const PairHit &hit, const uint8_t *pi,
+                                                      uint8_t *cw)
+{
+    pair_flips(code, hit, pi, [=](uint32_t i) { cw[i] ^= 1; });
 }
 
 /* ---------------------------------------------------- the flat table */
@@ -912,15 +948,18 @@ __device__ __forceinline__ bool flat_test(const typename Syn<W>::T *__restrict__
     return true;
 }
 
-/* Flips of flat pattern t into the staged codeword. */
-__device__ __forceinline__ void apply_flat_flips(const OrbgDeviceCode &code, uint32_t t,
-                                                 const uint8_t *pi, uint8_t *cw)
+/* Flips of flat pattern t on the hard decision of llr, already in cw. */
+template <bool LS>
+__device__ __forceinline__ void write_flat_flips(const OrbgDeviceCode &code, uint32_t t,
+                                                 const uint8_t *pi, const float *llr, uint8_t *cw)
 {
     const uint2 e = __ldg(reinterpret_cast<const uint2 *>(code.flat) + (t - 1));
     for (int i = 0; i < ORBG_FLAT_POS; i++) {
         const int q = flat_pos(e, i);
-        if (q)
-            cw[pi[q - 1]] ^= 1;
+        if (q == 0)
+            break; /* positions come first, zeros after */
+        const int idx = pi[q - 1];
+        cw[idx] = llr_at<LS>(llr, idx) > 0.0f ? 0 : 1;
     }
 }
 
@@ -929,11 +968,12 @@ __device__ __forceinline__ void apply_flat_flips(const OrbgDeviceCode &code, uin
 /*
  * Decode one block with one warp: the flat table, then the bands
  * (search_bands) while no hit is known and the next one starts within
- * `budget`.  A block still open after them is not written: its index is
+ * `budget`.  A block still open after them is left: its index is
  * appended to heavy[] for decode_block_cta, with its reliability order and
  * starting syndrome in the handover record of the same slot when one is free
  * (hand_cap; bit 63 of the heavy[] entry says so); with heavy NULL the
- * caller takes it up.  Returns whether the block was written.  LS: llr
+ * caller takes it up.  Its codeword bytes hold the hard decision by then.
+ * Returns whether the block was finished.  LS: llr
  * points into shared memory (the batched kernel stages it there).
  */
 template <int K, int W, bool LS = false, bool ROLL = true>
@@ -948,9 +988,9 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
     typedef typename Syn<W>::T T;
     const int n = code.n;
     BlockSmem<W> sm(bsm, n);
-    uint32_t key[K];
+    uint32_t key[K]; /* the bits of |L| until they are needed as sort keys */
     bool nan;
-    const T s0 = load_block<K, W, LS>(code, llr, key, sm.cw, lane, &nan);
+    const T s0 = load_block<K, W, LS>(code, llr, key, cw_out, lane, &nan);
     PairHit hit{ORBG_NONE, ORBG_NONE, 0u}; /* prefix NONE: a flat-table hit */
     bool flat_mine = false;
     bool done = true;
@@ -962,6 +1002,9 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
          * so the first step with a hit holds the answer.  Ranks are
          * extracted as the steps need them (one more than needed, so that a
          * tie across the boundary is seen); a tie sorts everything exactly. */
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            key[k] = make_key<K>(key[k], k * 32 + lane);
         sort_lane<K>(key);
         if (lane == 0) {
             sm.h[-1] = szero<T>();
@@ -1070,18 +1113,12 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
         return false;
     }
     const bool found = !nan && hit.t <= cap;
-    if (found) {
+    if (found && hit.t > 1u) {
+        __syncwarp(); /* after the other lanes' stores of the hard decision */
         if (flat_mine)
-            apply_flat_flips(code, hit.t, sm.pi, sm.cw);
+            write_flat_flips<LS>(code, hit.t, sm.pi, llr, cw_out);
         else if (hit.pre != ORBG_NONE && lane == 0)
-            apply_pair_flips(code, hit, sm.pi, sm.cw);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-        int i = k * 32 + lane;
-        if (i < n)
-            cw_out[i] = sm.cw[i];
+            write_pair_flips(code, hit, sm.pi, llr, cw_out);
     }
     if (lane == 0) {
         *q_out = nan ? 0u : found ? hit.t : cap;
@@ -1092,8 +1129,8 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
 }
 
 /* The block loaded and sorted by one warp (rare: a block past phase 1's
- * handover records, and the plain form's open ones): hard decision, order,
- * permuted columns and *s0.  Returns 0, 1 for a code word, 2 for a NaN
+ * handover records, and the plain form's open ones): order, permuted columns
+ * and *s0.  Returns 0, 1 for a code word, 2 for a NaN
  * block. */
 template <int K, int W>
 __device__ __noinline__ int load_and_sort_k(const OrbgDeviceCode &code, const float *llr,
@@ -1104,11 +1141,12 @@ __device__ __noinline__ int load_and_sort_k(const OrbgDeviceCode &code, const fl
     const BlockSmem<W> sm(bsm, n);
     uint32_t key[K];
     bool nan;
-    *s0 = load_block<K, W>(code, llr, key, sm.cw, lane, &nan);
+    *s0 = load_block<K, W>(code, llr, key, nullptr, lane, &nan);
     if (nan)
         return 2;
     if (sz(*s0))
         return 1;
+    make_keys<K, false>(llr, n, lane, key);
     sort_block<K>(key, llr, n, lane);
     build_perm<K, W>(code, key, sm, lane);
     return 0;
@@ -1126,7 +1164,8 @@ __device__ __forceinline__ int load_and_sort(const OrbgDeviceCode &code, const f
 /* ------------------------------------------------ one CTA, one block */
 
 /*
- * All warps of the CTA decode one block.  Its order comes from phase 1's
+ * All warps of the CTA decode one block whose hard decision is in cw_out
+ * already (phase 1 wrote it).  Its order comes from phase 1's
  * handover record, or warp 0 loads and sorts; all threads then build the
  * subset tables of the light positions and the filter of the block's pairs
  * (several in turn for an order of more than kPairChunk pairs); then
@@ -1156,7 +1195,6 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
         /* phase 1's handover record: the block's order and starting
          * syndrome; every thread takes a share of the positions */
         for (int i = (int)threadIdx.x; i < n; i += (int)blockDim.x) {
-            sm.cw[i] = __ldg(llr + i) > 0.0f ? 1 : 0;
             const int idx = (int)rec[i];
             sm.pi[i] = (uint8_t)idx;
             const T col = load_col<W>(code.hcol, idx);
@@ -1312,10 +1350,7 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
     const bool is_nan = best == ORBG_NONE - 1;
     const bool hit = !is_nan && best <= cap;
     if (start == ORBG_NONE && hit && mine.t == best)
-        apply_pair_flips(code, mine, sm.pi, sm.cw);
-    __syncthreads();
-    for (int i = warp * 32 + lane; i < n; i += nwarps * 32)
-        cw_out[i] = sm.cw[i];
+        toggle_pair_flips(code, mine, sm.pi, cw_out);
     if (warp == 0 && lane == 0) {
         *q_out = is_nan ? 0u : hit ? best : cap;
         *ab_out = is_nan ? 2 : hit ? 0 : 1;

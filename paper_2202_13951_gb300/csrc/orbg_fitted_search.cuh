@@ -780,6 +780,9 @@ __device__ void prepare_fitted_block(const OrbgDeviceCode &code, const float *__
     } else if (sz(s0) && rec_out == nullptr) {
         q = 1; /* the hard decision is a code word: query 1, whatever the model */
     } else {
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            key[k] = make_key<K>(key[k], k * 32 + lane);
         sort_block<K>(key, llr, n, lane);
 #pragma unroll
         for (int k = 0; k < K; k++) {

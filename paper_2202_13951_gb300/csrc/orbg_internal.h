@@ -66,6 +66,9 @@
 /* What a kernel needs of one code (passed by value or from a device array). */
 struct OrbgDeviceCode {
     const uint32_t *hcol;        /* [n][w32]: column j of H, row i at bit i%32 of word i/32 */
+    const uint32_t *hrow;        /* [w32][K][32]: 32 received positions of 32 rows of H, K words
+                                  * a row (n <= 32, 64, 128, 256: 1, 2, 4, 8): bit j % 32 of
+                                  * entry (i / 32, j / 32, i % 32) is H[i][j] */
     const uint16_t *pairs;       /* [npairs] a0 | b0 << 8, 0-based, by (weight, a, b) */
     const uint32_t *pinfo;       /* [npairs] its group of equally heavy pairs | first pair of the
                                   * group << 16 */
