@@ -68,6 +68,8 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
     /* the warp's own pairs (search_band) */
     uint32_t *filter = reinterpret_cast<uint32_t *>(smem + nwarps * (bstride + 2 * kSlot * 4) +
                                                   warp * kWarpPairBytes);
+    uint32_t *list = reinterpret_cast<uint32_t *>(
+        smem + nwarps * (bstride + 2 * kSlot * 4 + kWarpPairBytes) + warp * key_list_bytes<K>());
     const int64_t n0 = ONE ? code0.n : codes[0].n;
 
     /* the queue's slots: all B (< 2^32), or (range_count: the per-bucket
@@ -159,8 +161,8 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
         /* the 256-key sort stays rolled; the others are unrolled */
         if (ONE) {
             decode_block_warp<K, W, true, (K >= 8)>(code0, l, out, q + b, ab + b, cap, budget, bsm,
-                                                    lane, filter, heavy, &counters[1], b_base + b,
-                                                    hand, hand_cap);
+                                                    lane, filter, list, heavy, &counters[1],
+                                                    b_base + b, hand, hand_cap);
         } else if (cid < 0 || cid >= ncodes) {
             if (lane == 0) {
                 q[b] = 0u;
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
             /* the block's descriptor is read where it is used (a register
              * copy of it spilled) */
             decode_block_warp<K, W, true, (K >= 8)>(codes[cid], l, out, q + b, ab + b, cap, budget,
-                                                    bsm, lane, filter, heavy, &counters[1],
+                                                    bsm, lane, filter, list, heavy, &counters[1],
                                                     b_base + b, hand, hand_cap);
         }
         __syncwarp(); /* slot is free before it is refilled */
@@ -190,7 +192,8 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
  * and its own pairs. */
 template <int K> constexpr uint32_t warp_smem_bytes(uint32_t bstride)
 {
-    return bstride + 2u * 32u * K * (uint32_t)sizeof(float) + kWarpPairBytes;
+    return bstride + 2u * 32u * K * (uint32_t)sizeof(float) + kWarpPairBytes +
+           key_list_bytes<K>();
 }
 
 /* Phase 1 of one decoder variant (K, W): the blocks of sort buckets

@@ -480,13 +480,61 @@ __device__ __forceinline__ void sort_lane(uint32_t (&key)[K])
         }
 }
 
+/* The lane's keys, ascending: its smallest, and how the next ones follow.
+ * Up to four keys shift down in registers; eight (n > 128) go to a list in
+ * shared memory, where taking one costs a load instead of eight moves and
+ * the registers are free for the search (about 20 warp instructions a rank
+ * in registers, 13 with the list).  The list ends on a key past all. */
+template <int K> constexpr bool kKeyList = K >= 8;
+template <int K> __host__ __device__ constexpr uint32_t key_list_bytes() { return kKeyList<K> ? (K + 1) * 128u : 0u; }
+template <int K> struct LaneKeys {
+    uint32_t key[K];
+    __device__ __forceinline__ LaneKeys(const uint32_t (&sorted)[K], uint32_t *, int)
+    {
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            key[k] = sorted[k];
+    }
+    __device__ __forceinline__ uint32_t first() const { return key[0]; }
+    __device__ __forceinline__ void take(bool mine)
+    {
+        if (mine) {
+#pragma unroll
+            for (int k = 0; k + 1 < K; k++)
+                key[k] = key[k + 1];
+            key[K - 1] = 0xFFFFFFFFu;
+        }
+    }
+};
+template <> struct LaneKeys<8> {
+    uint32_t cur;
+    const uint32_t *at;
+    __device__ __forceinline__ LaneKeys(const uint32_t (&sorted)[8], uint32_t *list, int lane)
+    {
+#pragma unroll
+        for (int k = 1; k < 8; k++)
+            list[k * 32 + lane] = sorted[k];
+        list[8 * 32 + lane] = 0xFFFFFFFFu;
+        cur = sorted[0];
+        at = list + 32 + lane;
+    }
+    __device__ __forceinline__ uint32_t first() const { return cur; }
+    __device__ __forceinline__ void take(bool mine)
+    {
+        if (mine) {
+            cur = *at;
+            at += 32;
+        }
+    }
+};
+
 /* Extracts ranks have .. upto-1 (upto <= 64): lane r keeps rank r's key in
  * mine[0], rank r + 32's in mine[1].  Returns true if two consecutive ranks
  * (this call's or the last earlier one, in *prev) have equal truncated
  * reliabilities: then the truncated order may differ from the exact one and
  * the caller sorts exactly instead. */
 template <int K>
-__device__ __forceinline__ bool extract_ranks(uint32_t (&key)[K], int have, int upto,
+__device__ __forceinline__ bool extract_ranks(LaneKeys<K> &keys, int have, int upto,
                                               uint32_t *prev, uint32_t (&mine)[2], int lane)
 {
     typedef KeyBits<K> KB;
@@ -496,14 +544,9 @@ __device__ __forceinline__ bool extract_ranks(uint32_t (&key)[K], int have, int 
     for (int half = 0; half < 2; half++) {
         const int end = min(upto, 32 * half + 32);
         for (int r = max(have, 32 * half); r < end; r++) {
-            const uint32_t g = __reduce_min_sync(FULL_MASK, key[0]);
+            const uint32_t g = __reduce_min_sync(FULL_MASK, keys.first());
             tie |= (g >> KB::IB) == (pv >> KB::IB);
-            if (key[0] == g) {
-#pragma unroll
-                for (int k = 0; k + 1 < K; k++)
-                    key[k] = key[k + 1];
-                key[K - 1] = 0xFFFFFFFFu;
-            }
+            keys.take(keys.first() == g);
             if (lane == r - 32 * half)
                 mine[half] = g;
             pv = g;
@@ -972,7 +1015,7 @@ __device__ __forceinline__ void write_flat_flips(const OrbgDeviceCode &code, uin
  * appended to heavy[] for decode_block_cta, with its reliability order and
  * starting syndrome in the handover record of the same slot when one is free
  * (hand_cap; bit 63 of the heavy[] entry says so); with heavy NULL the
- * caller takes it up.  Its codeword bytes hold the hard decision by then.
+ * caller takes it up.  list: key_list_bytes<K>() bytes.  Its codeword bytes hold the hard decision by then.
  * Returns whether the block was finished.  LS: llr
  * points into shared memory (the batched kernel stages it there).
  */
@@ -981,6 +1024,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
                                   uint8_t *__restrict__ cw_out, uint32_t *__restrict__ q_out,
                                   uint8_t *__restrict__ ab_out, uint32_t cap, uint32_t budget,
                                   unsigned char *__restrict__ bsm, int lane, uint32_t *filter,
+                                  uint32_t *list,
                                   unsigned long long *heavy, unsigned long long *heavy_count,
                                   unsigned long long block_index,
                                   unsigned char *hand = nullptr, uint32_t hand_cap = 0)
@@ -1006,6 +1050,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
         for (int k = 0; k < K; k++)
             key[k] = make_key<K>(key[k], k * 32 + lane);
         sort_lane<K>(key);
+        LaneKeys<K> keys(key, list, lane);
         if (lane == 0) {
             sm.h[-1] = szero<T>();
             if (W > 1)
@@ -1055,7 +1100,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
             if (upto > have) {
                 /* a tie among the ranks, or more than 64, sorts everything
                  * exactly */
-                if (upto > 64 || extract_ranks<K>(key, have, upto, &prev, mine_key, lane)) {
+                if (upto > 64 || extract_ranks<K>(keys, have, upto, &prev, mine_key, lane)) {
                     make_keys<K, LS>(llr, n, lane, key);
                     sort_block<K, LS, ROLL>(key, llr, n, lane);
                     build_perm<K, W>(code, key, sm, lane);

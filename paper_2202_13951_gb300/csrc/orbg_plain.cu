@@ -35,10 +35,11 @@ __global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
     const int64_t b = b0 + warp;
     if (b < B) {
         const int64_t off = b * (int64_t)code.n;
-        unsigned char *own = smem + warp * (bstride + kWarpPairBytes);
+        unsigned char *own = smem + warp * (bstride + kWarpPairBytes + key_list_bytes<K>());
         const bool done = decode_block_warp<K, W, false, (K >= 8)>(
             code, llr + off, cw + off, q + b, ab + b, cap, cap, own, lane,
-            reinterpret_cast<uint32_t *>(own + bstride), nullptr, nullptr, 0ull);
+            reinterpret_cast<uint32_t *>(own + bstride),
+            reinterpret_cast<uint32_t *>(own + bstride + kWarpPairBytes), nullptr, nullptr, 0ull);
         if (!done && lane == 0)
             atomicOr(&s_open, 1u << warp);
     }
@@ -57,7 +58,7 @@ cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t
                            uint8_t *cw, uint32_t *q, uint8_t *ab, cudaStream_t st)
 {
     const uint32_t bstride = block_smem_bytes(code.n, W);
-    size_t smem = (size_t)(bstride + kWarpPairBytes) * kPlainWarps;
+    size_t smem = (size_t)(bstride + kWarpPairBytes + key_list_bytes<K>()) * kPlainWarps;
     const size_t cta = (size_t)bstride + pair_smem_bytes(code.npairs);
     if (smem < cta)
         smem = cta;
