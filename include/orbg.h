@@ -271,7 +271,8 @@ ORBG_API int orbg_decode_batched_noalloc(const orbg_codeset *set,
  *   warps_per_cta   phase 1: warps per CTA, one block per warp (1..16; 0 = 8)
  *   ctas_per_sm     phase 1: resident CTAs per SM (0 = as many as fit)
  *   blocks_per_grab phase 1: blocks a warp takes per work-queue atomic
- *                   (1..1024; 0 = 4)
+ *                   (1..1024; 0 = 4), fewer in a batch of less than eight
+ *                   grabs a warp; likewise warps_per_cta in one of few blocks
  *   warp_budget     phase 1: a single warp searches its block's order in bands
  *                   (for basic ORBGRAND up to query 256, 2,375 and 16,857) and
  *                   hands the block to phase 2 before a band that starts past

@@ -35,9 +35,15 @@ using namespace orbg_dev;
 
 constexpr int kCounters = ORBG_BATCHED_COUNTERS;
 
-/* resident phase-1 CTAs per SM the register allocation is sized for */
+/* Resident phase-1 CTAs per SM the register allocation is sized for: four
+ * for one code of up to 128 keys and one-word syndromes (64 registers; shared
+ * memory allows it), else three.  Measured on 400,000 BCH(127,113) blocks:
+ * four 340 us, three 368, two 431; where the descriptor is read per block the
+ * kernels spill at 64 (three serving codes, 8,191 blocks: four 190 us, three
+ * 170; the four mixed codes with n = 256 at four 2,769 us, at three 2,431, at
+ * two 2,541). */
 #ifndef ORBG_PHASE1_MIN_CTAS
-#define ORBG_PHASE1_MIN_CTAS 3
+#define ORBG_PHASE1_MIN_CTAS(K, W, ONE) ((ONE) && (K) < 8 && (W) == 1 ? 4 : 3)
 #endif
 
 /* ONE: every block is the code in the kernel's parameters; otherwise each
@@ -45,7 +51,7 @@ constexpr int kCounters = ORBG_BATCHED_COUNTERS;
  * W (one decoder variant per launch, the blocks taken from their sort
  * buckets). */
 template <int K, int W, bool ONE>
-__global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel(
+__global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS(K, W, ONE)) orbg_batched_kernel(
     const OrbgDeviceCode *__restrict__ codes, int ncodes, const int32_t *__restrict__ code_id,
     const int64_t *__restrict__ llr_off, const float *__restrict__ llr, int64_t B, uint32_t cap,
     uint32_t budget, uint8_t *__restrict__ cw, const int64_t *__restrict__ cw_off,
@@ -53,7 +59,7 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
     unsigned long long *__restrict__ queue, unsigned long long *__restrict__ heavy,
     const uint32_t *__restrict__ perm,
     unsigned char *__restrict__ hand, uint32_t hand_cap, unsigned long long b_base,
-    uint32_t bstride, int grab, const uint32_t *__restrict__ range_count,
+    uint32_t bstride, int grab, int ahead, const uint32_t *__restrict__ range_count,
     int blo, int bhi, const __grid_constant__ OrbgDeviceCode code0)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -148,19 +154,21 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
         return cid;
     };
 
+    /* ahead: the next block is taken and its LLRs copied in while this one is
+     * decoded; a batch of few blocks a warp leaves it to the others until
+     * this one is done */
     uint32_t b = next_block();
     int slot = 0;
     int cid = stage(b, slot);
     while (b != kNone) {
-        const uint32_t bn = next_block();
-        const int cidn = stage(bn, slot ^ 1);
+        uint32_t bn = ahead ? next_block() : kNone;
+        int cidn = stage(bn, slot ^ 1);
         __pipeline_wait_prior(1); /* block b's copies have landed */
         __syncwarp();
         uint8_t *out = cw + (cw_off ? cw_off[b] : (int64_t)b * n0);
         const float *l = ring + slot * kSlot;
-        /* the 256-key sort stays rolled; the others are unrolled */
         if (ONE) {
-            decode_block_warp<K, W, true, (K >= 8)>(code0, l, out, q + b, ab + b, cap, budget, bsm,
+            decode_block_warp<K, W, true>(code0, l, out, q + b, ab + b, cap, budget, bsm,
                                                     lane, filter, list, heavy, &counters[1],
                                                     b_base + b, hand, hand_cap);
         } else if (cid < 0 || cid >= ncodes) {
@@ -171,11 +179,15 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS) orbg_batched_kernel
         } else {
             /* the block's descriptor is read where it is used (a register
              * copy of it spilled) */
-            decode_block_warp<K, W, true, (K >= 8)>(codes[cid], l, out, q + b, ab + b, cap, budget,
+            decode_block_warp<K, W, true>(codes[cid], l, out, q + b, ab + b, cap, budget,
                                                     bsm, lane, filter, list, heavy, &counters[1],
                                                     b_base + b, hand, hand_cap);
         }
         __syncwarp(); /* slot is free before it is refilled */
+        if (!ahead) {
+            bn = next_block();
+            cidn = stage(bn, slot ^ 1);
+        }
         b = bn;
         cid = cidn;
         slot ^= 1;
@@ -196,6 +208,45 @@ template <int K> constexpr uint32_t warp_smem_bytes(uint32_t bstride)
            key_list_bytes<K>();
 }
 
+/* How a phase-1 launch of B blocks is cut: warps per CTA, queue slots per
+ * grab, whether warps take blocks ahead, and the grid.  A batch of few blocks
+ * is spread over the SMs and shared out block by block: with the tuned grab
+ * of four, 257 blocks of BCH(127,113) ran four after another on 65 warps of
+ * nine SMs.  Measured with it and without: three serving codes, 8,191 blocks,
+ * 170 -> 121 us. */
+struct Cut {
+    int wpc, grab, ahead, grid;
+};
+template <typename Kern>
+int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
+{
+    int dev = 0, sms = 1;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return (int)e;
+    int wpc = a.warps_per_cta > 0 ? (a.warps_per_cta > 8 ? 8 : a.warps_per_cta) : 8;
+    const int64_t spread = (a.B + 2 * sms - 1) / (2 * sms); /* two CTAs an SM */
+    if (wpc > spread)
+        wpc = (int)spread;
+    int rc = orbg_grid_for((const void *)kern, wpc * 32, (size_t)per_warp * wpc, a.ctas_per_sm,
+                           &c->grid);
+    if (rc != 0)
+        return rc;
+    const int64_t warps = (int64_t)c->grid * wpc;
+    int64_t g = a.grab < 1 ? 1 : a.grab;
+    const int64_t fair = a.B / (8 * warps); /* eight grabs a warp or more */
+    if (g > fair)
+        g = fair > 0 ? fair : 1;
+    c->wpc = wpc;
+    c->grab = (int)g;
+    c->ahead = a.B > 4 * warps;
+    const int64_t need = ((a.B + g - 1) / g + wpc - 1) / wpc;
+    if (c->grid > need)
+        c->grid = (int)(need > 0 ? need : 1);
+    return 0;
+}
+
 /* Phase 1 of one decoder variant (K, W): the blocks of sort buckets
  * [blo, bhi) of ss.perm (blo < 0: every block, in order), on its own queue.
  * pdl: the launch may begin while the previous launch in the stream (the
@@ -204,27 +255,19 @@ template <int K, int W>
 int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned long long *queue,
                    int blo, int bhi, int pdl)
 {
-    const int wpc = a.warps_per_cta > 0 ? (a.warps_per_cta > 8 ? 8 : a.warps_per_cta) : 8;
-    const int g = a.grab < 1 ? 1 : a.grab;
     const int nk = a.n_max < 32 * K ? a.n_max : 32 * K;
     const uint32_t bstride = block_smem_bytes(nk, W);
     auto k1 = orbg_batched_kernel<K, W, false>;
-    const size_t smem1 = (size_t)warp_smem_bytes<K>(bstride) * wpc;
-    int grid = 0;
-    int rc = orbg_grid_for((const void *)k1, wpc * 32, smem1, a.ctas_per_sm, &grid);
+    Cut c;
+    const int rc = cut_launch(k1, a, warp_smem_bytes<K>(bstride), &c);
     if (rc != 0)
         return rc;
-    if (blo < 0) {
-        const int64_t need = ((a.B + g - 1) / g + wpc - 1) / wpc;
-        if (grid > need)
-            grid = (int)(need > 0 ? need : 1);
-    }
     const bool sorted = blo >= 0;
     OrbgDeviceCode c0{};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)(wpc * 32));
-    cfg.dynamicSmemBytes = smem1;
+    cfg.gridDim = dim3((unsigned)c.grid);
+    cfg.blockDim = dim3((unsigned)(c.wpc * 32));
+    cfg.dynamicSmemBytes = (size_t)warp_smem_bytes<K>(bstride) * c.wpc;
     cfg.stream = (cudaStream_t)a.stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -235,15 +278,13 @@ int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned lon
         &cfg, k1, a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, a.budget, a.cw,
         a.cw_off, a.q, a.ab, ss.counters, queue, ss.heavy,
         sorted ? (const uint32_t *)ss.perm : (const uint32_t *)nullptr, ss.hand, ss.hand_cap,
-        (unsigned long long)a.scratch_base, bstride, g,
+        (unsigned long long)a.scratch_base, bstride, c.grab, c.ahead,
         sorted ? (const uint32_t *)ss.count : (const uint32_t *)nullptr, blo, bhi, c0);
 }
 
 template <int KMAX, int WMAX, bool ONE>
 cudaError_t launch_t(const OrbgBatchedArgs &a)
 {
-    const int wpc = a.warps_per_cta > 0 ? (a.warps_per_cta > 8 ? 8 : a.warps_per_cta) : 8;
-    const int g = a.grab < 1 ? 1 : a.grab;
     const uint32_t bstride = block_smem_bytes(a.n_max, a.w32_max);
     const OrbgScratch sc =
         orbg_scratch_layout(a.scratch, a.scratch_B > 0 ? a.scratch_B : a.B, a.ncodes);
@@ -251,10 +292,10 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
     unsigned long long *heavy = sc.heavy;
     cudaStream_t st = (cudaStream_t)a.stream;
     cudaError_t e;
-    int grid = 0, rc;
+    int rc;
     if (a.stage == 2) {
         /* phase 2 over the open blocks every chunk's phase 1 listed */
-        return launch_heavy_t<WMAX, ONE>(a, counters, heavy, sc.hand);
+        return launch_heavy_t<WMAX, ONE>(a, counters, heavy, sc.hand, false);
     }
     /* this launch's slot: its queue heads, bucket counts and cursors, and
      * its blocks' part of the order array */
@@ -295,17 +336,14 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
         }
     } else {
         auto k1 = orbg_batched_kernel<KMAX, WMAX, true>;
-        const size_t smem1 = (size_t)warp_smem_bytes<KMAX>(bstride) * wpc;
-        if ((rc = orbg_grid_for((const void *)k1, wpc * 32, smem1, a.ctas_per_sm, &grid)) != 0)
+        Cut c;
+        if ((rc = cut_launch(k1, a, warp_smem_bytes<KMAX>(bstride), &c)) != 0)
             return (cudaError_t)rc;
-        int64_t units = (a.B + g - 1) / g;
-        int64_t need = (units + wpc - 1) / wpc;
-        if (grid > need) grid = (int)(need > 0 ? need : 1);
-        k1<<<grid, wpc * 32, smem1, st>>>(a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B,
-                                          a.cap, a.budget, a.cw, a.cw_off, a.q, a.ab, counters,
-                                          queue, heavy, nullptr, sc.hand, sc.hand_cap,
-                                          (unsigned long long)a.scratch_base, bstride, g, nullptr,
-                                          0, 0, *a.code0);
+        k1<<<c.grid, c.wpc * 32, (size_t)warp_smem_bytes<KMAX>(bstride) * c.wpc, st>>>(
+            a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, a.budget, a.cw, a.cw_off,
+            a.q, a.ab, counters, queue, heavy, nullptr, sc.hand, sc.hand_cap,
+            (unsigned long long)a.scratch_base, bstride, c.grab, c.ahead, nullptr, 0, 0,
+            *a.code0);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }
@@ -314,7 +352,7 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
      * length) */
     if (a.stage == 1)
         return cudaSuccess; /* phase 2 comes later, over every chunk's list */
-    return launch_heavy_t<WMAX, ONE>(a, counters, heavy, sc.hand);
+    return launch_heavy_t<WMAX, ONE>(a, counters, heavy, sc.hand, true);
 }
 
 /* Phases 1 and 2 for keys-per-lane bound KMAX and syndrome width WMAX: one

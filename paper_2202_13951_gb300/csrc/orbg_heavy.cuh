@@ -37,6 +37,8 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
     const int lane = threadIdx.x & 31;
     const int nwarps = blockDim.x >> 5;
     const int64_t n0 = ONE ? code0.n : codes[0].n;
+    /* launched while phase 1 finishes: its list is complete after this */
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (;;) {
         if (threadIdx.x == 0) {
             const unsigned long long nheavy = *((volatile unsigned long long *)&counters[1]);
@@ -84,7 +86,7 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
 
 template <int WMAX, bool ONE>
 cudaError_t launch_heavy_t(const OrbgBatchedArgs &a, unsigned long long *counters,
-                           const unsigned long long *heavy, const unsigned char *hand)
+                           const unsigned long long *heavy, const unsigned char *hand, bool pdl)
 {
     auto k2 = orbg_heavy_kernel<WMAX, ONE>;
     const int hw = a.heavy_warps > 0 ? a.heavy_warps : 8;
@@ -98,11 +100,20 @@ cudaError_t launch_heavy_t(const OrbgBatchedArgs &a, unsigned long long *counter
     OrbgDeviceCode c0{};
     if (ONE)
         c0 = *a.code0;
-    k2<<<grid, hw * 32, smem, (cudaStream_t)a.stream>>>(a.d_codes, a.ncodes, a.code_id,
-                                                        a.llr_off, a.llr, a.cap, a.cw, a.cw_off,
-                                                        a.q, a.ab, counters, heavy, hand, bstride,
-                                                        c0);
-    return cudaGetLastError();
+    /* pdl: the launch before it in the stream is its phase 1, which lets it
+     * come on as the queue runs empty */
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)(hw * 32));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = (cudaStream_t)a.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k2, a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.cap,
+                              a.cw, a.cw_off, a.q, a.ab, counters, heavy, hand, bstride, c0);
 }
 
 }  // namespace orbg_batched_impl

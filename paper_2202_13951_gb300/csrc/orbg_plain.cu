@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
     if (b < B) {
         const int64_t off = b * (int64_t)code.n;
         unsigned char *own = smem + warp * (bstride + kWarpPairBytes + key_list_bytes<K>());
-        const bool done = decode_block_warp<K, W, false, (K >= 8)>(
+        const bool done = decode_block_warp<K, W, false>(
             code, llr + off, cw + off, q + b, ab + b, cap, cap, own, lane,
             reinterpret_cast<uint32_t *>(own + bstride),
             reinterpret_cast<uint32_t *>(own + bstride + kWarpPairBytes), nullptr, nullptr, 0ull);
