@@ -1279,11 +1279,17 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
  * of it in stage 2's longest warps, 35.6 in the CTAs' walks), 1.7 ms with
  * the longer searches here; 100,000 BCH(127,113) blocks 4.4 -> 1.5 ms.
  */
+/* classes of the prefixes' tree (see kClasses): it is small, and each class
+ * walks all its depth-1 nodes */
+#ifndef ORBG_FS_CLASSES
+#define ORBG_FS_CLASSES 16
+#endif
+constexpr int kFsClasses = ORBG_FS_CLASSES;
 constexpr int kFsTop = 4095;          /* largest weight counted */
 constexpr uint32_t kFsCountMax = 1u << 26; /* counts are exact below, and no cap is above */
 constexpr uint32_t kFsChunk = 7168;   /* pairs in the set at once: load 0.44 */
 constexpr uint32_t kFsBand = 32768;   /* patterns of the first band */
-constexpr uint32_t kFsTied = 8192;    /* entries of the tied-patterns count */
+constexpr uint32_t kFsTied = 1u << kFsSetBits; /* entries of the tied-patterns count */
 
 /* Dynamic shared memory of the CTA. */
 template <int W> struct FpSmem {
@@ -1332,38 +1338,60 @@ template <int W> __host__ __device__ constexpr uint32_t fp_smem_bytes()
 }
 
 /* cum[r] = patterns of weight <= r (the empty one included), r <= top,
- * exact below kFsCountMax, held there above.  x, y: top + 1 words each. */
-__device__ __forceinline__ void count_weights(const uint32_t *rho, int n, uint32_t top, uint32_t *x,
-                                              uint32_t *y, uint32_t *cum)
+ * exact below kFsCountMax, held there above; mall[j]: the least weight of
+ * positions >= j.  From the last position to the first, in place: position p
+ * of weight a adds the sets of later positions shifted by a, which are the
+ * empty one and sets of weight mall[p + 1] or more, so that only r = a and r
+ * >= a + mall[p + 1] change (a quarter of the entries where the weights rise
+ * evenly). */
+__device__ __forceinline__ void count_weights(const uint32_t *rho, const uint32_t *mall, int n,
+                                              uint32_t top, uint32_t *cum)
 {
-    for (uint32_t r = threadIdx.x; r <= top; r += blockDim.x)
-        x[r] = r == 0u;
+    constexpr int kPer = (kFsTop + 32 * kWarps) / (32 * kWarps); /* entries of a thread */
+    for (uint32_t r = threadIdx.x; r <= top; r += 32 * kWarps)
+        cum[r] = r == 0u;
     __syncthreads();
-    for (int j = 1; j <= n; j += 2) {
-        /* two positions at a time: rho[n + 1] is out of reach */
-        const uint32_t a = rho[j], b = rho[j + 1], ab = a + b;
-        if (a > top && b > top)
+    bool stale = false; /* thread 0 changed an entry since the last barrier */
+    for (int p = n; p >= 1; p--) {
+        const uint32_t a = rho[p], lo = a + mall[p + 1];
+        if (a > top)
             continue;
-        for (uint32_t r = threadIdx.x; r <= top; r += blockDim.x) {
-            uint32_t v = x[r];
-            if (r >= a)
-                v += x[r - a];
-            if (r >= b)
-                v += x[r - b];
-            if (r >= ab)
-                v += x[r - ab];
-            y[r] = min(v, kFsCountMax);
+        if (lo > top) {
+            if (threadIdx.x == 0)
+                cum[a]++;
+            stale = true;
+            continue;
+        }
+        if (stale)
+            __syncthreads();
+        stale = false;
+        uint32_t v[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; i++) {
+            const uint32_t r = lo + threadIdx.x + (uint32_t)i * 32u * kWarps;
+            if (lo + (uint32_t)i * 32u * kWarps > top)
+                break;
+            v[i] = r <= top ? min(cum[r] + cum[r - a], kFsCountMax) : 0u;
         }
         __syncthreads();
-        uint32_t *t = x;
-        x = y;
-        y = t;
+#pragma unroll
+        for (int i = 0; i < kPer; i++) {
+            const uint32_t r = lo + threadIdx.x + (uint32_t)i * 32u * kWarps;
+            if (lo + (uint32_t)i * 32u * kWarps > top)
+                break;
+            if (r <= top)
+                cum[r] = v[i];
+        }
+        if (threadIdx.x == 0 && a < lo)
+            cum[a]++;
+        __syncthreads();
     }
+    __syncthreads();
     if (threadIdx.x < 32u) {
         uint32_t run = 0;
         for (uint32_t base = 0; base <= top; base += 32u) {
             const uint32_t r = base + threadIdx.x;
-            uint32_t v = r <= top ? x[r] : 0u;
+            uint32_t v = r <= top ? cum[r] : 0u;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const uint32_t o = __shfl_up_sync(FULL_MASK, v, d);
@@ -1395,9 +1423,12 @@ __device__ __forceinline__ uint32_t weight_holding(const uint32_t *cum, uint32_t
 
 /* The patterns of weight R before the T positions v (less one, ascending):
  * fewer positions, or as many and lexicographically smaller; T (R + 1) <=
- * kFsTied.  x, y: that many words each.  Every thread returns the count. */
-__device__ __forceinline__ uint32_t count_tied(const uint32_t *rho, int n, uint32_t R, int T,
-                                               const uint8_t *v, uint32_t *x, uint32_t *y,
+ * kFsTied.  x[t (R + 1) + r] counts the sets of t positions of weight r, from
+ * the last position to the first as count_weights does; t positions weigh t
+ * mall[p] or more, so the rows of more positions join late.  Every thread
+ * returns the count. */
+__device__ __forceinline__ uint32_t count_tied(const uint32_t *rho, const uint32_t *mall, int n,
+                                               uint32_t R, int T, const uint8_t *v, uint32_t *x,
                                                uint32_t *s_acc)
 {
     const uint32_t row = R + 1u;
@@ -1426,18 +1457,21 @@ __device__ __forceinline__ uint32_t count_tied(const uint32_t *rho, int n, uint3
         }
         if (a > R)
             continue;
-        for (int t = 0; t < T; t++)
-            for (uint32_t r = threadIdx.x; r <= R; r += blockDim.x) {
-                uint32_t c = x[(uint32_t)t * row + r];
-                if (t > 0 && r >= a)
-                    c += x[(uint32_t)(t - 1) * row + (r - a)];
-                y[(uint32_t)t * row + r] = c;
-            }
-        __syncthreads();
-        uint32_t *s = x;
-        x = y;
-        y = s;
+        __syncthreads(); /* thread 0 has read its entry */
+        const uint32_t least = mall[p + 1];
+        /* rows of most positions first: each reads the one before it */
+        for (int t = T - 1; t >= 2; t--) {
+            const uint32_t lo = a + (uint32_t)(t - 1) * least; /* < 2^32: least <= 2^30 */
+            if (least > R || lo > R)
+                continue;
+            for (uint32_t r = lo + threadIdx.x; r <= R; r += blockDim.x)
+                x[(uint32_t)t * row + r] += x[(uint32_t)(t - 1) * row + (r - a)];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0 && T > 1)
+            x[row + a]++; /* read by others after the barrier above, next time round */
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
         for (int t = 0; t < T; t++)
             acc += x[(uint32_t)t * row + R];
@@ -1559,28 +1593,13 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                 fp.m3[8 * lane + 1 + i] = v[i];
         }
         __syncthreads();
-        /* the weight of the cap-th pattern */
-        uint32_t top = 511u, Rcap;
-        for (;;) {
-            count_weights(sm.rho, n, top, fp.set, fp.set + (kFsTop + 1), fp.cum);
-            Rcap = weight_holding(fp.cum, top, cap);
-            if (Rcap <= top || top >= (uint32_t)kFsTop)
-                break;
-            top = min(2u * top + 1u, (uint32_t)kFsTop);
-        }
-        if (Rcap > top) {
-            /* fewer than cap patterns in all, or weights past the count */
-            if (threadIdx.x == 0)
-                sc.rest[atomicAdd(&sc.cnt[6], 1ull)] = open;
-            continue;
-        }
         /* single positions: thread j - 1 tests position j */
         int32_t bR = kNoHit;
         int bT = 0;
         bool guard = false;
         {
             const int j = (int)threadIdx.x + 1;
-            if (j <= n && sm.rho[j] <= Rcap &&
+            if (j <= n && sm.rho[j] <= (uint32_t)kFsTop &&
                 (W == 1 ? sm.c0[j] == syn_key(s0) : sz(sx(sm.h[j], s0)))) {
                 bR = (int32_t)sm.rho[j];
                 bT = 1;
@@ -1589,9 +1608,23 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
             }
         }
         __syncthreads();
-        uint32_t Rb = 0;
+        uint32_t Rb = 0, top = 0;
+        bool counted = true;
         for (uint32_t goal = min(cap, kFsBand);; goal = goal > cap / 16u ? cap : goal * 16u) {
-            Rb = weight_holding(fp.cum, top, goal); /* <= Rcap */
+            /* the weight that holds the goal-th pattern */
+            for (;;) {
+                if (top != 0u) {
+                    Rb = weight_holding(fp.cum, top, goal);
+                    if (Rb <= top || top >= (uint32_t)kFsTop)
+                        break;
+                }
+                top = top == 0u ? 319u : min(2u * top + 1u, (uint32_t)kFsTop);
+                count_weights(sm.rho, fp.mall, n, top, fp.cum);
+            }
+            if (Rb > top) {
+                counted = false; /* fewer patterns in all, or weights past the count */
+                break;
+            }
             /* chunks of pairs by weight: (slo, shi] */
             int32_t slo = -1;
             while (slo < (int32_t)Rb) {
@@ -1601,8 +1634,9 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                         fp.set[r] = 0u;
                     __syncthreads();
                     for (int a = 1 + warp; a < n; a += kWarps)
-                        for (int c = a + 1 + lane; c <= n; c += 32) {
-                            const uint32_t s = sm.rho[a] + sm.rho[c];
+                        for (int c0 = a + 1; c0 <= n && sm.rho[a] + fp.mall[c0] <= Rb; c0 += 32) {
+                            const int c = c0 + lane;
+                            const uint32_t s = c <= n ? sm.rho[a] + sm.rho[c] : kRhoInf;
                             if ((int32_t)s > slo && s <= Rb)
                                 atomicAdd(fp.set + s, 1u);
                         }
@@ -1648,8 +1682,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                 }
                 __syncthreads();
                 for (int a = 1 + warp; a < n; a += kWarps)
-                    for (int c = a + 1 + lane; c <= n; c += 32) {
-                        const int32_t s = (int32_t)(sm.rho[a] + sm.rho[c]);
+                    for (int c0 = a + 1; c0 <= n && sm.rho[a] + fp.mall[c0] <= (uint32_t)shi;
+                         c0 += 32) {
+                        const int c = c0 + lane;
+                        const int32_t s = (int32_t)(c <= n ? sm.rho[a] + sm.rho[c] : kRhoInf);
                         if (s > slo && s <= shi)
                             fs_insert<W>(sm, fp.set, a, c);
                     }
@@ -1676,11 +1712,11 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                     if (lane == 0)
                         k = atomicAdd(&s_next, 1u);
                     k = __shfl_sync(FULL_MASK, k, 0);
-                    if (k >= (unsigned)kClasses)
+                    if (k >= (unsigned)kFsClasses)
                         break;
                     const int32_t Rk = min((int32_t)Rb, *((volatile int32_t *)&s_R));
                     const int32_t was = __reduce_min_sync(FULL_MASK, bR);
-                    tree_pass<W, kFsPairs, kClasses>(walk, n, s0, Rk, 0, 0, lane, steps, &bR, &bT,
+                    tree_pass<W, kFsPairs, kFsClasses>(walk, n, s0, Rk, 0, 0, lane, steps, &bR, &bT,
                                                      &guard, (int)k, &pairs);
                     const int32_t now = __reduce_min_sync(FULL_MASK, bR);
                     if (lane == 0 && now < was)
@@ -1691,8 +1727,14 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                 if (s_R <= (int32_t)Rb && slo + 1 > s_R)
                     break; /* later pairs are heavier than the hit (uniform) */
             }
-            if (s_R <= (int32_t)Rb || Rb >= Rcap)
+            if (s_R <= (int32_t)Rb || goal >= cap)
                 break;
+        }
+        if (!counted) {
+            __syncthreads(); /* everyone has left the search before s_R changes */
+            if (threadIdx.x == 0)
+                sc.rest[atomicAdd(&sc.cnt[6], 1ull)] = open;
+            continue;
         }
         const int32_t R = s_R;
         const bool hit = R <= (int32_t)Rb;
@@ -1740,8 +1782,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
         uint32_t rank = 0xFFFFFFFFu;
         if (hit) {
             rank = 1u + (R > 0 ? fp.cum[R - 1] : 0u) +
-                   count_tied(sm.rho, n, (uint32_t)R, Tb, team.pos[win], fp.set, fp.set + kFsTied,
-                              &s_acc);
+                   count_tied(sm.rho, fp.mall, n, (uint32_t)R, Tb, team.pos[win], fp.set, &s_acc);
             if (warp == 0 && lane < Tb)
                 sm.best[lane] = team.pos[win][lane];
         }
