@@ -209,13 +209,21 @@ template <int K> constexpr uint32_t warp_smem_bytes(uint32_t bstride)
 }
 
 /* How a phase-1 launch of B blocks is cut: warps per CTA, queue slots per
- * grab, whether warps take blocks ahead, and the grid.  A batch of few blocks
+ * grab, whether warps take blocks ahead, the grid, and how far a warp takes
+ * its block.  A batch of few blocks
  * is spread over the SMs and shared out block by block: with the tuned grab
  * of four, 257 blocks of BCH(127,113) ran four after another on 65 warps of
  * nine SMs.  Measured with it and without: three serving codes, 8,191 blocks,
- * 170 -> 121 us. */
+ * 170 -> 121 us.  While phase 2's CTAs are not all busy, a block goes there
+ * early: up to two blocks a resident warp after the flat table, up to eight
+ * after the first band.  us, flat / first band / both bands: BCH(127,113),
+ * 257 blocks 34 / 38 / 49, 100,000 186 / 133 / 148, 400,000 632 / 391 / 350;
+ * three serving codes, 8,191 blocks 103 / 105 / 122; four mixed codes, 33,000
+ * blocks 197 / 175 / 205, 100,000 460 / 380 / 361 (3,648 warps; 4,864 for the
+ * one code). */
 struct Cut {
     int wpc, grab, ahead, grid;
+    uint32_t budget;
 };
 template <typename Kern>
 int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
@@ -241,6 +249,11 @@ int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
     c->wpc = wpc;
     c->grab = (int)g;
     c->ahead = a.B > 4 * warps;
+    c->budget = a.budget;
+    if (a.B <= 2 * warps)
+        c->budget = a.budget < 1u ? a.budget : 1u;
+    else if (a.B <= 8 * warps)
+        c->budget = a.budget < ORBG_FLAT_MAX + 1u ? a.budget : ORBG_FLAT_MAX + 1u;
     const int64_t need = ((a.B + g - 1) / g + wpc - 1) / wpc;
     if (c->grid > need)
         c->grid = (int)(need > 0 ? need : 1);
@@ -275,7 +288,7 @@ int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned lon
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     return (int)cudaLaunchKernelEx(
-        &cfg, k1, a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, a.budget, a.cw,
+        &cfg, k1, a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, c.budget, a.cw,
         a.cw_off, a.q, a.ab, ss.counters, queue, ss.heavy,
         sorted ? (const uint32_t *)ss.perm : (const uint32_t *)nullptr, ss.hand, ss.hand_cap,
         (unsigned long long)a.scratch_base, bstride, c.grab, c.ahead,
@@ -340,7 +353,7 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
         if ((rc = cut_launch(k1, a, warp_smem_bytes<KMAX>(bstride), &c)) != 0)
             return (cudaError_t)rc;
         k1<<<c.grid, c.wpc * 32, (size_t)warp_smem_bytes<KMAX>(bstride) * c.wpc, st>>>(
-            a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, a.budget, a.cw, a.cw_off,
+            a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, c.budget, a.cw, a.cw_off,
             a.q, a.ab, counters, queue, heavy, nullptr, sc.hand, sc.hand_cap,
             (unsigned long long)a.scratch_base, bstride, c.grab, c.ahead, nullptr, 0, 0,
             *a.code0);
