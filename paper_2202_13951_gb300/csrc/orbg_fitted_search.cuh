@@ -396,11 +396,10 @@ __device__ __forceinline__ bool node_pair_lex_less(const uint8_t *stk, int lane,
 }
 
 /* What a pass over prefixes needs besides the node arrays: the block's pairs
- * of weights slo < s <= shi in a hash set (2^kFsSetBits 32-bit slots, linear
+ * of weights slo < s <= shi in a hash set (2^SB 32-bit slots, linear
  * probing; an entry is a 16-bit tag, the hash bits below the slot's, over
  * a - 1 and b - 1), and the least weight tb[j] that a pair of the set after
  * position j can have. */
-constexpr int kFsSetBits = 14;
 constexpr uint32_t kFsEmpty = 0xFFFFFFFFu;
 struct FsPairs {
     const uint32_t *tb;
@@ -411,32 +410,32 @@ struct FsPairs {
  * golden ratio */
 __device__ __forceinline__ uint32_t fs_hash(uint32_t v) { return v * 0x9E3779B1u; }
 
-__device__ __forceinline__ uint32_t fs_tag(uint32_t hash)
+template <int SB> __device__ __forceinline__ uint32_t fs_tag(uint32_t hash)
 {
-    return (hash << kFsSetBits) & 0xFFFF0000u;
+    return (hash << SB) & 0xFFFF0000u;
 }
 
 /* Entry with the tag of key v, or kFsEmpty (a filter: fs_match checks). */
-__device__ __forceinline__ uint32_t fs_find(const uint32_t *set, uint32_t v)
+template <int SB> __device__ __forceinline__ uint32_t fs_find(const uint32_t *set, uint32_t v)
 {
-    const uint32_t x = fs_hash(v), tag = fs_tag(x);
-    uint32_t slot = x >> (32 - kFsSetBits);
+    const uint32_t x = fs_hash(v), tag = fs_tag<SB>(x);
+    uint32_t slot = x >> (32 - SB);
     uint32_t e = set[slot];
     while (e != kFsEmpty && ((e ^ tag) & 0xFFFF0000u) != 0u) {
-        slot = (slot + 1u) & ((1u << kFsSetBits) - 1u);
+        slot = (slot + 1u) & ((1u << SB) - 1u);
         e = set[slot];
     }
     return e;
 }
 
 /* The set's pair whose whole syndrome is `full` (key v): a | b << 16, 1-based, or 0. */
-template <int W>
+template <int W, int SB>
 __device__ __noinline__ uint32_t fs_match(const uint32_t *set, const uint32_t *c0,
                                           const typename Syn<W>::T *h, uint32_t v,
                                           typename Syn<W>::T full)
 {
-    const uint32_t x = fs_hash(v), tag = fs_tag(x);
-    uint32_t slot = x >> (32 - kFsSetBits);
+    const uint32_t x = fs_hash(v), tag = fs_tag<SB>(x);
+    uint32_t slot = x >> (32 - SB);
     for (;;) {
         const uint32_t e = set[slot];
         if (e == kFsEmpty)
@@ -446,7 +445,7 @@ __device__ __noinline__ uint32_t fs_match(const uint32_t *set, const uint32_t *c
             if (W == 1 ? (c0[a] ^ c0[b]) == v : sz(sx(sx(h[a], h[b]), full)))
                 return a | b << 16;
         }
-        slot = (slot + 1u) & ((1u << kFsSetBits) - 1u);
+        slot = (slot + 1u) & ((1u << SB) - 1u);
     }
 }
 
@@ -481,7 +480,7 @@ __device__ __noinline__ typename Syn<W>::T node_syndrome(const FsSmem<W> &sm, in
  * the big subtrees of the least reliable positions are shared out evenly.
  */
 enum { kFsSearch = 0, kFsRank = 1, kFsPairs = 2 };
-template <int W, int MODE, int P>
+template <int W, int MODE, int P, int SB = 14>
 __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0, int32_t Rhi,
                               int32_t Rb, int Tb, int lane, uint32_t steps, int32_t *bR,
                               int *bT, bool *guard, int w, const FsPairs *pr = nullptr)
@@ -521,10 +520,10 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
             active && R + (PAIRS ? pr->tb[jt] : 0u) <= (uint32_t)Rhi &&
             (P == 1 || t != 1 || (jt - 1) % P == w);
         if (PAIRS) {
-            const bool cand = tested && fs_find(pr->set, syn) != kFsEmpty;
+            const bool cand = tested && fs_find<SB>(pr->set, syn) != kFsEmpty;
             if (__any_sync(FULL_MASK, cand)) {
                 if (cand) {
-                    const uint32_t ab = fs_match<W>(
+                    const uint32_t ab = fs_match<W, SB>(
                         pr->set, sm.c0, sm.h, syn,
                         W == 1 ? szero<typename Syn<W>::T>()
                                : node_syndrome<W>(sm, lane, t, jt, s0));
@@ -669,7 +668,7 @@ __device__ uint32_t tree_pass(const FsSmem<W> &sm, int n, typename Syn<W>::T s0,
                     const bool inner = jm < n && Rs + sm.msuf[jm + 1] <= (uint32_t)Rhi;
                     const bool own =
                         PAIRS ? Rs + pr->tb[jm] <= (uint32_t)Rhi &&
-                                    fs_find(pr->set, sp ^ sm.c0[jm]) != kFsEmpty
+                                    fs_find<SB>(pr->set, sp ^ sm.c0[jm]) != kFsEmpty
                               : Rs <= (uint32_t)Rhi &&
                                     (RANK ? Rs == (uint32_t)Rb : (sp ^ sm.c0[jm]) == 0u);
                     if (inner || own) {
@@ -1258,7 +1257,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
  * million patterns of a three-line model) looks up each one's syndrome,
  * which tests every pattern it starts.  Of several pairs of one syndrome the
  * set keeps the first in the order (weight, a, b): exchanging a later one in
- * a hit for it gives an earlier hit.  Orders of more than kFsChunk pairs up
+ * a hit for it gives an earlier hit.  Orders of more than kFsChunk<K> pairs up
  * to a band's bound take the pairs in chunks of rising weight, each with its
  * own walk.
  *
@@ -1287,14 +1286,21 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
 constexpr int kFsClasses = ORBG_FS_CLASSES;
 constexpr int kFsTop = 4095;          /* largest weight counted */
 constexpr uint32_t kFsCountMax = 1u << 26; /* counts are exact below, and no cap is above */
-constexpr uint32_t kFsChunk = 7168;   /* pairs in the set at once: load 0.44 */
 constexpr uint32_t kFsBand = 32768;   /* patterns of the first band */
-constexpr uint32_t kFsTied = 1u << kFsSetBits; /* entries of the tied-patterns count */
+/* The set's slots for codes of K keys per lane, and how many pairs it takes
+ * at once (load 0.44); the same words hold the tied-patterns count.  Half the
+ * slots from n > 64 on let three CTAs share an SM instead of two (20,000
+ * CA-Polar[256,234] blocks 1,430 -> 1,357 us); a short code's weights reach
+ * further, and with half the count's entries a quarter of its blocks would
+ * go to the tree search (80,000 RLC(64,51) blocks of four lines 709 -> 921). */
+template <int K> constexpr int kFsSetBits = K >= 4 ? 13 : 14;
+template <int K> constexpr uint32_t kFsChunk = 7u << (kFsSetBits<K> - 4);
+template <int K> constexpr uint32_t kFsTied = 1u << kFsSetBits<K>;
 
 /* Dynamic shared memory of the CTA. */
-template <int W> struct FpSmem {
+template <int K, int W> struct FpSmem {
     uint32_t *cum;   /* [kFsTop + 1] patterns of weight <= r */
-    uint32_t *set;   /* [2^kFsSetBits]; also the counts' work space */
+    uint32_t *set;   /* [2^kFsSetBits<K>]; also the tied count */
     uint32_t *mpair; /* [258] least pair weight after position j */
     uint32_t *m3;    /* [258] least rho_v + mpair[v] over v >= j */
     uint32_t *mall;  /* [258] least rho over positions >= j */
@@ -1309,7 +1315,7 @@ template <int W> struct FpSmem {
             p += (bytes + 15) & ~(size_t)15;
             return r;
         };
-        set = (uint32_t *)take(4u << kFsSetBits);
+        set = (uint32_t *)take(4u << kFsSetBits<K>);
         cum = (uint32_t *)take(4 * (kFsTop + 1));
         sm.h = (typename Syn<W>::T *)take(W > 1 ? 258 * sizeof(typename Syn<W>::T) : 0);
         mpair = (uint32_t *)take(258 * 4);
@@ -1330,9 +1336,9 @@ template <int W> struct FpSmem {
         sm.anch = nullptr;
     }
 };
-template <int W> __host__ __device__ constexpr uint32_t fp_smem_bytes()
+template <int K, int W> __host__ __device__ constexpr uint32_t fp_smem_bytes()
 {
-    return (4u << kFsSetBits) + 4u * (kFsTop + 1) +
+    return (4u << kFsSetBits<K>) + 4u * (kFsTop + 1) +
            (W > 1 ? (258u * 4u * W + 15u) / 16u * 16u : 0u) + 7u * ((258u * 4u + 15u) / 16u * 16u) +
            96u + 256u + 256u + 32u + 2u * 32u * 32u * kWarps;
 }
@@ -1483,16 +1489,16 @@ __device__ __forceinline__ uint32_t count_tied(const uint32_t *rho, const uint32
 
 /* The pair (a, b) of key v into the set; the first of a syndrome in the
  * order (weight, a, b) stays. */
-template <int W>
+template <int W, int SB>
 __device__ __forceinline__ void fs_insert(const FsSmem<W> &sm, uint32_t *set, int a, int b)
 {
     const uint32_t v = sm.c0[a] ^ sm.c0[b];
     typename Syn<W>::T full = szero<typename Syn<W>::T>();
     if (W > 1)
         full = sx(sm.h[a], sm.h[b]);
-    const uint32_t x = fs_hash(v), e = fs_tag(x) | (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1);
+    const uint32_t x = fs_hash(v), e = fs_tag<SB>(x) | (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1);
     const uint32_t mine = (sm.rho[a] + sm.rho[b]) << 16 | (e & 0xFFFFu);
-    uint32_t slot = x >> (32 - kFsSetBits);
+    uint32_t slot = x >> (32 - SB);
     for (;;) {
         uint32_t old = atomicCAS(set + slot, kFsEmpty, e);
         if (old == kFsEmpty)
@@ -1508,12 +1514,12 @@ __device__ __forceinline__ void fs_insert(const FsSmem<W> &sm, uint32_t *set, in
                 return;
             old = was;
         }
-        slot = (slot + 1u) & ((1u << kFsSetBits) - 1u);
+        slot = (slot + 1u) & ((1u << SB) - 1u);
     }
 }
 
 template <int K, int W>
-__global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
+__global__ void __launch_bounds__(kWarps * 32, K >= 4 ? 3 : 2) orbg_fitpair_kernel(
     const __grid_constant__ OrbgDeviceCode code, const float *__restrict__ llr, int64_t B,
     uint32_t cap, uint8_t *__restrict__ cw, uint32_t *__restrict__ q,
     uint8_t *__restrict__ ab, unsigned char *__restrict__ scratch)
@@ -1526,7 +1532,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
     __shared__ uint32_t s_next, s_acc;
     __shared__ int s_win, s_T;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    FpSmem<W> fp(smem, warp);
+    FpSmem<K, W> fp(smem, warp);
     const FsSmem<W> &sm = fp.sm;
     FsSmem<W> walk = fp.sm;
     walk.msuf = fp.lb;
@@ -1629,7 +1635,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
             int32_t slo = -1;
             while (slo < (int32_t)Rb) {
                 int32_t shi = (int32_t)Rb;
-                if (n * (n - 1) / 2 > (int)kFsChunk) {
+                if (n * (n - 1) / 2 > (int)kFsChunk<K>) {
                     for (uint32_t r = threadIdx.x; r <= Rb; r += blockDim.x)
                         fp.set[r] = 0u;
                     __syncthreads();
@@ -1642,7 +1648,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                         }
                     __syncthreads();
                     if (warp == 0) {
-                        /* the largest shi with at most kFsChunk pairs (a weight
+                        /* the largest shi with at most kFsChunk<K> pairs (a weight
                          * has far fewer) */
                         uint32_t run = 0;
                         int32_t lim = (int32_t)Rb;
@@ -1656,7 +1662,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                                     v += o;
                             }
                             const uint32_t over =
-                                __ballot_sync(FULL_MASK, run + v > kFsChunk && r <= Rb);
+                                __ballot_sync(FULL_MASK, run + v > kFsChunk<K> && r <= Rb);
                             if (over) {
                                 lim = (int32_t)base + __ffs(over) - 2;
                                 break;
@@ -1670,7 +1676,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                     shi = s_win;
                 }
                 uint4 *clear = reinterpret_cast<uint4 *>(fp.set);
-                for (uint32_t r = threadIdx.x; r < (1u << kFsSetBits) / 4u; r += blockDim.x)
+                for (uint32_t r = threadIdx.x; r < (1u << kFsSetBits<K>) / 4u; r += blockDim.x)
                     clear[r] = make_uint4(kFsEmpty, kFsEmpty, kFsEmpty, kFsEmpty);
                 for (int j = (int)threadIdx.x; j <= n + 1; j += (int)blockDim.x) {
                     const uint32_t least = (uint32_t)(slo + 1);
@@ -1687,12 +1693,12 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                         const int c = c0 + lane;
                         const int32_t s = (int32_t)(c <= n ? sm.rho[a] + sm.rho[c] : kRhoInf);
                         if (s > slo && s <= shi)
-                            fs_insert<W>(sm, fp.set, a, c);
+                            fs_insert<W, kFsSetBits<K>>(sm, fp.set, a, c);
                     }
                 __syncthreads();
                 if (threadIdx.x == 0) {
                     /* the empty prefix: a pair alone */
-                    const uint32_t m = fs_match<W>(fp.set, sm.c0, sm.h, syn_key(s0), s0);
+                    const uint32_t m = fs_match<W, kFsSetBits<K>>(fp.set, sm.c0, sm.h, syn_key(s0), s0);
                     if (m) {
                         const int pa = (int)(m & 0xFFFFu), pb = (int)(m >> 16);
                         const int32_t R = (int32_t)(sm.rho[pa] + sm.rho[pb]);
@@ -1716,7 +1722,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
                         break;
                     const int32_t Rk = min((int32_t)Rb, *((volatile int32_t *)&s_R));
                     const int32_t was = __reduce_min_sync(FULL_MASK, bR);
-                    tree_pass<W, kFsPairs, kFsClasses>(walk, n, s0, Rk, 0, 0, lane, steps, &bR, &bT,
+                    tree_pass<W, kFsPairs, kFsClasses, kFsSetBits<K>>(walk, n, s0, Rk, 0, 0, lane, steps, &bR, &bT,
                                                      &guard, (int)k, &pairs);
                     const int32_t now = __reduce_min_sync(FULL_MASK, bR);
                     if (lane == 0 && now < was)
@@ -1774,7 +1780,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) orbg_fitpair_kernel(
         }
         __syncthreads();
         const int win = s_win, Tb = s_T;
-        if (win == -2 || (hit && (uint32_t)Tb * ((uint32_t)R + 1u) > kFsTied)) {
+        if (win == -2 || (hit && (uint32_t)Tb * ((uint32_t)R + 1u) > kFsTied<K>)) {
             if (threadIdx.x == 0)
                 sc.rest[atomicAdd(&sc.cnt[6], 1ull)] = open;
             continue;
@@ -1808,7 +1814,7 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
     if (rc == 0)
         rc = orbg_grid_for((const void *)k2, kWarps * 32, smem, 0, &g2);
     if (rc == 0)
-        rc = orbg_grid_for((const void *)k3, kWarps * 32, fp_smem_bytes<W>(), 0, &g3);
+        rc = orbg_grid_for((const void *)k3, kWarps * 32, fp_smem_bytes<K, W>(), 0, &g3);
     if (rc == 0)
         rc = orbg_grid_for((const void *)k4, kWarps * 32, smem, 0, &g4);
     if (rc != 0)
@@ -1833,7 +1839,7 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
     k2<<<g2, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return (int)e;
-    k3<<<g3, kWarps * 32, fp_smem_bytes<W>(), st>>>(code, llr, B, cap, cw, q, ab, scratch);
+    k3<<<g3, kWarps * 32, fp_smem_bytes<K, W>(), st>>>(code, llr, B, cap, cw, q, ab, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return (int)e;
     k4<<<g4, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
