@@ -76,10 +76,13 @@ constexpr uint32_t kRhoInf = 1u << 30;      /* weight of a position never reache
 constexpr int32_t kRmax = (1 << 26) - 1;    /* heaviest reliability weight searched */
 constexpr int kLeafRun = 3;                /* leaf siblings tested per step besides the node */
 /* Nodes a one-warp pass may test before a CTA takes over (a quarter of the
- * cap if less).  Measured, us a call, three lines, 100,000 BCH(127,113) and
- * 20,000 CA-Polar[256,234] blocks: 256 1,658 and 1,991; 512 1,533 and 1,861;
- * 1024 1,469 and 1,699; 2048 1,505 and 1,732; 4096 1,746 and 1,946. */
-constexpr uint32_t kSplit = 1024;
+ * cap if less): kSplit, or kSplitSmall where a batch has at most two blocks a
+ * resident warp and the CTAs wait for work.  Measured, us a call, three lines,
+ * 100,000 BCH(127,113) and 20,000 CA-Polar[256,234] blocks, and 3,000 BCH
+ * blocks of two lines: 256 1,415, 1,473 and 223; 512 1,361, 1,353 and 242;
+ * 1024 1,340, 1,386 and 330. */
+constexpr uint32_t kSplit = 512;
+constexpr uint32_t kSplitSmall = 256;
 constexpr int32_t kNoHit = 0x7FFFFFFF;
 constexpr int kBlockRange = ORBG_BLOCK_RANGE; /* abandoned[] value: beyond the search range */
 
@@ -1167,12 +1170,12 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitprep_kernel(
 }
 
 /* Stage 2, persistent over the open list that stage 1 filled, one warp per
- * block; a block whose search grows past min(kSplit, cap / 4) nodes without
+ * block; a block whose search grows past `split` nodes without
  * a member is left to stage 3. */
 template <int K, int W>
 __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_kernel(
     const __grid_constant__ OrbgDeviceCode code, const float *__restrict__ llr, int64_t B,
-    uint32_t cap, uint8_t *__restrict__ cw, uint32_t *__restrict__ q,
+    uint32_t cap, uint32_t split, uint8_t *__restrict__ cw, uint32_t *__restrict__ q,
     uint8_t *__restrict__ ab, unsigned char *__restrict__ scratch)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1181,7 +1184,6 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_kernel(
     const FsScratch sc(scratch, B);
     const unsigned long long nopen = sc.cnt[1];
     const int n = code.n;
-    const uint32_t split = min(kSplit, cap / 4u);
     for (;;) {
         unsigned long long i = 0;
         if (lane == 0)
@@ -1819,6 +1821,8 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
         rc = orbg_grid_for((const void *)k4, kWarps * 32, smem, 0, &g4);
     if (rc != 0)
         return rc;
+    const uint32_t most = B <= 2 * (int64_t)g2 * kWarps ? kSplitSmall : kSplit;
+    const uint32_t split = most < cap / 4u ? most : cap / 4u;
     const int64_t need = (B + kWarps - 1) / kWarps;
     if (g1 > need)
         g1 = (int)need;
@@ -1836,7 +1840,7 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
                                       scratch);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return (int)e;
-    k2<<<g2, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
+    k2<<<g2, kWarps * 32, smem, st>>>(code, llr, B, cap, split, cw, q, ab, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return (int)e;
     k3<<<g3, kWarps * 32, fp_smem_bytes<K, W>(), st>>>(code, llr, B, cap, cw, q, ab, scratch);
