@@ -555,6 +555,7 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
         d.band_ranks[i] = tb.band_ranks[i];
         d.band_end[i] = tb.band_end[i];
     }
+    d.ranks = tb.ranks;
     d.lead_pairs = tb.lead_pairs;
     d.lead_end = tb.lead_end;
     d.nflat = tb.nflat;

@@ -402,6 +402,12 @@ __device__ __forceinline__ void sort_lane(uint32_t (&key)[K])
         }
 }
 
+/* Ranks taken one at a time at most; beyond, a full sort is cheaper.  A
+ * handover to phase 2 at cap 1e6 needs 82: sorted in full, 256 keys cost
+ * phase 1 a bitonic network and, in one block of three, a second one on exact
+ * keys for a tie somewhere among them. */
+constexpr int kMostRanks = 128;
+
 /* The lane's keys, ascending: its smallest, and how the next ones follow.
  * Up to four keys shift down in registers; eight (n > 128) go to a list in
  * shared memory, where taking one costs a load instead of eight moves and
@@ -450,50 +456,40 @@ template <> struct LaneKeys<8> {
     }
 };
 
-/* Extracts ranks have .. upto-1 (upto <= 64): lane r keeps rank r's key in
- * mine[0], rank r + 32's in mine[1].  Returns true if two consecutive ranks
- * (this call's or the last earlier one, in *prev) have equal truncated
- * reliabilities: then the truncated order may differ from the exact one and
- * the caller sorts exactly instead. */
+/* Extracts ranks have .. upto-1: pi[r] is rank r's received index.  Returns
+ * true if two consecutive ranks (this call's or the last earlier one, in
+ * *prev) have equal truncated reliabilities: then the truncated order may
+ * differ from the exact one and the caller sorts exactly instead. */
 template <int K>
 __device__ __forceinline__ bool extract_ranks(LaneKeys<K> &keys, int have, int upto,
-                                              uint32_t *prev, uint32_t (&mine)[2], int lane)
+                                              uint32_t *prev, uint8_t *pi)
 {
     typedef KeyBits<K> KB;
     bool tie = false;
     uint32_t pv = *prev;
-#pragma unroll
-    for (int half = 0; half < 2; half++) {
-        const int end = min(upto, 32 * half + 32);
-        for (int r = max(have, 32 * half); r < end; r++) {
-            const uint32_t g = __reduce_min_sync(FULL_MASK, keys.first());
-            tie |= (g >> KB::IB) == (pv >> KB::IB);
-            keys.take(keys.first() == g);
-            if (lane == r - 32 * half)
-                mine[half] = g;
-            pv = g;
-        }
+    for (int r = have; r < upto; r++) {
+        const uint32_t g = __reduce_min_sync(FULL_MASK, keys.first());
+        tie |= (g >> KB::IB) == (pv >> KB::IB);
+        const bool mine = keys.first() == g;
+        if (mine)
+            pi[r] = (uint8_t)(g & KB::IMASK);
+        keys.take(mine);
+        pv = g;
     }
     *prev = pv;
     return tie;
 }
 
-/* Permuted columns of ranks lo .. hi-1 from the lanes holding them. */
-template <int K, int W>
-__device__ __forceinline__ void perm_ranks(const OrbgDeviceCode &code, const uint32_t (&mine)[2],
-                                           int lo, int hi, const BlockSmem<W> &sm, int lane)
+/* Permuted columns of ranks lo .. hi-1, whose received indices are in pi. */
+template <int W>
+__device__ __forceinline__ void perm_ranks(const OrbgDeviceCode &code, int lo, int hi,
+                                           const BlockSmem<W> &sm, int lane)
 {
-#pragma unroll
-    for (int half = 0; half < 2; half++) {
-        const int r = lane + 32 * half;
-        if (r >= lo && r < hi) {
-            const int idx = (int)(mine[half] & KeyBits<K>::IMASK);
-            sm.pi[r] = (uint8_t)idx;
-            const typename Syn<W>::T col = load_col<W>(code.hcol, idx);
-            sm.h[r] = col;
-            if (W > 1)
-                sm.h0[r] = syn_key(col);
-        }
+    for (int r = lo + lane; r < hi; r += 32) {
+        const typename Syn<W>::T col = load_col<W>(code.hcol, (int)sm.pi[r]);
+        sm.h[r] = col;
+        if (W > 1)
+            sm.h0[r] = syn_key(col);
     }
 }
 
@@ -978,7 +974,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
             if (W > 1)
                 sm.h0[-1] = 0u;
         }
-        uint32_t prev = 0xFFFFFFFFu, mine_key[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+        uint32_t prev = 0xFFFFFFFFu;
         uint32_t base = 0, tested = 1u, np = 0;
         int k = -1; /* the band; -1: the flat table */
 #pragma unroll 1
@@ -1015,20 +1011,21 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     if (heavy == nullptr)
                         break;
                     k = ORBG_BANDS;
-                    upto = n; /* the handover record holds them all */
+                    upto = (int)code.ranks + 1; /* the handover record */
                 }
             }
             upto = min(upto, n);
             if (upto > have) {
-                /* a tie among the ranks, or more than 64, sorts everything
-                 * exactly */
-                if (upto > 64 || extract_ranks<K>(keys, have, upto, &prev, mine_key, lane)) {
+                /* a tie among the ranks, or more than kMostRanks, sorts
+                 * everything exactly */
+                if (upto > kMostRanks || extract_ranks<K>(keys, have, upto, &prev, sm.pi)) {
                     make_keys<K, LS>(llr, n, lane, key);
                     sort_block<K, LS>(key, llr, n, lane);
                     build_perm<K, W>(code, key, sm, lane);
                     have = n;
                 } else {
-                    perm_ranks<K, W>(code, mine_key, have, upto, sm, lane);
+                    __syncwarp();
+                    perm_ranks<W>(code, have, upto, sm, lane);
                     have = upto;
                 }
                 __syncwarp();
@@ -1068,7 +1065,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
             const bool keep = slot < (unsigned long long)hand_cap;
             if (keep) {
                 unsigned char *rec = hand + slot * ORBG_HANDOVER_BYTES;
-                for (int e = lane; e < n; e += 32)
+                for (int e = lane; e < (int)code.ranks; e += 32)
                     rec[e] = sm.pi[e];
                 if (lane == 0)
                     *reinterpret_cast<T *>(rec + 256) = s0;
@@ -1159,9 +1156,10 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
     uint32_t *filter = reinterpret_cast<uint32_t *>(pair_sm + kMaskBytes);
     uint32_t *set = filter + (1u << fbits) / 32u;
     if (rec != nullptr) {
-        /* phase 1's handover record: the block's order and starting
-         * syndrome; every thread takes a share of the positions */
-        for (int i = (int)threadIdx.x; i < n; i += (int)blockDim.x) {
+        /* phase 1's handover record: the leading part of the block's order
+         * that its patterns use, and the starting syndrome; every thread
+         * takes a share of the positions */
+        for (int i = (int)threadIdx.x; i < (int)code.ranks; i += (int)blockDim.x) {
             const int idx = (int)rec[i];
             sm.pi[i] = (uint8_t)idx;
             const T col = load_col<W>(code.hcol, idx);
@@ -1193,7 +1191,7 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
     if (start == ORBG_NONE) {
         const T s0 = *s_s0;
         const uint32_t s0w = syn_key(s0);
-        mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x, (uint32_t)n);
+        mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x, code.ranks);
         if (mine.t != ORBG_NONE)
             atomicMin(s_best, mine.t);
         const uint4 light = __ldg(reinterpret_cast<const uint4 *>(code.light));

@@ -89,6 +89,7 @@ struct OrbgDeviceCode {
     uint32_t band_pre[ORBG_BANDS];   /* prefixes, */
     uint32_t band_ranks[ORBG_BANDS]; /* sorted positions they and the band's patterns take, */
     uint32_t band_end[ORBG_BANDS];   /* and the first query index past the band */
+    uint32_t ranks;              /* sorted positions any pattern of the order takes */
     uint32_t lead_pairs;         /* phase 2: pairs of the order's leading part, */
     uint32_t lead_end;           /* and the first query index past it */
     const uint32_t *flat;        /* [2 * nflat] flat-table patterns, 8 bytes each */
@@ -114,7 +115,7 @@ struct OrbgTables {
     uint32_t npre = 0, nflat = 0;
     uint32_t band_pairs[ORBG_BANDS] = {}, band_pre[ORBG_BANDS] = {};
     uint32_t band_ranks[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
-    uint32_t lead_pairs = 0, lead_end = 0;
+    uint32_t ranks = 0, lead_pairs = 0, lead_end = 0;
     uint64_t patterns = 0;  /* query indices covered (last index) */
 };
 /* The tables for the order of increasing reliability weight J0 w + beta W

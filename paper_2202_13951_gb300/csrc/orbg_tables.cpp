@@ -423,6 +423,9 @@ struct TableBuilder {
                 top = std::max(top, (uint32_t)(out->pairs[i] >> 8) + 1u);
             out->band_ranks[k] = top;
         }
+        for (int j = 1; j <= n; j++)
+            if (rho[(size_t)j] <= Rmax)
+                out->ranks = (uint32_t)j;
         /* phase 2's leading part, likewise, where one CTA's set does not hold
          * all pairs */
         uint32_t np = (uint32_t)out->pairs.size();
