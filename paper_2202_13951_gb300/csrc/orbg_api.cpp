@@ -32,6 +32,7 @@ struct orbg_codeset {
     uint32_t npairs_max;
     orbg_tuning tuning;
     std::vector<int> n_of;       /* n of each code, host copy */
+    std::vector<OrbgDeviceCode> by_bucket; /* var.by_bucket */
     OrbgDeviceCode code0;        /* host copy of code 0's descriptor */
     uint32_t cap_min;
     int device;
@@ -715,6 +716,12 @@ int orbg_codeset_create(const orbg_code *const *codes, int ncodes, orbg_codeset 
             v.bhi[v.n - 1] = j + 1;
         }
         v.bhi[v.n - 1] = ncodes + 1; /* ids outside the set go with the last variant */
+    }
+    if (ncodes <= ORBG_MAX_VARIANTS) {
+        s->by_bucket.resize((size_t)ncodes);
+        for (int i = 0; i < ncodes; i++)
+            s->by_bucket[(size_t)bucket[(size_t)i]] = descs[(size_t)i];
+        s->var.by_bucket = s->by_bucket.data();
     }
     cudaError_t e;
     if ((e = cudaGetDevice(&s->device)) != cudaSuccess ||

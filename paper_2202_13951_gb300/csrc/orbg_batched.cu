@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kSortThreads) orbg_code_count_kernel(
 __global__ void __launch_bounds__(kSortThreads) orbg_code_scatter_kernel(
     const int32_t *__restrict__ code_id, const int32_t *__restrict__ bucket, int64_t B, int ncodes,
     const uint32_t *__restrict__ count, uint32_t *__restrict__ cursor,
-    uint32_t *__restrict__ perm)
+    uint32_t *__restrict__ perm, uint32_t *__restrict__ q, uint8_t *__restrict__ ab)
 {
     extern __shared__ uint32_t sh[];
     uint32_t *base = sh;              /* [ncodes + 1] first slot of each code */
@@ -97,8 +97,14 @@ __global__ void __launch_bounds__(kSortThreads) orbg_code_scatter_kernel(
     for (int i = threadIdx.x; i <= ncodes; i += blockDim.x)
         local[i] = local[i] ? base[i] + atomicAdd(&cursor[i], local[i]) : 0u;
     __syncthreads();
-    for (int64_t b = lo + threadIdx.x; b < hi; b += blockDim.x)
-        perm[atomicAdd(&local[sort_bucket(code_id, bucket, b, ncodes)], 1u)] = (uint32_t)b;
+    for (int64_t b = lo + threadIdx.x; b < hi; b += blockDim.x) {
+        const int k = sort_bucket(code_id, bucket, b, ncodes);
+        perm[atomicAdd(&local[k], 1u)] = (uint32_t)b;
+        if (q != nullptr && k == ncodes) {
+            q[b] = 0u;
+            ab[b] = 2;
+        }
+    }
 }
 
 /* one warp per heavy-list entry; the lanes copy the codeword bytes */
@@ -169,7 +175,7 @@ int orbg_launch_heavy_gather(const OrbgDeviceCode *d_codes, const int32_t *code_
 }
 
 int orbg_launch_code_sort(const int32_t *code_id, const int32_t *bucket, int64_t B, int ncodes,
-                          const OrbgScratch &s, void *stream)
+                          const OrbgScratch &s, uint32_t *q, uint8_t *ab, void *stream)
 {
     cudaStream_t st = (cudaStream_t)stream;
     const size_t sh1 = sizeof(uint32_t) * (size_t)(ncodes + 1);
@@ -187,17 +193,18 @@ int orbg_launch_code_sort(const int32_t *code_id, const int32_t *bucket, int64_t
         return (int)e;
     const int64_t g2 = (B + kSortChunk - 1) / kSortChunk;
     orbg_code_scatter_kernel<<<(unsigned)g2, kSortThreads, 2 * sh1, st>>>(
-        code_id, bucket, B, ncodes, s.count, s.cursor, s.perm);
+        code_id, bucket, B, ncodes, s.count, s.cursor, s.perm, q, ab);
     return (int)cudaGetLastError();
 }
 
 int orbg_launch_exact(int K, int W, const OrbgBatchedArgs &a, const OrbgScratch &s,
-                      unsigned long long *queue, int blo, int bhi, int pdl)
+                      unsigned long long *queue, int blo, int bhi, int pdl,
+                      const OrbgDeviceCode *one)
 {
 #define ORBG_EX(KK)                                                                         \
-    return W <= 1   ? orbg_launch_exact_k##KK##w1(a, s, queue, blo, bhi, pdl)       \
-           : W == 2 ? orbg_launch_exact_k##KK##w2(a, s, queue, blo, bhi, pdl)       \
-                    : orbg_launch_exact_k##KK##w4(a, s, queue, blo, bhi, pdl);
+    return W <= 1   ? orbg_launch_exact_k##KK##w1(a, s, queue, blo, bhi, pdl, one)       \
+           : W == 2 ? orbg_launch_exact_k##KK##w2(a, s, queue, blo, bhi, pdl, one)       \
+                    : orbg_launch_exact_k##KK##w4(a, s, queue, blo, bhi, pdl, one);
     if (K <= 1)
         ORBG_EX(1)
     if (K == 2)

@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(256, ORBG_PHASE1_MIN_CTAS(K, W, ONE)) orbg_bat
                                                   warp * kWarpPairBytes);
     uint32_t *list = reinterpret_cast<uint32_t *>(
         smem + nwarps * (bstride + 2 * kSlot * 4 + kWarpPairBytes) + warp * key_list_bytes<K>());
-    const int64_t n0 = ONE ? code0.n : codes[0].n;
+    /* the dense layout's stride: the set's first code's length */
+    const int64_t n0 = ONE && !range_count ? code0.n : codes[0].n;
 
     /* the queue's slots: all B (< 2^32), or (range_count: the per-bucket
      * counts of the sort into perm) the slots of buckets [blo, bhi) */
@@ -263,20 +264,21 @@ int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
 /* Phase 1 of one decoder variant (K, W): the blocks of sort buckets
  * [blo, bhi) of ss.perm (blo < 0: every block, in order), on its own queue.
  * pdl: the launch may begin while the previous launch in the stream (the
- * previous variant's) finishes its last blocks. */
+ * previous variant's) finishes its last blocks.  one: all of them are this
+ * code. */
 template <int K, int W>
 int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned long long *queue,
-                   int blo, int bhi, int pdl)
+                   int blo, int bhi, int pdl, const OrbgDeviceCode *one)
 {
     const int nk = a.n_max < 32 * K ? a.n_max : 32 * K;
     const uint32_t bstride = block_smem_bytes(nk, W);
-    auto k1 = orbg_batched_kernel<K, W, false>;
+    auto k1 = one ? orbg_batched_kernel<K, W, true> : orbg_batched_kernel<K, W, false>;
     Cut c;
     const int rc = cut_launch(k1, a, warp_smem_bytes<K>(bstride), &c);
     if (rc != 0)
         return rc;
     const bool sorted = blo >= 0;
-    OrbgDeviceCode c0{};
+    const OrbgDeviceCode c0 = one ? *one : OrbgDeviceCode{};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)c.grid);
     cfg.blockDim = dim3((unsigned)(c.wpc * 32));
@@ -334,16 +336,26 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
     }
     if constexpr (!ONE) {
         /* per-block codes: one launch per decoder variant, each a kernel of
-         * that variant alone; with several variants the blocks are first
+         * that variant alone, or per code; with several the blocks are first
          * grouped by variant (a counting sort by bucket), and each launch
          * after the first may start while the one before finishes */
-        const bool sorted = a.var.n > 1;
+        const bool per_code =
+            a.var.by_bucket != nullptr && a.ncodes > 1 &&
+            a.B >= (int64_t)ORBG_PER_CODE_BLOCKS * a.ncodes;
+        const bool sorted = per_code || a.var.n > 1;
         if (sorted && (rc = orbg_launch_code_sort(a.code_id, a.var.d_bucket, a.B, a.ncodes, ss,
-                                                  st)) != 0)
+                                                  per_code ? a.q : nullptr, a.ab, st)) != 0)
             return (cudaError_t)rc;
-        for (int v = 0; v < a.var.n; v++) {
-            rc = orbg_launch_exact(a.var.k[v], a.var.w[v], a, ss, vqueue + v,
-                                   sorted ? a.var.blo[v] : -1, a.var.bhi[v], v > 0);
+        const int launches = per_code ? a.ncodes : a.var.n;
+        for (int v = 0; v < launches; v++) {
+            if (per_code) {
+                const OrbgDeviceCode &one = a.var.by_bucket[v];
+                const int k = one.n <= 32 ? 1 : one.n <= 64 ? 2 : one.n <= 128 ? 4 : 8;
+                rc = orbg_launch_exact(k, one.w32, a, ss, vqueue + v, v, v + 1, v > 0, &one);
+            } else {
+                rc = orbg_launch_exact(a.var.k[v], a.var.w[v], a, ss, vqueue + v,
+                                       sorted ? a.var.blo[v] : -1, a.var.bhi[v], v > 0, nullptr);
+            }
             if (rc != 0)
                 return (cudaError_t)rc;
         }

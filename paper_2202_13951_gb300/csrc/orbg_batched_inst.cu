@@ -27,8 +27,8 @@ int ORBG_INST_NAME(ORBG_INST_K, ORBG_INST_W)(const OrbgBatchedArgs &a)
 
 int ORBG_INST_NAME_EX(ORBG_INST_K, ORBG_INST_W)(const OrbgBatchedArgs &a, const OrbgScratch &s,
                                                 unsigned long long *queue, int blo, int bhi,
-                                                int pdl)
+                                                int pdl, const OrbgDeviceCode *one)
 {
     return orbg_batched_impl::launch_exact_t<ORBG_INST_K, ORBG_INST_W>(a, s, queue, blo, bhi,
-                                                                       pdl);
+                                                                       pdl, one);
 }

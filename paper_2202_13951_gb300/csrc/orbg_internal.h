@@ -165,7 +165,16 @@ struct OrbgVariants {
     int k[ORBG_MAX_VARIANTS], w[ORBG_MAX_VARIANTS];
     int blo[ORBG_MAX_VARIANTS], bhi[ORBG_MAX_VARIANTS];
     const int32_t *d_bucket; /* [ncodes] */
+    const OrbgDeviceCode *by_bucket; /* host: the descriptor of each bucket's code, for sets of up
+                                      * to ORBG_MAX_VARIANTS codes, else NULL */
 };
+/* A mixed-code call of at least this many blocks per code of such a set
+ * launches phase 1 per code, each with its descriptor in the kernel's
+ * parameters, and not per variant with descriptors read from memory block by
+ * block (four codes, 1,000,000 blocks: 2,392 -> 2,216 us); a smaller one pays
+ * more for the launches and their ends (four codes of one variant, 100,003
+ * blocks: 685 -> 712 us). */
+#define ORBG_PER_CODE_BLOCKS 65536
 struct OrbgBatchedArgs {
     const OrbgDeviceCode *d_codes;
     const OrbgDeviceCode *code0;
@@ -203,12 +212,14 @@ int orbg_launch_batched(const OrbgBatchedArgs &args);
 /* orbg_batched_inst.cu, one per (keys per lane K, syndrome words W): both
  * phases, and phase 1 of that decoder variant alone over sort buckets
  * [blo, bhi) (blo < 0: every block) on `queue` (pdl: the launch may begin
- * while the previous one in the stream finishes). */
+ * while the previous one in the stream finishes; one: all of those blocks are
+ * this code, else NULL). */
 struct OrbgScratch;
 #define ORBG_DECLARE_BATCHED(K, W)                                                   \
     int orbg_launch_batched_k##K##w##W(const OrbgBatchedArgs &a);                    \
     int orbg_launch_exact_k##K##w##W(const OrbgBatchedArgs &a, const OrbgScratch &s, \
-                                     unsigned long long *queue, int blo, int bhi, int pdl);
+                                     unsigned long long *queue, int blo, int bhi, int pdl,  \
+                                     const OrbgDeviceCode *one);
 ORBG_DECLARE_BATCHED(1, 1) ORBG_DECLARE_BATCHED(1, 2) ORBG_DECLARE_BATCHED(1, 4)
 ORBG_DECLARE_BATCHED(2, 1) ORBG_DECLARE_BATCHED(2, 2) ORBG_DECLARE_BATCHED(2, 4)
 ORBG_DECLARE_BATCHED(4, 1) ORBG_DECLARE_BATCHED(4, 2) ORBG_DECLARE_BATCHED(4, 4)
@@ -263,12 +274,15 @@ inline OrbgScratch orbg_scratch_layout(void *base, int64_t B, int ncodes)
 /* Order the blocks of a mixed-code call by the bucket of their code
  * (bucket[code id]; ids outside the set go to bucket ncodes): a counting
  * sort into perm, so that each decoder variant's blocks hold consecutive
- * slots and one launch per variant decodes them; returns a cudaError_t. */
+ * slots and one launch per variant or code decodes them; with q and ab given,
+ * blocks of ids outside the set are written there (0, ORBG_BLOCK_NAN).
+ * Returns a cudaError_t. */
 int orbg_launch_code_sort(const int32_t *code_id, const int32_t *bucket, int64_t B, int ncodes,
-                          const OrbgScratch &s, void *stream);
+                          const OrbgScratch &s, uint32_t *q, uint8_t *ab, void *stream);
 /* orbg_launch_exact_k*w* for keys per lane K and syndrome words W. */
 int orbg_launch_exact(int K, int W, const OrbgBatchedArgs &a, const OrbgScratch &s,
-                      unsigned long long *queue, int blo, int bhi, int pdl);
+                      unsigned long long *queue, int blo, int bhi, int pdl,
+                      const OrbgDeviceCode *one);
 /* Outputs of the blocks phase 2 decoded, gathered after the last launch of a
  * batch whose other results already went to the host.  At `out` (memory the
  * device writes, here host-mapped) the heavy list's length (uint64).  With

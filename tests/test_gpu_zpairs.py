@@ -10,7 +10,7 @@ import oracle
 from paper_2202_13951_gb300 import workloads
 from test_gpu_parity import assert_same, gpu_batched, gpu_plain, orbg  # noqa: F401
 
-pytest.importorskip("torch")
+torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
@@ -84,3 +84,33 @@ def test_prefix_of_more_positions_than_a_record(orbg):  # noqa: F811
     c = orbg.Code(H, max_query_cap=cap, model=model)
     assert_same(gpu_plain(orbg, c, llr, cap), want)
     assert_same(gpu_batched(orbg, orbg.CodeSet([c]), llr, cap), want)
+
+
+def test_per_code_launches(orbg):  # noqa: F811
+    """A call large enough for one phase-1 launch per code, dense (one
+    stride) with ids outside the set: each code's blocks as alone, the others
+    flagged, their codewords untouched."""
+    B, n, cap = 2 * 65536 + 5, 48, 20000
+    codes = [workloads.rlc(n, 34, 81), workloads.rlc(n, 30, 82)]
+    objs = [orbg.Code(c.H, max_query_cap=cap) for c in codes]
+    rng = np.random.default_rng(83)
+    cid = rng.integers(0, 2, B).astype(np.int32)
+    bad = rng.choice(B, 50, replace=False)
+    cid[bad] = rng.choice([-1, 2, 1 << 20], 50)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(84)
+    llr = 4.0 * (-1.0 + 0.5 * torch.randn((B, n), generator=gen, device="cuda"))
+    cs = orbg.CodeSet(objs)
+    cw, q, ab = orbg.decode_batched(cs, llr, cap, code_id=torch.from_numpy(cid).cuda())
+    torch.cuda.synchronize()
+    for j, c in enumerate(objs):
+        at = torch.from_numpy(np.nonzero(cid == j)[0]).cuda()
+        alone = orbg.decode_batched(orbg.CodeSet([c]), llr[at].contiguous(), cap)
+        for got, want in zip((cw[at], q[at], ab[at]), alone):
+            assert torch.equal(got, want)
+        pick = at[:40].cpu().numpy()
+        want = oracle.decode_batch(codes[j].H, llr[at[:40]].cpu().numpy(), cap)[:3]
+        assert_same((cw.cpu().numpy()[pick], q.cpu().numpy().astype(np.int64)[pick],
+                     ab.cpu().numpy()[pick]), want)
+    at = torch.from_numpy(bad).cuda()
+    assert (q[at] == 0).all() and (ab[at] == 2).all() and (cw[at] == 255).all()
