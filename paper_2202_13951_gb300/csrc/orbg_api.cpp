@@ -557,8 +557,9 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
         d.band_end[i] = tb.band_end[i];
     }
     d.ranks = tb.ranks;
-    d.lead_pairs = tb.lead_pairs;
-    d.lead_end = tb.lead_end;
+    d.chunk = tb.chunk;
+    std::copy(tb.cut_pairs, tb.cut_pairs + ORBG_CUTS, d.cut_pairs);
+    std::copy(tb.cut_end, tb.cut_end + ORBG_CUTS, d.cut_end);
     d.nflat = tb.nflat;
     c->dev.max_cap = cap;
     c->dev.n = n;
@@ -687,7 +688,7 @@ int orbg_codeset_create(const orbg_code *const *codes, int ncodes, orbg_codeset 
         s->n_max = std::max(s->n_max, codes[i]->n);
         s->w32_max = std::max(s->w32_max, codes[i]->w32);
         s->cap_min = std::min(s->cap_min, codes[i]->max_cap);
-        s->npairs_max = std::max(s->npairs_max, codes[i]->dev.npairs);
+        s->npairs_max = std::max(s->npairs_max, codes[i]->dev.chunk);
     }
     /* the decoder variants the kernels specialise on: keys per lane from n
      * (n <= 32, 64, 128, 256: 1, 2, 4, 8) and the syndrome words (1, 2, or

@@ -1,8 +1,8 @@
 /*
- * orbg_batched.cu -- the batched form's launcher: picks the instantiation
- * (orbg_batched_inst.cu, kernels in orbg_batched.cuh) by the longest code
- * and widest syndrome of the call, and the grid-size helper the persistent
- * kernels share.
+ * orbg_batched.cu -- the batched form's launcher (it picks the instantiation,
+ * orbg_batched_inst.cu, by the longest code and widest syndrome of the call),
+ * the code sort of mixed calls, the gather of phase 2's outputs for host
+ * buffers, and the grid-size helper the persistent kernels share.
  */
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -224,7 +224,7 @@ int orbg_launch_batched(const OrbgBatchedArgs &args)
         /* every block is code 0: size everything for it alone */
         a.n_max = a.code0->n;
         a.w32_max = a.code0->w32;
-        a.npairs_max = a.code0->npairs;
+        a.npairs_max = a.code0->chunk;
     }
 #define ORBG_BW(K)                                           \
     return a.w32_max <= 1   ? orbg_launch_batched_k##K##w1(a) \

@@ -8,15 +8,16 @@
  *      reliability key (FP32 bits of |L_i|, i) (Sec. III-A); starting
  *      syndrome s0 = H y (Sec. I).  If s0 = 0, y is a codeword and query 1
  *      (the zero pattern) decodes: no sort is needed;
- *   2. the reliability order pi (Sec. III-A): for blocks decided inside the
- *      flat table only its leading ranks, extracted as warp minima; else a
- *      warp bitonic sort of the keys in registers (the paper names bitonic
- *      sorting networks as one option, Sec. IV-B);
+ *   2. the reliability order pi (Sec. III-A): its leading ranks, as many as
+ *      the stage of the search uses, extracted as warp minima; only an order
+ *      that uses more than 128 of them takes a warp bitonic sort of the keys
+ *      (the paper names bitonic sorting networks as one option, Sec. IV-B);
  *   3. permuted columns hperm[p] = H[:, pi_p] into shared memory, after a
  *      zero column read by unused prefix slots;
  *   4. past the flat table, every pattern of weight >= 2 is a prefix and a
- *      pair of its last two positions: the block's pairs go into a hash set
- *      of their syndromes, and each prefix is one look-up of s0 (+) prefix
+ *      pair of its last two positions: the block's pairs go into a filter
+ *      of their syndromes (and, in a CTA, a hash set behind it), and each
+ *      prefix is one look-up of s0 (+) prefix
  *      (orbg_internal.h says why the first pair of a syndrome is enough, how
  *      a hit's query index is formed and when no later prefix can beat it);
  *   5. codeword y (+) z* (or y if abandoned), query count, abandon flag.
@@ -58,17 +59,6 @@ template <typename T> __device__ __forceinline__ T szero();
 template <> __device__ __forceinline__ uint32_t szero<uint32_t>() { return 0u; }
 template <> __device__ __forceinline__ uint2 szero<uint2>() { return make_uint2(0u, 0u); }
 template <> __device__ __forceinline__ uint4 szero<uint4>() { return make_uint4(0u, 0u, 0u, 0u); }
-
-__device__ __forceinline__ uint32_t shfl_xor_all(uint32_t v, int m) { return __shfl_xor_sync(FULL_MASK, v, m); }
-__device__ __forceinline__ uint2 shfl_xor_all(uint2 v, int m)
-{
-    return make_uint2(__shfl_xor_sync(FULL_MASK, v.x, m), __shfl_xor_sync(FULL_MASK, v.y, m));
-}
-__device__ __forceinline__ uint4 shfl_xor_all(uint4 v, int m)
-{
-    return make_uint4(__shfl_xor_sync(FULL_MASK, v.x, m), __shfl_xor_sync(FULL_MASK, v.y, m),
-                      __shfl_xor_sync(FULL_MASK, v.z, m), __shfl_xor_sync(FULL_MASK, v.w, m));
-}
 
 template <int W>
 __device__ __forceinline__ typename Syn<W>::T load_col(const uint32_t *__restrict__ hcol, int j)
@@ -116,10 +106,6 @@ template <int W> struct BlockSmem {
         pi = p;
     }
 };
-
-__device__ __forceinline__ uint32_t first_word(uint32_t v) { return v; }
-__device__ __forceinline__ uint32_t first_word(uint2 v) { return v.x; }
-__device__ __forceinline__ uint32_t first_word(uint4 v) { return v.x; }
 
 /* A 32-bit key of a syndrome, linear over GF(2) so that the key of a sum is
  * the XOR of the keys; the syndrome itself up to 32 bits.  Longer ones add
@@ -382,12 +368,11 @@ __device__ __forceinline__ void build_perm(const OrbgDeviceCode &code, const uin
 /* ------------------------------------- step 2': the leading ranks only */
 
 /*
- * Most blocks finish inside the flat table, whose patterns flip only the
- * ORBG_FLAT_RANKS least reliable positions.  For those the full sort is
- * replaced by extracting the smallest keys one at a time (a warp minimum
- * per rank) until the ranks a flat step needs are known; the full sort runs
- * only when the walk leaves the flat table.  Each lane first sorts its own
- * K keys, so its smallest is key[0].
+ * Each stage of the search (a flat step, a band, the handover to a CTA)
+ * reaches only so many of the least reliable positions.  Instead of a full
+ * sort the smallest keys are extracted one at a time, a warp minimum per
+ * rank, until the ranks the stage needs are known.  Each lane first sorts
+ * its own K keys, so its smallest is key[0].
  */
 template <int K>
 __device__ __forceinline__ void sort_lane(uint32_t (&key)[K])
@@ -539,8 +524,7 @@ constexpr uint32_t kWarpFilterBits = 14;
 constexpr uint32_t kWarpFilterBytes = (1u << kWarpFilterBits) / 8u;
 constexpr uint32_t kWarpPairBytes = kWarpFilterBytes + ((ORBG_BAND2_PAIRS * 4u + 15u) & ~15u);
 
-/* A CTA's for a code of `npairs` pairs, taken in chunks of at most
- * kPairChunk: at least 64 bits a pair (2^17 for the 1,640 of cap 1e6), and a
+/* A CTA's for `npairs` pairs at once, at most kPairChunk: at least 64 bits a pair (2^17 for the 1,640 of cap 1e6), and a
  * hash set behind it of at least two slots a pair, linear probing, in which
  * every lane finds its own pair (codes of few parity bits hit often).  An
  * entry is the pair's index in the chunk (low 12 bits) under the hash bits
@@ -550,9 +534,8 @@ constexpr uint32_t kPairChunk = ORBG_PAIR_CHUNK; /* 4095: entry kEmpty is never 
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 __host__ __device__ __forceinline__ uint32_t pair_filter_bits(uint32_t npairs)
 {
-    const uint32_t np = npairs < kPairChunk ? npairs : kPairChunk;
     uint32_t b = 12;
-    while (b < 18 && (1u << b) < 64u * np)
+    while (b < 18 && (1u << b) < 64u * npairs)
         b++;
     return b;
 }
@@ -655,29 +638,75 @@ __device__ __forceinline__ uint32_t pattern_index(const OrbgDeviceCode &code, ui
     return __ldg(code.start + at) + (id - a);
 }
 
-/* Query index of prefix i with the first of `np` pairs (their keys in
- * `keys`) that makes it a hit, and that pair in *pair, or ORBG_NONE; v: the
- * key to find.  The whole warp together (rare: kept out of line). */
-template <int W>
-__device__ __noinline__ uint32_t resolve_listed(const OrbgDeviceCode &code,
-                                                const typename Syn<W>::T *h,
-                                                typename Syn<W>::T s0, uint32_t i,
-                                                const uint32_t *keys, uint32_t v, uint32_t np,
-                                                int lane, uint32_t *pair)
+/* The warp's best of its lanes' hits, in every lane. */
+__device__ __forceinline__ PairHit warp_best(const PairHit &mine)
 {
-    for (uint32_t base = 0; base < np; base += 32u) {
-        const uint32_t k = base + (uint32_t)lane;
-        uint32_t f = __ballot_sync(FULL_MASK, k < np && keys[k] == v);
-        for (; f; f &= f - 1u) {
-            const uint32_t id = base + (uint32_t)__ffs(f) - 1u;
-            const uint32_t p = __ldg(code.pairs + id);
-            if (W == 1 || sz(sx(sx(h[p & 0xFFu], h[p >> 8]), prefix_target<W>(code, h, s0, i)))) {
-                *pair = id;
-                return pattern_index(code, i, id, p);
+    PairHit h;
+    h.t = __reduce_min_sync(FULL_MASK, mine.t);
+    const int src = __ffs(__ballot_sync(FULL_MASK, mine.t == h.t)) - 1;
+    h.pre = __shfl_sync(FULL_MASK, mine.pre, src);
+    h.pair = __shfl_sync(FULL_MASK, mine.pair, src);
+    return h;
+}
+
+/* The best of `best` and the hits of a warp's step: lanes f look for their
+ * key v among the first `np` pairs (their keys in `keys`), and the first of a
+ * key gives the index with the lane's prefix i.  One lane after the other,
+ * each with the whole warp; from kManyHits on (codes of few parity bits) and
+ * where the key is the syndrome, every lane for itself and all together: in
+ * turn, each would wait for its loads again (60,000 blocks of a (256,248)
+ * code, whose look-ups hit in three of five lanes: 173 -> 82 us; of a
+ * (256,244) code 173 -> 154, from seven hits on 171; with fewer than four
+ * BCH(127,113), a hit a step, gains nothing).  Kept out of line: most steps
+ * have none. */
+constexpr int kManyHits = 4;
+template <int W>
+__device__ __noinline__ PairHit resolve_step(const OrbgDeviceCode &code,
+                                             const typename Syn<W>::T *h,
+                                             typename Syn<W>::T s0, uint32_t i,
+                                             const uint32_t *keys, uint32_t v, uint32_t np,
+                                             uint32_t f, int lane, PairHit best)
+{
+    if (W == 1 && __popc(f) >= kManyHits) {
+        const uint4 *k4 = reinterpret_cast<const uint4 *>(keys);
+        uint32_t id = ORBG_NONE;
+#pragma unroll 4
+        for (uint32_t k = (np + 3u) / 4u; k-- > 0u;) {
+            const uint4 q = k4[k];
+            id = q.w == v ? 4u * k + 3u : id;
+            id = q.z == v ? 4u * k + 2u : id;
+            id = q.y == v ? 4u * k + 1u : id;
+            id = q.x == v ? 4u * k : id;
+        }
+        PairHit mine{ORBG_NONE, i, id};
+        if ((f >> lane & 1u) && id < np)
+            mine.t = pattern_index(code, i, id, __ldg(code.pairs + id));
+        __syncwarp();
+        mine = warp_best(mine);
+        return mine.t < best.t ? mine : best;
+    }
+    for (; f; f &= f - 1u) {
+        const int src = __ffs(f) - 1;
+        const uint32_t key = __shfl_sync(FULL_MASK, v, src);
+        const uint32_t pre = __shfl_sync(FULL_MASK, i, src);
+        bool found = false;
+        for (uint32_t base = 0; base < np && !found; base += 32u) {
+            const uint32_t k = base + (uint32_t)lane;
+            uint32_t same = __ballot_sync(FULL_MASK, k < np && keys[k] == key);
+            for (; same && !found; same &= same - 1u) {
+                const uint32_t id = base + (uint32_t)__ffs(same) - 1u;
+                const uint32_t p = __ldg(code.pairs + id);
+                if (W > 1 && !sz(sx(sx(h[p & 0xFFu], h[p >> 8]),
+                                    prefix_target<W>(code, h, s0, pre))))
+                    continue;
+                found = true;
+                const uint32_t t = pattern_index(code, pre, id, p);
+                if (t < best.t)
+                    best = PairHit{t, pre, id};
             }
         }
     }
-    return ORBG_NONE;
+    return best;
 }
 
 /* The same from a CTA's hash set of the pairs from lo, each lane for itself. */
@@ -731,17 +760,6 @@ __device__ __forceinline__ PairHit single_hits(const OrbgDeviceCode &code,
     return best;
 }
 
-/* The warp's best of its lanes' hits, in every lane. */
-__device__ __forceinline__ PairHit warp_best(const PairHit &mine)
-{
-    PairHit h;
-    h.t = __reduce_min_sync(FULL_MASK, mine.t);
-    const int src = __ffs(__ballot_sync(FULL_MASK, mine.t == h.t)) - 1;
-    h.pre = __shfl_sync(FULL_MASK, mine.pre, src);
-    h.pair = __shfl_sync(FULL_MASK, mine.pair, src);
-    return h;
-}
-
 /*
  * One warp searches band k of its block: the band's pairs from np on go into
  * its filter, then every prefix of the band is looked up, unless `best` or
@@ -793,19 +811,10 @@ __device__ __forceinline__ PairHit search_band(const OrbgDeviceCode &code,
                 break;
             v ^= sm.h0[(int)(((j < 4 ? r.x : r.y) >> (8 * (j & 3))) & 0xFFu) - 1];
         }
-        uint32_t f = __ballot_sync(FULL_MASK, i < npre && filter_has(filter, kWarpFilterBits, v));
-        for (; f; f &= f - 1u) {
-            const int src = __ffs(f) - 1;
-            uint32_t pair = 0;
-            const uint32_t t =
-                resolve_listed<W>(code, sm.h, s0, g * ORBG_GROUP + (uint32_t)src, keys,
-                                  __shfl_sync(FULL_MASK, v, src), hi, lane, &pair);
-            if (t < best.t) {
-                best.t = t;
-                best.pre = g * ORBG_GROUP + (uint32_t)src;
-                best.pair = pair;
-            }
-        }
+        const uint32_t f =
+            __ballot_sync(FULL_MASK, i < npre && filter_has(filter, kWarpFilterBits, v));
+        if (f)
+            best = resolve_step<W>(code, sm.h, s0, i, keys, v, hi, f, lane, best);
     }
     return best;
 }
@@ -1132,12 +1141,13 @@ __device__ __forceinline__ int load_and_sort(const OrbgDeviceCode &code, const f
  * already (phase 1 wrote it).  Its order comes from phase 1's
  * handover record, or warp 0 loads and sorts; all threads then build the
  * subset tables of the light positions and the filter of the block's pairs
- * (several in turn for an order of more than kPairChunk pairs); then
+ * (several in turn for an order of more than kPairChunk pairs: its cuts, then
+ * chunks); then
  * warp w looks up the prefixes of groups w, w + nw, w + 2 nw, ...  Each warp
  * stops at its first group whose floor is at least the shared best (or above
  * the cap): floors never decrease with the group index and the best never
  * increases, so no group that could hold the final best is skipped.
- * pair_sm: pair_smem_bytes(code.npairs) bytes.
+ * pair_sm: pair_smem_bytes(code.chunk) bytes.
  */
 template <int W>
 __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__restrict__ llr,
@@ -1152,7 +1162,7 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
     const int n = code.n;
     BlockSmem<W> sm(bsm, n);
     uint32_t *mask = reinterpret_cast<uint32_t *>(pair_sm);
-    const uint32_t fbits = pair_filter_bits(code.npairs), bits = pair_slot_bits(code.npairs);
+    const uint32_t fbits = pair_filter_bits(code.chunk), bits = pair_slot_bits(code.chunk);
     uint32_t *filter = reinterpret_cast<uint32_t *>(pair_sm + kMaskBytes);
     uint32_t *set = filter + (1u << fbits) / 32u;
     if (rec != nullptr) {
@@ -1208,24 +1218,26 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
         }
         const uint4 *gm = reinterpret_cast<const uint4 *>(code.gmeta);
         const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre);
-        /* first the pairs and prefixes of the order's leading part alone, most
-         * blocks' share; then the rest, chunk by chunk of pairs */
+        /* all pairs at once; or up to one cut after the other, then the rest
+         * chunk by chunk */
         uint32_t lo = 0, hi = 0;
-        bool lead = true;
+        int cut = code.chunk < code.npairs ? 0 : ORBG_CUTS;
 #pragma unroll 1
-        while (hi < code.npairs || lead) {
-            uint32_t end = ORBG_NONE;
-            if (lead && code.lead_pairs < code.npairs) {
-                hi = code.lead_pairs;
-                end = code.lead_end;
+        for (;;) {
+            const uint32_t from = hi;
+            uint32_t end = ORBG_NONE, limit = ORBG_NONE;
+            bool fresh = cut == 0;
+            if (cut < ORBG_CUTS) {
+                hi = code.cut_pairs[cut];
+                end = code.cut_end[cut];
+                /* the last cut's pairs are looked up in full: the chunk ends
+                 * with them */
+                limit = ++cut < ORBG_CUTS ? end : ORBG_NONE;
             } else {
-                /* after the lead, all pairs again: its filter holds them */
-                lo = lead || hi == code.lead_pairs ? 0u : hi;
-                hi = min(code.npairs, lo + kPairChunk);
+                lo = hi;
+                hi = min(code.npairs, lo + code.chunk);
+                fresh = true;
             }
-            const bool fresh = lead || lo != 0u;
-            const uint32_t from = fresh ? lo : code.lead_pairs;
-            lead = false;
             if (fresh) {
                 uint4 *clear = reinterpret_cast<uint4 *>(filter);
                 for (uint32_t i = threadIdx.x; i < (1u << fbits) / 128u; i += blockDim.x)
@@ -1254,7 +1266,7 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
                 const uint4 m = nm;
                 const uint2 r0 = nr0, r1 = nr1;
                 const uint32_t best = *((volatile uint32_t *)s_best);
-                if (m.x >= min(best, end) || m.x > cap)
+                if (m.x >= min(best, limit) || m.x > cap)
                     break;
                 /* the warp's next groups, loaded while these are searched */
                 const uint32_t gn = g + (uint32_t)nwarps;
@@ -1306,7 +1318,8 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
                 }
             }
             __syncthreads(); /* the filter is free before the next pairs */
-            if (end != ORBG_NONE && (*((volatile uint32_t *)s_best) < end || end > cap))
+            if (hi >= code.npairs ||
+                (end != ORBG_NONE && (*((volatile uint32_t *)s_best) < end || end > cap)))
                 break; /* every pattern before `end` is covered (uniform) */
         }
     }

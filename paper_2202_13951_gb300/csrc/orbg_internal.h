@@ -7,10 +7,13 @@
  * code as prefixes and pairs.  A pattern of weight w >= 2 is its prefix P,
  * the first w - 2 positions, and the pair a < b of the last two.  With h_j
  * the parity-check column of sorted position j, it is a hit iff h_a ^ h_b =
- * s0 ^ sum over P of h: the pairs of a block go into a hash set of their
- * syndromes, and one look-up per prefix then tests every pattern the prefix
- * starts, of whatever weight.  A search up to 1,004,225 queries (cap 1e6, n
- * >= 82) makes 15,552 look-ups over 1,640 pairs.
+ * s0 ^ sum over P of h: the pairs of a block go into a filter or hash set of
+ * their syndromes, and one look-up per prefix then tests every pattern the
+ * prefix starts, of whatever weight.  A search up to 1,004,225 queries (cap
+ * 1e6, n >= 82) makes 15,552 look-ups over 1,640 pairs.  Testing its patterns
+ * one by one was bound by the integer pipes: CA-Polar(128,94), 100,000 blocks
+ * at 3-6 dB and 119,000 queries a block, took 4,720 us, 12e9 tests; with the
+ * look-ups it takes 955 us.
  *
  * Only one pair per syndrome matters, the first in the order (weight, a, b):
  * if the first hit of the order is P + {a, b} and a pair {c, d} before {a, b}
@@ -46,19 +49,24 @@
 #define ORBG_BAND2_PAIRS 500
 #define ORBG_PRE1_MAX 1024
 /* Phase 2 (a CTA a block) holds up to ORBG_PAIR_CHUNK pairs at a time.  An
- * order of more takes its first ORBG_LEAD_PAIRS alone before all of them in
- * chunks: most blocks end there (three-segment model of BCH(127,113), 6,441
- * pairs: 216 -> 190 us on 100,000 blocks); with one chunk the repeated
- * look-ups cost more (CA-Polar(128,94) 1,030 -> 1,110 us). */
+ * order of more takes ORBG_SPLIT_CHUNK at a time, and of the first ones the
+ * leading ORBG_LEAD_PAIRS alone before the others (the cuts of a search:
+ * most blocks end at one of them).  Three-segment model of BCH(127,113),
+ * 6,441 pairs, us on 100,000 and 300,000 blocks: all pairs in chunks of 4,095
+ * 216 and -, its first 900 before them 180 and 434, both cuts 161 and 360;
+ * where one chunk holds all, a cut only repeats look-ups (CA-Polar(128,94)
+ * 1,030 -> 1,110 us). */
 #define ORBG_PAIR_CHUNK 4095
+#define ORBG_SPLIT_CHUNK 2047
 #define ORBG_LEAD_PAIRS 900
+#define ORBG_CUTS 2
 
 /* The flat table: the first `nflat` patterns of the order, 8 bytes each:
  * up to 7 positions, 1-based (0 = unused), then a byte describing the
  * pattern's step of 32: bits 0-4 the number of sorted ranks the step needs
  * (the largest position of that step or an earlier one, at most
  * ORBG_FLAT_RANKS), bits 5-7 the step's largest Hamming weight.  A warp
- * tests 32 consecutive patterns per step before it turns to runs. */
+ * tests 32 consecutive patterns per step before it turns to the bands. */
 #define ORBG_FLAT_MAX 256
 #define ORBG_FLAT_POS 7
 #define ORBG_FLAT_RANKS 31
@@ -90,8 +98,9 @@ struct OrbgDeviceCode {
     uint32_t band_ranks[ORBG_BANDS]; /* sorted positions they and the band's patterns take, */
     uint32_t band_end[ORBG_BANDS];   /* and the first query index past the band */
     uint32_t ranks;              /* sorted positions any pattern of the order takes */
-    uint32_t lead_pairs;         /* phase 2: pairs of the order's leading part, */
-    uint32_t lead_end;           /* and the first query index past it */
+    uint32_t chunk;              /* phase 2: pairs held at once; where that is not all, */
+    uint32_t cut_pairs[ORBG_CUTS]; /* the pairs of each cut, the last one a chunk, */
+    uint32_t cut_end[ORBG_CUTS]; /* and the first query index past it */
     const uint32_t *flat;        /* [2 * nflat] flat-table patterns, 8 bytes each */
     uint32_t nflat;
     uint32_t max_cap;
@@ -115,7 +124,7 @@ struct OrbgTables {
     uint32_t npre = 0, nflat = 0;
     uint32_t band_pairs[ORBG_BANDS] = {}, band_pre[ORBG_BANDS] = {};
     uint32_t band_ranks[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
-    uint32_t ranks = 0, lead_pairs = 0, lead_end = 0;
+    uint32_t ranks = 0, chunk = 0, cut_pairs[ORBG_CUTS] = {}, cut_end[ORBG_CUTS] = {};
     uint64_t patterns = 0;  /* query indices covered (last index) */
 };
 /* The tables for the order of increasing reliability weight J0 w + beta W
@@ -191,7 +200,7 @@ struct OrbgBatchedArgs {
     uint8_t *ab;
     unsigned long long *scratch;
     int warps_per_cta, ctas_per_sm, grab, heavy_warps;
-    uint32_t npairs_max;         /* most pairs of a code of the set */
+    uint32_t npairs_max;         /* most pairs phase 2 holds at once for a code of the set */
     void *stream;
     /* Staged calls (the host-buffer pipeline: phase 1 chunk by chunk as the
      * LLRs arrive, then one phase 2 over every chunk's open blocks).
@@ -240,9 +249,10 @@ ORBG_DECLARE_BATCHED(8, 1) ORBG_DECLARE_BATCHED(8, 2) ORBG_DECLARE_BATCHED(8, 4)
 #define ORBG_MAX_CODES 1024      /* codes in one set */
 size_t orbg_batched_scratch_bytes(int64_t B, int ncodes);
 /* Then, 16-byte aligned, up to ORBG_HANDOVER_MAX handover records: for the
- * i-th block phase 1 leaves open, its reliability order (256 bytes: the
- * received index of each sorted position) and its starting syndrome (16
- * bytes), so that phase 2 need not sort the block again. */
+ * i-th block phase 1 leaves open, the leading `ranks` positions of its
+ * reliability order (room for 256 bytes: the received index of each sorted
+ * position) and its starting syndrome (16 bytes), so that phase 2 need not
+ * order the block again.  Blocks past the records are loaded and sorted. */
 #define ORBG_HANDOVER_MAX 32768
 #define ORBG_HANDOVER_BYTES 272
 struct OrbgScratch {
@@ -347,10 +357,10 @@ int orbg_fit_map_lines(const int32_t *models, int64_t B, int32_t top, const int3
                        int32_t *cid, void *stream);
 /* The per-block fitted decoder (orbg_fitted_search_inst.cu, one per keys per
  * lane K): every block fitted (Sec. III-E) and searched in its own order, in
- * three launches; scratch: orbg_fitsearch_scratch_bytes(B) device bytes
- * (counters, the list of blocks the second launch searches, the list of
- * those it leaves to the third, and for each open block a handover record
- * of ORBG_FIT_HAND_BYTES: order, model, starting syndrome).
+ * four launches; scratch: orbg_fitsearch_scratch_bytes(B) device bytes
+ * (counters; the lists of blocks the second, third and fourth launch search;
+ * for each open block a handover record of ORBG_FIT_HAND_BYTES: order, model,
+ * starting syndrome).
  * Return a cudaError_t value. */
 #define ORBG_FIT_HAND_BYTES 384
 inline size_t orbg_fitsearch_scratch_bytes(int64_t B)

@@ -18,12 +18,14 @@ namespace {
  * all (after the first band).  Measured, us a call on 10,000 and 100,000
  * BCH(127,113) blocks: eight warps, first band 45 and 178; both bands 66 and
  * 200; four warps, first band 55 and 186; flat table alone 62 and 221; two
- * warps, both bands 80 and 259. */
+ * warps, both bands 80 and 259.  Four CTAs an SM for one-word syndromes (64
+ * registers): 100,000 of those 188 -> 178, 60,000 blocks of a (200,176) code
+ * 237 -> 215. */
 constexpr int kPlainWarps = 8;
 constexpr uint32_t kPlainBudget = ORBG_FLAT_MAX + 1;
 
 template <int K, int W>
-__global__ void __launch_bounds__(32 * kPlainWarps) orbg_plain_kernel(
+__global__ void __launch_bounds__(32 * kPlainWarps, W == 1 ? 4 : 1) orbg_plain_kernel(
     const __grid_constant__ OrbgDeviceCode code, const float *__restrict__ llr, int64_t B,
     uint32_t cap, uint8_t *__restrict__ cw, uint32_t *__restrict__ q, uint8_t *__restrict__ ab,
     uint32_t bstride)
@@ -65,7 +67,7 @@ cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t
 {
     const uint32_t bstride = block_smem_bytes(code.n, W);
     size_t smem = (size_t)(bstride + kWarpPairBytes + key_list_bytes<K>()) * kPlainWarps;
-    const size_t cta = (size_t)bstride + pair_smem_bytes(code.npairs);
+    const size_t cta = (size_t)bstride + pair_smem_bytes(code.chunk);
     if (smem < cta)
         smem = cta;
     int64_t grid = (B + kPlainWarps - 1) / kPlainWarps;

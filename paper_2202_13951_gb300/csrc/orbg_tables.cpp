@@ -426,15 +426,20 @@ struct TableBuilder {
         for (int j = 1; j <= n; j++)
             if (rho[(size_t)j] <= Rmax)
                 out->ranks = (uint32_t)j;
-        /* phase 2's leading part, likewise, where one CTA's set does not hold
-         * all pairs */
-        uint32_t np = (uint32_t)out->pairs.size();
-        if (np > ORBG_PAIR_CHUNK)
-            np = ORBG_LEAD_PAIRS;
-        while (np > 0 && np < out->pairs.size() && out->pgroup[np] == out->pgroup[np - 1])
-            np--;
-        out->lead_pairs = np;
-        out->lead_end = first_at(np < out->pairs.size() ? gsum[out->pgroup[np]] : past);
+        /* phase 2's cuts, likewise, where one CTA's set does not hold all
+         * pairs */
+        out->chunk = (uint32_t)out->pairs.size();
+        if (out->chunk > ORBG_PAIR_CHUNK) {
+            out->chunk = ORBG_SPLIT_CHUNK;
+            const uint32_t to[ORBG_CUTS] = {ORBG_LEAD_PAIRS, ORBG_SPLIT_CHUNK};
+            for (int k = 0; k < ORBG_CUTS; k++) {
+                uint32_t np = to[k];
+                while (np > 0 && out->pgroup[np] == out->pgroup[np - 1])
+                    np--;
+                out->cut_pairs[k] = np;
+                out->cut_end[k] = first_at(gsum[out->pgroup[np]]);
+            }
+        }
         make_flat();
         return 0;
     }

@@ -39,6 +39,11 @@ CASES = {
     # 32,385 pairs of n = 255, eight sets
     "eight_pair_chunks": (lambda: workloads.rlc(255, 231, 78).H, 255, 4.5, 60000,
                           ((), (40000,), (1,))),
+    # 6,441 pairs: the first 900, the first 2,047, then chunk by chunk
+    "cuts_of_an_order": (lambda: workloads.rlc(127, 109, 81).H, 127, 2.5, 1_000_000,
+                         ((7, 17), (3, 37, 58), (5, 2, 1))),
+    # most look-ups of a band hit
+    "many_hits_a_step": (lambda: workloads.rlc(256, 247, 82).H, 256, 5.0, 20000, None),
     "weightless_positions": (lambda: workloads.rlc(60, 40, 80).H, 60, 2.5, 30000,
                              ((20, 40), (-3, 10, 0), (3, 1, 2))),
 }
