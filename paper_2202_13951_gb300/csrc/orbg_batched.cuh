@@ -15,10 +15,11 @@
  * Both phases compute the exact first hit of the same query order, so the
  * result equals the plain form's block for block.
  *
- * ONE: every block belongs to one code, passed by value as a kernel
- * parameter (constant bank) and decoded with its exact keys-per-lane K and
- * syndrome width W; otherwise each block's code comes from the device array
- * and K, W are dispatched per block up to KMAX, WMAX.
+ * Every launch of phase 1 decodes one decoder variant (keys per lane K,
+ * syndrome width W); a mixed-code call sorts its blocks by code and launches
+ * per variant, or per code where each code has blocks enough.  ONE: all
+ * blocks are one code, passed by value as a kernel parameter (constant bank);
+ * otherwise each block's descriptor is read from the device array.
  */
 #pragma once
 #include <cuda_runtime.h>
@@ -244,7 +245,11 @@ int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
         return rc;
     const int64_t warps = (int64_t)c->grid * wpc;
     int64_t g = a.grab < 1 ? 1 : a.grab;
-    const int64_t fair = a.B / (8 * warps); /* eight grabs a warp or more */
+    /* eight grabs a warp or more; two for one code of up to 16 parity bits,
+     * whose blocks search alike and are short beside a grab's wait (60,000
+     * blocks of a (64,52) code: 90 -> 67 us; three serving codes, 50,000
+     * blocks, two 334, eight 299) */
+    const int64_t fair = a.B / ((a.code0 && a.code0->r <= 16 ? 2 : 8) * warps);
     if (g > fair)
         g = fair > 0 ? fair : 1;
     c->wpc = wpc;
