@@ -777,21 +777,27 @@ class Job:
                     1 if w <= 1 else 2 if w == 2 else 4))
         return len(kw)
 
+    def phase1_launches(self):
+        """Phase-1 launches of a call with code ids: one per code from 65,536
+        blocks a code on (sets of 2 to 12 codes), else one per variant."""
+        nc = len(self.codes)
+        return nc if 1 < nc <= 12 and self.B >= 65536 * nc else self.variants()
+
     def launches_per_step(self):
         """Kernels of this library launched by one step: per-block codes
-        (code ids) run phase 1 as one launch per decoder variant, after a
-        two-kernel grouping by variant when there are several; phase 2 is
-        one launch (whatever the budget: it also decodes the blocks whose
-        phase-1 walk ran past the warp's own triple table)."""
+        (code ids) run phase 1 as one launch per decoder variant, or per code
+        of large calls, after a two-kernel grouping by code when there are
+        several; phase 2 is one launch (whatever the budget: it also decodes
+        the blocks open after a warp's last band)."""
         if self.form == "plain":
             return 1
         if self.search:
-            return 3  # fit, one-warp search of the open blocks, CTA search of the long ones
+            return 4  # fit, one-warp search, pair look-ups by CTAs, their tree search
         phase2 = 1
         if self.fitted is not None:
             return 3 + 1 + phase2  # fit, mark, map; one variant (handles of one code); phase 2
         if self.off_np is not None:
-            v = self.variants()
+            v = self.phase1_launches()
             return (2 if v > 1 else 0) + v + phase2
         return 1 + phase2
 
@@ -799,13 +805,14 @@ class Job:
         if self.form == "plain":
             return "orbg_plain_kernel"
         if self.search:
-            return "orbg_fitprep_kernel + orbg_fitsearch_kernel + orbg_fitsearch_cta_kernel"
+            return ("orbg_fitprep_kernel + orbg_fitsearch_kernel + orbg_fitpair_kernel + "
+                    "orbg_fitsearch_cta_kernel")
         names = "orbg_batched_kernel + orbg_heavy_kernel"
         if self.fitted is not None:
             return "orbg_fit_kernel + line marking + " + names
-        if self.off_np is not None and self.variants() > 1:
-            names = ("orbg_batched_kernel (one launch per decoder variant) + orbg_heavy_kernel "
-                     "+ the two code-sort kernels")
+        if self.off_np is not None and self.phase1_launches() > 1:
+            names = ("orbg_batched_kernel (%d launches, per code or decoder variant) + "
+                     "orbg_heavy_kernel + the two code-sort kernels" % self.phase1_launches())
         return names
 
     def autotune(self):
@@ -994,9 +1001,11 @@ def bench_ours(args, rank, world, local):
                               "integer ops per step = sum_t W32 (w_t + 1) + B n ceil(log2 n) "
                               "= %s, which charges each column XOR as one op although one "
                               "3-input lop3 can retire two, and charges every query in full "
-                              "although the triple-range walk tests sixteen queries with "
-                              "about thirty instructions (so frac can exceed 1 on "
-                              "search-heavy work); peak = measured lop3 lanes/clk/SM (%s) x "
+                              "although one look-up of a prefix's syndrome among the "
+                              "block's pairs tests every query that the prefix starts, "
+                              "about 65 at cap 1e6 (so achieved counts the queries' "
+                              "equivalent and frac exceeds 1 on search-heavy work: "
+                              "issued_frac is the hardware's own utilisation); peak = measured lop3 lanes/clk/SM (%s) x "
                               "%d SMs x %.0f MHz (the median SM clock sampled during the "
                               "timed steps); issued_frac = the ALU pipe's issue utilisation "
                               "(ncu, time-weighted over the step's kernels, same source "
@@ -1009,7 +1018,7 @@ def bench_ours(args, rank, world, local):
         "smem_peak": {"bytes_per_clk_per_sm": smem_bpc,
                       "tb_s": (smem_bpc * sms * run_mhz * 1e6 / 1e12) if smem_bpc else None,
                       "what": "measured 64-bit conflict-free shared loads (the search's "
-                              "column and triple-table reads are shared loads)"},
+                              "column, filter and pair-set reads are shared loads)"},
     }
     if e2e:
         line["e2e"] = e2e

@@ -130,8 +130,7 @@ ORBG_API int orbg_load_code_line(const uint8_t *mat, int kind, int n, int k,
  * zero).  Ties: Hamming weight ascending, then positions lexicographically;
  * the empty pattern is query 1.  The orders of orbg_load_code and
  * orbg_load_code_line are the one-segment cases (J_0 = J0, beta_1 =
- * beta), built here without triple runs.  Every decode entry point decodes
- * in the handle's order.  Arrays are read during the call only.  Errors as
+ * beta).  Every decode entry point decodes in the handle's order.  Arrays are read during the call only.  Errors as
  * orbg_load_code; EINVAL for a model out of range; ELIMIT when the order
  * up to max_query_cap needs a position above 255 in a pattern's leading
  * positions or more than 22 flipped positions.
@@ -150,7 +149,9 @@ ORBG_API int orbg_code_info(const orbg_code *code, int *n, int *k,
                    uint32_t *max_query_cap, uint8_t *H_out);
 
 /*
- * Plain form: one launch, one warp per block, blocks in a static grid.
+ * Plain form: one launch, one warp per block, blocks in a static grid; a
+ * block its warp does not finish early in the order is searched by all warps
+ * of its CTA, inside the same launch.
  *   llr       : [B][n] FP32 LLRs, row-major, LLR = log f(Y|1)/f(Y|0).
  *   B         : number of blocks (0 is a no-op).
  *   query_cap : 1..max_query_cap of the handle; abandon after this many
@@ -192,15 +193,16 @@ ORBG_API int orbg_codeset_free(orbg_codeset *set);
  *   max_query_cap.
  * The call uses 287 + 16 ncodes + 12 B + 272 min(B, 32768) bytes of
  * stream-ordered device scratch (queue counters, per-code block counts, the
- * list of still-open blocks, the blocks' order grouped by decoder variant,
- * and the reliability order of up to 32,768 still-open blocks, which the
- * second launch reuses), allocated on cuda_stream from the library's pool
+ * list of still-open blocks, the blocks' order grouped by code,
+ * and the leading reliability order of up to 32,768 still-open blocks, which
+ * the second launch reuses), allocated on cuda_stream from the library's pool
  * (orbg_pool_trim).  With code_id given, the first launch is one launch per
  * decoder variant among the set's codes (length class n <= 32, 64, 128,
- * 256 and syndrome width 1, 2 or 3-4 words), each of that variant alone;
- * with several variants the blocks are first grouped by variant on the
- * device, and each variant's launch may begin while the previous one
- * finishes (programmatic dependent launch).  A code id outside the set
+ * 256 and syndrome width 1, 2 or 3-4 words), each of that variant alone, or
+ * one per code where a set of up to twelve codes has 65,536 blocks or more
+ * for each; with several such launches the blocks are first grouped by code on
+ * the device, and each launch, the second phase's too, may begin while the
+ * previous one finishes (programmatic dependent launch).  A code id outside the set
  * gives its block queries 0 and flag ORBG_BLOCK_NAN with its codeword
  * bytes untouched (with host layout arrays and offsets: ORBG_EINVAL).
  * Host buffers (staged through stream-ordered device copies): a call with
@@ -406,7 +408,7 @@ ORBG_API int orbg_probe_int_lanes(double *lanes_per_clk_per_sm);
  * Roofline probe for shared memory: bytes per SM per clock that 64-bit
  * shared loads deliver (a warp reads 32 consecutive 8-byte words, so no
  * bank conflicts), measured with clock64 on every SM of the current
- * device.  The column and triple-table reads of the search are shared
+ * device.  The search's column, filter and pair-set reads are shared
  * loads.  Synchronous; allocates and frees a small buffer.  The library's
  * own addition; the paper has no counterpart.
  */
@@ -415,10 +417,9 @@ ORBG_API int orbg_probe_smem_bytes(double *bytes_per_clk_per_sm);
 /*
  * The query order this library decodes in, for inspection and tests: the
  * first `count` noise patterns for length n (1..256), expanded from the
- * same tables the kernels read (table 0: the one-warp-per-block table;
- * table 1: the CTA table of the batched form's second phase; both hold
- * the same order; table 2: the flat table of the leading patterns both
- * start with, which stops after at most 256 patterns).  out: host memory, [count][n+1] int32 rows
+ * same tables the kernels read (tables 0 and 1: the prefixes and pairs that
+ * warps and CTAs look up, both the same; table 2: the flat table of the
+ * leading patterns, which stops after at most 256 patterns).  out: host memory, [count][n+1] int32 rows
  * holding w, then the w flipped positions (1-based, in increasing
  * reliability order, ascending), then zeros.  Returns the number of rows
  * written (fewer than count once the 2^n patterns run out), or a negative
@@ -433,8 +434,7 @@ ORBG_API int64_t orbg_query_order_line(int n, uint32_t count, int table, int32_t
                                        int32_t beta, int32_t *out);
 
 /* The same for the m-segment order of orbg_load_code_model (Sec. III-D,
- * Eq. relest_seg); the model's arguments as there.  Tables 0 and 1 are the
- * same run list. */
+ * Eq. relest_seg); the model's arguments as there. */
 ORBG_API int64_t orbg_query_order_model(int n, uint32_t count, int table, int m,
                                         const int32_t *anchors, const int32_t *J,
                                         const int32_t *beta, int32_t *out);
@@ -497,7 +497,7 @@ ORBG_API int orbg_fitted_free(orbg_fitted *f);
  * Full ORBGRAND with a piece-wise linear model fitted to each block, any
  * number of lines (Sec. III-E, Eq. Q, Eq. quant, then the order of Sec.
  * III-D, Eq. relest_seg): the paper's 1- to 4-line variants of Sec. IV.
- * One launch; per block, on the device: the reliability sort, the fit of
+ * Four launches; per block, on the device: the reliability sort, the fit of
  * orbg_fit_models (same anchors, same quantisation, plain or J-divisible),
  * and a search of the block's own order -- noise patterns by increasing
  * reliability weight (the sum over flipped sorted positions j of
@@ -516,8 +516,10 @@ ORBG_API int orbg_fitted_free(orbg_fitted *f);
  *   need reliability weights above 2^26 - 1 (far beyond any cap's reach
  *   for a model fitted to AWGN blocks) before its result is known, or its
  *   search exceeded its step guard; codeword = hard decision, queries = 0.
- * Device-buffer calls are asynchronous on cuda_stream and use 8 bytes of
- * stream-ordered device scratch (the work-queue counter).
+ * Device-buffer calls are asynchronous on cuda_stream and use 64 + 396 B bytes
+ * (and up to 45 of padding) of stream-ordered device scratch (the work queues'
+ * counters, three lists of blocks, and each open block's order, model and
+ * starting syndrome).
  * Errors: EINVAL, ELIMIT (query_cap above ORBG_MAX_QUERY_CAP), ENOMEM,
  * ECUDA; ENAN only for host-buffer calls, as orbg_decode.
  */

@@ -1,17 +1,19 @@
 /*
  * orbg_fitted_search.cuh -- full ORBGRAND with a piece-wise linear model
  * fitted to each block (Sec. III-E), searched in that block's own order
- * (Sec. III-D), one warp per block.
+ * (Sec. III-D).
  *
- * Per block, in three launches (each kernel's code stays small enough for
+ * Per block, in four launches (each kernel's code stays small enough for
  * the instruction cache: in one fused kernel the fit's double-precision code
  * and the search's tree walk, run by different warps of an SM at once, made
  * instruction fetch the largest stall).  The first launch does steps 1-3
  * and finishes the blocks that need no search; the second takes the others
  * from an open list, with their order and model in a handover record, one
  * warp per block; a block whose search grows long there goes to the third,
- * where all warps of a CTA search it (so the few longest blocks, which one
- * warp each would finish long after the rest, end sooner):
+ * where all warps of a CTA search it by pair look-ups (orbg_fitpair_kernel);
+ * the few that one does not cover (weights past its counting table, too many
+ * patterns tied at the hit's weight, an order of fewer patterns than the cap)
+ * go to the fourth, where a CTA walks the whole tree:
  *   1. load, hard decision y, starting syndrome s0 = H y (as the other
  *      decoders: load_block);
  *   2. the exact reliability order pi (sort_block) and the ordered curve
@@ -42,8 +44,8 @@
  * branch of a lane that is about to take its "add" branch; a lane at a leaf
  * also tests up to kLeafRun of the leaf's later siblings in the same step
  * while they are leaves too (the lanes stay in step: a longer inner run
- * would hold the other lanes).  When the warps of a CTA share a block, the
- * tree is cut into kClasses classes by the sets' second positions (modulo
+ * would hold the other lanes).  When the warps of a CTA share a block, in
+ * the third and fourth launch, the tree is cut into kClasses classes by the sets' second positions (modulo
  * kClasses; the singletons by their position), the warps take classes from
  * a counter, and each pass's node counts and least member are combined over
  * the warps.
