@@ -1067,78 +1067,77 @@ def bench_ours(args, rank, world, local):
 PROFILES = {
     "mixed/batched/basic": {
         "kernels": "batched",
-        "digest": "2c12445a5d48257a47c952b322d3bff627fe866c08f362acfe76301aa124f4ac",
-        # the step's kernels' DRAM bytes on 250,000 blocks (222.4 MB), x 4
+        "digest": "2b7fa358e689f06afe597eb1495cab852cb72e6aaf8cfe1e460f4c4be06034fb",
+        # the step's kernels' DRAM bytes on 270,000 blocks (215.4 MB), / 0.27;
         # ALU pipe issue share per kernel, weighted by the full-size step's
-        # time shares (phase 2 62.6 % x 0.542, phase 1 n = 256 42.7 % x 0.367,
-        # n = 128 36.5 % x 0.056, n = 64 32.9 % x 0.033)
-        "traffic_bytes_per_step": 889.6e6,
-        "issued_frac": 0.527,
-        "source": "profiles/orbg_batched_mixed_250k_full.md, "
+        # times (phase 2 41.2 %, phase 1 42.1, 40.3, 38.3 and 35.1 %)
+        "traffic_bytes_per_step": 797.8e6,
+        "issued_frac": 0.406,
+        "source": "profiles/orbg_batched_mixed_270k_full.md, "
                   "profiles/orbg_batched_mixed_1m_launches.md",
     },
     "bch/batched/fitted3": {
         "kernels": "fitsearch",
-        "digest": "de5fe7c9402f8746661f22207cfd249604b74f2bced388ba6bcd2e522d9358f9",
-        # 346.4 MB on 280,000 blocks, x 400,000 / 280,000
-        "traffic_bytes_per_step": 494.9e6,
-        "issued_frac": 0.317,
+        "digest": "504f9fa9f3bf485e491fe1748e7a3a7213df3ec528db3da1c2189cc391a70d6b",
+        # 357.2 MB on 280,000 blocks, x 400,000 / 280,000
+        "traffic_bytes_per_step": 510.3e6,
+        "issued_frac": 0.301,
         "source": "profiles/orbg_fitsearch_bch127_3line_280k_full.md",
     },
     "bch/batched/basic": {
         "kernels": "batched",
-        "digest": "2c12445a5d48257a47c952b322d3bff627fe866c08f362acfe76301aa124f4ac",
-        # 166.8 MB on the captured case, x 1.4286
-        "traffic_bytes_per_step": 238.3e6,
-        "issued_frac": 0.554,
+        "digest": "2b7fa358e689f06afe597eb1495cab852cb72e6aaf8cfe1e460f4c4be06034fb",
+        # 164.7 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 235.3e6,
+        "issued_frac": 0.540,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "bch/plain/basic": {
         "kernels": "plain",
-        "digest": "c529c1ef75f6f3ff68d8e84ae7a9ed48dd5b78b9e935a6f10120dd8354ec41b8",
-        # 165.0 MB on the captured case, x 1.4286
-        "traffic_bytes_per_step": 235.7e6,
-        "issued_frac": 0.344,
+        "digest": "557f1892bc18a25958700daa1bf2596c13982ee7b4e793fe4fa0e896c8d3bb5a",
+        # 165.4 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 236.3e6,
+        "issued_frac": 0.346,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "bch/batched/line": {
         "kernels": "batched",
-        "digest": "2c12445a5d48257a47c952b322d3bff627fe866c08f362acfe76301aa124f4ac",
-        # 169.1 MB on the captured case, x 1.4286
-        "traffic_bytes_per_step": 241.6e6,
-        "issued_frac": 0.557,
+        "digest": "2b7fa358e689f06afe597eb1495cab852cb72e6aaf8cfe1e460f4c4be06034fb",
+        # 167.9 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 239.9e6,
+        "issued_frac": 0.465,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "bch/batched/model": {
         "kernels": "batched",
-        "digest": "2c12445a5d48257a47c952b322d3bff627fe866c08f362acfe76301aa124f4ac",
-        # 166.4 MB on the captured case, x 1.4286
-        "traffic_bytes_per_step": 237.7e6,
-        "issued_frac": 0.614,
+        "digest": "2b7fa358e689f06afe597eb1495cab852cb72e6aaf8cfe1e460f4c4be06034fb",
+        # 170.7 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 243.8e6,
+        "issued_frac": 0.442,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "bch/batched/fitted1": {
         "kernels": "fitline",
-        "digest": "97ba7642ce2a3a88e76f54600d1b4350c6c75f61b0d9d555182f9b108aa4bd8b",
-        # 399.9 MB on the captured case, x 1.4286
-        "traffic_bytes_per_step": 571.3e6,
-        "issued_frac": 0.414,
+        "digest": "a757a5e9ada471cf7735ada42cc43455978fc65b9a68ddb60d8fde81a3f68fcf",
+        # 396.8 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 566.9e6,
+        "issued_frac": 0.382,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "paper256/batched/basic": {
         "kernels": "batched",
-        "digest": "2c12445a5d48257a47c952b322d3bff627fe866c08f362acfe76301aa124f4ac",
-        # 207.0 MB on the captured case, x 2.8571
-        "traffic_bytes_per_step": 591.4e6,
-        "issued_frac": 0.598,
+        "digest": "2b7fa358e689f06afe597eb1495cab852cb72e6aaf8cfe1e460f4c4be06034fb",
+        # 367.9 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 525.5e6,
+        "issued_frac": 0.404,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "capolar256/batched/fitted3": {
         "kernels": "fitsearch",
-        "digest": "de5fe7c9402f8746661f22207cfd249604b74f2bced388ba6bcd2e522d9358f9",
-        # 363.9 MB on the captured case, x 2.8571
-        "traffic_bytes_per_step": 1039.7e6,
-        "issued_frac": 0.305,
+        "digest": "504f9fa9f3bf485e491fe1748e7a3a7213df3ec528db3da1c2189cc391a70d6b",
+        # 380.5 MB on the captured case, x 2.8571
+        "traffic_bytes_per_step": 1087.2e6,
+        "issued_frac": 0.306,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
 }
