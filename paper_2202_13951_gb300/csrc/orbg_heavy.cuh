@@ -1,8 +1,8 @@
 /*
  * orbg_heavy.cuh -- phase 2 of the batched form: every CTA takes one block
  * left open by phase 1 at a time and searches it with all its warps
- * (decode_block_cta in orbg_decode_block.cuh).  Included by the
- * orbg_batched_k*.cu translation units; ONE as in orbg_batched.cuh.
+ * (decode_block_cta in orbg_decode_block.cuh).  Included by
+ * orbg_batched.cuh, whose ONE it shares.
  */
 #pragma once
 #include <cuda_runtime.h>
