@@ -9,6 +9,22 @@
 
 #include "orbg_internal.h"
 
+int orbg_allow_smem(const void *kern, size_t smem)
+{
+    cudaFuncAttributes fa;
+    cudaError_t e;
+    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return (int)e;
+    if (smem + fa.sharedSizeBytes <= 48 * 1024)
+        return 0; /* static + dynamic past 48 KB: opt in */
+    int dev = 0, most = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
+            cudaSuccess)
+        return (int)e;
+    return (int)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     most - (int)fa.sharedSizeBytes);
+}
+
 int orbg_grid_for(const void *kern, int threads, size_t smem, int ctas_per_sm, int *grid_out)
 {
     int dev = 0, sms = 0, occ = 0;
@@ -16,12 +32,9 @@ int orbg_grid_for(const void *kern, int threads, size_t smem, int ctas_per_sm, i
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return (int)e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return (int)e;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return (int)e;
-    if (smem + fa.sharedSizeBytes > 48 * 1024) { /* static + dynamic past 48 KB: opt in */
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return (int)e;
-    }
+    const int rc = orbg_allow_smem(kern, smem);
+    if (rc != 0)
+        return rc;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (e != cudaSuccess) return (int)e;
     if (occ < 1) return (int)cudaErrorInvalidConfiguration;

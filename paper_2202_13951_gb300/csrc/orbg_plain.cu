@@ -74,11 +74,10 @@ cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t
     if (grid > 0x7FFFFFFF)
         return cudaErrorInvalidValue;
     auto k = orbg_plain_kernel<K, W>;
-    if (smem > 47 * 1024) { /* static + dynamic past 48 KB: opt in */
-        const cudaError_t e = cudaFuncSetAttribute(
-            k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess)
-            return e;
+    if (smem > 47 * 1024) { /* with the static part past 48 KB, perhaps */
+        const int rc = orbg_allow_smem((const void *)k, smem);
+        if (rc != 0)
+            return (cudaError_t)rc;
     }
     k<<<(unsigned)grid, kPlainWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, bstride);
     return cudaGetLastError();
