@@ -558,6 +558,7 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
     }
     d.ranks = tb.ranks;
     d.chunk = tb.chunk;
+    d.scan = tb.scan;
     std::copy(tb.cut_pairs, tb.cut_pairs + ORBG_CUTS, d.cut_pairs);
     std::copy(tb.cut_end, tb.cut_end + ORBG_CUTS, d.cut_end);
     d.nflat = tb.nflat;

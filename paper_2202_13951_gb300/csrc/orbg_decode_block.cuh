@@ -1134,6 +1134,124 @@ __device__ __forceinline__ int load_and_sort(const OrbgDeviceCode &code, const f
                            : load_and_sort_k<8, W>(code, llr, bsm, lane, s0);
 }
 
+/* ------------------------------------ few prefixes, many pairs: a scan */
+
+/*
+ * The CTA's search of an order with code.scan set (the models that come close
+ * to ordering by Hamming weight): thousands of pairs, and too few prefixes to
+ * pay for inserting them.  The pairs are gone through in their order instead:
+ *   - alone, which covers every pattern before the first prefix of a position
+ *     (cut_end[0]): the first kScanLead of them, then, where any pair of
+ *     columns makes up s0 at all, the others.  Whether one does takes each
+ *     thread one comparison a row of pairs, its columns in registers, where a
+ *     pair of the list takes ten instructions;
+ *   - then with the prefixes' targets (s0 and the prefix's columns) in the
+ *     filter and the set, one look-up a pair.  All prefixes of a target stay
+ *     in the set: which of them comes first depends on the pair.
+ * The empty prefix's index of a pair bounds from below every hit of that pair
+ * and later ones.  100,000 blocks of a (255,231) code at 4.5-7 dB and cap
+ * 1e5, 32,385 pairs and 45 prefixes: in hash sets of 2,047 pairs 4,400 us,
+ * patterns one by one 1,160, pair by pair here 1,650, with the rows 770.
+ */
+constexpr uint32_t kScanLead = 2048;
+template <int W>
+__device__ __noinline__ PairHit scan_pairs(const OrbgDeviceCode &code, const BlockSmem<W> sm,
+                                           const typename Syn<W>::T s0, uint32_t cap,
+                                           uint32_t *filter, uint32_t fbits, uint32_t *set,
+                                           uint32_t bits, volatile uint32_t *s_best, int warp,
+                                           int lane, int nwarps, PairHit mine)
+{
+    const uint32_t s0w = syn_key(s0);
+    const uint32_t *two = reinterpret_cast<const uint32_t *>(code.pairs);
+    auto take = [&](uint32_t pre, uint32_t id, uint32_t p) {
+        const uint32_t t = pattern_index(code, pre, id, p);
+        if (t < mine.t) {
+            mine = PairHit{t, pre, id};
+            atomicMin(const_cast<uint32_t *>(s_best), t);
+        }
+    };
+    auto first_of = [&](uint32_t id) {
+        return __ldg(code.start + (__ldg(code.pinfo + id) & 0xFFFFu));
+    };
+    /* 64 pairs a warp step, two a lane; a pair is always the same thread's */
+    const uint32_t step = (uint32_t)nwarps * 64u;
+    auto alone = [&](uint32_t lo, uint32_t hi) {
+#pragma unroll 1
+        for (uint32_t base = lo + (uint32_t)warp * 64u; base < hi; base += step) {
+            const uint32_t id = base + 2u * (uint32_t)lane;
+            const uint32_t p2 = id < hi ? __ldg(two + (id >> 1)) : 0u;
+#pragma unroll
+            for (uint32_t u = 0; u < 2; u++) {
+                const uint32_t p = u ? p2 >> 16 : p2 & 0xFFFFu;
+                if ((sm.h0[p & 0xFFu] ^ sm.h0[p >> 8]) == s0w && id + u < hi &&
+                    (W == 1 || sz(sx(sx(sm.h[p & 0xFFu], sm.h[p >> 8]), s0))))
+                    take(0u, id + u, p);
+            }
+        }
+        __syncthreads();
+    };
+    const uint32_t lead = min(code.cut_pairs[0], kScanLead / step * step);
+    alone(0u, lead);
+    if (lead < code.cut_pairs[0] && *s_best >= first_of(lead)) {
+        uint32_t col[8];
+        bool any = false;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const uint32_t i = (uint32_t)(k * 32 + lane);
+            col[k] = sm.h0[i < code.ranks ? i : 0u];
+        }
+        for (uint32_t i = (uint32_t)warp; i < code.ranks; i += (uint32_t)nwarps) {
+            const uint32_t t = s0w ^ sm.h0[i];
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                any |= col[k] == t;
+        }
+        if (__syncthreads_or(any))
+            alone(lead, code.cut_pairs[0]);
+    }
+    if (*s_best < code.cut_end[0] || code.cut_end[0] > cap)
+        return mine; /* every pattern before that index is covered (uniform) */
+    for (uint32_t i = threadIdx.x; i < (1u << fbits) / 32u; i += blockDim.x)
+        filter[i] = 0u;
+    for (uint32_t i = threadIdx.x; i < (1u << bits); i += blockDim.x)
+        set[i] = kEmpty;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < code.npre; i += blockDim.x) {
+        const uint32_t v = syn_key(prefix_target<W>(code, sm.h, s0, i));
+        filter_add(filter, fbits, v);
+        const uint32_t x = pair_hash(v);
+        uint32_t slot = x >> (32u - bits);
+        while (atomicCAS(set + slot, kEmpty, slot_tag(x, bits) | i) != kEmpty)
+            slot = (slot + 1u) & ((1u << bits) - 1u);
+    }
+    __syncthreads();
+    const uint32_t end = code.cut_pairs[1];
+#pragma unroll 1
+    for (uint32_t base = (uint32_t)warp * 64u; base < end; base += step) {
+        const uint32_t from = first_of(base);
+        if (from >= *s_best || from > cap)
+            break;
+        const uint32_t id = base + 2u * (uint32_t)lane;
+        const uint32_t p2 = id < end ? __ldg(two + (id >> 1)) : 0u;
+#pragma unroll 1
+        for (uint32_t u = 0; u < 2; u++) {
+            const uint32_t p = u ? p2 >> 16 : p2 & 0xFFFFu;
+            const uint32_t v = sm.h0[p & 0xFFu] ^ sm.h0[p >> 8];
+            if (id + u >= end || !filter_has(filter, fbits, v))
+                continue;
+            const uint32_t x = pair_hash(v), tag = slot_tag(x, bits);
+            for (uint32_t slot = x >> (32u - bits); set[slot] != kEmpty;
+                 slot = (slot + 1u) & ((1u << bits) - 1u)) {
+                const uint32_t e = set[slot], pre = e & kIdMask;
+                if ((e ^ tag) <= kIdMask && sz(sx(sx(sm.h[p & 0xFFu], sm.h[p >> 8]),
+                                                  prefix_target<W>(code, sm.h, s0, pre))))
+                    take(pre, id + u, p);
+            }
+        }
+    }
+    return mine;
+}
+
 /* ------------------------------------------------ one CTA, one block */
 
 /*
@@ -1142,7 +1260,7 @@ __device__ __forceinline__ int load_and_sort(const OrbgDeviceCode &code, const f
  * handover record, or warp 0 loads and sorts; all threads then build the
  * subset tables of the light positions and the filter of the block's pairs
  * (several in turn for an order of more than kPairChunk pairs: its cuts, then
- * chunks); then
+ * chunks; scan_pairs takes one of many pairs and few prefixes); then
  * warp w looks up the prefixes of groups w, w + nw, w + 2 nw, ...  Each warp
  * stops at its first group whose floor is at least the shared best (or above
  * the cap): floors never decrease with the group index and the best never
@@ -1204,123 +1322,128 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
         mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x, code.ranks);
         if (mine.t != ORBG_NONE)
             atomicMin(s_best, mine.t);
-        const uint4 light = __ldg(reinterpret_cast<const uint4 *>(code.light));
-        for (uint32_t e = threadIdx.x; e < 512u; e += blockDim.x) {
-            const uint32_t w0 = e < 256u ? light.x : light.z, w1 = e < 256u ? light.y : light.w;
-            uint32_t v = 0;
-#pragma unroll
-            for (int b = 0; b < 8; b++) {
-                const int p = (int)(((b < 4 ? w0 : w1) >> (8 * (b & 3))) & 0xFFu);
-                const uint32_t c = sm.h0[p - 1];
-                v ^= e >> b & 1u ? c : 0u;
-            }
-            mask[e] = v;
-        }
-        const uint4 *gm = reinterpret_cast<const uint4 *>(code.gmeta);
-        const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre);
-        /* all pairs at once; or up to one cut after the other, then the rest
-         * chunk by chunk */
-        uint32_t lo = 0, hi = 0;
-        int cut = code.chunk < code.npairs ? 0 : ORBG_CUTS;
-#pragma unroll 1
-        for (;;) {
-            const uint32_t from = hi;
-            uint32_t end = ORBG_NONE, limit = ORBG_NONE;
-            bool fresh = cut == 0;
-            if (cut < ORBG_CUTS) {
-                hi = code.cut_pairs[cut];
-                end = code.cut_end[cut];
-                /* the last cut's pairs are looked up in full: the chunk ends
-                 * with them */
-                limit = ++cut < ORBG_CUTS ? end : ORBG_NONE;
-            } else {
-                lo = hi;
-                hi = min(code.npairs, lo + code.chunk);
-                fresh = true;
-            }
-            if (fresh) {
-                uint4 *clear = reinterpret_cast<uint4 *>(filter);
-                for (uint32_t i = threadIdx.x; i < (1u << fbits) / 128u; i += blockDim.x)
-                    clear[i] = make_uint4(0u, 0u, 0u, 0u);
-                clear = reinterpret_cast<uint4 *>(set);
-                for (uint32_t i = threadIdx.x; i < (1u << bits) / 4u; i += blockDim.x)
-                    clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
-            }
-            __syncthreads();
-            for (uint32_t id = from + threadIdx.x; id < hi; id += blockDim.x)
-                insert_pair<W>(code, sm, filter, fbits, set, bits, lo, id);
-            __syncthreads();
-            /* two groups a warp step: their loads overlap, and the step's
-             * overhead is shared (60 -> 48 warp instructions a group) */
-            const uint32_t ng2 = (code.ngroups + 1u) / 2u;
-            uint32_t g = (uint32_t)warp;
-            uint4 nm = make_uint4(ORBG_NONE, 0u, ORBG_NONE, 0u);
-            uint2 nr0 = make_uint2(0u, 0u), nr1 = nr0;
-            if (g < ng2) {
-                nm = __ldg(gm + g);
-                nr0 = __ldg(pre + g * 64u + (uint32_t)lane);
-                nr1 = __ldg(pre + g * 64u + 32u + (uint32_t)lane);
-            }
-#pragma unroll 1
-            for (; g < ng2; g += (uint32_t)nwarps) {
-                const uint4 m = nm;
-                const uint2 r0 = nr0, r1 = nr1;
-                const uint32_t best = *((volatile uint32_t *)s_best);
-                if (m.x >= min(best, limit) || m.x > cap)
-                    break;
-                /* the warp's next groups, loaded while these are searched */
-                const uint32_t gn = g + (uint32_t)nwarps;
-                if (gn < ng2) {
-                    nm = __ldg(gm + gn);
-                    nr0 = __ldg(pre + gn * 64u + (uint32_t)lane);
-                    nr1 = __ldg(pre + gn * 64u + 32u + (uint32_t)lane);
+        if (code.scan) {
+            mine = scan_pairs<W>(code, sm, s0, cap, filter, fbits, set, bits, s_best, warp, lane,
+                                 nwarps, mine);
+        } else {
+            const uint4 light = __ldg(reinterpret_cast<const uint4 *>(code.light));
+            for (uint32_t e = threadIdx.x; e < 512u; e += blockDim.x) {
+                const uint32_t w0 = e < 256u ? light.x : light.z, w1 = e < 256u ? light.y : light.w;
+                uint32_t v = 0;
+    #pragma unroll
+                for (int b = 0; b < 8; b++) {
+                    const int p = (int)(((b < 4 ? w0 : w1) >> (8 * (b & 3))) & 0xFFu);
+                    const uint32_t c = sm.h0[p - 1];
+                    v ^= e >> b & 1u ? c : 0u;
                 }
-                const uint32_t i = g * 64u + (uint32_t)lane;
-                uint32_t v0 = s0w ^ mask[r0.x & 0xFFu] ^ mask[256u + ((r0.x >> 8) & 0xFFu)];
-                uint32_t v1 = s0w ^ mask[r1.x & 0xFFu] ^ mask[256u + ((r1.x >> 8) & 0xFFu)];
-                const int kmax = (int)max(m.y & 0xFFu, m.w & 0xFFu);
-#pragma unroll
-                for (int j = 0; j < ORBG_PRE_POS; j++) {
-                    if (j >= kmax)
+                mask[e] = v;
+            }
+            const uint4 *gm = reinterpret_cast<const uint4 *>(code.gmeta);
+            const uint2 *pre = reinterpret_cast<const uint2 *>(code.pre);
+            /* all pairs at once; or up to one cut after the other, then the rest
+             * chunk by chunk */
+            uint32_t lo = 0, hi = 0;
+            int cut = code.chunk < code.npairs ? 0 : ORBG_CUTS;
+    #pragma unroll 1
+            for (;;) {
+                const uint32_t from = hi;
+                uint32_t end = ORBG_NONE, limit = ORBG_NONE;
+                bool fresh = cut == 0;
+                if (cut < ORBG_CUTS) {
+                    hi = code.cut_pairs[cut];
+                    end = code.cut_end[cut];
+                    /* the last cut's pairs are looked up in full: the chunk ends
+                     * with them */
+                    limit = ++cut < ORBG_CUTS ? end : ORBG_NONE;
+                } else {
+                    lo = hi;
+                    hi = min(code.npairs, lo + code.chunk);
+                    fresh = true;
+                }
+                if (fresh) {
+                    uint4 *clear = reinterpret_cast<uint4 *>(filter);
+                    for (uint32_t i = threadIdx.x; i < (1u << fbits) / 128u; i += blockDim.x)
+                        clear[i] = make_uint4(0u, 0u, 0u, 0u);
+                    clear = reinterpret_cast<uint4 *>(set);
+                    for (uint32_t i = threadIdx.x; i < (1u << bits) / 4u; i += blockDim.x)
+                        clear[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+                }
+                __syncthreads();
+                for (uint32_t id = from + threadIdx.x; id < hi; id += blockDim.x)
+                    insert_pair<W>(code, sm, filter, fbits, set, bits, lo, id);
+                __syncthreads();
+                /* two groups a warp step: their loads overlap, and the step's
+                 * overhead is shared (60 -> 48 warp instructions a group) */
+                const uint32_t ng2 = (code.ngroups + 1u) / 2u;
+                uint32_t g = (uint32_t)warp;
+                uint4 nm = make_uint4(ORBG_NONE, 0u, ORBG_NONE, 0u);
+                uint2 nr0 = make_uint2(0u, 0u), nr1 = nr0;
+                if (g < ng2) {
+                    nm = __ldg(gm + g);
+                    nr0 = __ldg(pre + g * 64u + (uint32_t)lane);
+                    nr1 = __ldg(pre + g * 64u + 32u + (uint32_t)lane);
+                }
+    #pragma unroll 1
+                for (; g < ng2; g += (uint32_t)nwarps) {
+                    const uint4 m = nm;
+                    const uint2 r0 = nr0, r1 = nr1;
+                    const uint32_t best = *((volatile uint32_t *)s_best);
+                    if (m.x >= min(best, limit) || m.x > cap)
                         break;
-                    const uint32_t p0 = j < 2 ? r0.x >> (16 + 8 * j) : r0.y >> (8 * (j - 2));
-                    const uint32_t p1 = j < 2 ? r1.x >> (16 + 8 * j) : r1.y >> (8 * (j - 2));
-                    v0 ^= sm.h0[(int)(p0 & 0xFFu) - 1];
-                    v1 ^= sm.h0[(int)(p1 & 0xFFu) - 1];
-                }
-                if (kmax > ORBG_PRE_POS) {
-                    const uint2 *ext = reinterpret_cast<const uint2 *>(code.pext);
-                    const uint2 x0 = __ldg(ext + i), x1 = __ldg(ext + i + 32u);
-                    for (int j = 0; j < 8; j++) {
-                        v0 ^= sm.h0[(int)(((j < 4 ? x0.x : x0.y) >> (8 * (j & 3))) & 0xFFu) - 1];
-                        v1 ^= sm.h0[(int)(((j < 4 ? x1.x : x1.y) >> (8 * (j & 3))) & 0xFFu) - 1];
+                    /* the warp's next groups, loaded while these are searched */
+                    const uint32_t gn = g + (uint32_t)nwarps;
+                    if (gn < ng2) {
+                        nm = __ldg(gm + gn);
+                        nr0 = __ldg(pre + gn * 64u + (uint32_t)lane);
+                        nr1 = __ldg(pre + gn * 64u + 32u + (uint32_t)lane);
                     }
-                }
-                const bool maybe0 = filter_has(filter, fbits, v0);
-                const bool maybe1 = filter_has(filter, fbits, v1);
-                if (__any_sync(FULL_MASK, maybe0 | maybe1)) {
-#pragma unroll 1
-                    for (int w = 0; w < 2; w++) {
-                        const uint32_t iw = i + 32u * (uint32_t)w;
-                        if (!(w ? maybe1 : maybe0) || iw >= code.npre)
-                            continue;
-                        uint32_t pair = 0;
-                        const uint32_t t = resolve_hashed<W>(code, sm.h, s0, iw, set, bits,
-                                                             w ? v1 : v0, lo, &pair);
-                        if (t < mine.t) {
-                            mine.t = t;
-                            mine.pre = iw;
-                            mine.pair = pair;
-                            atomicMin(s_best, t);
+                    const uint32_t i = g * 64u + (uint32_t)lane;
+                    uint32_t v0 = s0w ^ mask[r0.x & 0xFFu] ^ mask[256u + ((r0.x >> 8) & 0xFFu)];
+                    uint32_t v1 = s0w ^ mask[r1.x & 0xFFu] ^ mask[256u + ((r1.x >> 8) & 0xFFu)];
+                    const int kmax = (int)max(m.y & 0xFFu, m.w & 0xFFu);
+    #pragma unroll
+                    for (int j = 0; j < ORBG_PRE_POS; j++) {
+                        if (j >= kmax)
+                            break;
+                        const uint32_t p0 = j < 2 ? r0.x >> (16 + 8 * j) : r0.y >> (8 * (j - 2));
+                        const uint32_t p1 = j < 2 ? r1.x >> (16 + 8 * j) : r1.y >> (8 * (j - 2));
+                        v0 ^= sm.h0[(int)(p0 & 0xFFu) - 1];
+                        v1 ^= sm.h0[(int)(p1 & 0xFFu) - 1];
+                    }
+                    if (kmax > ORBG_PRE_POS) {
+                        const uint2 *ext = reinterpret_cast<const uint2 *>(code.pext);
+                        const uint2 x0 = __ldg(ext + i), x1 = __ldg(ext + i + 32u);
+                        for (int j = 0; j < 8; j++) {
+                            v0 ^= sm.h0[(int)(((j < 4 ? x0.x : x0.y) >> (8 * (j & 3))) & 0xFFu) - 1];
+                            v1 ^= sm.h0[(int)(((j < 4 ? x1.x : x1.y) >> (8 * (j & 3))) & 0xFFu) - 1];
                         }
                     }
-                    __syncwarp();
+                    const bool maybe0 = filter_has(filter, fbits, v0);
+                    const bool maybe1 = filter_has(filter, fbits, v1);
+                    if (__any_sync(FULL_MASK, maybe0 | maybe1)) {
+    #pragma unroll 1
+                        for (int w = 0; w < 2; w++) {
+                            const uint32_t iw = i + 32u * (uint32_t)w;
+                            if (!(w ? maybe1 : maybe0) || iw >= code.npre)
+                                continue;
+                            uint32_t pair = 0;
+                            const uint32_t t = resolve_hashed<W>(code, sm.h, s0, iw, set, bits,
+                                                                 w ? v1 : v0, lo, &pair);
+                            if (t < mine.t) {
+                                mine.t = t;
+                                mine.pre = iw;
+                                mine.pair = pair;
+                                atomicMin(s_best, t);
+                            }
+                        }
+                        __syncwarp();
+                    }
                 }
+                __syncthreads(); /* the filter is free before the next pairs */
+                if (hi >= code.npairs ||
+                    (end != ORBG_NONE && (*((volatile uint32_t *)s_best) < end || end > cap)))
+                    break; /* every pattern before `end` is covered (uniform) */
             }
-            __syncthreads(); /* the filter is free before the next pairs */
-            if (hi >= code.npairs ||
-                (end != ORBG_NONE && (*((volatile uint32_t *)s_best) < end || end > cap)))
-                break; /* every pattern before `end` is covered (uniform) */
         }
     }
     __syncthreads();

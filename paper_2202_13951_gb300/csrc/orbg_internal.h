@@ -60,6 +60,13 @@
 #define ORBG_SPLIT_CHUNK 2047
 #define ORBG_LEAD_PAIRS 900
 #define ORBG_CUTS 2
+/* An order of many pairs alone (at least phase 1's 500) and few prefixes, up
+ * to ORBG_SCAN_PREFIXES and half as many as pairs, is searched the other way
+ * round, the prefixes held and the pairs gone through (scan_pairs).  Lines on
+ * n = 127, 100,000 blocks, hash sets of pairs / scan, us: J_0 = 9000 (8,001
+ * pairs, 51 prefixes) 640 / 332; J_0 = 50 at cap 1e6 (7,952 and 2,384) 303 /
+ * 486, since every block that reaches the prefixes inserts them all. */
+#define ORBG_SCAN_PREFIXES 2047
 
 /* The flat table: the first `nflat` patterns of the order, 8 bytes each:
  * up to 7 positions, 1-based (0 = unused), then a byte describing the
@@ -98,9 +105,13 @@ struct OrbgDeviceCode {
     uint32_t band_ranks[ORBG_BANDS]; /* sorted positions they and the band's patterns take, */
     uint32_t band_end[ORBG_BANDS];   /* and the first query index past the band */
     uint32_t ranks;              /* sorted positions any pattern of the order takes */
-    uint32_t chunk;              /* phase 2: pairs held at once; where that is not all, */
+    uint32_t chunk;              /* phase 2: pairs (scan: prefixes) held at once; where that is not
+                                  * all pairs, */
     uint32_t cut_pairs[ORBG_CUTS]; /* the pairs of each cut, the last one a chunk, */
     uint32_t cut_end[ORBG_CUTS]; /* and the first query index past it */
+    uint32_t scan;               /* phase 2 holds the prefixes and goes through the pairs: the
+                                  * first cut_pairs[0] alone, which covers the queries before
+                                  * cut_end[0], then the first cut_pairs[1] with every prefix */
     const uint32_t *flat;        /* [2 * nflat] flat-table patterns, 8 bytes each */
     uint32_t nflat;
     uint32_t max_cap;
@@ -125,6 +136,7 @@ struct OrbgTables {
     uint32_t band_pairs[ORBG_BANDS] = {}, band_pre[ORBG_BANDS] = {};
     uint32_t band_ranks[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
     uint32_t ranks = 0, chunk = 0, cut_pairs[ORBG_CUTS] = {}, cut_end[ORBG_CUTS] = {};
+    uint32_t scan = 0;
     uint64_t patterns = 0;  /* query indices covered (last index) */
 };
 /* The tables for the order of increasing reliability weight J0 w + beta W

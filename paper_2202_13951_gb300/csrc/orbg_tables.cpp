@@ -397,14 +397,35 @@ struct TableBuilder {
                 out->gmeta[2 * (size_t)(i / ORBG_GROUP)] = first_at(p.m);
         }
         npre1 = std::min<uint32_t>(npre1, ORBG_PRE1_MAX);
+        const long past = Rmax + 1;
+        const uint32_t npairs = (uint32_t)out->pairs.size();
+        /* the first weight of a prefix that holds a position, and the pairs
+         * below it */
+        const long first = npre > 1 ? pre[ord[1]].m : past;
+        uint32_t alone = 0;
+        while (alone < npairs && gsum[out->pgroup[alone]] < first)
+            alone++;
+        if (alone >= ORBG_BAND2_PAIRS && npre <= ORBG_SCAN_PREFIXES && npre <= npairs / 2) {
+            out->scan = 1;
+            out->cut_pairs[0] = alone;
+            out->cut_end[0] = first_at(first);
+            /* then the pairs that prefixes of positions take, or all, if the
+             * first ones are not */
+            uint32_t most = 0, np = npairs;
+            for (uint32_t i = 1; i < npre; i++)
+                most = std::max(most, g0[(size_t)pre[ord[i]].q] + out->pmeta[2 * i + 2] -
+                                          out->pmeta[2 * i]);
+            while (alone == npairs && np > 0 && out->pgroup[np - 1] >= most)
+                np--;
+            out->cut_pairs[1] = np;
+        }
         /* phase 1's bands: the pairs of the leading groups; the first weight
          * not covered by them and the leading prefixes; how many prefixes
          * and positions the patterns below it take */
         const uint32_t aim[ORBG_BANDS] = {ORBG_BAND1_PAIRS, ORBG_BAND2_PAIRS};
-        const long past = Rmax + 1;
         const long lim1 = npre1 < npre ? pre[ord[npre1]].m : past;
         for (int k = 0; k < ORBG_BANDS; k++) {
-            uint32_t np = std::min<uint32_t>(aim[k], (uint32_t)out->pairs.size());
+            uint32_t np = std::min(aim[k], npairs);
             while (np > 0 && np < out->pairs.size() && out->pgroup[np] == out->pgroup[np - 1])
                 np--;
             const long end =
@@ -428,8 +449,8 @@ struct TableBuilder {
                 out->ranks = (uint32_t)j;
         /* phase 2's cuts, likewise, where one CTA's set does not hold all
          * pairs */
-        out->chunk = (uint32_t)out->pairs.size();
-        if (out->chunk > ORBG_PAIR_CHUNK) {
+        out->chunk = out->scan ? npre : (uint32_t)out->pairs.size();
+        if (!out->scan && out->chunk > ORBG_PAIR_CHUNK) {
             out->chunk = ORBG_SPLIT_CHUNK;
             const uint32_t to[ORBG_CUTS] = {ORBG_LEAD_PAIRS, ORBG_SPLIT_CHUNK};
             for (int k = 0; k < ORBG_CUTS; k++) {
