@@ -328,12 +328,12 @@ int orbg_launch_heavy_gather(const OrbgDeviceCode *d_codes, const int32_t *code_
                              const uint8_t *ab, const OrbgScratch &s, unsigned char *out,
                              uint32_t cap, int n_max, uint8_t *to_cw, uint32_t *to_q,
                              uint8_t *to_ab, void *stream);
-/* Lets launches of kern take `smem` bytes of dynamic shared memory.  The limit
- * is an attribute of the kernel on its device, which host threads with other
- * sizes share: it is only ever set to the most the device gives, so that no
- * call lowers it between another's setting and launch (which then fails).
- * Returns a cudaError_t. */
-int orbg_allow_smem(const void *kern, size_t smem);
+/* The grid of a persistent launch of kern: as many CTAs as are resident, or
+ * ctas_per_sm of them on each SM.  Lets launches of kern take the `smem` bytes
+ * of dynamic shared memory too: the limit is an attribute of the kernel on its
+ * device, which host threads with other sizes share, and is only ever set to
+ * the most the device gives, so that no call lowers it between another's
+ * setting and launch (which then fails).  Returns a cudaError_t. */
 int orbg_grid_for(const void *kern, int threads, size_t smem, int ctas_per_sm, int *grid_out);
 
 /* A named range on the NVTX timeline for the span of a scope (header-only

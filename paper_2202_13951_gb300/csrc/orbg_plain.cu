@@ -74,11 +74,10 @@ cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t
     if (grid > 0x7FFFFFFF)
         return cudaErrorInvalidValue;
     auto k = orbg_plain_kernel<K, W>;
-    if (smem > 47 * 1024) { /* with the static part past 48 KB, perhaps */
-        const int rc = orbg_allow_smem((const void *)k, smem);
-        if (rc != 0)
-            return (cudaError_t)rc;
-    }
+    int resident; /* not needed: the grid is the blocks' */
+    const int rc = orbg_grid_for((const void *)k, kPlainWarps * 32, smem, 0, &resident);
+    if (rc != 0)
+        return (cudaError_t)rc;
     k<<<(unsigned)grid, kPlainWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, bstride);
     return cudaGetLastError();
 }
