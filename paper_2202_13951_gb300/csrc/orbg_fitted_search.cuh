@@ -82,9 +82,22 @@ constexpr int kLeafRun = 3;                /* leaf siblings tested per step besi
  * resident warp and the CTAs wait for work.  Measured, us a call, three lines,
  * 100,000 BCH(127,113) and 20,000 CA-Polar[256,234] blocks, and 3,000 BCH
  * blocks of two lines: 256 1,415, 1,473 and 223; 512 1,361, 1,353 and 242;
- * 1024 1,340, 1,386 and 330. */
+ * 1024 1,340, 1,386 and 330.  (A pass tests about four times as many as
+ * the one before, from 70 on.)
+ * kSplitFew in a batch of so few positions that
+ * its longest search mostly ends there, where a CTA's takes 60 us more for a
+ * single block: up to kFewPositions, and past 14 parity bits, where a hit by
+ * chance does not end a long search, up to kFewBlocks.  One and three lines,
+ * us, 256 / 1024 / no handover: BCH 100 blocks 120, 122 / 94, 116 / 94, 115,
+ * 300 blocks 151, 154 / 95, 117 / 95, 116, 1,000 blocks 157, 166 / 234, 263 /
+ * 1,614, 860; a (256,244) code 10 blocks 162, 170 / 139, 148 / 140, 149, 300
+ * blocks 212, 210 / 315, 286 / 492, 526; CA-Polar[256,234] 10 blocks 89, 184 /
+ * 89, 124 / 89, 125, 100 blocks 199, 204 / 240, 267 / 1,891, 348. */
 constexpr uint32_t kSplit = 512;
 constexpr uint32_t kSplitSmall = 256;
+constexpr uint32_t kSplitFew = 1024;
+constexpr int64_t kFewPositions = 38912; /* 128 for two blocks an SM */
+constexpr int64_t kFewBlocks = 32;
 constexpr int32_t kNoHit = 0x7FFFFFFF;
 constexpr int kBlockRange = ORBG_BLOCK_RANGE; /* abandoned[] value: beyond the search range */
 
@@ -1180,6 +1193,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_kernel(
     uint32_t cap, uint32_t split, uint8_t *__restrict__ cw, uint32_t *__restrict__ q,
     uint8_t *__restrict__ ab, unsigned char *__restrict__ scratch)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory"); /* the launch before it is done */
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FsSmem<W> sm(smem + warp * fs_warp_bytes<W>());
@@ -1219,6 +1233,7 @@ __global__ void __launch_bounds__(kWarps * 32, 3) orbg_fitsearch_cta_kernel(
     uint32_t cap, uint8_t *__restrict__ cw, uint32_t *__restrict__ q,
     uint8_t *__restrict__ ab, unsigned char *__restrict__ scratch)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory"); /* the launch before it is done */
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ FsTeam team;
     __shared__ unsigned long long s_i;
@@ -1529,6 +1544,7 @@ __global__ void __launch_bounds__(kWarps * 32, K >= 4 ? 3 : 2) orbg_fitpair_kern
     uint8_t *__restrict__ ab, unsigned char *__restrict__ scratch)
 {
     typedef typename Syn<W>::T T;
+    asm volatile("griddepcontrol.wait;" ::: "memory"); /* the launch before it is done */
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ FsTeam team;
     __shared__ unsigned long long s_i;
@@ -1823,7 +1839,10 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
         rc = orbg_grid_for((const void *)k4, kWarps * 32, smem, 0, &g4);
     if (rc != 0)
         return rc;
-    const uint32_t most = B <= 2 * (int64_t)g2 * kWarps ? kSplitSmall : kSplit;
+    const bool few = B * code.n <= kFewPositions && (code.r <= 14 || B <= kFewBlocks);
+    const uint32_t most = few                                   ? kSplitFew
+                          : B <= 2 * (int64_t)g2 * kWarps ? kSplitSmall
+                                                          : kSplit;
     const uint32_t split = most < cap / 4u ? most : cap / 4u;
     const int64_t need = (B + kWarps - 1) / kWarps;
     if (g1 > need)
@@ -1842,14 +1861,28 @@ int launch_fitsearch(const OrbgDeviceCode &code, const float *llr, int64_t B, ui
                                       scratch);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return (int)e;
-    k2<<<g2, kWarps * 32, smem, st>>>(code, llr, B, cap, split, cw, q, ab, scratch);
-    if ((e = cudaGetLastError()) != cudaSuccess)
+    /* the further launches come on while the one before ends (each waits for
+     * it first): four in a row cost a batch of ten blocks 3 us more than three */
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kWarps * 32);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3((unsigned)g2);
+    cfg.dynamicSmemBytes = smem;
+    if ((e = cudaLaunchKernelEx(&cfg, k2, code, llr, B, cap, split, cw, q, ab, scratch)) !=
+        cudaSuccess)
         return (int)e;
-    k3<<<g3, kWarps * 32, fp_smem_bytes<K, W>(), st>>>(code, llr, B, cap, cw, q, ab, scratch);
-    if ((e = cudaGetLastError()) != cudaSuccess)
+    cfg.gridDim = dim3((unsigned)g3);
+    cfg.dynamicSmemBytes = fp_smem_bytes<K, W>();
+    if ((e = cudaLaunchKernelEx(&cfg, k3, code, llr, B, cap, cw, q, ab, scratch)) != cudaSuccess)
         return (int)e;
-    k4<<<g4, kWarps * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, scratch);
-    return (int)cudaGetLastError();
+    cfg.gridDim = dim3((unsigned)g4);
+    cfg.dynamicSmemBytes = smem;
+    return (int)cudaLaunchKernelEx(&cfg, k4, code, llr, B, cap, cw, q, ab, scratch);
 }
 
 }  // namespace orbg_fitsearch
