@@ -500,6 +500,7 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
         delete c;
         return ORBG_ELIMIT;
     }
+    orbg_few_rows(&tb, n, r);
     cudaError_t e;
     if ((e = cudaGetDevice(&c->device)) != cudaSuccess) {
         delete c;
@@ -562,6 +563,7 @@ int load_code(const uint8_t *mat, int kind, int n, int k, uint32_t max_query_cap
     std::copy(tb.cut_pairs, tb.cut_pairs + ORBG_CUTS, d.cut_pairs);
     std::copy(tb.cut_end, tb.cut_end + ORBG_CUTS, d.cut_end);
     d.nflat = tb.nflat;
+    d.long_end = tb.long_end;
     c->dev.max_cap = cap;
     c->dev.n = n;
     c->dev.r = r;

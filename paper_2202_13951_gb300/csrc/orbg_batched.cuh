@@ -228,7 +228,8 @@ struct Cut {
     uint32_t budget;
 };
 template <typename Kern>
-int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
+int cut_launch(Kern kern, const OrbgBatchedArgs &a, const OrbgDeviceCode *one,
+               uint32_t per_warp, Cut *c)
 {
     int dev = 0, sms = 1;
     cudaError_t e;
@@ -256,9 +257,15 @@ int cut_launch(Kern kern, const OrbgBatchedArgs &a, uint32_t per_warp, Cut *c)
     c->grab = (int)g;
     c->ahead = a.B > 4 * warps;
     c->budget = a.budget;
-    if (a.B <= 2 * warps)
+    /* a code of few parity bits (long flat table) ends most searches by its
+     * first band: it stays, and the others are few enough for phase 2 up to
+     * forty blocks a warp.  us, flat / first band / both: a (64,56) code, 5,000
+     * blocks 25 / 20 / 19, a (48,38) code, 60,000 43 / 42 / 53, 200,000 82 / 74 /
+     * 74, 400,000 140 / 142 / 133, a (256,246) code, 60,000 142 / 93 / 103 */
+    const bool few_rows = one != nullptr && one->long_end != 0u;
+    if (a.B <= 2 * warps && !few_rows)
         c->budget = a.budget < 1u ? a.budget : 1u;
-    else if (a.B <= 8 * warps)
+    else if (a.B <= (few_rows ? 40 : 8) * warps)
         c->budget = a.budget < ORBG_FLAT_MAX + 1u ? a.budget : ORBG_FLAT_MAX + 1u;
     const int64_t need = ((a.B + g - 1) / g + wpc - 1) / wpc;
     if (c->grid > need)
@@ -279,7 +286,7 @@ int launch_exact_t(const OrbgBatchedArgs &a, const OrbgScratch &ss, unsigned lon
     const uint32_t bstride = block_smem_bytes(nk, W);
     auto k1 = one ? orbg_batched_kernel<K, W, true> : orbg_batched_kernel<K, W, false>;
     Cut c;
-    const int rc = cut_launch(k1, a, warp_smem_bytes<K>(bstride), &c);
+    const int rc = cut_launch(k1, a, one, warp_smem_bytes<K>(bstride), &c);
     if (rc != 0)
         return rc;
     const bool sorted = blo >= 0;
@@ -367,7 +374,7 @@ cudaError_t launch_t(const OrbgBatchedArgs &a)
     } else {
         auto k1 = orbg_batched_kernel<KMAX, WMAX, true>;
         Cut c;
-        if ((rc = cut_launch(k1, a, warp_smem_bytes<KMAX>(bstride), &c)) != 0)
+        if ((rc = cut_launch(k1, a, a.code0, warp_smem_bytes<KMAX>(bstride), &c)) != 0)
             return (cudaError_t)rc;
         k1<<<c.grid, c.wpc * 32, (size_t)warp_smem_bytes<KMAX>(bstride) * c.wpc, st>>>(
             a.d_codes, a.ncodes, a.code_id, a.llr_off, a.llr, a.B, a.cap, c.budget, a.cw, a.cw_off,

@@ -933,6 +933,49 @@ __device__ __forceinline__ void write_flat_flips(const OrbgDeviceCode &code, uin
     }
 }
 
+/* The flat table past its first part, queries from .. code.long_end - 1 in
+ * order, by one warp: the first hit, or ORBG_NONE (as flat_test, an entry with
+ * no positions is none).  128 queries a step, their entries loaded while the
+ * step before is tested: step by step of 32 as the first part, whose ranks are
+ * found on the way, a query cost three times as much. */
+template <int W>
+__device__ __noinline__ uint32_t search_long_flat(const OrbgDeviceCode &code,
+                                                  const typename Syn<W>::T *h, const uint32_t *h0,
+                                                  typename Syn<W>::T s0, uint32_t from, int lane)
+{
+    const uint2 *flat = reinterpret_cast<const uint2 *>(code.flat) - 1; /* 1-based */
+    const uint32_t end = code.long_end, s0w = syn_key(s0);
+    uint2 e[4], next[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const uint32_t t = from + 32u * u + (uint32_t)lane;
+        next[u] = t < end ? __ldg(flat + t) : make_uint2(0u, 0u);
+    }
+#pragma unroll 1
+    for (uint32_t base = from; base < end; base += 128u) {
+        uint32_t mine = ORBG_NONE;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            e[u] = next[u];
+            const uint32_t t = base + 128u + 32u * u + (uint32_t)lane;
+            next[u] = t < end ? __ldg(flat + t) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int u = 3; u >= 0; u--) {
+            uint32_t v = s0w;
+#pragma unroll
+            for (int i = 0; i < ORBG_FLAT_POS; i++)
+                v ^= h0[flat_pos(e[u], i) - 1];
+            if (v == 0u && (W == 1 || flat_test<W>(h, h0, s0, e[u], 0)))
+                mine = base + 32u * u + (uint32_t)lane;
+        }
+        const uint32_t first = __reduce_min_sync(FULL_MASK, mine);
+        if (first != ORBG_NONE)
+            return first;
+    }
+    return ORBG_NONE;
+}
+
 /* ------------------------------------------------ one warp, one block */
 
 /*
@@ -941,9 +984,10 @@ __device__ __forceinline__ void write_flat_flips(const OrbgDeviceCode &code, uin
  * `budget`.  A block still open after them is left: its index is
  * appended to heavy[] for decode_block_cta, with its reliability order and
  * starting syndrome in the handover record of the same slot when one is free
- * (hand_cap; bit 63 of the heavy[] entry says so); with heavy NULL the
- * caller takes it up.  list: key_list_bytes<K>() bytes.  Its codeword bytes hold the hard decision by then.
- * Returns whether the block was finished.  LS: llr
+ * (hand_cap; bit 63 of the heavy[] entry says so); with heavy NULL hand is
+ * its record and the caller takes it up.  Its codeword bytes hold the hard
+ * decision by then.  list: key_list_bytes<K>() bytes.  Returns whether the
+ * block was finished.  LS: llr
  * points into shared memory (the batched kernel stages it there).
  */
 template <int K, int W, bool LS = false>
@@ -1004,10 +1048,6 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     if (cap <= code.nflat)
                         break;
                     tested = code.nflat + 1u;
-                    uint4 *clear = reinterpret_cast<uint4 *>(filter);
-                    for (uint32_t i = (uint32_t)lane; i < kWarpFilterBytes / 16u; i += 32u)
-                        clear[i] = make_uint4(0u, 0u, 0u, 0u);
-                    __syncwarp();
                 }
                 for (k++; k < ORBG_BANDS && code.band_end[k] <= tested;)
                     k++;
@@ -1017,8 +1057,6 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     upto = (int)code.band_ranks[k] + 1;
                 } else {
                     done = false;
-                    if (heavy == nullptr)
-                        break;
                     k = ORBG_BANDS;
                     upto = (int)code.ranks + 1; /* the handover record */
                 }
@@ -1054,7 +1092,21 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     break;
                 }
                 base += 32u;
+            } else if (k == 0 && code.long_end != 0u) {
+                const uint32_t t = search_long_flat<W>(code, sm.h, sm.h0, s0, tested, lane);
+                if (t != ORBG_NONE) {
+                    hit.t = t;
+                    flat_mine = lane == 0;
+                    break;
+                }
+                tested = code.long_end;
             } else if (k < ORBG_BANDS) {
+                if (np == 0u) {
+                    uint4 *clear = reinterpret_cast<uint4 *>(filter);
+                    for (uint32_t i = (uint32_t)lane; i < kWarpFilterBytes / 16u; i += 32u)
+                        clear[i] = make_uint4(0u, 0u, 0u, 0u);
+                    __syncwarp();
+                }
                 hit = warp_best(single_hits<W>(code, sm.h, s0, (uint32_t)lane, 32u,
                                                code.band_ranks[k]));
                 hit = search_band<W>(code, sm, s0, cap, k, np, filter, lane, hit);
@@ -1081,6 +1133,11 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
             }
             if (lane == 0)
                 heavy[slot] = block_index | (keep ? 1ull << 63 : 0ull);
+        } else {
+            for (int e = lane; e < (int)code.ranks; e += 32)
+                hand[e] = sm.pi[e];
+            if (lane == 0)
+                *reinterpret_cast<T *>(hand + 256) = s0;
         }
         __syncwarp();
         return false;
@@ -1102,9 +1159,8 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
 }
 
 /* The block loaded and sorted by one warp (rare: a block past phase 1's
- * handover records, and the plain form's open ones): order, permuted columns
- * and *s0.  Returns 0, 1 for a code word, 2 for a NaN
- * block. */
+ * handover records): order, permuted columns and *s0.  Returns 0, 1 for a code
+ * word, 2 for a NaN block. */
 template <int K, int W>
 __device__ __noinline__ int load_and_sort_k(const OrbgDeviceCode &code, const float *llr,
                                             unsigned char *bsm, int lane,
@@ -1256,7 +1312,7 @@ __device__ __noinline__ PairHit scan_pairs(const OrbgDeviceCode &code, const Blo
 
 /*
  * All warps of the CTA decode one block whose hard decision is in cw_out
- * already (phase 1 wrote it).  Its order comes from phase 1's
+ * already (its warp wrote it).  Its order comes from the
  * handover record, or warp 0 loads and sorts; all threads then build the
  * subset tables of the light positions and the filter of the block's pairs
  * (several in turn for an order of more than kPairChunk pairs: its cuts, then

@@ -77,6 +77,19 @@
 #define ORBG_FLAT_MAX 256
 #define ORBG_FLAT_POS 7
 #define ORBG_FLAT_RANKS 31
+/* Codes of few parity bits, whose searches are short.  Up to ORBG_FEW_ROWS
+ * phase 2 takes at most ORBG_FEW_CHUNK pairs at a time, so that the plain form's
+ * CTAs of four warps are not held apart by the pair set's room; up to
+ * ORBG_LONG_FLAT_ROWS they go through the first band pattern by pattern (the
+ * flat table goes on to its end), since most of a band's look-ups would hit by
+ * chance.  Plain form, us, as other codes / so: (40,32), 3,000 and 60,000
+ * blocks at 4.5-7 dB, 14.8 and 34 / 9.2 and 27; (64,54), 60,000 blocks 52 / 44,
+ * 50,000 at 2-3 dB 172 / 119; with the long table alone 9.5 and 29.7, 48, 132;
+ * the chunk and four warps at 60,000 blocks, (64,51) 51 / 42, (128,116) 70 / 61
+ * (patterns one by one, 40 to 56, 68 and 104). */
+#define ORBG_LONG_FLAT_ROWS 10
+#define ORBG_FEW_ROWS 13
+#define ORBG_FEW_CHUNK 1023
 
 /* What a kernel needs of one code (passed by value or from a device array). */
 struct OrbgDeviceCode {
@@ -112,8 +125,9 @@ struct OrbgDeviceCode {
     uint32_t scan;               /* phase 2 holds the prefixes and goes through the pairs: the
                                   * first cut_pairs[0] alone, which covers the queries before
                                   * cut_end[0], then the first cut_pairs[1] with every prefix */
-    const uint32_t *flat;        /* [2 * nflat] flat-table patterns, 8 bytes each */
-    uint32_t nflat;
+    const uint32_t *flat;        /* flat-table patterns, 8 bytes each: the first nflat, and up to
+                                  * query long_end - 1 if that is not 0 */
+    uint32_t nflat, long_end;
     uint32_t max_cap;
     int32_t n;
     int32_t r;
@@ -132,7 +146,7 @@ struct OrbgTables {
     std::vector<uint32_t> gmeta, pmeta, start, single;
     uint8_t light[16] = {};
     std::vector<uint8_t> flat;           /* 8 bytes per pattern */
-    uint32_t npre = 0, nflat = 0;
+    uint32_t npre = 0, nflat = 0, long_end = 0;
     uint32_t band_pairs[ORBG_BANDS] = {}, band_pre[ORBG_BANDS] = {};
     uint32_t band_ranks[ORBG_BANDS] = {}, band_end[ORBG_BANDS] = {};
     uint32_t ranks = 0, chunk = 0, cut_pairs[ORBG_CUTS] = {}, cut_end[ORBG_CUTS] = {};
@@ -143,6 +157,10 @@ struct OrbgTables {
  * (one-line full ORBGRAND; J0 = 0, beta = 1 is basic ORBGRAND). */
 #define ORBG_MAX_LINE 1024
 int orbg_build_tables(int n, uint64_t cap, OrbgTables *out, long J0 = 0, long beta = 1);
+/* What codes of few parity bits r take instead (ORBG_FEW_ROWS,
+ * ORBG_LONG_FLAT_ROWS): smaller chunks of pairs, and the flat table over the
+ * first band too, if its patterns fit it. */
+void orbg_few_rows(OrbgTables *tb, int n, int r);
 /* The m-segment model of Eq. relest_seg: segment i = 1..m covers the
  * sorted positions I[i-1] < j <= I[i] (I[0] = 0, I[m] = n) and position j
  * weighs J[i-1] + beta[i-1] (j - I[i-1]); beta >= 1, J[i-1] >= -beta[i-1]. */

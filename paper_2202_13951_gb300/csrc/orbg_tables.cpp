@@ -580,6 +580,40 @@ int orbg_build_tables_model(int n, uint64_t cap, const OrbgModel &md, OrbgTables
     return build_order(n, rho, patterns, Rmax, true, out);
 }
 
+void orbg_few_rows(OrbgTables *tb, int n, int r)
+{
+    /* phase 2: fewer pairs at a time, two cuts as for an order of many */
+    if (r <= ORBG_FEW_ROWS && !tb->scan && tb->chunk > ORBG_FEW_CHUNK) {
+        tb->chunk = ORBG_FEW_CHUNK;
+        const uint32_t to[ORBG_CUTS] = {ORBG_BAND2_PAIRS, ORBG_FEW_CHUNK};
+        for (int k = 0; k < ORBG_CUTS; k++) {
+            uint32_t np = to[k];
+            while (np > 0 && tb->pgroup[np] == tb->pgroup[np - 1])
+                np--;
+            tb->cut_pairs[k] = np;
+            /* the empty prefix's first index of the group: the first pattern
+             * that takes one of its pairs */
+            tb->cut_end[k] = tb->start[tb->pgroup[np]];
+        }
+    }
+    const uint32_t end = tb->band_end[0];
+    if (r > ORBG_LONG_FLAT_ROWS || end <= tb->nflat + 1)
+        return;
+    std::vector<uint8_t> more((size_t)(end - 1 - tb->nflat) * 8, 0);
+    bool fits = true;
+    orbg_expand_tables(*tb, n, end - 1, [&](uint32_t t, const int *v, int w) {
+        fits &= w <= ORBG_FLAT_POS && (w == 0 || v[w - 1] <= 255);
+        if (t > tb->nflat && fits)
+            for (int i = 0; i < w; i++)
+                more[(size_t)(t - 1 - tb->nflat) * 8 + i] = (uint8_t)v[i];
+    });
+    if (!fits)
+        return;
+    tb->flat.resize((size_t)tb->nflat * 8);
+    tb->flat.insert(tb->flat.end(), more.begin(), more.end());
+    tb->long_end = end;
+}
+
 /* Calls f(t, positions, w) for every pattern of index t <= count: positions
  * 1-based, ascending.  Expanded from the tables the kernels read. */
 void orbg_expand_tables(const OrbgTables &tb, int n, uint64_t count,

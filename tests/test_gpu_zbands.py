@@ -1,7 +1,8 @@
 """Phase 1's two bands, and its hand-over after each of them, against the
 oracle.  A batch of at most two blocks a resident warp hands its blocks over
-after the flat table and one of at most eight after the first band, whatever
-the budget: here one warp an SM is resident and the batches are larger.
+after the flat table and one of at most eight (forty with few parity bits)
+after the first band, whatever the budget: here one warp an SM is resident and
+the batches are larger.
 Whole numbers: equal or wrong."""
 import numpy as np
 import pytest
@@ -62,7 +63,8 @@ def test_bands(orbg, name):  # noqa: F811
     cs = orbg.CodeSet([orbg.Code(H, max_query_cap=cap, line=line, model=model)])
     warps = torch.cuda.get_device_properties(0).multi_processor_count
     few = TILE * (2 * warps // TILE + 1)   # past two blocks a warp
-    many = TILE * (8 * warps // TILE + 1)  # past eight
+    past = 40 if H.shape[0] <= 10 else 8
+    many = TILE * (past * warps // TILE + 1)  # past that
     assert 2 * warps < few <= 8 * warps < many
     for B, budget in ((few, 1 << 25), (many, 1), (many, 1000), (many, 1 << 25)):
         orbg.orbg_codeset_set_tuning(cs.handle, orbg.OrbgTuning(1, 1, 4, budget, 8))
