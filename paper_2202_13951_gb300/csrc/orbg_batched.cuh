@@ -246,11 +246,15 @@ int cut_launch(Kern kern, const OrbgBatchedArgs &a, const OrbgDeviceCode *one,
         return rc;
     const int64_t warps = (int64_t)c->grid * wpc;
     int64_t g = a.grab < 1 ? 1 : a.grab;
-    /* eight grabs a warp or more; two for one code of up to 16 parity bits,
-     * whose blocks search alike and are short beside a grab's wait (60,000
-     * blocks of a (64,52) code: 90 -> 67 us; three serving codes, 50,000
-     * blocks, two 334, eight 299) */
-    const int64_t fair = a.B / ((a.code0 && a.code0->r <= 16 ? 2 : 8) * warps);
+    /* eight grabs a warp or more (three serving codes, 50,000 blocks, two 334
+     * us, eight 299); one code takes longer grabs, since its blocks search
+     * alike: two a warp up to 16 parity bits, whose blocks are short beside a
+     * grab's wait (60,000 blocks of a (64,52) code: 90 -> 67), else eight
+     * rounded in their favour (50,000 blocks of a (200,180) code at 8-9 dB, one
+     * at a time 47, two 31) */
+    const int64_t fair = !a.code0            ? a.B / (8 * warps)
+                         : a.code0->r <= 16 ? a.B / (2 * warps)
+                                            : (a.B + 8 * warps - 1) / (8 * warps);
     if (g > fair)
         g = fair > 0 ? fair : 1;
     c->wpc = wpc;
