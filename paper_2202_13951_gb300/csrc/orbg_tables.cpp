@@ -65,28 +65,33 @@ struct Order {
         long all = 0;
         for (long w : x)
             all += w;
-        const long top = std::min(all, kDenseMax);
-        std::vector<uint64_t> c((size_t)top + 1, 0);
-        c[0] = 1;
-        long reach = 0;
-        for (long w : x) {
-            reach = std::min(top, reach + w);
-            for (long R = reach; R >= w; R--)
-                c[(size_t)R] = std::min(kCountMax, c[(size_t)R] + c[(size_t)(R - w)]);
-        }
-        uint64_t sum = 0;
-        long last = 0;
-        for (long R = 0; R <= top; R++) {
-            if (!c[(size_t)R])
-                continue;
-            sum = std::min(kCountMax, sum + c[(size_t)R]);
-            last = R;
-            if (sum >= cap || (top == all && R == all)) {
-                *patterns = sum;
-                return last;
+        const long dense = std::min(all, kDenseMax);
+        /* few weights first: a cap of 1,000 reaches weight 26 */
+        for (long top = std::min(dense, 64l);; top = std::min(dense, 4 * top)) {
+            std::vector<uint64_t> c((size_t)top + 1, 0);
+            c[0] = 1;
+            long reach = 0;
+            for (long w : x) {
+                reach = std::min(top, reach + w);
+                for (long R = reach; R >= w; R--)
+                    c[(size_t)R] = std::min(kCountMax, c[(size_t)R] + c[(size_t)(R - w)]);
             }
+            uint64_t sum = 0;
+            long last = 0;
+            for (long R = 0; R <= top; R++) {
+                if (!c[(size_t)R])
+                    continue;
+                sum = std::min(kCountMax, sum + c[(size_t)R]);
+                last = R;
+                if (sum >= cap || (top == all && R == all)) {
+                    *patterns = sum;
+                    return last;
+                }
+            }
+            if (top == dense)
+                break;
         }
-        long lo = top + 1, hi = all; /* the depth is in [lo, hi] */
+        long lo = dense + 1, hi = all; /* the depth is in [lo, hi] */
         while (lo < hi) {
             const long mid = lo + (hi - lo) / 2;
             if (1 + count_from(0, mid, cap) >= cap)
@@ -113,8 +118,11 @@ struct TableBuilder {
     void make_pairs()
     {
         std::vector<std::pair<long, uint32_t>> v;
+        std::vector<long> least_from((size_t)n + 2, INT64_MAX / 4); /* over positions >= b */
+        for (int b = n; b >= 1; b--)
+            least_from[(size_t)b] = std::min(least_from[(size_t)b + 1], rho[(size_t)b]);
         for (int a = 1; a < n; a++)
-            for (int b = a + 1; b <= n; b++)
+            for (int b = a + 1; b <= n && rho[(size_t)a] + least_from[(size_t)b] <= Rmax; b++)
                 if (rho[(size_t)a] + rho[(size_t)b] <= Rmax)
                     v.push_back({rho[(size_t)a] + rho[(size_t)b],
                                  (uint32_t)(a - 1) << 8 | (uint32_t)(b - 1)});
