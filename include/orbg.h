@@ -274,12 +274,19 @@ ORBG_API int orbg_decode_batched_noalloc(const orbg_codeset *set,
  *   ctas_per_sm     phase 1: resident CTAs per SM (0 = as many as fit)
  *   blocks_per_grab phase 1: blocks a warp takes per work-queue atomic
  *                   (1..1024; 0 = 4), fewer in a batch of less than eight
- *                   grabs a warp; likewise warps_per_cta in one of few blocks
+ *                   grabs a warp (with one code of up to 16 parity bits, two);
+ *                   likewise warps_per_cta in one of few blocks
  *   warp_budget     phase 1: a single warp searches its block's order in bands
  *                   (for basic ORBGRAND up to query 256, 2,375 and 16,857) and
  *                   hands the block to phase 2 before a band that starts past
  *                   this query (0 = 16384), or after the last band, whatever
- *                   the budget; phase 2 runs in every call
+ *                   the budget; phase 2 runs in every call.  Small batches
+ *                   take less than they are given: up to two blocks a resident
+ *                   warp of a launch every search past the flat table goes to
+ *                   phase 2, up to eight every one past the first band (with
+ *                   one code of up to ten parity bits, past the first band up
+ *                   to forty).  The blocks counted are the whole call's, also
+ *                   where it launches per variant or per code
  *   heavy_warps     phase 2: warps per CTA sharing one block (1..16; 0 = 8)
  * None of these change any result.
  */

@@ -212,17 +212,18 @@ template <int K> constexpr uint32_t warp_smem_bytes(uint32_t bstride)
 
 /* How a phase-1 launch of B blocks is cut: warps per CTA, queue slots per
  * grab, whether warps take blocks ahead, the grid, and how far a warp takes
- * its block.  A batch of few blocks
- * is spread over the SMs and shared out block by block: with the tuned grab
- * of four, 257 blocks of BCH(127,113) ran four after another on 65 warps of
- * nine SMs.  Measured with it and without: three serving codes, 8,191 blocks,
- * 170 -> 121 us.  While phase 2's CTAs are not all busy, a block goes there
- * early: up to two blocks a resident warp after the flat table, up to eight
- * after the first band.  us, flat / first band / both bands: BCH(127,113),
- * 257 blocks 34 / 38 / 49, 100,000 186 / 133 / 148, 400,000 632 / 391 / 350;
- * three serving codes, 8,191 blocks 103 / 105 / 122; four mixed codes, 33,000
- * blocks 197 / 175 / 205, 100,000 460 / 380 / 361 (3,648 warps; 4,864 for the
- * one code). */
+ * its block.  A batch of few blocks is spread over the SMs and shared out
+ * block by block: with the tuned grab of four, 257 blocks of BCH(127,113) ran
+ * four after another on 65 warps of nine SMs.  Measured with it and without:
+ * three serving codes, 8,191 blocks, 170 -> 121 us.  While phase 2's CTAs are
+ * not all busy, a block goes there early: up to two blocks a resident warp
+ * after the flat table, up to eight after the first band, past that after
+ * both.  us, flat / first band / both: three serving codes, 8,191 blocks (2 a
+ * warp) 103 / 105 / 122; BCH(127,113), 257 blocks 34 / 38 / 49; four mixed
+ * codes, 33,000 blocks (9) 197 / 175 / 205, 100,000 (27) 460 / 380 / 361;
+ * BCH(127,113), 100,000 (21) 189 / 137 / 143, 400,000 (82) 645 / 406 / 345.
+ * Both bands pay from 27 and 82 blocks a warp on; where between nine and those
+ * is not measured, and just above eight the rule is the slower choice. */
 struct Cut {
     int wpc, grab, ahead, grid;
     uint32_t budget;

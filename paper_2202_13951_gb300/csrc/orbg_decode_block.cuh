@@ -500,8 +500,9 @@ __device__ __forceinline__ void make_keys(const float *__restrict__ llr, int n, 
  * hash set alone a warp step waited for its longest probe sequence (80 warp
  * instructions a step of 32 look-ups, 45 with the filter).  Both hashes are
  * multiplicative (the high bits of the key times an odd constant, the first
- * near 2^32 / golden ratio): the low bits of one product would repeat where
- * the code's columns differ in few rows.
+ * near 2^32 / golden ratio, the second the first multiplier of MurmurHash3's
+ * final mix, A. Appleby): the low bits of one product would repeat where the
+ * code's columns differ in few rows.
  */
 __device__ __forceinline__ uint32_t pair_hash(uint32_t v) { return v * 0x9E3779B1u; }
 __device__ __forceinline__ void filter_add(uint32_t *filter, uint32_t bits, uint32_t v)

@@ -210,9 +210,10 @@ struct OrbgVariants {
 /* A mixed-code call of at least this many blocks per code of such a set
  * launches phase 1 per code, each with its descriptor in the kernel's
  * parameters, and not per variant with descriptors read from memory block by
- * block (four codes, 1,000,000 blocks: 2,392 -> 2,216 us); a smaller one pays
- * more for the launches and their ends (four codes of one variant, 100,003
- * blocks: 685 -> 712 us). */
+ * block.  Measured at 250,000 blocks a code (four codes of three variants,
+ * 2,392 -> 2,216 us) and at 25,000 (four of one variant, 685 -> 712: the
+ * launches and their ends cost more); the line lies between the two, near
+ * their geometric mean. */
 #define ORBG_PER_CODE_BLOCKS 65536
 struct OrbgBatchedArgs {
     const OrbgDeviceCode *d_codes;

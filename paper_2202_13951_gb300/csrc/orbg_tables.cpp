@@ -181,7 +181,9 @@ struct TableBuilder {
 
     /* A model's order is limited to patterns of 20 positions, and of 22 where
      * the last two can be written as a + j da, b - j db of one run of
-     * patterns with bytes for a and b.  Is any pattern outside that? */
+     * patterns with bytes for a and b.  Is any pattern outside that?  (The
+     * tables here have no such runs and would hold these patterns; the orders
+     * that orbg_load_code_model has always refused stay refused.) */
     bool past_model_limit() const
     {
         for (const Prefix &p : pre) {
