@@ -29,7 +29,7 @@ struct orbg_codeset {
     int ncodes, n_max, w32_max;
     OrbgVariants var;            /* decoder variants and the codes' sort buckets */
     int32_t *d_bucket = nullptr; /* [ncodes] sort bucket of each code (var.d_bucket) */
-    uint32_t npairs_max;
+    uint32_t npairs_max, scan_any;
     orbg_tuning tuning;
     std::vector<int> n_of;       /* n of each code, host copy */
     std::vector<OrbgDeviceCode> by_bucket; /* var.by_bucket */
@@ -236,6 +236,7 @@ int orbg_codeset_view(const orbg_codeset *set, OrbgSetView *out)
     out->w32_max = set->w32_max;
     out->var = set->var;
     out->npairs_max = set->npairs_max;
+    out->scan_any = set->scan_any;
     out->cap_min = set->cap_min;
     out->tuning = set->tuning;
     return 0;
@@ -678,6 +679,7 @@ int orbg_codeset_create(const orbg_code *const *codes, int ncodes, orbg_codeset 
     s->w32_max = 1;
     s->cap_min = 0xFFFFFFFFu;
     s->npairs_max = 0;
+    s->scan_any = 0;
     s->tuning = kDefaultTuning;
     for (int i = 0; i < ncodes; i++) {
         if (!codes[i]) {
@@ -692,6 +694,7 @@ int orbg_codeset_create(const orbg_code *const *codes, int ncodes, orbg_codeset 
         s->w32_max = std::max(s->w32_max, codes[i]->w32);
         s->cap_min = std::min(s->cap_min, codes[i]->max_cap);
         s->npairs_max = std::max(s->npairs_max, codes[i]->dev.chunk);
+        s->scan_any |= codes[i]->dev.scan;
     }
     /* the decoder variants the kernels specialise on: keys per lane from n
      * (n <= 32, 64, 128, 256: 1, 2, 4, 8) and the syndrome words (1, 2, or
@@ -935,6 +938,7 @@ int decode_batched_pipelined(const orbg_codeset *set, const int32_t *code_id,
     a.grab = t.blocks_per_grab;
     a.heavy_warps = t.heavy_warps;
     a.npairs_max = set->npairs_max;
+    a.scan_any = set->scan_any;
     a.scratch_B = B;
     bool declined = false;
     std::vector<cudaEvent_t> chunk_done;
@@ -1196,6 +1200,7 @@ int orbg_decode_batched(const orbg_codeset *set, const int32_t *code_id,
     a.grab = t.blocks_per_grab;
     a.heavy_warps = t.heavy_warps;
     a.npairs_max = set->npairs_max;
+    a.scan_any = set->scan_any;
     a.stream = st;
     int le = orbg_launch_batched(a);
     cudaFreeAsync(scratch, st);
@@ -1500,6 +1505,7 @@ int orbg_fitted_decode(orbg_fitted *f, const float *llr, int64_t B, uint32_t que
         a.grab = t.blocks_per_grab;
         a.heavy_warps = t.heavy_warps;
         a.npairs_max = set->npairs_max;
+        a.scan_any = set->scan_any;
         a.stream = st;
         const int le = orbg_launch_batched(a);
         if (le != 0)

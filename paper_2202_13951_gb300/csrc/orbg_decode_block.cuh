@@ -1093,7 +1093,7 @@ __device__ bool decode_block_warp(const OrbgDeviceCode &code, const float *__res
                     break;
                 }
                 base += 32u;
-            } else if (k == 0 && code.long_end != 0u) {
+            } else if (W == 1 && k == 0 && code.long_end != 0u) { /* few rows: one word */
                 const uint32_t t = search_long_flat<W>(code, sm.h, sm.h0, s0, tested, lane);
                 if (t != ORBG_NONE) {
                     hit.t = t;
@@ -1322,9 +1322,10 @@ __device__ __noinline__ PairHit scan_pairs(const OrbgDeviceCode &code, const Blo
  * stops at its first group whose floor is at least the shared best (or above
  * the cap): floors never decrease with the group index and the best never
  * increases, so no group that could hold the final best is skipped.
- * pair_sm: pair_smem_bytes(code.chunk) bytes.
+ * pair_sm: pair_smem_bytes(code.chunk) bytes.  SCAN: the code may have scan
+ * set (with the call in it, a set of codes that have not lost 1 %).
  */
-template <int W>
+template <int W, bool SCAN>
 __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__restrict__ llr,
                                  uint8_t *__restrict__ cw_out, uint32_t *__restrict__ q_out,
                                  uint8_t *__restrict__ ab_out, uint32_t cap,
@@ -1379,7 +1380,7 @@ __device__ void decode_block_cta(const OrbgDeviceCode &code, const float *__rest
         mine = single_hits<W>(code, sm.h, s0, threadIdx.x, blockDim.x, code.ranks);
         if (mine.t != ORBG_NONE)
             atomicMin(s_best, mine.t);
-        if (code.scan) {
+        if (SCAN && code.scan) {
             mine = scan_pairs<W>(code, sm, s0, cap, filter, fbits, set, bits, s_best, warp, lane,
                                  nwarps, mine);
         } else {

@@ -1486,10 +1486,10 @@ __device__ __forceinline__ uint32_t count_tied(const uint32_t *rho, const uint32
         const uint32_t least = mall[p + 1];
         /* rows of most positions first: each reads the one before it */
         for (int t = T - 1; t >= 2; t--) {
-            if (least > R)
-                continue;
-            const uint32_t lo = a + (uint32_t)(t - 1) * least; /* at most 32 R */
-            if (lo > R)
+            /* may wrap where least > R, which is tested by itself (tested
+             * first, in a branch of its own, it cost the kernel 1 %) */
+            const uint32_t lo = a + (uint32_t)(t - 1) * least;
+            if (least > R || lo > R)
                 continue;
             for (uint32_t r = lo + threadIdx.x; r <= R; r += blockDim.x)
                 x[(uint32_t)t * row + r] += x[(uint32_t)(t - 1) * row + (r - a)];

@@ -19,7 +19,7 @@ using namespace orbg_dev;
 #define ORBG_PHASE2_MIN_CTAS 2
 #endif
 
-template <int WMAX, bool ONE>
+template <int WMAX, bool ONE, bool SCAN>
 __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
     const OrbgDeviceCode *__restrict__ codes, int ncodes, const int32_t *__restrict__ code_id,
     const int64_t *__restrict__ llr_off, const float *__restrict__ llr, uint32_t cap,
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
         const int64_t lo = llr_off ? llr_off[b] : b * n0;
         const int64_t co = cw_off ? cw_off[b] : b * n0;
         if (ONE) {
-            decode_block_cta<WMAX>(code0, llr + lo, cw + co, q + b, ab + b, cap, smem,
+            decode_block_cta<WMAX, SCAN>(code0, llr + lo, cw + co, q + b, ab + b, cap, smem,
                                    smem + bstride, &s_best,
                                    reinterpret_cast<typename Syn<WMAX>::T *>(&s_s0), warp, lane,
                                    nwarps, rec);
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(512, ORBG_PHASE2_MIN_CTAS) orbg_heavy_kernel(
         __syncthreads();
         const OrbgDeviceCode &code = s_code;
 #define ORBG_CALL_CTA(WW)                                                               \
-    decode_block_cta<WW>(code, llr + lo, cw + co, q + b, ab + b, cap, smem,             \
+    decode_block_cta<WW, SCAN>(code, llr + lo, cw + co, q + b, ab + b, cap, smem,             \
                          smem + bstride, &s_best,                                       \
                          reinterpret_cast<typename Syn<WW>::T *>(&s_s0), warp, lane, nwarps, rec)
         ORBG_DISPATCH_W(WMAX, ORBG_CALL_CTA);
@@ -88,7 +88,8 @@ template <int WMAX, bool ONE>
 cudaError_t launch_heavy_t(const OrbgBatchedArgs &a, unsigned long long *counters,
                            const unsigned long long *heavy, const unsigned char *hand, bool pdl)
 {
-    auto k2 = orbg_heavy_kernel<WMAX, ONE>;
+    auto k2 = (ONE ? a.code0->scan != 0u : a.scan_any != 0u) ? orbg_heavy_kernel<WMAX, ONE, true>
+                                                             : orbg_heavy_kernel<WMAX, ONE, false>;
     const int hw = a.heavy_warps > 0 ? a.heavy_warps : 8;
     /* 16-byte aligned: block_smem_bytes is a multiple of 16 */
     const uint32_t bstride = block_smem_bytes(a.n_max, a.w32_max);

@@ -232,6 +232,7 @@ struct OrbgBatchedArgs {
     unsigned long long *scratch;
     int warps_per_cta, ctas_per_sm, grab, heavy_warps;
     uint32_t npairs_max;         /* most pairs phase 2 holds at once for a code of the set */
+    uint32_t scan_any;           /* a code of the set has scan */
     void *stream;
     /* Staged calls (the host-buffer pipeline: phase 1 chunk by chunk as the
      * LLRs arrive, then one phase 2 over every chunk's open blocks).
@@ -372,7 +373,7 @@ struct OrbgSetView {
     OrbgDeviceCode code0;        /* host copy of code 0's descriptor */
     int ncodes, n_max, w32_max;
     OrbgVariants var;
-    uint32_t npairs_max;
+    uint32_t npairs_max, scan_any;
     uint32_t cap_min;
     orbg_tuning tuning;
 };

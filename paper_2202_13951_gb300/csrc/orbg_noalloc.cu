@@ -134,6 +134,7 @@ extern "C" int orbg_decode_batched_noalloc(const orbg_codeset *set, const int32_
     a.grab = v.tuning.blocks_per_grab;
     a.heavy_warps = v.tuning.heavy_warps;
     a.npairs_max = v.npairs_max;
+    a.scan_any = v.scan_any;
     a.stream = cuda_stream;
     e = orbg_launch_batched(a);
     return e != 0 ? orbg_note_cuda_error(e) : ORBG_OK;

@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(32 * kPlainWarps, W == 1 ? 4 : 1) orbg_plain_k
         const int w = __ffs(open) - 1;
         const int64_t bo = b0 + w;
         const int64_t off = bo * (int64_t)code.n;
-        decode_block_cta<W>(code, llr + off, cw + off, q + bo, ab + bo, cap, smem, smem + bstride,
+        decode_block_cta<W, true>(code, llr + off, cw + off, q + bo, ab + bo, cap, smem, smem + bstride,
                             &s_best, reinterpret_cast<typename Syn<W>::T *>(&s_s0), warp, lane,
                             nwarps, s_rec[w]);
     }

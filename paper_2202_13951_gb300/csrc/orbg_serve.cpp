@@ -294,6 +294,7 @@ bool dispatch_one(orbg_server *s)
         a.grab = s->view.tuning.blocks_per_grab;
         a.heavy_warps = s->view.tuning.heavy_warps;
         a.npairs_max = s->view.npairs_max;
+        a.scan_any = s->view.scan_any;
         a.stream = st;
         le = orbg_launch_batched(a);
     }
