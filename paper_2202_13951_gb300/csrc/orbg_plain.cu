@@ -84,10 +84,12 @@ cudaError_t launch_plain_t(const OrbgDeviceCode &code, const float *llr, int64_t
     if (grid > 0x7FFFFFFF)
         return cudaErrorInvalidValue;
     auto k = orbg_plain_kernel<K, W>;
-    int resident; /* not needed: the grid is the blocks' */
-    const int rc = orbg_grid_for((const void *)k, nw * 32, smem, 0, &resident);
-    if (rc != 0)
-        return (cudaError_t)rc;
+    if (smem > 45 * 1024) { /* with the static part past 48 KB, perhaps */
+        int resident;       /* not needed: the grid is the blocks' */
+        const int rc = orbg_grid_for((const void *)k, nw * 32, smem, 0, &resident);
+        if (rc != 0)
+            return (cudaError_t)rc;
+    }
     k<<<(unsigned)grid, nw * 32, smem, st>>>(code, llr, B, cap, cw, q, ab, bstride);
     return cudaGetLastError();
 }
