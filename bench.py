@@ -1096,10 +1096,10 @@ PROFILES = {
     },
     "bch/plain/basic": {
         "kernels": "plain",
-        "digest": "c0d26dfae9aaa035da2a2dc44b6c0ba71b326e2751a8360eb7762c46f19f01ff",
-        # 164.2 MB on the captured case, x 1.4286
-        "traffic_bytes_per_step": 234.6e6,
-        "issued_frac": 0.341,
+        "digest": "a3a72d88c65adef6cafea4f3511654bbc5bf58f783b2c65d99ace3da2574cc0f",
+        # 164.1 MB on the captured case, x 1.4286
+        "traffic_bytes_per_step": 234.4e6,
+        "issued_frac": 0.342,
         "source": "profiles/bench_workloads_traffic_alu.md",
     },
     "bch/batched/line": {
